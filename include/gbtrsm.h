@@ -96,7 +96,16 @@ typedef struct gb_plan {
  *  11 ldb >= max(1, m)
  *  12 stream
  * The plan is picked by the planner (cost model if loaded, else the
- * built-in default).  Asynchronous.
+ * built-in default).  Asynchronous.  Off-diagonal updates of 64 (FP64) / 128
+ * (FP32) products per entry or more run on the tensor cores, by exact
+ * products of 8-bit digits whose error is below that of the CUDA-core sum
+ * (input for which it would not be is found on the device and taken by the
+ * CUDA cores).  Their work space (14 (M + N) K bytes FP64, 6 (M + N) K FP32
+ * for the largest update, at most about 2 GiB) is taken from and given back
+ * to a stream-ordered pool of the library, which keeps up to 2.5 GiB
+ * (gb_mixed_workspace_release returns it); while `stream` is being captured,
+ * or when the memory is not to be had, the CUDA-core update is taken
+ * instead, which needs none.
  */
 int gb_dtrsm(int side, int uplo, int trans, int diag, int64_t m, int64_t n,
              double alpha, const double *A, int64_t lda, double *B,
@@ -258,7 +267,8 @@ int gb_set_lookahead(int on);
  * b.low -= L.mid x.up, with many right-hand sides): C = alpha*C - A*B with
  * A (M x K, lda), B (K x N, ldb) and C (M x N, ldc) column-major device
  * arrays of FP64 (dtype 0) or FP32 (dtype 1), alpha converted to the dtype;
- * DFMA / FFMA register-blocked kernel, asynchronous on `stream`.  The
+ * the kernels that a solve would take for the size (digit products on the
+ * tensor cores, or the DFMA / FFMA kernel), asynchronous on `stream`.  The
  * planner's analytic model times it (gemm(j) of Section V).  Returns 0, -1
  * for a bad dtype, -2..-4 for negative M, N, K, -5 / -7 / -9 for a NULL
  * operand that is needed, -6 / -8 / -10 for a leading dimension below its

@@ -7,6 +7,7 @@
 #include <mutex>
 #include "common.cuh"
 #include "driver.cuh"
+#include "gemm_digits.cuh"
 #include "plan.cuh"
 
 namespace gb {
@@ -33,7 +34,39 @@ int side_stream(cudaStream_t *out)
     return 0;
 }
 
+// A TS task larger than the diagonal kernel (64 rows) is itself solved: by
+// the recursive model down to that kernel, whose updates are wide enough for
+// the digit gemm, or, for a plan that asks for smaller blocks, blocked by
+// them.
+constexpr int64_t kTsRows = 64;
+template <class E, typename T>
+void expand_ts(E &e, int64_t b0, int64_t nr, int64_t nb, T a, bool fwd)
+{
+    if (nb < kTsRows) drive_blocked(e, b0, b0 + nr, nb, a, fwd);
+    else drive_recursive(e, b0, b0 + nr, 24, kTsRows, a, fwd);
+}
+
+// Executor that finds the work space of a schedule's largest digit gemm.
+template <typename T>
+struct DigitBytesExec {
+    int64_t nb, ncols;
+    bool forward;
+    size_t bytes = 0;
+    bool ok() const { return true; }
+    void ts(int64_t b0, int64_t nr, T a)
+    {
+        if (nr > kTsRows) expand_ts(*this, b0, nr, nb, a, forward);
+    }
+    void gemm(int64_t, int64_t M, int64_t, int64_t K, T)
+    {
+        if (digit_gemm_wanted<T>(M, ncols, K, 0)) bytes = std::max(bytes, digit_gemm_bytes<T>(M, ncols, K, 0));
+    }
+};
+
 // Executor that launches the kernels of each task on the canonical view.
+//
+// A gemm task large enough goes to the digit gemm (gemm_digits.cu), in its
+// work space; the others to the CUDA-core update, with lookahead:
 //
 // Lookahead (the overlap of the diagonal solve with the off-diagonal
 // updates that the paper's blocked model aims at, Section V-C, and names as
@@ -56,7 +89,9 @@ struct LaunchExec {
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_tail = nullptr;
     int64_t pend_lo = 0, pend_hi = 0;  // rows written by tails not yet waited for
-    LaunchExec(const Canon<T> &c_, int64_t nb_) : c(c_), nb(nb_) {}
+    size_t digit_bytes = 0;            // work space of the schedule's largest digit gemm (0: none)
+    DigitWorkspace dws;
+    LaunchExec(const Canon<T> &c_, int64_t nb_) : c(c_), nb(nb_), dws(c_.stream) {}
     ~LaunchExec()
     {
         if (ev_fork) cudaEventDestroy(ev_fork);
@@ -88,19 +123,28 @@ struct LaunchExec {
     void ts(int64_t b0, int64_t nr, T a)
     {
         if (status) return;
-        if (nr <= 64) {
+        if (nr <= kTsRows) {
             settle(b0, b0 + nr);
             if (!status) status = launch_diag_solve(c, b0, (int)nr, a);
             return;
         }
-        // A TS task larger than the diagonal kernel is itself solved blocked.
-        int64_t inner = nb < nr ? nb : 64;
-        if (inner > 64 && inner >= nr) inner = 64;
-        drive_blocked(*this, b0, b0 + nr, inner, a, c.forward);
+        expand_ts(*this, b0, nr, nb, a, c.forward);
     }
     void gemm(int64_t ci0, int64_t M, int64_t ak0, int64_t K, T a)
     {
         if (status) return;
+        // (decided on the whole task, so that lookahead does not change it)
+        if (digit_bytes && digit_gemm_wanted<T>(M, c.ncols, K, 0)) {
+            char *ws = dws.get(digit_bytes);
+            if (ws) {
+                settle(ci0, ci0 + M);
+                if (status) return;
+                const DigitGemm<T> g{M, c.ncols, K, mv_ptr(c, ci0, ak0), c.lda, !c.mt, bv_ptr(c, ak0, 0), c.ldb, c.left,
+                                     bv_ptr(c, ci0, 0), c.ldb, c.left, a, 0};
+                status = launch_digit_gemm<T>(g, ws, dws.size(), c.stream);
+                return;
+            }
+        }
         const int64_t h = nb;  // rows of the next diagonal block
         if (!lookahead || M <= 2 * h) {
             settle(ci0, ci0 + M);
@@ -176,6 +220,9 @@ int trsm_impl(int side, int uplo, int trans, int diag, int64_t m, int64_t n, T a
     // the blocked and recursive models on more than four blocks of rows
     if (g_lookahead.load() && p.driver != GB_DRIVER_ITERATIVE && k > 4 * p.nb)
         GB_TRY(e.enable_lookahead());
+    DigitBytesExec<T> db{p.nb, c.ncols, c.forward};
+    drive_plan(db, p.driver, k, p.nb, p.depth, alpha, c.forward);
+    e.digit_bytes = db.bytes;
     drive_plan(e, p.driver, k, p.nb, p.depth, alpha, c.forward);
     if (e.status) {
         e.join();  // leave no work of this call on the second stream unordered

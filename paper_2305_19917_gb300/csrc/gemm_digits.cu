@@ -1,0 +1,1004 @@
+// Off-diagonal update C = alpha*C - Aop*Bop of the plain FP64 / FP32 solve on
+// the tensor cores: the paper's gemm task (Section IV stage 2) by exact
+// integer digit products.
+//
+// What bounds the CUDA-core update (gemm_simt.cu) is the FP64 unit: two DFMA
+// per clock and SM, 1.26 TFLOP/s for the chip.  The BF16 tensor cores do
+// about 1700 TFLOP/s, so cutting both factors into 8-bit digits and forming
+// the digit products there is faster although 28 of them stand for one FP64
+// product (6 for FP32).  Three launches per update:
+//
+//  1. digits_kernel: row i of Aop (column j of Bop) is scaled by the power of
+//     two 2^-e that brings its largest entry below 1 and rounded to a
+//     fixed-point number of 8 P bits, P = 7 (FP64: 56 bits; an entry in the
+//     largest binade keeps all its 53) or 3 (FP32: 24 bits), cut into P
+//     balanced base-256 digits, each an integer |d| <= 128 (the top one
+//     <= 256) that BF16 holds exactly.
+//  2. digit_mma_kernel: per 128 x 128 tile of C the digit products S_pq =
+//     sum_k a_p x_q with p + q <= P + 1 (what is left out lies below 2^-8P of
+//     the largest product).  K advances in chunks of 256, over which every
+//     sum of one weight p + q stays an exact integer of at most 2^24 in the
+//     FP32 accumulators; so all pairs of one weight share an accumulator
+//     (FP64: 28 pairs in 12 accumulators, six passes over the chunk), and
+//     the chunk's sums are added into int64 sums T = sum 2^(W-8(p+q)) S_pq.
+//     The two lowest weights of FP64 (2^-56, 2^-64 of the product) are scaled
+//     and rounded before they are added; W is the largest weight for which T
+//     cannot overflow.  A pass multiplies slice a_p with [x_q; x_q+1]
+//     (N = 256: two weights at a time, two accumulators of 128 x 256, one
+//     drained while the other fills).
+//     When a tile's sums are complete C = alpha C - 2^(e_i+f_j-W) T follows
+//     in the same kernel, one rounding of T, while the tensor cores are at
+//     the next tile.
+//  3. digit_fallback_kernel: the tiles that pass 2 listed (usually none).
+//
+// Accuracy: each factor's rounding is at most 2^-57 (FP32 2^-25) of its row's
+// (column's) largest entry, independent of K, where the CUDA-core sum rounds
+// K times.  That is relative to the largest entries, not to each product: for
+// a sum in which large entries of Aop meet only small ones of Bop it would be
+// worse.  Pass 1 therefore counts the entries of every row and column within
+// 2^-4 of its largest; where the counts of a row and a column add up to more
+// than 5/4 K, at least K/4 products of the sum have both factors within 2^-4
+// of their largest ones, and sum |a||x| is of the order of K times the product
+// of the largest entries.  A tile with a row and a column for which that
+// cannot be said, with an infinity or a NaN, or with exponents near the ends
+// of the range, is listed for the last pass, which computes it with the
+// CUDA-core tile of gemm_tile.cuh: the operations of gemm_simt.cu.  So is a
+// tile whose bounded waits gave up.
+#include <mutex>
+#include <cuda_bf16.h>
+#include "common.cuh"
+#include "fixed.cuh"
+#include "gemm_digits.cuh"
+#include "gemm_tile.cuh"
+#include "tc_common.cuh"
+
+namespace gb {
+
+namespace {
+
+constexpr int BM = 128, BK = 64, STAGES = 4;
+constexpr int KC = 256;                        // K of one exact accumulation
+constexpr uint32_t TILE_BYTES = BM * BK * 2;   // one digit tile of 128 rows
+constexpr uint32_t STAGE_BYTES = 3 * TILE_BYTES;
+constexpr int EPI_WARPS = 16;                  // four column groups of 32 times the four TMEM lane groups
+constexpr int MMA_THREADS = 32 * (2 + EPI_WARPS);
+constexpr uint32_t XP_BYTES = 32 * 5 * 8;      // a warp's transpose buffer (row-major C)
+constexpr size_t MMA_SMEM = 1024 + STAGES * size_t(STAGE_BYTES) + EPI_WARPS * size_t(XP_BYTES) + 256;
+constexpr int DROWS = 32;                      // rows of one digits_kernel CTA
+constexpr int DTHREADS = 256;
+constexpr int kMaxCluster = 8;
+constexpr int kCntBad = -(1 << 28);            // a row the digits must not represent
+constexpr int kNear = 4;                       // "within 2^-4 of the largest"
+
+template <typename T>
+struct Fmt;
+template <>
+struct Fmt<double> {
+    static constexpr int P = 7;        // digits
+    static constexpr int BIAS = 1023;
+    static constexpr int EMAX = 400;   // |exponent of the largest entry| beyond which the CUDA cores take over
+    __device__ static int field(double a) { return bexp(a); }
+};
+template <>
+struct Fmt<float> {
+    static constexpr int P = 3;
+    static constexpr int BIAS = 127;
+    static constexpr int EMAX = 45;
+    __device__ static int field(float a) { return int((__float_as_uint(a) >> 23) & 0xFF); }
+};
+
+// Digits of a (exponent field of the row's largest entry: emax), most
+// significant first, as the bit patterns of exact FP32 integers.
+// e' = emax - BIAS + 1: |a| < 2^e', N = round(a 2^(8P - e')).
+__device__ __forceinline__ void digits_of(double a, int emax, uint32_t (&d)[7])
+{
+    const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(a));
+    const int E = int((b >> 52) & 0x7FF);
+    const unsigned long long mant = E ? ((b & ((1ull << 52) - 1)) | (1ull << 52)) : 0ull;
+    const int r = emax - E - 3;  // N = mant 2^-r
+    unsigned long long n;
+    if (r <= 0) n = mant << (-r);  // r >= -3
+    else if (r >= 56) n = 0;
+    else n = (mant + (1ull << (r - 1))) >> r;
+    const long long N = (b >> 63) ? -static_cast<long long>(n) : static_cast<long long>(n);
+    int x = int(uint32_t(N) & 0xFFFFFFu);
+#pragma unroll
+    for (int p = 6; p >= 4; p--) {
+        const int q = bal8(x);
+        d[p] = small_int_f32bits(q);
+        x = (x - q) >> 8;
+    }
+    const long long y64 = (N >> 24) + x;  // |y64| <= 2^32
+    const int q3 = bal8(int(uint32_t(y64)));
+    d[3] = small_int_f32bits(q3);
+    int y = int((y64 - q3) >> 8);         // |y| <= 2^24 + 1
+#pragma unroll
+    for (int p = 2; p >= 1; p--) {
+        const int q = bal8(y);
+        d[p] = small_int_f32bits(q);
+        y = (y - q) >> 8;
+    }
+    d[0] = small_int_f32bits(y);          // |y| <= 256
+}
+__device__ __forceinline__ void digits_of(float a, int emax, uint32_t (&d)[3])
+{
+    const uint32_t b = __float_as_uint(a);
+    const int E = int((b >> 23) & 0xFF);
+    const uint32_t mant = E ? ((b & 0x7FFFFFu) | 0x800000u) : 0u;
+    const int r = emax - E;
+    uint32_t n;
+    if (r <= 0) n = mant;
+    else if (r >= 26) n = 0;
+    else n = (mant + (1u << (r - 1))) >> r;
+    int x = (b >> 31) ? -int(n) : int(n);
+#pragma unroll
+    for (int p = 2; p >= 1; p--) {
+        const int q = bal8(x);
+        d[p] = small_int_f32bits(q);
+        x = (x - q) >> 8;
+    }
+    d[0] = small_int_f32bits(x);
+}
+
+// ---- pass 1: digits ----------------------------------------------------------
+
+// One factor: R(r, k), r < rows, k < K; contiguous along k (kc) or along r.
+template <typename T>
+struct DigitSrc {
+    const T *src;
+    int64_t ld;
+    int kc;
+    int rows;             // valid rows; rp = padded to 128
+    int rp;
+    __nv_bfloat16 *out;   // P planes of rp x kp, row-major
+    int *e;               // exponent e' per row
+    int *cnt;             // entries within 2^-kNear of the largest; kCntBad; >= 2K for a zero or padding row
+};
+
+// cp.async-free: what bounds this kernel is the latency of its loads (8 per
+// thread in flight) and the integer work of the digits.  A CTA takes 32 rows
+// and a share of K; the CTAs of one row block form a cluster along K (so that
+// a few rows of a long K still fill the chip) and exchange the rows' largest
+// exponents and counts through distributed shared memory.  The second read of
+// the tile comes from L2.
+template <typename T>
+__global__ void __launch_bounds__(DTHREADS, sizeof(T) == 8 ? 3 : 4)
+digits_kernel(DigitSrc<T> a, DigitSrc<T> x, int ablocks, int K, int kp, int *zero, int nzero)
+{
+    constexpr int P = Fmt<T>::P;
+    __shared__ T t[DROWS][65];
+    __shared__ int key[DROWS];   // 2 * largest exponent field + (any nonzero entry)
+    __shared__ int num[DROWS];
+    __shared__ int emx[DROWS];
+    const int tid = threadIdx.x;
+    const bool isa = int(blockIdx.x) < ablocks;
+    const DigitSrc<T> s = isa ? a : x;
+    const int r0 = (isa ? blockIdx.x : blockIdx.x - ablocks) * DROWS;
+    const int rank = blockIdx.y, ncta = gridDim.y;  // the cluster is the grid's y extent
+    const int ntile = kp / BK, per = (ntile + ncta - 1) / ncta;
+    const int t0 = min(rank * per, ntile), t1 = min(t0 + per, ntile);
+
+    if (tid < DROWS) {
+        key[tid] = 0;
+        num[tid] = 0;
+    }
+    tc::pdl_wait();
+    tc::pdl_launch_dependents();
+    // the tiles' words of pass 2
+    for (int z = (blockIdx.x * gridDim.y + blockIdx.y) * DTHREADS + tid; z < nzero; z += gridDim.x * gridDim.y * DTHREADS)
+        zero[z] = 0;
+    __syncthreads();
+    auto load = [&](int tile, T (&v)[8]) {
+        const int kb = tile * BK;
+#pragma unroll
+        for (int u = 0; u < 8; u++) {
+            const int r = s.kc ? (tid >> 6) + 4 * u : (tid & 31);
+            const int k = kb + (s.kc ? (tid & 63) : (tid >> 5) + 8 * u);
+            const bool in = r0 + r < s.rows && k < K;
+            v[u] = in ? (s.kc ? s.src[k + int64_t(r0 + r) * s.ld] : s.src[r0 + r + int64_t(k) * s.ld]) : T(0);
+        }
+    };
+    // largest exponent field of every row
+    int mx[8];
+#pragma unroll
+    for (int u = 0; u < 8; u++) mx[u] = 0;
+    T v[8];
+    for (int tile = t0; tile < t1; tile++) {
+        load(tile, v);
+#pragma unroll
+        for (int u = 0; u < 8; u++) mx[u] = max(mx[u], 2 * Fmt<T>::field(v[u]) + (v[u] != T(0) ? 1 : 0));
+    }
+    if (s.kc) {  // a warp's lanes share the rows (tid >> 6) + 4u
+#pragma unroll
+        for (int u = 0; u < 8; u++) {
+            const int w = __reduce_max_sync(0xffffffffu, mx[u]);
+            if ((tid & 31) == 0) atomicMax(&key[(tid >> 6) + 4 * u], w);
+        }
+    } else {
+#pragma unroll
+        for (int u = 1; u < 8; u++) mx[0] = max(mx[0], mx[u]);
+        atomicMax(&key[tid & 31], mx[0]);
+    }
+    auto cluster_sync = [&]() {
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    };
+    // p of cluster CTA c's copy of a shared variable
+    auto peer = [&](const int *p, int c) {
+        uint32_t ad;
+        int r;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ad) : "r"(tc::smem_u32(p)), "r"(c));
+        asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(r) : "r"(ad) : "memory");
+        return r;
+    };
+    cluster_sync();
+    if (tid < DROWS) {
+        int m = 0;
+        for (int c = 0; c < ncta; c++) m = max(m, peer(&key[tid], c));
+        emx[tid] = m;
+    }
+    __syncthreads();
+    // digits, 8 consecutive k of one row per thread and tile
+    const int row = tid >> 3, lk = (tid & 7) * 8;
+    const int em = emx[row] >> 1;
+    int near = 0;
+    const size_t plane = size_t(s.rp) * size_t(kp);
+    for (int tile = t0; tile < t1; tile++) {
+        load(tile, v);
+        __syncthreads();  // the previous tile has been read
+#pragma unroll
+        for (int u = 0; u < 8; u++) {
+            const int r = s.kc ? (tid >> 6) + 4 * u : (tid & 31);
+            const int k = s.kc ? (tid & 63) : (tid >> 5) + 8 * u;
+            t[r][k] = v[u];
+        }
+        __syncthreads();
+        uint32_t w[P][4];
+#pragma unroll
+        for (int u = 0; u < 8; u += 2) {
+            uint32_t d0[P], d1[P];
+            const T a0 = t[row][lk + u], a1 = t[row][lk + u + 1];
+            digits_of(a0, em, d0);
+            digits_of(a1, em, d1);
+            near += (Fmt<T>::field(a0) + kNear >= em && a0 != T(0)) + (Fmt<T>::field(a1) + kNear >= em && a1 != T(0));
+#pragma unroll
+            for (int p = 0; p < P; p++) w[p][u >> 1] = pack_hi16(d0[p], d1[p]);
+        }
+        __nv_bfloat16 *o = s.out + size_t(r0 + row) * size_t(kp) + size_t(tile * BK + lk);
+#pragma unroll
+        for (int p = 0; p < P; p++)
+            *reinterpret_cast<uint4 *>(o + p * plane) = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) near += __shfl_xor_sync(0xffffffffu, near, o);
+    if ((tid & 7) == 0) num[row] = near;
+    cluster_sync();
+    if (rank == 0 && tid < DROWS) {
+        int c = 0;
+        for (int q = 0; q < ncta; q++) c += peer(&num[tid], q);
+        const int k2 = emx[tid], f = k2 >> 1, e = f - Fmt<T>::BIAS;
+        if (k2 == 0) c = 2 * K;                                         // a zero row: exact
+        else if (f == 0 || e > Fmt<T>::EMAX || e < -Fmt<T>::EMAX) c = kCntBad;  // infinities and NaN too
+        s.cnt[r0 + tid] = c;
+        s.e[r0 + tid] = k2 == 0 ? 0 : e + 1;
+    }
+    cluster_sync();  // no CTA leaves while its shared memory may be read
+}
+
+// ---- pass 2: digit products ----------------------------------------------------
+
+// The schedule of a chunk: products in order, grouped into passes (pass j:
+// weight j + 2 in the low half of the accumulator, j + 3 in the high half).
+// Product o takes A slice p(o) (0-based) with X slices q(o) and q(o) + 1 into
+// both halves (o < TWO), or with X slice q(o) alone into the high half.
+template <typename T>
+struct Sched;
+template <>
+struct Sched<double> {  // (p, q): (0,0) | (1,0) | (0,2) (2,0) | (1,2) (3,0) | (0,4) (2,2) (4,0) |
+                        // (1,4) (3,2) (5,0) and alone (0,6) (2,4) (4,2) (6,0)
+    static constexpr int NP = 6, NO = 16, TWO = 12;
+    __device__ static int p(int o) { return int(0x6420531420312010ull >> (4 * o)) & 15; }
+    __device__ static int q(int o) { return int(0x0246024024020200ull >> (4 * o)) & 15; }
+    __device__ static int first(int j) { return int(0x10090604020100ull >> (8 * j)) & 255; }
+};
+template <>
+struct Sched<float> {  // (0,0) | (1,0) and alone (0,2) (2,0)
+    static constexpr int NP = 2, NO = 4, TWO = 2;
+    __device__ static int p(int o) { return (0x2010 >> (4 * o)) & 15; }
+    __device__ static int q(int o) { return (0x0200 >> (4 * o)) & 15; }
+    __device__ static int first(int j) { return (0x040100 >> (8 * j)) & 255; }
+};
+
+// The tiles' words, cleared by pass 1: [0] number of listed tiles, then per
+// tile: partial sums stored (split > 1), listed or not, and the list; last the
+// bounded waits' status (nobody reads it: a tile whose wait gave up is listed).
+struct TileWords {
+    int *count, *done, *listed, *list;
+};
+
+template <typename T>
+struct MmaArgs {
+    DigitGemm<T> g;
+    long long *Tg;      // split > 1: planes of tile-blocked partial sums (128 x 128, column-major)
+    const int *cnt_a, *cnt_x, *e_a, *e_x;
+    TileWords w;
+    int kp, nMt, nNt, ntiles, W, split;
+    int *status;
+};
+
+// Tile (m, n) number t of the launch: grouped rasterisation of the full
+// grid, or the triangle's tiles (a >= b; lower: m = a, upper: n = a).
+__device__ __forceinline__ void digit_tile(int t, int nMt, int nNt, int tri, int &m, int &n)
+{
+    if (tri == 0) {
+        tc::raster_grouped(t, nMt, nNt, 8, m, n);
+        return;
+    }
+    int a = int((sqrtf(8.0f * float(t) + 1.0f) - 1.0f) * 0.5f);
+    while (a * (a + 1) / 2 > t) a--;
+    while ((a + 1) * (a + 2) / 2 <= t) a++;
+    const int b = t - a * (a + 1) / 2;
+    m = tri == 1 ? a : b;
+    n = tri == 1 ? b : a;
+}
+
+__device__ __forceinline__ double scale_sum(double, long long t, int e) { return scaled_i64_to_f64(t, e); }
+// |T| 2^e with a normal scale factor (EMAX bounds e): one rounding, of T
+__device__ __forceinline__ float scale_sum(float, long long t, int e)
+{
+    return __ll2float_rn(t) * __int_as_float((e + 127) << 23);
+}
+
+// One work item of a CTA: a tile and a share of its K chunks.
+struct Item {
+    int tile, i0, j0, sp, ch0, ch1;
+    bool skip;  // the digits may not represent this tile
+};
+// Evaluated by every warp for itself (all lanes).
+template <typename T>
+__device__ __forceinline__ Item digit_item(const MmaArgs<T> &a, int w, int lane)
+{
+    Item it;
+    it.tile = w % a.ntiles;
+    it.sp = w / a.ntiles;
+    int m, n;
+    digit_tile(it.tile, a.nMt, a.nNt, a.g.tri, m, n);
+    it.i0 = m * BM;
+    it.j0 = n * BM;
+    const int nch = (a.kp + KC - 1) / KC, per = (nch + a.split - 1) / a.split;
+    it.ch0 = min(it.sp * per, nch);
+    it.ch1 = min(it.ch0 + per, nch);
+    const int4 ca = reinterpret_cast<const int4 *>(a.cnt_a + it.i0)[lane];
+    const int4 cx = reinterpret_cast<const int4 *>(a.cnt_x + it.j0)[lane];
+    const int ma = __reduce_min_sync(0xffffffffu, min(min(ca.x, ca.y), min(ca.z, ca.w)));
+    const int mx = __reduce_min_sync(0xffffffffu, min(min(cx.x, cx.y), min(cx.z, cx.w)));
+    const int K = int(a.g.K);
+    it.skip = ma < 0 || mx < 0 || ma + mx < K + K / 4;
+    return it;
+}
+
+// An integer S held in FP32, |S| <= 2^26, as the integer S + kIntBias modulo
+// 2^32 (positive as a signed number): S is cut at bit 12, and each part added
+// to 1.5 2^23 stands in the low bits of the sum.  Float-to-integer conversions
+// run at a small fraction of the FP32 rate here: with them a drained
+// accumulator pair took about 8000 clocks.
+constexpr float kMagic = 12582912.0f;  // 1.5 2^23 = 0x4B400000
+constexpr unsigned long long kIntBias = 0x4B400000ull;
+__device__ __forceinline__ uint32_t biased_int(float S)
+{
+    const float h = fmaf(S, 1.0f / 4096.0f, kMagic);    // round(S / 2^12) + magic
+    const float f = h - (kMagic + 3072.0f);             // round(S / 2^12) - 3072
+    const float l = fmaf(f, -4096.0f, S);               // S - 2^12 round(S / 2^12) + magic
+    // 2^12 times the magic's bits is 0 modulo 2^32
+    return __float_as_uint(h) * 4096u + __float_as_uint(l);
+}
+
+// Persistent: one CTA per SM walks the items w = blockIdx.x, + gridDim.x, ...
+// Warp 0 issues the TMA loads, warp 1 the MMAs, warps 2-17 drain the
+// accumulators and finish C.  What bounds it: the tensor cores (28 x 2 flop
+// per multiply-add of the product), fed with 48 KB of digits per 512 clocks;
+// the drains (12 half accumulators per 28.7k clocks of MMAs) go on beside them.
+// Sixteen drain warps hide the latencies of the accumulators' loads.
+template <typename T>
+__global__ void __launch_bounds__(MMA_THREADS, 1)
+digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmX,
+                 const __grid_constant__ MmaArgs<T> a)
+{
+    using S = Sched<T>;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *xpose = base + STAGES * STAGE_BYTES;
+    uint64_t *full = reinterpret_cast<uint64_t *>(xpose + EPI_WARPS * XP_BYTES);
+    uint64_t *empty = full + STAGES;
+    uint64_t *accf = empty + STAGES;  // [2]
+    uint64_t *acce = accf + 2;        // [2]
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(acce + 2);
+    __shared__ int abort_flag;
+    __shared__ int last_flag;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nitems = a.ntiles * a.split;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; s++) {
+            tc::mbar_init(&full[s], 1);
+            tc::mbar_init(&empty[s], 1);  // one MMA commit
+        }
+        for (int b = 0; b < 2; b++) {
+            tc::mbar_init(&accf[b], 1);
+            tc::mbar_init(&acce[b], EPI_WARPS);  // one arrival per epilogue warp
+        }
+        abort_flag = 0;
+        tc::fence_barrier_init();
+    }
+    if (warp == 1) tc::tmem_alloc(tslot, 512);
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    const uint32_t tmem = *tslot;
+    volatile int *ab = &abort_flag;
+    tc::pdl_wait();
+    tc::pdl_launch_dependents();
+
+    if (warp == 0) {
+        if (lane == 0) {
+            tc::tma_prefetch_desc(&tmA);
+            tc::tma_prefetch_desc(&tmX);
+        }
+        int n = 0;
+        int ok = 1;
+        for (int w = blockIdx.x; w < nitems && ok; w += gridDim.x) {
+            const Item it = digit_item(a, w, lane);
+            if (it.skip) continue;
+            if (lane == 0) {
+                for (int c = it.ch0; c < it.ch1 && ok; c++) {
+                    const int kb = c * KC, ke = min(kb + KC, a.kp);
+                    for (int o = 0; o < S::NO && ok; o++) {
+                        const int p = S::p(o), q = S::q(o);
+                        const bool two = o < S::TWO;
+                        for (int kk = kb; kk < ke; kk += BK, n++) {
+                            const int s = n % STAGES;
+                            const uint32_t ph = (n / STAGES) & 1;
+                            ok = tc::mbar_wait(&empty[s], ph ^ 1, ab, a.status, tc::TC_TIMEOUT_PRODUCER);
+                            if (!ok) break;
+                            uint8_t *st = base + s * STAGE_BYTES;
+                            tc::mbar_arrive_expect_tx(&full[s], (two ? 3u : 2u) * TILE_BYTES);
+                            tc::tma_load_3d(&tmA, &full[s], st, kk, it.i0, p);
+                            tc::tma_load_3d(&tmX, &full[s], st + TILE_BYTES, kk, it.j0, q);
+                            if (two) tc::tma_load_3d(&tmX, &full[s], st + 2 * TILE_BYTES, kk, it.j0, q + 1);
+                        }
+                    }
+                }
+            }
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+        }
+        if (lane == 0) {
+            // tail: wait until the MMAs released every stage, so that no
+            // commit is still on its way to this CTA's barriers when it exits
+            for (int t = 0; t < STAGES && ok; t++, n++) {
+                const int s = n % STAGES;
+                const uint32_t ph = (n / STAGES) & 1;
+                ok = tc::mbar_wait(&empty[s], ph ^ 1, ab, a.status, tc::TC_TIMEOUT_PRODUCER);
+            }
+            // after a wait that gave up: the copies still in flight land
+            // before this CTA's shared memory is given away (bounded)
+            if (!ok)
+                for (int t = n > STAGES ? n - STAGES : 0; t < n; t++)
+                    for (int spin = 0; spin < (1 << 16) && !tc::mbar_try_wait(&full[t % STAGES], (t / STAGES) & 1); spin++) {
+                    }
+        }
+    } else if (warp == 1) {
+        const uint64_t d0 = tc::desc_kmajor_sw128(tc::smem_u32(base));
+        const uint32_t idesc256 = tc::idesc_bf16_f32(BM, 256), idesc128 = tc::idesc_bf16_f32(BM, 128);
+        int n = 0, cp = 0;
+        int ok = 1;
+        for (int w = blockIdx.x; w < nitems && ok; w += gridDim.x) {
+            const Item it = digit_item(a, w, lane);
+            if (it.skip) continue;
+            if (lane == 0) {
+                for (int c = it.ch0; c < it.ch1 && ok; c++) {
+                    const int kb = c * KC, ke = min(kb + KC, a.kp);
+                    const int nk = (ke - kb) / BK;
+                    for (int j = 0; j < S::NP && ok; j++, cp++) {
+                        const int buf = cp & 1;
+                        ok = tc::mbar_wait(&acce[buf], ((cp >> 1) & 1) ^ 1, ab, a.status, tc::TC_TIMEOUT_MMA);
+                        if (!ok) break;
+                        tc::tc_fence_after();
+                        const uint32_t acc = tmem + uint32_t(buf * 256);
+                        const int o0 = S::first(j), o1 = S::first(j + 1);
+                        for (int o = o0; o < o1 && ok; o++) {
+                            const bool two = o < S::TWO;
+                            const uint32_t d = two ? acc : acc + 128u;
+                            const uint32_t idesc = two ? idesc256 : idesc128;
+                            for (int kt = 0; kt < nk; kt++, n++) {
+                                const int s = n % STAGES;
+                                ok = tc::mbar_wait(&full[s], (n / STAGES) & 1, ab, a.status, tc::TC_TIMEOUT_MMA);
+                                if (!ok) break;
+                                tc::tc_fence_after();
+                                // the start address field counts 16-byte units: a
+                                // 32-byte step along K adds 2
+                                const uint64_t da = d0 + uint64_t(uint32_t(s) * (STAGE_BYTES >> 4));
+                                const uint64_t db = da + uint64_t(TILE_BYTES >> 4);
+                                tc::mma_f16(d, da, db, idesc, o != o0 || kt != 0);
+#pragma unroll
+                                for (int kk = 1; kk < BK / 16; kk++)
+                                    tc::mma_f16(d, da + uint64_t(2 * kk), db + uint64_t(2 * kk), idesc, 1);
+                                tc::mma_commit(&empty[s]);
+                            }
+                        }
+                        if (ok) tc::mma_commit(&accf[buf]);
+                    }
+                }
+            }
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+        }
+    } else {
+        const int q = warp & 3;                 // TMEM lane group this warp may read
+        const int cg = (warp - 2) >> 2;         // columns [32 cg, 32 cg + 32) of the tile
+        const bool first = threadIdx.x == 64;   // speaks for the epilogue warps
+        T *xp = reinterpret_cast<T *>(xpose + (warp - 2) * XP_BYTES);
+        const uint32_t lbase = tmem + (uint32_t(q * 32) << 16) + uint32_t(cg * 32);
+        int ok = 1, cp = 0;
+        for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
+            const Item it = digit_item(a, w, lane);
+            if (it.skip || !ok) {
+                if (first && atomicExch(&a.w.listed[it.tile], 1) == 0) a.w.list[atomicAdd(a.w.count, 1)] = it.tile;
+                continue;
+            }
+            // Sums start at minus what the conversions below add: kIntBias 2^s
+            // for every half accumulator of weight 2^s (modulo 2^64).
+            long long T64[32];
+            {
+                unsigned long long bias = 0;
+#pragma unroll
+                for (int j = 0; j < S::NP; j++)
+#pragma unroll
+                    for (int h = 0; h < 2; h++) {
+                        const int s = a.W - 8 * (j + 2 + h);
+                        if (s >= 0) bias += kIntBias << s;
+                        else if (h == 1) bias += kIntBias;
+                    }
+                bias *= (unsigned long long)(it.ch1 - it.ch0);
+#pragma unroll
+                for (int c = 0; c < 32; c++) T64[c] = static_cast<long long>(0ull - bias);
+            }
+            // T += S 2^s over the 32 columns at tb
+            auto add_half = [&](uint32_t tb, int s) {
+#pragma unroll
+                for (int c0 = 0; c0 < 32; c0 += 8) {
+                    uint32_t r[8];
+                    tc::tmem_ld8(tb + c0, r);
+                    tc::tmem_ld_wait();
+                    if (s >= 32) {
+#pragma unroll
+                        for (int e = 0; e < 8; e++)
+                            T64[c0 + e] += static_cast<long long>(
+                                static_cast<unsigned long long>(biased_int(__uint_as_float(r[e])) << (s - 32)) << 32);
+                    } else {
+                        const int m = 1 << s;
+#pragma unroll
+                        for (int e = 0; e < 8; e++)
+                            T64[c0 + e] += static_cast<long long>(int(biased_int(__uint_as_float(r[e])))) * m;
+                    }
+                }
+            };
+            for (int c = it.ch0; c < it.ch1 && ok; c++) {
+#pragma unroll 1
+                for (int j = 0; j < S::NP; j++, cp++) {
+                    const int buf = cp & 1;
+                    ok = tc::mbar_wait(&accf[buf], (cp >> 1) & 1, ab, a.status, tc::TC_TIMEOUT_EPILOGUE);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    tc::tc_fence_after();
+                    const uint32_t tb = lbase + uint32_t(buf * 256);
+                    const int s1 = a.W - 8 * (j + 2), s2 = s1 - 8;
+                    if (s1 >= 0) add_half(tb, s1);
+                    if (sizeof(T) == 4 || s2 >= 0) {
+                        add_half(tb + 128, s2);
+                    } else {
+                        // a weight below the sums' last bit: scaled, and both
+                        // halves rounded as one number when neither is above it
+                        // (|S| 2^s2 <= 2^25-4: the sum stays within 2^22)
+                        const float m1 = s1 < 0 ? __int_as_float((127 + s1) << 23) : 0.f;
+                        const float m2 = __int_as_float((127 + s2) << 23);
+#pragma unroll
+                        for (int c0 = 0; c0 < 32; c0 += 8) {
+                            uint32_t r1[8], r2[8];
+                            tc::tmem_ld8(tb + c0, r1);
+                            tc::tmem_ld8(tb + 128 + c0, r2);
+                            tc::tmem_ld_wait();
+#pragma unroll
+                            for (int e = 0; e < 8; e++)
+                                T64[c0 + e] += __float_as_int(
+                                    fmaf(__uint_as_float(r1[e]), m1, __uint_as_float(r2[e]) * m2) + kMagic);
+                        }
+                    }
+                    tc::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(&acce[buf]);
+                }
+            }
+            // one answer for all sixteen warps (a bounded wait that gave up
+            // in one of them leaves the tile to the last pass)
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS) : "memory");
+            ok = ok && *ab == 0;
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS) : "memory");
+            if (!ok) {
+                if (first && atomicExch(&a.w.listed[it.tile], 1) == 0) a.w.list[atomicAdd(a.w.count, 1)] = it.tile;
+                continue;
+            }
+            const int row = q * 32 + lane;
+            if (a.split > 1) {
+                // the partial sums of this share; the CTA that stores the
+                // tile's last one adds them all up (integers: in any order)
+                const size_t plane = size_t(a.ntiles) * (BM * BM);
+                long long *o = a.Tg + size_t(it.tile) * (BM * BM) + row + cg * 32 * BM;
+#pragma unroll
+                for (int c = 0; c < 32; c++) __stcg(o + it.sp * plane + c * BM, T64[c]);
+                __threadfence();
+                asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS) : "memory");
+                if (first) last_flag = atomicAdd(&a.w.done[it.tile], 1) == a.split - 1;
+                asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS) : "memory");
+                const bool last = last_flag != 0;
+                if (!last) continue;
+                __threadfence();
+                for (int sp = 0; sp < a.split; sp++) {
+                    if (sp == it.sp) continue;
+#pragma unroll
+                    for (int c = 0; c < 32; c++) T64[c] += __ldcg(o + sp * plane + c * BM);
+                }
+            }
+            const DigitGemm<T> &g = a.g;
+            const int64_t i = int64_t(it.i0) + row, jb = int64_t(it.j0) + cg * 32;
+            const int ei = a.e_a[i] - a.W;
+            if (g.cl) {
+                // lanes hold consecutive rows: 256-byte accesses
+#pragma unroll
+                for (int c0 = 0; c0 < 32; c0 += 4) {
+                    T old[4];
+                    bool in[4];
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        const int64_t j = jb + c0 + u;
+                        in[u] = i < g.M && j < g.N && !(g.tri == 1 && j > i) && !(g.tri == 2 && j < i);
+                        old[u] = in[u] ? g.C[i + j * g.ldc] : T(0);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; u++) {
+                        const int64_t j = jb + c0 + u;
+                        const T v = scale_sum(T(0), T64[c0 + u], ei + a.e_x[j]);
+                        const T r = (g.alpha == T(1)) ? old[u] - v : g.alpha * old[u] - v;
+                        if (in[u]) g.C[i + j * g.ldc] = r;
+                    }
+                }
+            } else {
+                // row-major: 32 bytes of a row at a time, through the warp's
+                // transpose buffer
+                constexpr int NC = int(32 / sizeof(T)), LX = NC + 1, LPR = 32 / NC;
+                static_assert(32 * LX * sizeof(T) <= XP_BYTES, "transpose buffer");
+#pragma unroll
+                for (int c0 = 0; c0 < 32; c0 += NC) {
+#pragma unroll
+                    for (int u = 0; u < NC; u++)
+                        xp[lane * LX + u] = scale_sum(T(0), T64[c0 + u], ei + a.e_x[jb + c0 + u]);
+                    __syncwarp();
+                    T old[NC];
+                    const int64_t j = jb + c0 + lane % NC;
+#pragma unroll
+                    for (int u = 0; u < NC; u++) {
+                        const int64_t ii = int64_t(it.i0) + q * 32 + lane / NC + u * LPR;
+                        const bool in = ii < g.M && j < g.N && !(g.tri == 1 && j > ii) && !(g.tri == 2 && j < ii);
+                        old[u] = in ? g.C[j + ii * g.ldc] : T(0);
+                    }
+#pragma unroll
+                    for (int u = 0; u < NC; u++) {
+                        const int64_t ii = int64_t(it.i0) + q * 32 + lane / NC + u * LPR;
+                        const bool in = ii < g.M && j < g.N && !(g.tri == 1 && j > ii) && !(g.tri == 2 && j < ii);
+                        const T v = xp[(lane / NC + u * LPR) * LX + lane % NC];
+                        if (in) g.C[j + ii * g.ldc] = (g.alpha == T(1)) ? old[u] - v : g.alpha * old[u] - v;
+                    }
+                    __syncwarp();
+                }
+            }
+        }
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc::tc_fence_after();
+        tc::tmem_dealloc(tmem, 512);
+    }
+}
+
+// ---- pass 3: the listed tiles on the CUDA cores ------------------------------------
+
+template <typename T, bool AM, bool BC, bool CL>
+__global__ void __launch_bounds__(256)
+digit_fallback_kernel(DigitGemm<T> g, TileWords w, int nMt, int nNt)
+{
+    constexpr int FB = GemmTile<T>::BM, PER = BM / FB;
+    __shared__ __align__(16) T smem[gemm_tile_smem<T>()];
+    tc::pdl_wait();
+    tc::pdl_launch_dependents();
+    const int n = *w.count * PER * PER;
+    for (int t = blockIdx.x; t < n; t += gridDim.x) {
+        const int tile = w.list[t / (PER * PER)], sub = t % (PER * PER);
+        int m_blk, n_blk;
+        digit_tile(tile, nMt, nNt, g.tri, m_blk, n_blk);
+        const int64_t i0 = int64_t(m_blk) * BM + (sub % PER) * FB, j0 = int64_t(n_blk) * BM + (sub / PER) * FB;
+        if (i0 >= g.M || j0 >= g.N || (g.tri == 1 && j0 > i0 + FB - 1) || (g.tri == 2 && i0 > j0 + FB - 1)) continue;
+        gemm_tile<T, AM, BC, CL>(smem, i0, j0, g.M, g.N, g.K, g.A, g.lda, g.B, g.ldb, g.C, g.ldc, g.alpha, g.tri);
+        __syncthreads();
+    }
+}
+
+// ---- host ------------------------------------------------------------------------
+
+inline int64_t up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
+
+// SMs of the current device.
+inline int sm_count()
+{
+    static PerDeviceOnce n;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
+    int v = n.done[dev].load(std::memory_order_relaxed);
+    if (!v && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) n.done[dev].store(v);
+    return v > 0 ? v : 152;
+}
+
+// Largest piece of one launch sequence: the digits of both factors and the
+// sums stay within the work space's cap, K within 16384 (the sums' weight W).
+constexpr size_t kWsCap = size_t(2) << 30;
+constexpr int64_t kMaxK = 16384;
+
+struct Piece {
+    int64_t mc, nc, kc;  // extents of one piece (mc, nc multiples of 128 unless whole)
+    int split;
+    size_t bytes;
+};
+
+template <typename T>
+size_t piece_bytes(int64_t M, int64_t N, int64_t K, int tri, int split)
+{
+    constexpr int P = Fmt<T>::P;
+    const size_t mp = size_t(up(M, BM)), np = size_t(up(N, BM)), kp = size_t(up(K, BK));
+    const size_t nt = tri ? (mp / BM) * (mp / BM + 1) / 2 : (mp / BM) * (np / BM);
+    size_t b = 256 + 2 * P * mp * kp + (tri ? 0 : 2 * P * np * kp) + (split > 1 ? size_t(split) * nt * BM * BM * 8 : 0);
+    b += 4 * (2 * mp + 2 * np) + 4 * (3 * nt + 2) + 8 * 256;
+    return b;
+}
+
+// K is split over CTAs (with a plane of sums each) while the tiles alone leave
+// SMs idle and a CTA keeps at least two chunks of 256.
+inline int pick_split(int64_t ntiles, int64_t K)
+{
+    const int64_t nch = (K + KC - 1) / KC;
+    int64_t s = 152 / ntiles;
+    if (s > nch / 2) s = nch / 2;
+    if (s > 8) s = 8;
+    return s < 1 ? 1 : int(s);
+}
+
+template <typename T>
+Piece plan_piece(int64_t M, int64_t N, int64_t K, int tri)
+{
+    Piece p;
+    p.kc = K < kMaxK ? K : kMaxK;
+    p.mc = M;
+    p.nc = N;
+    // halve the longer of the two extents until the piece fits (a triangle is not cut)
+    while (!tri && piece_bytes<T>(p.mc, p.nc, p.kc, 0, 1) > kWsCap && (p.mc > 1024 || p.nc > 1024)) {
+        if (p.nc >= p.mc) p.nc = up((p.nc + 1) / 2, BM);
+        else p.mc = up((p.mc + 1) / 2, BM);
+    }
+    const int64_t mt = up(p.mc, BM) / BM, nt = up(p.nc, BM) / BM;
+    p.split = pick_split(tri ? mt * (mt + 1) / 2 : mt * nt, p.kc);
+    p.bytes = piece_bytes<T>(p.mc, p.nc, p.kc, tri, p.split);
+    return p;
+}
+
+template <typename T>
+int launch_fallback(const DigitGemm<T> &g, const TileWords &w, int nMt, int nNt, int ntiles, cudaStream_t s)
+{
+    void (*k)(DigitGemm<T>, TileWords, int, int) = nullptr;
+    if (g.am && g.bc && g.cl) k = digit_fallback_kernel<T, true, true, true>;
+    else if (g.am && !g.bc && !g.cl) k = digit_fallback_kernel<T, true, false, false>;
+    else if (!g.am && g.bc && g.cl) k = digit_fallback_kernel<T, false, true, true>;
+    else if (!g.am && !g.bc && !g.cl) k = digit_fallback_kernel<T, false, false, false>;
+    else if (g.am && !g.bc && g.cl) k = digit_fallback_kernel<T, true, false, true>;  // P P^T
+    if (!k) return GB_STATUS_CUDA_ERROR;
+    constexpr int PER = BM / GemmTile<T>::BM;
+    const int grid = ntiles * PER * PER < 304 ? ntiles * PER * PER : 304;
+    return check(launch_pdl(k, dim3((unsigned)grid), dim3(256), 0, s, g, w, nMt, nNt));
+}
+
+template <typename T>
+int digit_piece(const DigitGemm<T> &g, char *ws, size_t ws_bytes, int split, cudaStream_t s)
+{
+    constexpr int P = Fmt<T>::P;
+    const int64_t mp = up(g.M, BM), np = g.tri ? mp : up(g.N, BM), kp = up(g.K, BK);
+    const int nMt = int(mp / BM), nNt = int(np / BM);
+    const int64_t nt = g.tri ? int64_t(nMt) * (nMt + 1) / 2 : int64_t(nMt) * nNt;
+    size_t off = 0;
+    auto take = [&](size_t b) {
+        char *p = ws + off;
+        off += (b + 255) & ~size_t(255);
+        return p;
+    };
+    __nv_bfloat16 *da = reinterpret_cast<__nv_bfloat16 *>(take(size_t(2) * P * mp * kp));
+    __nv_bfloat16 *dx = g.tri ? da : reinterpret_cast<__nv_bfloat16 *>(take(size_t(2) * P * np * kp));
+    long long *Tg = reinterpret_cast<long long *>(take(split > 1 ? size_t(split) * nt * BM * BM * 8 : 0));
+    int *ea = reinterpret_cast<int *>(take(4 * size_t(mp))), *ca = reinterpret_cast<int *>(take(4 * size_t(mp)));
+    int *ex = g.tri ? ea : reinterpret_cast<int *>(take(4 * size_t(np)));
+    int *cx = g.tri ? ca : reinterpret_cast<int *>(take(4 * size_t(np)));
+    int *words = reinterpret_cast<int *>(take(4 * (3 * size_t(nt) + 2)));
+    const TileWords w{words, words + 1, words + 1 + nt, words + 1 + 2 * nt};
+    if (off > ws_bytes || nt * split > 0x3fffffff) return GB_STATUS_CUDA_ERROR;
+
+    CUtensorMap ta, tx;
+    {
+        const uint32_t box[3] = {BK, BM, 1};
+        uint64_t dims[3] = {uint64_t(kp), uint64_t(mp), uint64_t(P)};
+        uint64_t strides[2] = {uint64_t(kp) * 2, uint64_t(mp) * uint64_t(kp) * 2};
+        GB_TRY(encode_tmap(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, da, dims, strides, box));
+        dims[1] = uint64_t(np);
+        strides[1] = uint64_t(np) * uint64_t(kp) * 2;
+        GB_TRY(encode_tmap(&tx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, dx, dims, strides, box));
+    }
+    // weight of the sums: |T| <= 1.02 K 2^W < 2^63, at most 52 (the last weight
+    // but one is then scaled by 2^-4 or less, which keeps it in the range of
+    // its conversion)
+    int W = sizeof(T) == 8 ? 52 : 32;
+    if (sizeof(T) == 8)
+        for (int64_t k = 1024; k < g.K; k *= 2) W--;
+    {
+        LaunchScope ls(KK_CONVERT, s, 0,
+                       (sizeof(T) + 2.0 * P) * (double(g.M) + (g.tri ? 0.0 : double(g.N))) * double(g.K));
+        DigitSrc<T> sa{g.A, g.lda, g.am ? 0 : 1, int(g.M), int(mp), da, ea, ca};
+        DigitSrc<T> sx{g.B, g.ldb, g.bc ? 1 : 0, int(g.N), int(np), dx, ex, cx};
+        const int ab = int(mp / DROWS), xb = g.tri ? 0 : int(np / DROWS);
+        const int64_t ktiles = kp / BK;
+        int cl = 1;
+        while (cl < kMaxCluster && ktiles >= 4 * cl && int64_t(ab + xb) * cl < 1216) cl *= 2;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(ab + xb), (unsigned)cl);
+        cfg.blockDim = dim3(DTHREADS);
+        cfg.stream = s;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = 1;
+        attr[1].val.clusterDim.y = (unsigned)cl;
+        attr[1].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 2;
+        GB_CUDA(cudaLaunchKernelEx(&cfg, digits_kernel<T>, sa, sx, ab, int(g.K), int(kp), words, int(2 * nt + 1)));
+    }
+    {
+        static PerDeviceOnce attr;
+        GB_TRY(smem_attr_once(attr, digit_mma_kernel<T>, MMA_SMEM));
+        constexpr double pairs = P == 7 ? 28.0 : 6.0;
+        LaunchScope ls(KK_GEMM_TC, s, 2.0 * pairs * double(nt) * BM * BM * double(kp), 8.0 * double(nt) * BM * BM);
+        MmaArgs<T> a{g, Tg, ca, cx, ea, ex, w, int(kp), nMt, nNt, int(nt), W, split, words + 3 * nt + 1};
+        const int64_t items = nt * split;
+        GB_CUDA(launch_pdl(digit_mma_kernel<T>, dim3((unsigned)(items < sm_count() ? items : sm_count())), dim3(MMA_THREADS),
+                           MMA_SMEM, s, ta, tx, a));
+    }
+    LaunchScope ls(KK_GEMM_SIMT, s, 0, 0);
+    return launch_fallback<T>(g, w, nMt, nNt, int(nt), s);
+}
+
+cudaMemPool_t digit_pool()
+{
+    static cudaMemPool_t pool[64] = {nullptr};
+    static std::mutex mu;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!pool[dev]) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.handleTypes = cudaMemHandleTypeNone;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t p;
+        if (cudaMemPoolCreate(&p, &props) != cudaSuccess) return nullptr;
+        // freed work spaces up to this many bytes stay with the pool, the
+        // rest goes back to the driver when the stream is next synchronised
+        uint64_t thr = kWsCap + kWsCap / 4;
+        cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &thr);
+        pool[dev] = p;
+    }
+    return pool[dev];
+}
+
+}  // namespace
+
+char *DigitWorkspace::get(size_t bytes)
+{
+    if (state_ < 0) return nullptr;
+    if (state_ == 0) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s_, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+            state_ = -1;
+            return nullptr;
+        }
+        state_ = 1;
+    }
+    if (size_ >= bytes) return p_;
+    release();
+    cudaMemPool_t pool = digit_pool();
+    void *p = nullptr;
+    if (!pool || cudaMallocFromPoolAsync(&p, bytes, pool, s_) != cudaSuccess) {
+        cudaGetLastError();  // no memory: the CUDA-core update needs none
+        state_ = -1;
+        return nullptr;
+    }
+    p_ = static_cast<char *>(p);
+    size_ = bytes;
+    return p_;
+}
+
+void DigitWorkspace::release()
+{
+    if (p_) cudaFreeAsync(p_, s_);
+    p_ = nullptr;
+    size_ = 0;
+}
+
+void digit_pool_trim()
+{
+    cudaMemPool_t pool = digit_pool();
+    if (pool) cudaMemPoolTrimTo(pool, 0);
+}
+
+// FP64: from K = 64 on at every M and N: measured, 64 x 32 x 64 takes 40 us
+// (CUDA cores 74), 64 x 256 x 512 82 (531), 2048 x 8192 x 64 0.22 ms (1.79),
+// 2048 x 8192 x 2048 1.7 ms (55).  FP32: from K = 128, where the digits'
+// rounding (1.7e-7 of a normally distributed sum) falls below that of the
+// CUDA-core sum (2.1e-7; at K = 64 it would be above), and from 64 x 256
+// outputs, where they are the faster ones: 64 x 256 x 128 30 us (36), 512 x
+// 8192 x 128 44 (94), 2048 x 8192 x 2048 0.56 ms (2.6).
+template <typename T>
+bool digit_gemm_wanted(int64_t M, int64_t N, int64_t K, int)
+{
+    if (sizeof(T) == 8) return K >= 64;
+    return K >= 128 && (double(M) * double(N) >= 16384.0 || K >= 512);
+}
+
+template <typename T>
+size_t digit_gemm_bytes(int64_t M, int64_t N, int64_t K, int tri)
+{
+    return plan_piece<T>(M, N, K, tri).bytes;
+}
+
+template <typename T>
+int launch_digit_gemm(const DigitGemm<T> &g, char *ws, size_t ws_bytes, cudaStream_t s)
+{
+    const Piece pc = plan_piece<T>(g.M, g.N, g.K, g.tri);
+    for (int64_t i = 0; i < g.M; i += pc.mc)
+        for (int64_t j = 0; j < g.N; j += pc.nc)
+            for (int64_t k = 0; k < g.K; k += pc.kc) {
+                DigitGemm<T> d = g;
+                d.M = g.M - i < pc.mc ? g.M - i : pc.mc;
+                d.N = g.N - j < pc.nc ? g.N - j : pc.nc;
+                d.K = g.K - k < pc.kc ? g.K - k : pc.kc;
+                d.A = g.am ? g.A + i + k * g.lda : g.A + k + i * g.lda;
+                d.B = g.bc ? g.B + k + j * g.ldb : g.B + j + k * g.ldb;
+                d.C = g.cl ? g.C + i + j * g.ldc : g.C + j + i * g.ldc;
+                if (k > 0) d.alpha = T(1);
+                // a ragged last piece needs no more than the full one
+                GB_TRY(digit_piece<T>(d, ws, ws_bytes, pc.split, s));
+            }
+    return 0;
+}
+
+template bool digit_gemm_wanted<double>(int64_t, int64_t, int64_t, int);
+template bool digit_gemm_wanted<float>(int64_t, int64_t, int64_t, int);
+template size_t digit_gemm_bytes<double>(int64_t, int64_t, int64_t, int);
+template size_t digit_gemm_bytes<float>(int64_t, int64_t, int64_t, int);
+template int launch_digit_gemm<double>(const DigitGemm<double> &, char *, size_t, cudaStream_t);
+template int launch_digit_gemm<float>(const DigitGemm<float> &, char *, size_t, cudaStream_t);
+
+}  // namespace gb

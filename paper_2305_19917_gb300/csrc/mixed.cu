@@ -33,6 +33,8 @@
 #include <cuda_fp8.h>
 #include "common.cuh"
 #include "driver.cuh"
+#include "fixed.cuh"
+#include "gemm_digits.cuh"
 #include "mixed.cuh"
 
 namespace gb {
@@ -66,12 +68,6 @@ constexpr int kZSlots = 3;
 constexpr int kBand = 128;     // FP32 band of diagonal 128-blocks (column-major per block)
 constexpr int kLeaf = 1024;    // default leaf order of the BF16 low-precision solve (one leaf kernel launch each)
 
-// Library fallback of the integer-built conversions below, for results
-// outside the normal double range.  Kept out of line: inlined, the compiler
-// may evaluate it on every element (its int -> double conversion and scaling
-// run on the FP64 pipe) and select the result afterwards.
-__device__ __noinline__ double ldexp_i64_slow(long long t, int e) { return ldexp(static_cast<double>(t), e); }
-
 // z * 2^e as a double for |z| < 2^31 (exact: no rounding), built with 32-bit
 // integer operations (an int -> double conversion runs on the FP64 pipe,
 // which retires two operations per clock and SM); results outside the
@@ -88,31 +84,6 @@ __device__ __forceinline__ double scaled_i32_to_f64(int z, int e)
     const unsigned hi = sign | (unsigned(ex + 1023) << 20) | (m >> 12);
     const unsigned lo = m << 20;
     return __hiloint2double(int(hi), int(lo));
-}
-
-// T * 2^e rounded to the nearest double (ties to even), i.e. the value of
-// ldexp((double)T, e), for |T| < 2^63, built with integer operations (the
-// FP64 pipe retires two operations per clock and SM); results outside the
-// normal exponent range take the library path.
-__device__ __forceinline__ double scaled_i64_to_f64(long long T, int e)
-{
-    if (T == 0) return 0.0;
-    const unsigned long long sign = T < 0 ? (1ull << 63) : 0ull;
-    const unsigned long long u = T < 0 ? 0ull - static_cast<unsigned long long>(T) : static_cast<unsigned long long>(T);
-    const int lz = __clzll(static_cast<long long>(u));
-    int msb = 63 - lz;
-    const unsigned long long m = u << lz;  // leading one at bit 63
-    unsigned long long keep = m >> 11;     // 53 significant bits
-    const unsigned long long rem = m & 0x7FFull;
-    if (rem > 0x400ull || (rem == 0x400ull && (keep & 1ull))) keep++;
-    if (keep >> 53) {  // rounded up to the next power of two
-        keep >>= 1;
-        msb++;
-    }
-    const int ex = msb + e;
-    if (ex < -1022 || ex > 1023) return ldexp_i64_slow(T, e);
-    return __longlong_as_double(static_cast<long long>(sign | (static_cast<unsigned long long>(ex + 1023) << 52) |
-                                                       (keep & ((1ull << 52) - 1))));
 }
 
 // x rounded to the nearest float (ties to even), as __double2float_rn(x),
@@ -215,12 +186,6 @@ __device__ void load_tile(const View &v, int64_t i0, int64_t c0, double (*t)[65]
 // diagonal block of i0 (the residual kernel reads up to that column).
 __device__ __forceinline__ bool tile_needed(int64_t i0, int64_t c0) { return c0 < ((i0 >> 7) << 7) + 128; }
 
-// Biased binary exponent field of a double (0 for zero / subnormal).
-__device__ __forceinline__ int bexp(double a)
-{
-    return int((static_cast<unsigned long long>(__double_as_longlong(a)) >> 52) & 0x7FF);
-}
-
 // Pass 1: row exponents.  e_i = E + 2 where 2^E <= max_{c<i} |Mv'(i,c)| <
 // 2^(E+1), so every strictly-lower entry satisfies |a| < 2^(e_i - 1): the
 // strictly lower part only, so that small off-diagonal entries keep all their
@@ -298,20 +263,6 @@ __device__ __forceinline__ long long fixed48(double a, int e)
     return (b >> 63) ? -n : n;
 }
 
-// Balanced base-256 digit of x: the d in [-128, 127] with d = x (mod 256).
-__device__ __forceinline__ int bal8(int x) { return ((x + 128) & 255) - 128; }
-// The FP32 bit pattern of an integer |d| < 2^22, exactly: d added to the
-// integer bits of 1.5 2^23 adds d to that value, which is then subtracted.
-__device__ __forceinline__ uint32_t small_int_f32bits(int d)
-{
-    return __float_as_uint(__int_as_float(0x4B400000 + d) - 12582912.0f);
-}
-// Two BF16 in one word from FP32 patterns whose low 16 bits are zero (the
-// high halves are then the BF16 values exactly): lo_elem first.
-__device__ __forceinline__ uint32_t pack_hi16(uint32_t lo_elem, uint32_t hi_elem)
-{
-    return __byte_perm(lo_elem, hi_elem, 0x7632);
-}
 // Round-to-nearest-even BF16 bit pattern of a double, from the two 32-bit
 // halves of its bit pattern (as d2bf16: results below the BF16 normal range
 // flush to zero, overflow gives infinity, NaN stays NaN).
@@ -1162,9 +1113,10 @@ extern "C" int gb_mixed_workspace_release(void *stream)
     GB_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return GB_STATUS_CUDA_ERROR;
     gb::DeviceWorkspace &w = gb::g_ws[dev];
-    if (!w.base) return 0;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     GB_CUDA(cudaStreamSynchronize(s));
+    gb::digit_pool_trim();
+    if (!w.base) return 0;
     GB_CUDA(cudaFreeAsync(w.base, s));
     w.base = nullptr;
     w.size = 0;

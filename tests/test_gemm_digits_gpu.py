@@ -1,0 +1,113 @@
+"""The off-diagonal update by digit products on the tensor cores
+(gb_gemm_update's path from K = 64 in FP64, from K = 128 in FP32) against
+numpy in extended precision: tile and chunk edges, the split of K, both
+factors' layouts (through the solve's other tests) and the inputs that the
+digits must leave to the CUDA cores.
+
+Tolerance, from the format: a factor is rounded at 2^-(8P+1) of its row's
+(column's) scale, at most twice the largest entry (P = 7 digits FP64, 3
+FP32), the pairs left out add (P - 1) 2^(14-8(P+2)) of the scales' product per
+term at most, and the tiles taken by digits hold at least K/4 terms of 2^-10
+of the largest product each: |error| <= 2^-41 (FP64), 2^-13 (FP32) of
+sum |a||x| in the worst case.  Dense random factors stay far below it: the
+factors' roundings are independent, about 2^-(8P) of sqrt(K) products, checked
+as 2^-50 and 2^-21 of the factors' norms (CUDA-core sums round K times)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+WORST = {0: 2.0 ** -41, 1: 2.0 ** -13}
+NORM = {0: 2.0 ** -50, 1: 2.0 ** -21}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2305_19917_gb300 import build
+    build.build()
+
+
+def _update(dtype, A, B, C, alpha):
+    import torch
+    from paper_2305_19917_gb300 import api
+    td = torch.float64 if dtype == 0 else torch.float32
+    dev = [api.to_device_colmajor(x, td) for x in (A, B, C)]
+    (M, K), N = A.shape, B.shape[1]
+    st = api.gb_gemm_update(dtype, M, N, K, dev[0].data_ptr(), M, dev[1].data_ptr(), K, dev[2].data_ptr(), M, alpha,
+                            torch.cuda.current_stream().cuda_stream)
+    assert st == 0
+    torch.cuda.synchronize()
+    return dev[2].cpu().numpy()
+
+
+def _factors(dtype, M, N, K, seed):
+    nt = np.float64 if dtype == 0 else np.float32
+    r = np.random.default_rng(seed)
+    return (r.uniform(-1, 1, (M, K)).astype(nt), r.standard_normal((K, N)).astype(nt),
+            r.standard_normal((M, N)).astype(nt))
+
+
+SIZES = [(1, 1, 128), (128, 128, 128), (129, 127, 191), (64, 300, 256), (127, 1, 257), (33, 65, 1000), (300, 260, 2100)]
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+@pytest.mark.parametrize("M,N,K", SIZES + [(100, 77, 64), (70, 50, 17000)])
+def test_dense_factors(dtype, M, N, K):
+    A, B, C = _factors(dtype, M, N, K, seed=M + N + K)
+    A *= np.exp2(np.arange(M) % 40 - 20).astype(A.dtype)[:, None]  # every row its own scale
+    got = _update(dtype, A, B, C, 0.5)
+    L = np.longdouble
+    prod = A.astype(L) @ B.astype(L)
+    bound = np.abs(A).astype(L) @ np.abs(B).astype(L)
+    u = L(2.0) ** (-53 if dtype == 0 else -24)
+    err = np.abs(got - (L(0.5) * C - prod))
+    assert np.all(err <= WORST[dtype] * bound + 2 * u * np.abs(got))
+    # sqrt(K) products: per row, |a_i| |B| in the 2-norms, and the old C
+    rows = np.sqrt(np.sum(A.astype(L) ** 2, axis=1)) * np.sqrt(np.sum(B.astype(L) ** 2))
+    rows += np.sqrt(np.sum(C.astype(L) ** 2, axis=1))
+    assert np.all(np.sqrt(np.sum(err ** 2, axis=1)) <= NORM[dtype] * rows * max(1.0, K / 4096))
+
+
+def _graded(A, B):
+    A[:, ::2] *= 2.0 ** -30   # large entries of A meet ...
+    B[1::2, :] *= 2.0 ** -30  # ... small ones of B: sum |a||x| is 2^-30 of the largest product
+
+
+def _sparse(A, B):
+    A[:, : A.shape[1] * 7 // 8] = 0
+
+
+def _infinite(A, B):
+    B[3, 5] = np.inf
+    A[7, 11] = np.nan
+
+
+def _huge(A, B):
+    e = 500 if A.dtype == np.float64 else 60
+    A *= A.dtype.type(2.0) ** e
+    B *= A.dtype.type(2.0) ** -e
+
+
+def _subnormal(A, B):
+    A[9, :] = np.finfo(A.dtype).smallest_subnormal * 5
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+@pytest.mark.parametrize("change", [_graded, _sparse, _infinite, _huge, _subnormal])
+def test_what_digits_cannot_hold(dtype, change):
+    """These tiles are computed by the CUDA cores: componentwise K u."""
+    M, N, K = 200, 300, 520
+    A, B, C = _factors(dtype, M, N, K, seed=5)
+    change(A, B)
+    C[:] = 0
+    got = _update(dtype, A, B, C, 1.0)
+    L = np.longdouble
+    with np.errstate(all="ignore"):
+        want = -(A.astype(L) @ B.astype(L))
+        bound = np.abs(A).astype(L) @ np.abs(B).astype(L)
+    ok = np.isfinite(want.astype(np.float64)) & np.isfinite(bound.astype(np.float64))
+    # an infinity reaches its column (or row) and nothing else
+    assert np.array_equal(np.isfinite(got), ok)
+    u = 2.0 ** (-53 if dtype == 0 else -24)
+    tiny = np.finfo(A.dtype).smallest_subnormal
+    assert np.all(np.abs(got - want)[ok] <= K * (u * bound[ok] + tiny))
