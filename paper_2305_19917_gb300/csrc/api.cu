@@ -8,6 +8,7 @@
 #include "common.cuh"
 #include "driver.cuh"
 #include "gemm_digits.cuh"
+#include "panel.cuh"
 #include "plan.cuh"
 
 namespace gb {
@@ -34,16 +35,31 @@ int side_stream(cudaStream_t *out)
     return 0;
 }
 
-// A TS task larger than the diagonal kernel (64 rows) is itself solved: by
-// the recursive model down to that kernel, whose updates are wide enough for
-// the digit gemm, or, for a plan that asks for smaller blocks, blocked by
-// them.
-constexpr int64_t kTsRows = 64;
+// Rows of the largest TS task solved by one kernel: the panel kernel's (FP64
+// 512, FP32 1024), halved while its multiply-adds outside the two halves (r^2 / 4
+// per right-hand side, FP64 252 per clock on the whole chip, FP32 about 10000)
+// take longer than the digit gemm that would replace them (50 and 30 us at
+// these sizes).  FP64 beyond 2432 right-hand sides: the 64-row diagonal kernel
+// (512 rows: 2400 right-hand sides 504 us with panels, 607 with it; 4096 962
+// with panels of 16, 646 with it).
+template <typename T>
+int64_t ts_rows(int64_t ncols)
+{
+    if (sizeof(T) == 8 && ncols > 2432) return 64;
+    const double split = sizeof(T) == 8 ? 1.0e8 : 2.3e9;
+    int64_t r = kPanelRows<T>;
+    while (r > 64 && double(r) * double(r) * double(ncols) > split) r /= 2;
+    return r;
+}
+
+// A larger TS task is itself solved: by the recursive model down to such
+// tasks, whose updates are wide enough for the digit gemm, or, for a plan
+// that asks for smaller blocks, blocked by them.
 template <class E, typename T>
 void expand_ts(E &e, int64_t b0, int64_t nr, int64_t nb, T a, bool fwd)
 {
-    if (nb < kTsRows) drive_blocked(e, b0, b0 + nr, nb, a, fwd);
-    else drive_recursive(e, b0, b0 + nr, 24, kTsRows, a, fwd);
+    if (nb < 64) drive_blocked(e, b0, b0 + nr, nb, a, fwd);
+    else drive_recursive(e, b0, b0 + nr, 24, ts_rows<T>(e.columns()), a, fwd);
 }
 
 // Executor that finds the work space of a schedule's largest digit gemm.
@@ -53,9 +69,10 @@ struct DigitBytesExec {
     bool forward;
     size_t bytes = 0;
     bool ok() const { return true; }
+    int64_t columns() const { return ncols; }
     void ts(int64_t b0, int64_t nr, T a)
     {
-        if (nr > kTsRows) expand_ts(*this, b0, nr, nb, a, forward);
+        if (nr > ts_rows<T>(ncols)) expand_ts(*this, b0, nr, nb, a, forward);
     }
     void gemm(int64_t, int64_t M, int64_t, int64_t K, T)
     {
@@ -98,6 +115,7 @@ struct LaunchExec {
         if (ev_tail) cudaEventDestroy(ev_tail);
     }
     bool ok() const { return status == 0; }
+    int64_t columns() const { return c.ncols; }
     int enable_lookahead()
     {
         GB_TRY(side_stream(&side));
@@ -123,9 +141,11 @@ struct LaunchExec {
     void ts(int64_t b0, int64_t nr, T a)
     {
         if (status) return;
-        if (nr <= kTsRows) {
+        if (nr <= ts_rows<T>(c.ncols)) {
             settle(b0, b0 + nr);
-            if (!status) status = launch_diag_solve(c, b0, (int)nr, a);
+            if (status) return;
+            if (sizeof(T) == 8 && c.ncols > 2432) status = launch_diag_solve(c, b0, (int)nr, a);
+            else status = launch_panel_solve(c, b0, (int)nr, a);
             return;
         }
         expand_ts(*this, b0, nr, nb, a, c.forward);

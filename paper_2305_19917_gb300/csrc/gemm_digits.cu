@@ -163,7 +163,7 @@ struct DigitSrc {
 // the tile comes from L2.
 template <typename T>
 __global__ void __launch_bounds__(DTHREADS, sizeof(T) == 8 ? 3 : 4)
-digits_kernel(DigitSrc<T> a, DigitSrc<T> x, int ablocks, int K, int kp, int *zero, int nzero)
+digits_kernel(DigitSrc<T> a, DigitSrc<T> x, int ablocks, int K, int kp, int *zero, int nzero, ulonglong2 *sums, int64_t nsums)
 {
     constexpr int P = Fmt<T>::P;
     __shared__ T t[DROWS][65];
@@ -184,9 +184,13 @@ digits_kernel(DigitSrc<T> a, DigitSrc<T> x, int ablocks, int K, int kp, int *zer
     }
     tc::pdl_wait();
     tc::pdl_launch_dependents();
-    // the tiles' words of pass 2
-    for (int z = (blockIdx.x * gridDim.y + blockIdx.y) * DTHREADS + tid; z < nzero; z += gridDim.x * gridDim.y * DTHREADS)
-        zero[z] = 0;
+    // the tiles' words and sums of pass 2
+    {
+        const int64_t z0 = int64_t(blockIdx.x * gridDim.y + blockIdx.y) * DTHREADS + tid;
+        const int64_t step = int64_t(gridDim.x) * gridDim.y * DTHREADS;
+        for (int64_t z = z0; z < nzero; z += step) zero[z] = 0;
+        for (int64_t z = z0; z < nsums; z += step) sums[z] = make_ulonglong2(0ull, 0ull);
+    }
     __syncthreads();
     auto load = [&](int tile, T (&v)[8]) {
         const int kb = tile * BK;
@@ -243,7 +247,7 @@ digits_kernel(DigitSrc<T> a, DigitSrc<T> x, int ablocks, int K, int kp, int *zer
     int near = 0;
     const size_t plane = size_t(s.rp) * size_t(kp);
     for (int tile = t0; tile < t1; tile++) {
-        load(tile, v);
+        if (t1 - t0 > 1) load(tile, v);  // (a single tile is still in registers)
         __syncthreads();  // the previous tile has been read
 #pragma unroll
         for (int u = 0; u < 8; u++) {
@@ -318,7 +322,7 @@ struct TileWords {
 template <typename T>
 struct MmaArgs {
     DigitGemm<T> g;
-    long long *Tg;      // split > 1: planes of tile-blocked partial sums (128 x 128, column-major)
+    long long *Tg;      // split > 1: the tiles' sums (128 x 128, column-major), cleared by pass 1
     const int *cnt_a, *cnt_x, *e_a, *e_x;
     TileWords w;
     int kp, nMt, nNt, ntiles, W, split;
@@ -348,9 +352,9 @@ __device__ __forceinline__ float scale_sum(float, long long t, int e)
     return __ll2float_rn(t) * __int_as_float((e + 127) << 23);
 }
 
-// One work item of a CTA: a tile and a share of its K chunks.
+// One work item of a CTA: a tile and a share [k0, k1) of K, taken in chunks of KC.
 struct Item {
-    int tile, i0, j0, sp, ch0, ch1;
+    int tile, i0, j0, sp, k0, k1;
     bool skip;  // the digits may not represent this tile
 };
 // Evaluated by every warp for itself (all lanes).
@@ -364,9 +368,9 @@ __device__ __forceinline__ Item digit_item(const MmaArgs<T> &a, int w, int lane)
     digit_tile(it.tile, a.nMt, a.nNt, a.g.tri, m, n);
     it.i0 = m * BM;
     it.j0 = n * BM;
-    const int nch = (a.kp + KC - 1) / KC, per = (nch + a.split - 1) / a.split;
-    it.ch0 = min(it.sp * per, nch);
-    it.ch1 = min(it.ch0 + per, nch);
+    const int kt = a.kp / BK, per = (kt + a.split - 1) / a.split;
+    it.k0 = min(it.sp * per, kt) * BK;
+    it.k1 = min(it.k0 + per * BK, a.kp);
     const int4 ca = reinterpret_cast<const int4 *>(a.cnt_a + it.i0)[lane];
     const int4 cx = reinterpret_cast<const int4 *>(a.cnt_x + it.j0)[lane];
     const int ma = __reduce_min_sync(0xffffffffu, min(min(ca.x, ca.y), min(ca.z, ca.w)));
@@ -450,8 +454,8 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             const Item it = digit_item(a, w, lane);
             if (it.skip) continue;
             if (lane == 0) {
-                for (int c = it.ch0; c < it.ch1 && ok; c++) {
-                    const int kb = c * KC, ke = min(kb + KC, a.kp);
+                for (int kb = it.k0; kb < it.k1 && ok; kb += KC) {
+                    const int ke = min(kb + KC, it.k1);
                     for (int o = 0; o < S::NO && ok; o++) {
                         const int p = S::p(o), q = S::q(o);
                         const bool two = o < S::TWO;
@@ -495,8 +499,8 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             const Item it = digit_item(a, w, lane);
             if (it.skip) continue;
             if (lane == 0) {
-                for (int c = it.ch0; c < it.ch1 && ok; c++) {
-                    const int kb = c * KC, ke = min(kb + KC, a.kp);
+                for (int kb = it.k0; kb < it.k1 && ok; kb += KC) {
+                    const int ke = min(kb + KC, it.k1);
                     const int nk = (ke - kb) / BK;
                     for (int j = 0; j < S::NP && ok; j++, cp++) {
                         const int buf = cp & 1;
@@ -557,7 +561,7 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         if (s >= 0) bias += kIntBias << s;
                         else if (h == 1) bias += kIntBias;
                     }
-                bias *= (unsigned long long)(it.ch1 - it.ch0);
+                bias *= (unsigned long long)((it.k1 - it.k0 + KC - 1) / KC);
 #pragma unroll
                 for (int c = 0; c < 32; c++) T64[c] = static_cast<long long>(0ull - bias);
             }
@@ -581,7 +585,7 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     }
                 }
             };
-            for (int c = it.ch0; c < it.ch1 && ok; c++) {
+            for (int kb = it.k0; kb < it.k1 && ok; kb += KC) {
 #pragma unroll 1
                 for (int j = 0; j < S::NP; j++, cp++) {
                     const int buf = cp & 1;
@@ -628,12 +632,11 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             }
             const int row = q * 32 + lane;
             if (a.split > 1) {
-                // the partial sums of this share; the CTA that stores the
-                // tile's last one adds them all up (integers: in any order)
-                const size_t plane = size_t(a.ntiles) * (BM * BM);
-                long long *o = a.Tg + size_t(it.tile) * (BM * BM) + row + cg * 32 * BM;
+                // the partial sums of this share are added into the tile's
+                // (integers: in any order); the CTA that comes last finishes
+                auto *o = reinterpret_cast<unsigned long long *>(a.Tg) + size_t(it.tile) * (BM * BM) + row + cg * 32 * BM;
 #pragma unroll
-                for (int c = 0; c < 32; c++) __stcg(o + it.sp * plane + c * BM, T64[c]);
+                for (int c = 0; c < 32; c++) atomicAdd(o + c * BM, static_cast<unsigned long long>(T64[c]));
                 __threadfence();
                 asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS) : "memory");
                 if (first) last_flag = atomicAdd(&a.w.done[it.tile], 1) == a.split - 1;
@@ -641,11 +644,8 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 const bool last = last_flag != 0;
                 if (!last) continue;
                 __threadfence();
-                for (int sp = 0; sp < a.split; sp++) {
-                    if (sp == it.sp) continue;
 #pragma unroll
-                    for (int c = 0; c < 32; c++) T64[c] += __ldcg(o + sp * plane + c * BM);
-                }
+                for (int c = 0; c < 32; c++) T64[c] = static_cast<long long>(__ldcg(o + c * BM));
             }
             const DigitGemm<T> &g = a.g;
             const int64_t i = int64_t(it.i0) + row, jb = int64_t(it.j0) + cg * 32;
@@ -763,20 +763,21 @@ size_t piece_bytes(int64_t M, int64_t N, int64_t K, int tri, int split)
     constexpr int P = Fmt<T>::P;
     const size_t mp = size_t(up(M, BM)), np = size_t(up(N, BM)), kp = size_t(up(K, BK));
     const size_t nt = tri ? (mp / BM) * (mp / BM + 1) / 2 : (mp / BM) * (np / BM);
-    size_t b = 256 + 2 * P * mp * kp + (tri ? 0 : 2 * P * np * kp) + (split > 1 ? size_t(split) * nt * BM * BM * 8 : 0);
+    size_t b = 256 + 2 * P * mp * kp + (tri ? 0 : 2 * P * np * kp) + (split > 1 ? nt * BM * BM * 8 : 0);
     b += 4 * (2 * mp + 2 * np) + 4 * (3 * nt + 2) + 8 * 256;
     return b;
 }
 
-// K is split over CTAs (with a plane of sums each) while the tiles alone leave
-// SMs idle and a CTA keeps at least two chunks of 256.
+// K is split over CTAs, down to 64 of it each, while the tiles alone leave SMs
+// idle: 9 tiles of K = 512 on 72 CTAs instead of 9.
 inline int pick_split(int64_t ntiles, int64_t K)
 {
-    const int64_t nch = (K + KC - 1) / KC;
+    const int64_t kt = (K + BK - 1) / BK;
     int64_t s = 152 / ntiles;
-    if (s > nch / 2) s = nch / 2;
-    if (s > 8) s = 8;
-    return s < 1 ? 1 : int(s);
+    if (s > kt) s = kt;
+    if (s < 2) return 1;
+    const int64_t per = (kt + s - 1) / s;
+    return int((kt + per - 1) / per);
 }
 
 template <typename T>
@@ -827,7 +828,7 @@ int digit_piece(const DigitGemm<T> &g, char *ws, size_t ws_bytes, int split, cud
     };
     __nv_bfloat16 *da = reinterpret_cast<__nv_bfloat16 *>(take(size_t(2) * P * mp * kp));
     __nv_bfloat16 *dx = g.tri ? da : reinterpret_cast<__nv_bfloat16 *>(take(size_t(2) * P * np * kp));
-    long long *Tg = reinterpret_cast<long long *>(take(split > 1 ? size_t(split) * nt * BM * BM * 8 : 0));
+    long long *Tg = reinterpret_cast<long long *>(take(split > 1 ? size_t(nt) * BM * BM * 8 : 0));
     int *ea = reinterpret_cast<int *>(take(4 * size_t(mp))), *ca = reinterpret_cast<int *>(take(4 * size_t(mp)));
     int *ex = g.tri ? ea : reinterpret_cast<int *>(take(4 * size_t(np)));
     int *cx = g.tri ? ca : reinterpret_cast<int *>(take(4 * size_t(np)));
@@ -859,7 +860,7 @@ int digit_piece(const DigitGemm<T> &g, char *ws, size_t ws_bytes, int split, cud
         const int ab = int(mp / DROWS), xb = g.tri ? 0 : int(np / DROWS);
         const int64_t ktiles = kp / BK;
         int cl = 1;
-        while (cl < kMaxCluster && ktiles >= 4 * cl && int64_t(ab + xb) * cl < 1216) cl *= 2;
+        while (cl < kMaxCluster && ktiles >= (int64_t(ab + xb) * cl < 304 ? 2 : 4) * cl && int64_t(ab + xb) * cl < 1216) cl *= 2;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(ab + xb), (unsigned)cl);
         cfg.blockDim = dim3(DTHREADS);
@@ -873,7 +874,8 @@ int digit_piece(const DigitGemm<T> &g, char *ws, size_t ws_bytes, int split, cud
         attr[1].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 2;
-        GB_CUDA(cudaLaunchKernelEx(&cfg, digits_kernel<T>, sa, sx, ab, int(g.K), int(kp), words, int(2 * nt + 1)));
+        GB_CUDA(cudaLaunchKernelEx(&cfg, digits_kernel<T>, sa, sx, ab, int(g.K), int(kp), words, int(2 * nt + 1),
+                                   reinterpret_cast<ulonglong2 *>(Tg), split > 1 ? nt * (BM * BM / 2) : int64_t(0)));
     }
     {
         static PerDeviceOnce attr;

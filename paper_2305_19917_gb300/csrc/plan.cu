@@ -1,7 +1,7 @@
 // Planner: picks driver, block size nb and recursion depth for a shape.
 //
 // Without a cost model the built-in default is used (recursive halving to
-// leaves of ~512 rows, blocked leaves with nb = 64).  With a model loaded
+// leaves of ~512 rows).  With a model loaded
 // (gb_plan_set_model) every candidate of the standard set is scored by the
 // cost-model network on the GPU (one inference launch over all candidates)
 // and the argmin of the predicted time is taken; the choice is cached per
@@ -26,20 +26,18 @@ namespace {
 constexpr int kFeat = 17;
 const int kNbs[6] = {16, 32, 64, 128, 256, 512};
 
+// One TS task up to the panel kernel's order (512 rows, FP32 1024), else
+// recursive halving to tasks of at least 512 rows, which are solved down to
+// the panel or diagonal kernel's rows inside (api.cu).
 gb_plan default_plan(int dtype, int64_t k)
 {
-    (void)dtype;
     gb_plan p;
     p.reserved = 0;
-    p.nb = 64;
-    if (k <= 512) {
-        p.driver = GB_DRIVER_BLOCKED;
-        p.depth = 0;
-        return p;
-    }
-    int d = 0;
-    while ((k >> (d + 1)) >= 512 && d < 8) d++;
+    p.nb = 512;
     p.driver = GB_DRIVER_RECURSIVE;
+    int d = 0;
+    if (k > (dtype == GB_DTYPE_F32 ? 1024 : 512))
+        while ((k >> (d + 1)) >= 512 && d < 8) d++;
     p.depth = d;
     return p;
 }
