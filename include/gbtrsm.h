@@ -281,13 +281,14 @@ int gb_gemm_update(int dtype, int64_t M, int64_t N, int64_t K, const void *A,
 /*
  * gb_dpotrf / gb_spotrf: Cholesky factorisation on this library's
  * triangular solve -- the use the paper names for its TS machinery (Section
- * VIII, future work), with the recursive computation model of Section V-A:
- * split A's order in two (first part a multiple of 64), factorise the first
- * diagonal block, solve the off-diagonal panel against it with gb_dtrsm /
- * gb_strsm (side Right, Lower, transposed: L21 = A21 L11^-T; or side Left,
- * Upper, transposed: U12 = U11^-T A12), update the trailing block by a SYRK
- * (A22 -= L21 L21^T, or U12^T U12; its triangle only), recurse; leaves of at
- * most 64 columns are factorised by one CTA in shared memory.
+ * VIII, future work), with the recursive computation model of Section V-A on
+ * panels of columns that reach down to the last row: the left half (its
+ * columns a multiple of 64), the update of the right half's entries on and
+ * below the diagonal by the left half's rows (the gemm task), the right half;
+ * panels of at most 64 columns: the diagonal block by one CTA in shared
+ * memory, the rows below it by gb_dtrsm / gb_strsm (side Right, Lower,
+ * transposed: L21 = A21 L11^-T; or side Left, Upper, transposed: U12 =
+ * U11^-T A12).  Work space as for gb_dtrsm.
  *   1 uplo   GB_LOWER: A = L L^T, L over the lower triangle;
  *            GB_UPPER: A = U^T U, U over the upper triangle
  *   2 n      order of A, >= 0

@@ -150,6 +150,12 @@ template <typename T>
 int launch_gemm_update(const Canon<T> &c, int64_t ci0, int64_t M, int64_t ak0,
                        int64_t K, T alpha);
 
+// C -= P P[0:N, :]^T on and below the diagonal of C (M x N, N <= M; P is M x K;
+// am false: P and C stored transposed).
+template <typename T>
+int launch_gemm_trapezoid(bool am, int64_t M, int64_t N, int64_t K, const T *P, int64_t ldp, T *C, int64_t ldc,
+                          cudaStream_t s);
+
 // Bv = 0 (alpha == 0 quick path).
 template <typename T>
 int launch_zero(const Canon<T> &c);

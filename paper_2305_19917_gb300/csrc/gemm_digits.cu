@@ -330,19 +330,27 @@ struct MmaArgs {
 };
 
 // Tile (m, n) number t of the launch: grouped rasterisation of the full
-// grid, or the triangle's tiles (a >= b; lower: m = a, upper: n = a).
+// grid, or of the trapezoid n <= m, its triangle first.
 __device__ __forceinline__ void digit_tile(int t, int nMt, int nNt, int tri, int &m, int &n)
 {
-    if (tri == 0) {
-        tc::raster_grouped(t, nMt, nNt, 8, m, n);
+    if (tri) {
+        const int head = nNt * (nNt + 1) / 2;
+        if (t < head) {
+            m = int((sqrtf(8.0f * float(t) + 1.0f) - 1.0f) * 0.5f);
+            while (m * (m + 1) / 2 > t) m--;
+            while ((m + 1) * (m + 2) / 2 <= t) m++;
+            n = t - m * (m + 1) / 2;
+            return;
+        }
+        tc::raster_grouped(t - head, nMt - nNt, nNt, 8, m, n);
+        m += nNt;
         return;
     }
-    int a = int((sqrtf(8.0f * float(t) + 1.0f) - 1.0f) * 0.5f);
-    while (a * (a + 1) / 2 > t) a--;
-    while ((a + 1) * (a + 2) / 2 <= t) a++;
-    const int b = t - a * (a + 1) / 2;
-    m = tri == 1 ? a : b;
-    n = tri == 1 ? b : a;
+    tc::raster_grouped(t, nMt, nNt, 8, m, n);
+}
+inline int64_t digit_tiles(int64_t nMt, int64_t nNt, int tri)
+{
+    return tri ? nNt * (nNt + 1) / 2 + (nMt - nNt) * nNt : nMt * nNt;
 }
 
 __device__ __forceinline__ double scale_sum(double, long long t, int e) { return scaled_i64_to_f64(t, e); }
@@ -659,7 +667,7 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
                     for (int u = 0; u < 4; u++) {
                         const int64_t j = jb + c0 + u;
-                        in[u] = i < g.M && j < g.N && !(g.tri == 1 && j > i) && !(g.tri == 2 && j < i);
+                        in[u] = i < g.M && j < g.N && !(g.tri && j > i);
                         old[u] = in[u] ? g.C[i + j * g.ldc] : T(0);
                     }
 #pragma unroll
@@ -686,13 +694,13 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
                     for (int u = 0; u < NC; u++) {
                         const int64_t ii = int64_t(it.i0) + q * 32 + lane / NC + u * LPR;
-                        const bool in = ii < g.M && j < g.N && !(g.tri == 1 && j > ii) && !(g.tri == 2 && j < ii);
+                        const bool in = ii < g.M && j < g.N && !(g.tri && j > ii);
                         old[u] = in ? g.C[j + ii * g.ldc] : T(0);
                     }
 #pragma unroll
                     for (int u = 0; u < NC; u++) {
                         const int64_t ii = int64_t(it.i0) + q * 32 + lane / NC + u * LPR;
-                        const bool in = ii < g.M && j < g.N && !(g.tri == 1 && j > ii) && !(g.tri == 2 && j < ii);
+                        const bool in = ii < g.M && j < g.N && !(g.tri && j > ii);
                         const T v = xp[(lane / NC + u * LPR) * LX + lane % NC];
                         if (in) g.C[j + ii * g.ldc] = (g.alpha == T(1)) ? old[u] - v : g.alpha * old[u] - v;
                     }
@@ -725,7 +733,7 @@ digit_fallback_kernel(DigitGemm<T> g, TileWords w, int nMt, int nNt)
         int m_blk, n_blk;
         digit_tile(tile, nMt, nNt, g.tri, m_blk, n_blk);
         const int64_t i0 = int64_t(m_blk) * BM + (sub % PER) * FB, j0 = int64_t(n_blk) * BM + (sub / PER) * FB;
-        if (i0 >= g.M || j0 >= g.N || (g.tri == 1 && j0 > i0 + FB - 1) || (g.tri == 2 && i0 > j0 + FB - 1)) continue;
+        if (i0 >= g.M || j0 >= g.N || (g.tri && j0 > i0 + FB - 1)) continue;
         gemm_tile<T, AM, BC, CL>(smem, i0, j0, g.M, g.N, g.K, g.A, g.lda, g.B, g.ldb, g.C, g.ldc, g.alpha, g.tri);
         __syncthreads();
     }
@@ -762,7 +770,7 @@ size_t piece_bytes(int64_t M, int64_t N, int64_t K, int tri, int split)
 {
     constexpr int P = Fmt<T>::P;
     const size_t mp = size_t(up(M, BM)), np = size_t(up(N, BM)), kp = size_t(up(K, BK));
-    const size_t nt = tri ? (mp / BM) * (mp / BM + 1) / 2 : (mp / BM) * (np / BM);
+    const size_t nt = size_t(digit_tiles(int64_t(mp / BM), int64_t(np / BM), tri));
     size_t b = 256 + 2 * P * mp * kp + (tri ? 0 : 2 * P * np * kp) + (split > 1 ? nt * BM * BM * 8 : 0);
     b += 4 * (2 * mp + 2 * np) + 4 * (3 * nt + 2) + 8 * 256;
     return b;
@@ -787,13 +795,13 @@ Piece plan_piece(int64_t M, int64_t N, int64_t K, int tri)
     p.kc = K < kMaxK ? K : kMaxK;
     p.mc = M;
     p.nc = N;
-    // halve the longer of the two extents until the piece fits (a triangle is not cut)
+    // halve the longer of the two extents until the piece fits (of a triangle, K)
     while (!tri && piece_bytes<T>(p.mc, p.nc, p.kc, 0, 1) > kWsCap && (p.mc > 1024 || p.nc > 1024)) {
         if (p.nc >= p.mc) p.nc = up((p.nc + 1) / 2, BM);
         else p.mc = up((p.mc + 1) / 2, BM);
     }
-    const int64_t mt = up(p.mc, BM) / BM, nt = up(p.nc, BM) / BM;
-    p.split = pick_split(tri ? mt * (mt + 1) / 2 : mt * nt, p.kc);
+    while (tri && piece_bytes<T>(M, N, p.kc, 1, 1) > kWsCap && p.kc > 1024) p.kc = up((p.kc + 1) / 2, BK);
+    p.split = pick_split(digit_tiles(up(p.mc, BM) / BM, up(p.nc, BM) / BM, tri), p.kc);
     p.bytes = piece_bytes<T>(p.mc, p.nc, p.kc, tri, p.split);
     return p;
 }
@@ -806,7 +814,8 @@ int launch_fallback(const DigitGemm<T> &g, const TileWords &w, int nMt, int nNt,
     else if (g.am && !g.bc && !g.cl) k = digit_fallback_kernel<T, true, false, false>;
     else if (!g.am && g.bc && g.cl) k = digit_fallback_kernel<T, false, true, true>;
     else if (!g.am && !g.bc && !g.cl) k = digit_fallback_kernel<T, false, false, false>;
-    else if (g.am && !g.bc && g.cl) k = digit_fallback_kernel<T, true, false, true>;  // P P^T
+    else if (g.am && !g.bc && g.cl) k = digit_fallback_kernel<T, true, false, true>;    // P P^T
+    else if (!g.am && g.bc && !g.cl) k = digit_fallback_kernel<T, false, true, false>;  // the same, stored transposed
     if (!k) return GB_STATUS_CUDA_ERROR;
     constexpr int PER = BM / GemmTile<T>::BM;
     const int grid = ntiles * PER * PER < 304 ? ntiles * PER * PER : 304;
@@ -817,9 +826,9 @@ template <typename T>
 int digit_piece(const DigitGemm<T> &g, char *ws, size_t ws_bytes, int split, cudaStream_t s)
 {
     constexpr int P = Fmt<T>::P;
-    const int64_t mp = up(g.M, BM), np = g.tri ? mp : up(g.N, BM), kp = up(g.K, BK);
+    const int64_t mp = up(g.M, BM), np = up(g.N, BM), kp = up(g.K, BK);
     const int nMt = int(mp / BM), nNt = int(np / BM);
-    const int64_t nt = g.tri ? int64_t(nMt) * (nMt + 1) / 2 : int64_t(nMt) * nNt;
+    const int64_t nt = digit_tiles(nMt, nNt, g.tri);
     size_t off = 0;
     auto take = [&](size_t b) {
         char *p = ws + off;
@@ -842,8 +851,10 @@ int digit_piece(const DigitGemm<T> &g, char *ws, size_t ws_bytes, int split, cud
         uint64_t dims[3] = {uint64_t(kp), uint64_t(mp), uint64_t(P)};
         uint64_t strides[2] = {uint64_t(kp) * 2, uint64_t(mp) * uint64_t(kp) * 2};
         GB_TRY(encode_tmap(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, da, dims, strides, box));
-        dims[1] = uint64_t(np);
-        strides[1] = uint64_t(np) * uint64_t(kp) * 2;
+        if (!g.tri) {
+            dims[1] = uint64_t(np);
+            strides[1] = uint64_t(np) * uint64_t(kp) * 2;
+        }
         GB_TRY(encode_tmap(&tx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, dx, dims, strides, box));
     }
     // weight of the sums: |T| <= 1.02 K 2^W < 2^63, at most 52 (the last weight

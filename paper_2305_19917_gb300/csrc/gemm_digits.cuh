@@ -10,8 +10,9 @@ namespace gb {
 // One update C = alpha*C - Aop*Bop, C of M x N, K products per entry.
 // am: Aop(i,k) = A[i + k lda] (else A[k + i lda]); bc: Bop(k,j) = B[k + j ldb]
 // (else B[j + k ldb]); cl: C(i,j) = C[i + j ldc] (else C[j + i ldc]).
-// tri: 0 all of C, 1 / 2 only its entries on and below / above the diagonal
-// (M == N; then Bop = Aop^T is read from the same digits, B is ignored).
+// tri: only the entries of C on and below its diagonal, with Bop = the first N
+// rows of Aop, transposed (N <= M; the same digits serve both; B and bc say
+// where the CUDA cores find it).
 template <typename T>
 struct DigitGemm {
     int64_t M, N, K;

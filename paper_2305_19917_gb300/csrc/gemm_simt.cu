@@ -20,6 +20,20 @@ gemm_update_kernel(int64_t M, int64_t N, int64_t K, const T *__restrict__ A, int
                                  M, N, K, A, lda, B, ldb, C, ldc, alpha, 0);
 }
 
+// The trapezoid of C on and below its diagonal, Bop = the first N rows of
+// Aop transposed: C(i, j) -= sum_k Aop(i, k) Aop(j, k).  AM: column-major
+// operands, else both stored transposed.
+template <typename T, bool AM>
+__global__ void __launch_bounds__(GemmTile<T>::NT)
+gemm_trapezoid_kernel(int64_t M, int64_t N, int64_t K, const T *__restrict__ P, int64_t ldp, T *__restrict__ C, int64_t ldc)
+{
+    constexpr int BM = GemmTile<T>::BM;
+    __shared__ __align__(16) T smem[gemm_tile_smem<T>()];
+    const int64_t m0 = int64_t(blockIdx.y) * BM, n0 = int64_t(blockIdx.x) * BM;
+    if (n0 > m0 + BM - 1) return;
+    gemm_tile<T, AM, !AM, AM>(smem, m0, n0, M, N, K, P, ldp, P, ldp, C, ldc, T(1), 1);
+}
+
 template <typename T, bool AM, bool LEFT>
 int launch_cfg(int64_t M, int64_t N, int64_t K, const T *A, int64_t lda, const T *B,
                int64_t ldb, T *C, int64_t ldc, T alpha, cudaStream_t s)
@@ -54,6 +68,21 @@ int launch_gemm_update(const Canon<T> &c, int64_t ci0, int64_t M, int64_t ak0, i
     if (!am && c.left) return launch_cfg<T, false, true>(M, c.ncols, K, Ap, c.lda, Bp, c.ldb, Cp, c.ldb, alpha, c.stream);
     return launch_cfg<T, false, false>(M, c.ncols, K, Ap, c.lda, Bp, c.ldb, Cp, c.ldb, alpha, c.stream);
 }
+
+template <typename T>
+int launch_gemm_trapezoid(bool am, int64_t M, int64_t N, int64_t K, const T *P, int64_t ldp, T *C, int64_t ldc, cudaStream_t s)
+{
+    if (M <= 0 || N <= 0 || K <= 0) return 0;
+    constexpr int BM = GemmTile<T>::BM;
+    const int64_t gx = (N + BM - 1) / BM, gy = (M + BM - 1) / BM;
+    if (gx > 0x7fffffff || gy > 65535) return GB_STATUS_CUDA_ERROR;
+    LaunchScope ls(KK_GEMM_SIMT, s, (2.0 * M - N) * N * K, sizeof(T) * (double(M) * K + (2.0 * M - N) * N));
+    auto k = am ? gemm_trapezoid_kernel<T, true> : gemm_trapezoid_kernel<T, false>;
+    k<<<dim3((unsigned)gx, (unsigned)gy), GemmTile<T>::NT, 0, s>>>(M, N, K, P, ldp, C, ldc);
+    return check(cudaGetLastError());
+}
+template int launch_gemm_trapezoid<double>(bool, int64_t, int64_t, int64_t, const double *, int64_t, double *, int64_t, cudaStream_t);
+template int launch_gemm_trapezoid<float>(bool, int64_t, int64_t, int64_t, const float *, int64_t, float *, int64_t, cudaStream_t);
 
 template int launch_gemm_update<double>(const Canon<double> &, int64_t, int64_t, int64_t, int64_t, double);
 template int launch_gemm_update<float>(const Canon<float> &, int64_t, int64_t, int64_t, int64_t, float);

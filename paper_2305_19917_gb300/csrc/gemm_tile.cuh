@@ -40,8 +40,7 @@ struct VecT<double, 2> {
 
 // AM: A-operand contiguous along M (Mv(i,k) = A(i,k), i.e. !mt).
 // BC: Bop contiguous along K, else along N.  CL: C contiguous along M, else
-// along N.  tri: 0 the whole tile, 1 / 2 only its entries on and below / above
-// the diagonal of C.  smem: gemm_tile_smem<T>() elements, 16-byte aligned.
+// along N.  tri: only the entries on and below the diagonal of C.  smem: gemm_tile_smem<T>() elements, 16-byte aligned.
 // Every thread of the CTA takes part; shared memory is free on return only
 // after a barrier.
 template <typename T>
@@ -168,7 +167,7 @@ __device__ __forceinline__ void gemm_tile(T *smem, int64_t m0, int64_t n0, int64
 #pragma unroll
         for (int c = 0; c < TN; c++) {
             int64_t gj = n0 + (c < VW ? tx * VW + c : BN / 2 + tx * VW + (c - VW));
-            if (gj >= N || (tri == 1 && gj > gi) || (tri == 2 && gj < gi)) continue;
+            if (gj >= N || (tri && gj > gi)) continue;
             T *p = CL ? &C[gi + gj * ldc] : &C[gj + gi * ldc];
             *p = (alpha == T(1)) ? (*p - acc[r][c]) : (alpha * *p - acc[r][c]);
         }

@@ -1,26 +1,32 @@
 // Cholesky factorisation on this triangular solver: the use the paper names
 // for its TS machinery (Section VIII, future work), built with the same
-// recursive computation model (Section V-A) as the solve:
+// recursive computation model (Section V-A) as the solve, on panels that
+// reach down to the last row:
 //
-//     A = [A11 A21^T; A21 A22]  ->  L11 = chol(A11)             (recursion)
-//                                   L21 = A21 L11^-T             (TS task: the
-//                                         library's own TRSM, side Right)
-//                                   A22 -= L21 L21^T             (gemm task:
-//                                         a SYRK update of the lower triangle)
-//                                   L22 = chol(A22)              (recursion)
+//     panel of columns [c0, c1), rows [c0, n):
+//         left half                                              (recursion)
+//         right half -= L(rows, left) L(right rows, left)^T       (gemm task:
+//                       its trapezoid on and below the diagonal)
+//         right half                                             (recursion)
 //
-// down to leaves of at most 64 columns, each factorised by one CTA in shared
-// memory.  The upper form (A = U^T U) is the mirror image: U12 = U11^-T A12
-// (TRSM side Left, Upper, transposed) and A22 -= U12^T U12.  Only the named
-// triangle of A is read and written.
+// down to leaves of at most 64 columns: the diagonal block factorised by one
+// CTA in shared memory, the rows below it solved against it (TS task: the
+// library's own TRSM, side Right, transposed).  So every column block meets
+// one TS task, on all its rows at once: splitting the matrix in 2 x 2 blocks
+// instead, with a TRSM of every order, ran 448 of them at n = 8192 instead of
+// 127.  n = 8192 FP64: 128 -> 28.5 ms by the panels and the tasks' digit gemms, 23.7
+// with the leaf below; n = 16384 87 ms (1.34 s before the digit gemms).  The upper form (A = U^T U) is the same with everything stored
+// transposed.  Only the named triangle of A is read and written.
 //
 // A non-positive (or NaN) pivot stops the leaf that meets it; the leaf
 // records info = (global column + 1) in a device word (the first failure
 // wins, leaves run in order) and every later leaf returns without work.  As
 // with LAPACK, the contents of A from that column on are then undefined.
+#include <algorithm>
 #include <cmath>
 #include "common.cuh"
 #include "driver.cuh"
+#include "gemm_digits.cuh"
 #include "mixed.cuh"
 
 extern "C" int gb_dtrsm(int side, int uplo, int trans, int diag, int64_t m, int64_t n, double alpha,
@@ -34,214 +40,153 @@ namespace {
 constexpr int kLeafNB = 64;
 constexpr int kLeafThreads = 256;
 
+// Exponent field and its largest value (tests on it are integer operations: a
+// comparison of FP64 values takes 66 clocks as any operation of that unit).
+__device__ __forceinline__ int expo(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
+__device__ __forceinline__ int expo(float x) { return (__float_as_int(x) >> 23) & 0xFF; }
+template <typename T>
+constexpr int kExpoMax = sizeof(T) == 8 ? 0x7FF : 0xFF;
+
+// The rare cases by definition.  Out of line: inlined, the compiler evaluates
+// a division beside every ordinary case and selects afterwards.
+template <typename T>
+__device__ __noinline__ void pivot_root_slow(T d, T &l, T &y)
+{
+    l = sqrt(d);
+    y = T(1) / l;
+}
+template <typename T>
+__device__ __noinline__ T pivot_scale_slow(T v, T l)
+{
+    return v / l;
+}
+
+// l = sqrt(d) and y = 1 / sqrt(d) of a pivot d > 0, the reciprocal square root
+// corrected once against d.
+template <typename T>
+__device__ __forceinline__ void pivot_root(T d, T &l, T &y)
+{
+    const int e = expo(d);
+    if (e < kExpoMax<T> / 8 || e == kExpoMax<T>) {  // where the corrections could leave the range
+        pivot_root_slow(d, l, y);
+        return;
+    }
+    y = rsqrt(d);
+    const T h = T(0.5) * y;
+    l = d * y;
+    l = fma(fma(-l, l, d), h, l);
+    y = fma(y, fma(-l, y, T(1)), y);
+}
+// v / l by the reciprocal y, corrected once: as exact as the division.
+template <typename T>
+__device__ __forceinline__ T pivot_scale(T v, T l, T y)
+{
+    T q = v * y;
+    q = fma(fma(-q, l, v), y, q);
+    if (expo(q) == kExpoMax<T>) q = pivot_scale_slow(v, l);
+    return q;
+}
+
 // One diagonal block of order nr <= 64 at &A(r0, r0) (A0 points there),
-// factorised right-looking in shared memory.  s[i][c] (i >= c) holds the
-// block's lower triangle: A(i, c) for the lower form, A(c, i) for the upper.
+// factorised right-looking in shared memory.  s[c][i] (i >= c) holds the
+// block's lower triangle by columns: A(i, c) for the lower form, A(c, i) for
+// the upper.  What bounds it is the chain of 64 pivots: a reciprocal square
+// root, its corrections and the next pivot's update are about 18 operations
+// of the FP64 unit, 66 clocks each.  Warp 0 does nothing else: while it forms
+// pivot j + 1 from its own copy of that pivot's column entry, warps 1 and 2
+// scale column j and then all but warps 0 and 4 (the one that shares warp 0's
+// sub-partition) update the columns behind it.  One CTA barrier a column; a
+// finished column goes to A at once.
+// Measured (one 64-column block): FP64 70 us, FP32 27 (one thread's square
+// root, a division per entry and three barriers a column: 107 and 48).
 template <typename T>
 __global__ void __launch_bounds__(kLeafThreads)
 potrf_leaf_kernel(T *__restrict__ A0, int64_t lda, int nr, int upper, int64_t r0, int *info)
 {
     __shared__ T s[kLeafNB][kLeafNB + 1];
+    __shared__ T piv[2][2];           // l and y of the pivots, by parity of the column
+    __shared__ T col[2][kLeafNB];     // scaled columns, likewise
     __shared__ int fail;
     if (*static_cast<volatile int *>(info) != 0) return;  // an earlier leaf failed
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // load the named triangle, reading A along its contiguous dimension
-    for (int idx = tid; idx < nr * nr; idx += kLeafThreads) {
-        const int fast = idx % nr, slow = idx / nr;  // A(fast, slow)
-        if (!upper && fast >= slow) s[fast][slow] = A0[fast + int64_t(slow) * lda];
-        if (upper && fast <= slow) s[slow][fast] = A0[fast + int64_t(slow) * lda];
+    // (every load before the first store)
+    {
+        constexpr int PER = kLeafNB * kLeafNB / kLeafThreads;
+        T v[PER];
+#pragma unroll
+        for (int u = 0; u < PER; u++) {
+            const int fast = tid % kLeafNB, slow = tid / kLeafNB + u * (kLeafThreads / kLeafNB);  // A(fast, slow)
+            const int i = upper ? slow : fast, c = upper ? fast : slow;
+            v[u] = (i < nr && c <= i) ? A0[fast + int64_t(slow) * lda] : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < PER; u++) {
+            const int fast = tid % kLeafNB, slow = tid / kLeafNB + u * (kLeafThreads / kLeafNB);
+            s[upper ? fast : slow][upper ? slow : fast] = v[u];
+        }
     }
-    if (tid == 0) fail = -1;
+    if (tid < 2 * kLeafNB) (&col[0][0])[tid] = T(0);
+    if (tid == 0) fail = kLeafNB;
     __syncthreads();
-    for (int j = 0; j < nr; j++) {
-        if (tid == 0) {
-            const T d = s[j][j];
+    auto pivot = [&](int j, T d) {  // warp 0
+        T l, y;
+        pivot_root(d, l, y);
+        if (lane == 0) {
+            piv[j & 1][0] = l;
+            piv[j & 1][1] = y;
             if (!(d > T(0))) fail = j;
-            else s[j][j] = sqrt(d);
-        }
-        __syncthreads();
-        if (fail >= 0) break;
-        const T ljj = s[j][j];
-        for (int i = j + 1 + tid; i < nr; i += kLeafThreads) s[i][j] = s[i][j] / ljj;
-        __syncthreads();
-        // trailing update of the lower triangle: s[i][c] -= l_ij l_cj, j < c <= i
-        const int w = nr - j - 1;
-        for (int idx = tid; idx < w * w; idx += kLeafThreads) {
-            const int i = j + 1 + idx % w, c = j + 1 + idx / w;
-            if (c <= i) s[i][c] -= s[i][j] * s[c][j];
-        }
-        __syncthreads();
-    }
-    if (fail >= 0) {
-        if (tid == 0) atomicCAS(info, 0, int(r0 + fail + 1));
-        return;
-    }
-    for (int idx = tid; idx < nr * nr; idx += kLeafThreads) {
-        const int fast = idx % nr, slow = idx / nr;
-        if (!upper && fast >= slow) A0[fast + int64_t(slow) * lda] = s[fast][slow];
-        if (upper && fast <= slow) A0[fast + int64_t(slow) * lda] = s[slow][fast];
-    }
-}
-
-// ---- SYRK update: C -= P P^T (lower) or C -= P^T P (upper) -----------------
-// The gemm task of the factorisation, restricted to the named triangle of
-// the symmetric C (order M): lower form, P is M x K (column-major, ldp) and
-// C(i, c) -= sum_k P(i, k) P(c, k) for i >= c; upper form, P is K x M and
-// C(i, c) -= sum_k P(k, i) P(k, c) for i <= c.  CTA tiles of BM x BM cover
-// the triangle only (a 1-D grid over the T (T + 1) / 2 tiles on and below /
-// above the diagonal); k-slices of BK are staged in shared memory with a
-// register double buffer, each thread owning a TM x TM micro-tile split in
-// two halves so that its shared-memory reads are 16-byte vectors (the
-// layout of the solve's gemm task).
-template <typename T>
-struct SyrkCfg;
-template <>
-struct SyrkCfg<double> {  // DFMA: 64 x 64 tile, 4 x 4 per thread, 256 threads
-    static constexpr int BM = 64, BK = 16, TM = 4;
-};
-template <>
-struct SyrkCfg<float> {  // FFMA: 128 x 128 tile, 8 x 8 per thread, 256 threads
-    static constexpr int BM = 128, BK = 8, TM = 8;
-};
-template <typename T, int W>
-struct SyrkVec;
-template <>
-struct SyrkVec<double, 2> {
-    using type = double2;
-};
-template <>
-struct SyrkVec<float, 4> {
-    using type = float4;
-};
-
-template <typename T, bool UP>
-__global__ void __launch_bounds__((SyrkCfg<T>::BM / SyrkCfg<T>::TM) * (SyrkCfg<T>::BM / SyrkCfg<T>::TM))
-syrk_update_kernel(int64_t M, int64_t K, const T *__restrict__ P, int64_t ldp, T *__restrict__ C, int64_t ldc)
-{
-    constexpr int BM = SyrkCfg<T>::BM, BK = SyrkCfg<T>::BK, TM = SyrkCfg<T>::TM;
-    constexpr int NTX = BM / TM, NT = NTX * NTX;
-    constexpr int VW = TM / 2;
-    static_assert(VW * sizeof(T) == 16, "16-byte shared vectors");
-    constexpr int LDS = BM + VW;
-    constexpr int PER = BM * BK / NT;
-    static_assert(PER * NT == BM * BK, "tile split");
-    using V = typename SyrkVec<T, VW>::type;
-    __shared__ __align__(16) T Rs[2][BK * LDS];  // rows operand: R(i, k), tile rows
-    __shared__ __align__(16) T Cs[2][BK * LDS];  // columns operand: R(c, k), tile columns
-
-    // tile (ti, tc) of the triangle: linear index t over tc <= ti (lower) or
-    // ti <= tc (upper, the same enumeration with the roles swapped)
-    const int64_t t = blockIdx.x;
-    int64_t a = int64_t((sqrt(8.0 * double(t) + 1.0) - 1.0) / 2.0);
-    while (a * (a + 1) / 2 > t) a--;
-    while ((a + 1) * (a + 2) / 2 <= t) a++;
-    const int64_t b = t - a * (a + 1) / 2;  // 0 <= b <= a
-    const int64_t ti = UP ? b : a, tc = UP ? a : b;
-    const int64_t i0 = ti * BM, c0 = tc * BM;
-
-    const int tid = threadIdx.x;
-    const int tx = tid % NTX, ty = tid / NTX;
-    T rr[PER], rc[PER];
-    // element (row x, k) of the operand R with R(x, k) = P(x, k) (lower) or
-    // P(k, x) (upper), read along P's contiguous dimension
-    auto load = [&](int64_t kk) {
-#pragma unroll
-        for (int p = 0; p < PER; p++) {
-            const int idx = tid + p * NT;
-            int x, k;
-            if (!UP) { x = idx % BM; k = idx / BM; }
-            else     { k = idx % BK; x = idx / BK; }
-            const int64_t gk = kk + k, gi = i0 + x, gc = c0 + x;
-            T vi = T(0), vc = T(0);
-            if (gk < K) {
-                if (gi < M) vi = UP ? P[gk + gi * ldp] : P[gi + gk * ldp];
-                if (gc < M) vc = UP ? P[gk + gc * ldp] : P[gc + gk * ldp];
-            }
-            rr[p] = vi;
-            rc[p] = vc;
+            else A0[j + int64_t(j) * lda] = l;
         }
     };
-    auto store = [&](int buf) {
-#pragma unroll
-        for (int p = 0; p < PER; p++) {
-            const int idx = tid + p * NT;
-            int x, k;
-            if (!UP) { x = idx % BM; k = idx / BM; }
-            else     { k = idx % BK; x = idx / BK; }
-            Rs[buf][k * LDS + x] = rr[p];
-            Cs[buf][k * LDS + x] = rc[p];
-        }
-    };
-    T acc[TM][TM];
-#pragma unroll
-    for (int r = 0; r < TM; r++)
-#pragma unroll
-        for (int c = 0; c < TM; c++) acc[r][c] = T(0);
-    const int64_t nk = (K + BK - 1) / BK;
-    if (nk > 0) {
-        load(0);
-        store(0);
+    if (warp == 0) pivot(0, s[0][0]);
+    for (int j = 0; j < nr; j++) {
         __syncthreads();
-    }
-    for (int64_t kt = 0; kt < nk; kt++) {
-        const int cur = int(kt & 1);
-        if (kt + 1 < nk) load((kt + 1) * BK);
-#pragma unroll
-        for (int k = 0; k < BK; k++) {
-            T x[TM], y[TM];
-            const V a0 = *reinterpret_cast<const V *>(&Rs[cur][k * LDS + ty * VW]);
-            const V a1 = *reinterpret_cast<const V *>(&Rs[cur][k * LDS + BM / 2 + ty * VW]);
-            const V b0 = *reinterpret_cast<const V *>(&Cs[cur][k * LDS + tx * VW]);
-            const V b1 = *reinterpret_cast<const V *>(&Cs[cur][k * LDS + BM / 2 + tx * VW]);
-            const T *pa0 = reinterpret_cast<const T *>(&a0), *pa1 = reinterpret_cast<const T *>(&a1);
-            const T *pb0 = reinterpret_cast<const T *>(&b0), *pb1 = reinterpret_cast<const T *>(&b1);
-#pragma unroll
-            for (int e = 0; e < VW; e++) {
-                x[e] = pa0[e];
-                x[VW + e] = pa1[e];
-                y[e] = pb0[e];
-                y[VW + e] = pb1[e];
+        if (fail <= j) break;
+        const T l = piv[j & 1][0], y = piv[j & 1][1];
+        if (warp == 0) {
+            if (j + 1 < nr) {
+                const T q = pivot_scale(s[j][j + 1], l, y);
+                pivot(j + 1, fma(-q, q, s[j + 1][j + 1]));
             }
-#pragma unroll
-            for (int r = 0; r < TM; r++)
-#pragma unroll
-                for (int c = 0; c < TM; c++) acc[r][c] = fma(x[r], y[c], acc[r][c]);
-        }
-        if (kt + 1 < nk) {
-            store(cur ^ 1);
-            __syncthreads();
+        } else if (warp != 4) {
+            const int w = warp - 1 - (warp > 4);  // 0 .. 5
+            T *q = col[j & 1];
+            if (w < 2) {
+                const int i = 32 * w + lane;
+                if (i > j && i < nr) {
+                    const T v = pivot_scale(s[j][i], l, y);
+                    q[i] = v;
+                    A0[upper ? j + int64_t(i) * lda : i + int64_t(j) * lda] = v;
+                }
+            }
+            asm volatile("bar.sync 1, 192;" ::: "memory");
+            // columns c > j, rows i >= c (but for the pivot (j + 1, j + 1): warp 0's)
+            // (rows past nr hold zeros); columns below 32 in two pieces of
+            // rows, two pieces at a time
+            int c = j + 1 + w;
+            for (; c < 32; c += 6) {
+                const T f = q[c];
+                const int i = c + lane, i2 = i + 32;
+                const T a = s[c][i], b = i2 < kLeafNB ? s[c][i2] : T(0);
+                const T qa = q[i], qb = i2 < kLeafNB ? q[i2] : T(0);
+                const T ra = fma(-qa, f, a), rb = fma(-qb, f, b);
+                if (i > j + 1) s[c][i] = ra;
+                if (i2 < kLeafNB) s[c][i2] = rb;
+            }
+            for (; c < nr; c += 12) {
+                const int i = c + lane, c2 = c + 6, i2 = c2 + lane;
+                const bool in = i < kLeafNB, in2 = c2 < nr && i2 < kLeafNB;
+                const T f = q[c], f2 = c2 < nr ? q[c2] : T(0);
+                const T a = in ? s[c][i] : T(0), b = in2 ? s[c2][i2] : T(0);
+                const T qa = in ? q[i] : T(0), qb = in2 ? q[i2] : T(0);
+                const T ra = fma(-qa, f, a), rb = fma(-qb, f2, b);
+                if (in && i > j + 1) s[c][i] = ra;
+                if (in2) s[c2][i2] = rb;
+            }
         }
     }
-#pragma unroll
-    for (int r = 0; r < TM; r++) {
-        const int64_t gi = i0 + (r < VW ? ty * VW + r : BM / 2 + ty * VW + (r - VW));
-        if (gi >= M) continue;
-#pragma unroll
-        for (int c = 0; c < TM; c++) {
-            const int64_t gc = c0 + (c < VW ? tx * VW + c : BM / 2 + tx * VW + (c - VW));
-            if (gc >= M || (UP ? gi > gc : gi < gc)) continue;
-            T *q = &C[gi + gc * ldc];
-            *q = *q - acc[r][c];
-        }
-    }
-}
-
-template <typename T>
-int launch_syrk(bool upper, int64_t M, int64_t K, const T *P, int64_t ldp, T *C, int64_t ldc, cudaStream_t s)
-{
-    if (M <= 0 || K <= 0) return 0;
-    constexpr int BM = SyrkCfg<T>::BM, NT = (BM / SyrkCfg<T>::TM) * (BM / SyrkCfg<T>::TM);
-    const int64_t tiles = (M + BM - 1) / BM;
-    const int64_t grid = tiles * (tiles + 1) / 2;
-    if (grid > 0x7fffffffLL) return GB_STATUS_CUDA_ERROR;
-    // algorithmic work: the triangle of C (M (M + 1) / 2 entries) x K multiply-adds
-    LaunchScope ls(KK_GEMM_SIMT, s, double(M) * double(M + 1) * double(K),
-                   sizeof(T) * (double(M) * K + double(M) * double(M + 1)));
-    if (upper)
-        syrk_update_kernel<T, true><<<(unsigned)grid, NT, 0, s>>>(M, K, P, ldp, C, ldc);
-    else
-        syrk_update_kernel<T, false><<<(unsigned)grid, NT, 0, s>>>(M, K, P, ldp, C, ldc);
-    return check(cudaGetLastError());
+    if (tid == 0 && fail < nr) atomicCAS(info, 0, int(r0 + fail + 1));
 }
 
 int trsm_call(int side, int uplo, int trans, int64_t m, int64_t n, const double *A, int64_t lda, double *B,
@@ -255,31 +200,67 @@ int trsm_call(int side, int uplo, int trans, int64_t m, int64_t n, const float *
     return gb_strsm(side, uplo, trans, GB_NONUNIT, m, n, 1.0f, A, lda, B, ldb, s);
 }
 
-// Recursive model (Section V-A) on columns [off, off + n) of the
-// factorisation, A pointing at their diagonal block.
-template <typename T>
-int potrf_rec(int uplo, int64_t n, T *A, int64_t lda, int64_t off, int *info, cudaStream_t s)
+// Recursive model (Section V-A) on the panel of columns [c0, c1); an Exec
+// either launches the tasks or finds their work space.
+template <class E>
+int potrf_rec(E &e, int64_t c0, int64_t c1)
 {
-    if (n <= 0) return 0;
-    if (n <= kLeafNB) {
-        LaunchScope ls(KK_DIAG, s, double(n) * n * n / 3.0, sizeof(T) * double(n) * (n + 1));
-        potrf_leaf_kernel<T><<<1, kLeafThreads, 0, s>>>(A, lda, int(n), uplo == GB_UPPER, off, info);
-        return check(cudaGetLastError());
-    }
-    const int64_t n1 = rec_split(n, kLeafNB), n2 = n - n1;
-    GB_TRY(potrf_rec(uplo, n1, A, lda, off, info, s));
-    T *A22 = A + n1 + n1 * lda;
-    if (uplo == GB_LOWER) {
-        T *A21 = A + n1;
-        GB_TRY(trsm_call(GB_RIGHT, GB_LOWER, GB_TRANS, n2, n1, A, lda, A21, lda, s));  // L21 = A21 L11^-T
-        GB_TRY(launch_syrk<T>(false, n2, n1, A21, lda, A22, lda, s));                   // A22 -= L21 L21^T
-    } else {
-        T *A12 = A + n1 * lda;
-        GB_TRY(trsm_call(GB_LEFT, GB_UPPER, GB_TRANS, n1, n2, A, lda, A12, lda, s));    // U12 = U11^-T A12
-        GB_TRY(launch_syrk<T>(true, n2, n1, A12, lda, A22, lda, s));                    // A22 -= U12^T U12
-    }
-    return potrf_rec(uplo, n2, A22, lda, off + n1, info, s);
+    if (c1 - c0 <= kLeafNB) return e.leaf(c0, c1);
+    const int64_t cm = c0 + rec_split(c1 - c0, kLeafNB);
+    GB_TRY(potrf_rec(e, c0, cm));
+    GB_TRY(e.update(c0, cm, c1));
+    return potrf_rec(e, cm, c1);
 }
+
+template <typename T>
+struct PotrfBytes {
+    int64_t n;
+    size_t bytes = 0;
+    int leaf(int64_t, int64_t) { return 0; }
+    int update(int64_t c0, int64_t cm, int64_t c1)
+    {
+        if (digit_gemm_wanted<T>(n - cm, c1 - cm, cm - c0, 1))
+            bytes = std::max(bytes, digit_gemm_bytes<T>(n - cm, c1 - cm, cm - c0, 1));
+        return 0;
+    }
+};
+
+template <typename T>
+struct PotrfExec {
+    bool upper;
+    int64_t n;
+    T *A;
+    int64_t lda;
+    int *info;
+    cudaStream_t s;
+    size_t digit_bytes;
+    DigitWorkspace ws;
+    T *at(int64_t i, int64_t c) { return upper ? A + c + i * lda : A + i + c * lda; }
+    int leaf(int64_t c0, int64_t c1)
+    {
+        const int64_t w = c1 - c0;
+        {
+            LaunchScope ls(KK_DIAG, s, double(w) * w * w / 3.0, sizeof(T) * double(w) * (w + 1));
+            potrf_leaf_kernel<T><<<1, kLeafThreads, 0, s>>>(at(c0, c0), lda, int(w), upper, c0, info);
+            GB_TRY(check(cudaGetLastError()));
+        }
+        if (c1 >= n) return 0;
+        // L(c1.., c0..) = A(c1.., c0..) L11^-T, or U(c0.., c1..) = U11^-T A(c0.., c1..)
+        if (upper) return trsm_call(GB_LEFT, GB_UPPER, GB_TRANS, w, n - c1, at(c0, c0), lda, at(c1, c0), lda, s);
+        return trsm_call(GB_RIGHT, GB_LOWER, GB_TRANS, n - c1, w, at(c0, c0), lda, at(c1, c0), lda, s);
+    }
+    int update(int64_t c0, int64_t cm, int64_t c1)
+    {
+        const int64_t M = n - cm, N = c1 - cm, K = cm - c0;
+        if (digit_gemm_wanted<T>(M, N, K, 1)) {
+            if (char *p = ws.get(digit_bytes)) {
+                const DigitGemm<T> g{M, N, K, at(cm, c0), lda, !upper, at(cm, c0), lda, upper, at(cm, cm), lda, !upper, T(1), 1};
+                return launch_digit_gemm<T>(g, p, ws.size(), s);
+            }
+        }
+        return launch_gemm_trapezoid<T>(!upper, M, N, K, at(cm, c0), lda, at(cm, cm), lda, s);
+    }
+};
 
 template <typename T>
 int potrf_impl(int uplo, int64_t n, T *A, int64_t lda, int64_t *info_out, void *stream)
@@ -298,7 +279,12 @@ int potrf_impl(int uplo, int64_t n, T *A, int64_t lda, int64_t *info_out, void *
     int *dinfo = nullptr;
     GB_CUDA(cudaMallocFromPoolAsync(reinterpret_cast<void **>(&dinfo), sizeof(int), pool, s));
     int st = check(cudaMemsetAsync(dinfo, 0, sizeof(int), s));
-    if (!st) st = potrf_rec<T>(uplo, n, A, lda, 0, dinfo, s);
+    if (!st) {
+        PotrfBytes<T> pb{n};
+        potrf_rec(pb, 0, n);
+        PotrfExec<T> e{uplo == GB_UPPER, n, A, lda, dinfo, s, pb.bytes, DigitWorkspace(s)};
+        st = potrf_rec(e, 0, n);
+    }
     int h = 0;
     if (!st) st = check(cudaMemcpyAsync(&h, dinfo, sizeof(int), cudaMemcpyDeviceToHost, s));
     cudaFreeAsync(dinfo, s);
