@@ -2,69 +2,59 @@
 // TS" (Section IV, many right-hand sides) generalised to many independent
 // problems of different order and width.
 //
-// Work units are (instance, chunk of CW right-hand sides); a chunk of an
-// order-k instance costs ~k^2 CW / 2 multiply-adds, so units are sorted by
-// k (largest first) and handed out through a device-side work queue: each
-// CTA of a persistent grid pops a ticket with one atomicAdd until the queue
-// is empty (no CTA ever waits on another).  A unit is solved entirely in
-// shared memory by its CTA with the blocked forward model of Section V-C in
-// left-looking order: for each 32-row diagonal block, one register-tiled
-// update with all solved blocks (the gemm tasks), then the 32 x 32 triangle
-// by warp-shuffle substitution (the TS task).  Backward problems are index
-// reversed and right-side problems transposed on the way in and out.
-// Instances of order above KMAX are solved by the regular driver.
+// Work units are (instance, chunk of CW right-hand sides, 16 FP64 / 32 FP32); a
+// chunk of an order-k instance costs ~k^2 CW / 2 multiply-adds, so units are
+// sorted by cost (largest first) and handed out through a device-side work
+// queue (atomic tickets; no CTA waits on another).  A unit is solved by the
+// blocked model of Section V-C in left-looking order on 32-row blocks, X in
+// shared memory, by a team of warps: warp w of n owns the block rows w, w + n,
+// ..., each taking its updates from the solved blocks as these are published
+// (no barrier inside a unit).  The more warps share a unit, the more of their
+// time goes into waiting for its chain of blocks; but X has to stay in shared
+// memory.  So teams are as small as that allows: the four warps of a CTA for
+// orders above 256, two above 128, one below (tile 1; half these orders with
+// tile 2), the CTA's X space divided among its teams.  Instances of order above KMAX are solved by the regular driver.
 //
-// Tile shapes (the autotuner's choice, gb_batched_autotune): in the gemm
-// tasks each thread owns RR rows x one 16-byte vector of right-hand sides
-// (PER = 2 FP64 / 4 FP32 columns), so a unit is CW = 8 PER RR right-hand
-// sides wide: RR = 1 gives 16 (FP64) / 32 (FP32) columns and two CTAs per
-// SM (109 KB of shared memory each); RR = 2 gives 32 / 64 columns, twice the
-// multiply-adds per shared-memory load, one CTA per SM.  A tiles are stored
-// k-major so that a thread's RR rows load as one vector.  A warp owns a few
-// whole columns of the block (its lanes the rows), so a step's A rows load
-// as whole wavefronts and its X vector as a broadcast, and the warps whose
-// columns lie past the last right-hand side of a chunk skip their products
-// (a chunk is often narrower than CW: the last one of every instance).
-//
-// FP32 solves the 32 x 32 diagonal blocks with their inverses: a first kernel
-// of the plan's graph inverts every diagonal block of every instance once per
-// run (one warp per block, one lane per column of the inverse, forward
-// substitution in registers), and the TS task of a unit becomes a product
-// with the inverse on the gemm tasks' register tiles -- the warp-shuffle
-// substitution, about four times the instructions of a gemm tile, dominated
-// the FP32 kernel's issue slots.  FP64 keeps the substitution: its DFMA rate,
-// not instruction issue, bounds it.
+// A lane holds one right-hand side and its rows of the block in registers, so
+// that the 32 x 32 triangle is solved by multiply-adds on independent rows,
+// without shuffles of partial sums or lanes masked off: in FP64, where an
+// instruction takes 66 clocks of its sub-partition whatever its active lanes
+// and the multiply-adds are the time, a block's triangle takes 18 instructions
+// per right-hand side instead of the 64 of a substitution with one row per
+// lane.  FP64: 16 right-hand sides times the two halves of the rows (odd and
+// even), Mv read from L1 / L2 as it is needed (two addresses per warp and load;
+// the loads hide behind the arithmetic).  FP32: 32 right-hand sides, tiles of
+// Mv through a ring of asynchronous copies, packed multiply-adds
+// (wide_tile.cuh); two CTAs of four warps fill an SM's shared memory, and the
+// latencies that eight warps leave open are the time.  Measured, 4096 uneven
+// instances (m log-uniform in [16, 512], n in [1, 256]): FP64 22.2 -> 16.4 ms
+// (the FP64 unit 89 % busy; 12.9 ms at its peak), FP32 1.79 -> 1.19 ms.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <vector>
 #include "common.cuh"
+#include "wide_tile.cuh"
 
 namespace gb {
 
 namespace {
 
-constexpr int KMAX = 512;   // largest order solved in shared memory
-constexpr int NBB = 32;     // diagonal block
-constexpr int NT = 256;     // threads per CTA
-constexpr int LT = NBB + 2; // k-major A tile: row stride of one k (keeps 8- and 16-byte alignment)
+constexpr int KMAX = 512;  // largest order solved in shared memory
+constexpr int NBB = 32;    // diagonal block
+constexpr int NW = 4;      // warps per CTA
+constexpr int NT = 32 * NW;
 
-// Tile shape of the gemm tasks: RR rows x PER columns per thread.
-template <typename T, int RR>
-struct BCfg {
-    static constexpr int PER = int(16 / sizeof(T));   // one 16-byte vector of right-hand sides
-    static constexpr int ROWG = NBB / RR;             // row groups of a block row
-    static constexpr int COLG = NT / ROWG;            // column groups
-    static constexpr int CW = COLG * PER;             // right-hand sides per unit
-    static constexpr int LX = CW + PER;               // row stride of X in shared memory
-    static_assert(ROWG * COLG == NT, "thread split");
-    static_assert(CW % 8 == 0, "warp split of the TS task");
-};
+template <typename T>
+constexpr int kChunk = sizeof(T) == 8 ? 16 : 32;  // right-hand sides per unit
+
+template <typename T>
+constexpr int kStride = sizeof(T) == 8 ? 16 : 33;  // row stride of X in shared memory (FP32: odd, read along rows too)
 
 template <typename T>
 struct Unit {
     const T *A;   // A of the instance
     T *B;         // B of the instance, offset to the chunk's first right-hand side
-    const T *Linv;  // inverses of the instance's 32 x 32 diagonal blocks (FP32), k-major 32 x 32 each
     int64_t lda, ldb;
     int k;        // order of the triangle
     int cw;       // right-hand sides in this chunk (<= CW)
@@ -72,383 +62,327 @@ struct Unit {
     T alpha;
 };
 
-
-// A tiles in the ring (NBUF - 1 in flight): the tiles stream from L2, whose
-// latency a short ring leaves exposed; FP32 tiles are half the size, so it
-// keeps twice as many.
+// Who solves a unit: warp `wid` of `nwu`, X of the unit at Xs, blocks solved so
+// far counted in *solved.
 template <typename T>
-constexpr int nbuf() { return sizeof(T) == 4 ? 8 : 4; }
-
-// Asynchronous copy of one element (4 or 8 bytes); `in` false writes zero.
-template <typename T>
-__device__ __forceinline__ void cp_async_elem(T *dst, const T *src, bool in)
-{
-    const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
-    const int n = in ? int(sizeof(T)) : 0;
-    if (sizeof(T) == 8)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-// Address of Mv'(i, j) of the forward view of unit u (index reversal for a
-// backward problem, transposition for mt).
-template <typename T>
-__device__ __forceinline__ const T *mv_addr(const Unit<T> &u, int i, int j)
-{
-    const bool mt = u.flags & 1, rev = u.flags & 2;
-    const int io = rev ? u.k - 1 - i : i, jo = rev ? u.k - 1 - j : j;
-    return mt ? u.A + jo + int64_t(io) * u.lda : u.A + io + int64_t(jo) * u.lda;
-}
-
-// A unit's tiles in sequence: block row jb, then tiles ib = 0..jb (ib < jb:
-// gemm tasks, ib == jb: the TS task); the position steps along the sequence.
-struct TilePos {
-    int jb = 0, ib = 0;
-    __device__ __forceinline__ void next()
-    {
-        if (ib == jb) {
-            jb++;
-            ib = 0;
-        } else {
-            ib++;
-        }
-    }
+struct Team {
+    int wid, nwu;
+    T *Xs;
+    T *ring;       // FP32: the warp's two tiles
+    T *inv;        // FP32: the warp's 32 inverse diagonal entries, and the entries
+    int *solved;
 };
-
-// Issue the asynchronous loads of tile (jb, ib) into buffer Tb (reading
-// along A's contiguous dimension): the gemm tiles in full, the TS tile on
-// and below its diagonal; everything else (and the ragged edge) reads as
-// zero.  Tb is k-major: Tb[kk * LT + rr] = Mv'(j0 + rr, i0 + kk).
-template <typename T>
-__device__ __forceinline__ void load_tile(const Unit<T> &u, int jb, int ib, T *Tb)
+// Until block kb of the unit is solved (bounded).
+__device__ __forceinline__ void await_block(int *solved, int kb, int &known, bool &gave_up)
 {
-    if (u.Linv && ib == jb) {
-        // the TS task's tile: the block's precomputed inverse (k-major 32 x
-        // 32 in global memory), in 8-byte pieces into the LT-strided layout
-        const T *src = u.Linv + size_t(jb) * NBB * NBB;
-        constexpr int PIECE = int(8 / sizeof(T));
-        for (int idx = threadIdx.x; idx < NBB * NBB / PIECE; idx += NT) {
-            const int kk = (idx * PIECE) / NBB, rr = (idx * PIECE) % NBB;
-            const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(Tb + kk * LT + rr));
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src + kk * NBB + rr) : "memory");
-        }
-        return;
+    for (int spin = 0; known <= kb && !gave_up; spin++) {
+        known = *static_cast<volatile int *>(solved);
+        if (spin > wide::kSpins) gave_up = true;
     }
-    const int j0 = jb * NBB, i0 = ib * NBB, k = u.k;
-    const bool mt = u.flags & 1;
-    if (ib < jb && j0 + NBB <= k) {
-        // a gemm tile inside the triangle: entry (fast, slow) of the copy
-        // sits at base + s fast + s lda slow (s = -1 for a backward problem),
-        // fast running along A's contiguous dimension
-        const bool rev = u.flags & 2;
-        const int x0 = mt ? i0 : j0, y0 = mt ? j0 : i0;  // origin along the contiguous / strided index
-        const int64_t sg = rev ? -1 : 1;
-        const T *base = u.A + (rev ? int64_t(k - 1 - x0) + int64_t(k - 1 - y0) * u.lda : int64_t(x0) + int64_t(y0) * u.lda);
-        const int fast = threadIdx.x % NBB;
-        const T *p = base + sg * (fast + int64_t(threadIdx.x / NBB) * u.lda);
-        const int64_t step = sg * int64_t(NT / NBB) * u.lda;
-#pragma unroll
-        for (int q = 0; q < NBB * NBB / NT; q++) {
-            const int slow = threadIdx.x / NBB + q * (NT / NBB);
-            const int rr = mt ? slow : fast, kk = mt ? fast : slow;
-            cp_async_elem(Tb + kk * LT + rr, p + q * step, true);
-        }
-        return;
+    __threadfence_block();
+}
+__device__ __forceinline__ void publish_block(int *solved, int b)
+{
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) {
+        __threadfence_block();
+        *static_cast<volatile int *>(solved) = b + 1;
     }
-    for (int idx = threadIdx.x; idx < NBB * NBB; idx += NT) {
-        const int fast = idx % NBB, slow = idx / NBB;
-        const int rr = mt ? slow : fast, kk = mt ? fast : slow;
-        const bool in = j0 + rr < k && i0 + kk < k && (ib < jb || kk <= rr);
-        cp_async_elem(Tb + kk * LT + rr, in ? mv_addr(u, j0 + rr, i0 + kk) : u.A, in);
-    }
+    __syncwarp();
 }
 
-// RR rows of a k-major A tile as one vector.
-template <typename T, int RR>
-struct RowVec {
-    T v[RR];
-};
-template <typename T, int RR>
-__device__ __forceinline__ void load_rows(const T *p, T (&a)[RR])
-{
-    if constexpr (RR * sizeof(T) == 16) {
-        const uint4 q = *reinterpret_cast<const uint4 *>(p);
-        const T *x = reinterpret_cast<const T *>(&q);
-#pragma unroll
-        for (int e = 0; e < RR; e++) a[e] = x[e];
-    } else if constexpr (RR * sizeof(T) == 8) {
-        const uint2 q = *reinterpret_cast<const uint2 *>(p);
-        const T *x = reinterpret_cast<const T *>(&q);
-#pragma unroll
-        for (int e = 0; e < RR; e++) a[e] = x[e];
-    } else {
-#pragma unroll
-        for (int e = 0; e < RR; e++) a[e] = p[e];
-    }
-}
+constexpr int XLD = kStride<float>;
 
-// acc += (rows r .. r + RR - 1 of the k-major tile Tb) x (32 rows of X from
-// xr, columns cq ..), software-pipelined: the operands of step kk + 2 are
-// loaded while step kk multiplies (two warps per scheduler leave the
-// shared-memory latency exposed otherwise).
-template <typename T, int RR, int PER, int LX>
-__device__ __forceinline__ void tile_fma(T (&acc)[RR][PER], const T *Tb, const T *xr, int r, int cq)
+// FP32, in solution order (a backward problem by negative strides), so that
+// one version of the unrolled steps serves every form: with one for each of
+// the four (rows or columns of A contiguous, forward or backward) instruction
+// fetch was the largest stall.
+__device__ __forceinline__ void solve_unit(const Unit<float> &u, const Team<float> &tm)
 {
-    constexpr int D = 3;  // operand sets in registers (2 steps ahead)
-    T a[D][RR], x[D][PER];
-    auto load = [&](int kk, int b) {
-        load_rows<T, RR>(Tb + kk * LT + r, a[b]);
-        const uint4 xv = *reinterpret_cast<const uint4 *>(xr + kk * LX + cq);
-        const T *xp = reinterpret_cast<const T *>(&xv);
+    using namespace wide;
+    const int lane = threadIdx.x & 31, k = u.k, nblk = (k + NB - 1) / NB;
+    const bool mt = u.flags & 1, rev = u.flags & 2, unitd = u.flags & 4, left = u.flags & 8;
+    int64_t sr = mt ? u.lda : 1, sc = mt ? 1 : u.lda, br = left ? 1 : u.ldb;
+    const int64_t bc = left ? u.ldb : 1;
+    const float *A = u.A;
+    float *B = u.B;
+    if (rev) {
+        A += int64_t(k - 1) * (sr + sc);
+        B += int64_t(k - 1) * br;
+        sr = -sr;
+        sc = -sc;
+        br = -br;
+    }
+    // A tile's copies run along A's contiguous dimension: 32 rows of a column,
+    // or (mt) 8 columns of 4 rows, which spreads the columns' stores over the
+    // banks.  Lane's entry (li, lk) of copy (x, y): row li + 4 x, column lk + 8 y,
+    // or row li, column x.
+    const int li = mt ? lane >> 3 : lane, lk = mt ? lane & 7 : 0;
+    const int64_t lsrc = li * sr + lk * sc;
+    const int ldst = lk * WLD + li;
+    auto load_tile = [&](int b, int kb, float *t) {
+        const float *src = A + int64_t(b) * NB * sr + int64_t(kb) * NB * sc + lsrc;
+        float *dst = t + ldst;
+        if (kb < b && (b + 1) * NB <= k) {
+            if (mt) {
+#pragma unroll 4
+                for (int y = 0; y < 4; y++)
 #pragma unroll
-        for (int e = 0; e < PER; e++) x[b][e] = xp[e];
+                    for (int x = 0; x < 8; x++) cp4(dst + 8 * y * WLD + 4 * x, src + (4 * x * sr + 8 * y * sc), true);
+            } else {
+#pragma unroll 8
+                for (int x = 0; x < NB; x++) cp4(dst + x * WLD, src + x * sc, true);
+            }
+            return;
+        }
+        // the last rows, and the strict triangle
+        const int rows = k - b * NB;
+        for (int s = 0; s < NB; s++) {
+            const int x = mt ? 4 * (s & 7) : 0, y = mt ? 8 * (s >> 3) : s;
+            const int i = li + x, c = lk + y;
+            const bool in = i < rows && (kb < b || c < i);
+            cp4(dst + y * WLD + x, in ? src + (x * sr + y * sc) : u.A, in);
+        }
     };
-    load(0, 0);
-    load(1, 1);
-#pragma unroll
-    for (int kk = 0; kk < NBB; kk++) {
-        if (kk + 2 < NBB) load(kk + 2, (kk + 2) % D);
-        const int b = kk % D;
-#pragma unroll
-        for (int q = 0; q < RR; q++)
-#pragma unroll
-            for (int e = 0; e < PER; e++) acc[q][e] += a[b][q] * x[b][e];
+    // the warp's tiles in order: block rows wid, wid + nwu, ...; in each kb = 0 .. b
+    int pb = tm.wid, pk = 0, pn = 0;
+    auto prefetch = [&]() {
+        if (pb < nblk) {
+            load_tile(pb, pk, tm.ring + (pn & 1) * TILE);
+            if (pk == pb) {
+                pb += tm.nwu;
+                pk = 0;
+            } else {
+                pk++;
+            }
+        }
+        pn++;
+        commit();
+    };
+    prefetch();
+    int n = 0, known = 0;
+    bool gave_up = false;
+    for (int b = tm.wid; b < nblk; b += tm.nwu) {
+        const int r0 = b * NB, rows = min(NB, k - r0);
+        // the rows' right-hand sides into their place in X
+        float *xs = tm.Xs + size_t(b) * NB * XLD;
+        {
+            const float *src = B + int64_t(r0) * br + (left ? lane * br : lane * bc);
+            const int64_t step = left ? bc : br;
+            const int ds = left ? 1 : XLD;
+            float *dst = xs + lane * (left ? XLD : 1);
+            const int cnt = left ? u.cw : rows;
+            const bool in = left ? lane < rows : lane < u.cw;
+            // (what the copies leave out is zero)
+#pragma unroll 8
+            for (int x = 0; x < NB; x++) cp4(dst + x * ds, (in && x < cnt) ? src + x * step : u.A, in && x < cnt);
+        }
+        commit();
+        {
+            const float dg = (!unitd && lane < rows) ? A[int64_t(r0 + lane) * (sr + sc)] : 1.f;
+            __syncwarp();
+            tm.inv[lane] = 1.f / dg;
+            tm.inv[NB + lane] = dg;
+        }
+        float *xb = xs + lane;
+        Sum<true> sum;
+        sum.clear();
+        for (int kb = 0; kb < b; kb++, n++) {
+            wait_all();
+            __syncwarp();
+            prefetch();  // into the buffer of tile n - 1, which every lane has read
+            if (tm.nwu > 1) await_block(tm.solved, kb, known, gave_up);
+            sum.update<XLD>(tm.ring + (n & 1) * TILE, tm.Xs + size_t(kb) * NB * XLD + lane);
+        }
+        wait_all();
+        __syncwarp();
+        prefetch();
+        substitute<true, true, XLD>(sum.t, tm.ring + (n & 1) * TILE, tm.inv, xb, 1.f);
+        n++;
+        // a reader that gave up (it cannot unless the device is broken) says
+        // so in every row from there on
+        if (gave_up) {
+            for (int i = 0; i < NB; i++) xb[i * XLD] = NAN;
+        }
+        publish_block(tm.solved, b);
+        {
+            float *dst = B + int64_t(r0) * br + (left ? lane * br : lane * bc);
+            const int64_t step = left ? bc : br;
+            const int ds = left ? 1 : XLD;
+            const float *src = xs + lane * (left ? XLD : 1);
+            const int cnt = left ? u.cw : rows;
+            if (left ? lane < rows : lane < u.cw) {
+#pragma unroll 8
+                for (int x = 0; x < cnt; x++) dst[x * step] = u.alpha * src[x * ds];
+            }
+        }
     }
+    wait_all();
+    __syncwarp();  // X, the ring and the inverses are free for the next unit
 }
 
-// smem: Xs[KMAX][LX], NBUF k-major tiles Ts[NBB][LT], inverse diagonal.
-template <typename T, int RR>
-__global__ void __launch_bounds__(NT)
-batched_kernel(const Unit<T> *__restrict__ units, int nunits, unsigned *__restrict__ ticket)
+// FP64, in solution order (a backward problem by negative strides): lane l
+// holds rows 2q + h (h = l / 16) of the block for right-hand side l % 16.
+__device__ __forceinline__ void solve_unit(const Unit<double> &u, const Team<double> &tm)
 {
-    using C = BCfg<T, RR>;
-    constexpr int CW = C::CW, LX = C::LX, PER = C::PER;
-    constexpr int TS = NBB * LT;
-    constexpr int CPW = CW / 8;  // columns per warp in the TS task
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *Xs = reinterpret_cast<T *>(smem_raw);
-    T *Ts = Xs + KMAX * LX;
-    constexpr int NBUF = nbuf<T>();
-    T *inv = Ts + NBUF * TS;
-    __shared__ int cur;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-
-    for (;;) {
-        if (tid == 0) cur = int(atomicAdd(ticket, 1u));
-        __syncthreads();
-        const int t = cur;
-        __syncthreads();
-        if (t >= nunits) return;
-        const Unit<T> u = units[t];
-        const int k = u.k, cw = u.cw;
-        const bool rev = u.flags & 2, unitd = u.flags & 4, left = u.flags & 8;
-        const int nblk = (k + NBB - 1) / NBB;
-        const int ntile = nblk * (nblk + 1) / 2;
-
-        // ---- Xs = Bv' (forward view of the chunk; alpha is applied on the
-        // way out), issued together with the first A tiles --------------------
-        // rows k .. 32*nblk-1 are zero: the ragged last block multiplies them
-        // by zero tile entries, and stale shared memory could hold a NaN
-        const int kr = nblk * NBB;
-        if (left) {
-            // contiguous along i: warp w takes columns w, w + 8, ..., its lanes the rows
-            for (int c = warp; c < CW; c += NT / 32) {
-                const T *bc = u.B + int64_t(c) * u.ldb;
-                for (int i = lane; i < kr; i += 32) {
-                    const bool in = c < cw && i < k;
-                    cp_async_elem(Xs + i * LX + c, in ? bc + (rev ? k - 1 - i : i) : u.B, in);
-                }
-            }
-        } else {
-            for (int idx = tid; idx < kr * CW; idx += NT) {  // contiguous along c (CW is a power of two)
-                const int c = idx % CW, i = idx / CW;
-                const int io = rev ? k - 1 - i : i;
-                const bool in = c < cw && i < k;
-                cp_async_elem(Xs + i * LX + c, in ? u.B + c + int64_t(io) * u.ldb : u.B, in);
-            }
+    constexpr int CW = kChunk<double>, NQ = NBB / 2;
+    const int lane = threadIdx.x & 31, h = lane >> 4, col = lane & 15;
+    const int k = u.k, nblk = (k + NBB - 1) / NBB;
+    const bool mt = u.flags & 1, rev = u.flags & 2, unitd = u.flags & 4, left = u.flags & 8;
+    int64_t sr = mt ? u.lda : 1, sc = mt ? 1 : u.lda, br = left ? 1 : u.ldb;
+    const double *A = u.A;
+    double *B = u.B + col * (left ? u.ldb : 1);
+    if (rev) {
+        A += int64_t(k - 1) * (sr + sc);
+        B += int64_t(k - 1) * br;
+        sr = -sr;
+        sc = -sc;
+        br = -br;
+    }
+    const bool incol = col < u.cw;
+    int known = 0;
+    bool gave_up = false;
+    for (int b = tm.wid; b < nblk; b += tm.nwu) {
+        const int r0 = b * NBB, nv = min(NBB, k - r0), nq = (nv + 1) / 2;
+        // entry (row 2q + h, column) of the block row; a row past the last one
+        // reads the row before it (its results are not used)
+        const double *Ar = A + int64_t(r0 + h) * sr;
+        const int64_t last = (nv & 1) && h ? (nv - 1) : -1;  // 2q of the lane's row past the end
+        auto row = [&](const double *p, int q) { return p[(2 * q == last ? int64_t(2 * q - 1) : int64_t(2 * q)) * sr]; };
+        double t[NQ], acc[NQ];
+#pragma unroll
+        for (int q = 0; q < NQ; q++) {
+            t[q] = (incol && 2 * q + h < nv) ? B[int64_t(r0 + 2 * q + h) * br] : 0.0;
+            acc[q] = 0.0;
         }
-        cp_async_commit();
-        TilePos pf;  // the next tile to load
-#pragma unroll 1
-        for (int q = 0; q < NBUF - 1; q++) {
-            if (q < ntile) {
-                load_tile(u, pf.jb, pf.ib, Ts + q * TS);
-                pf.next();
-            }
-            cp_async_commit();
-        }
-
-        // a warp owns PER * 32 / ROWG columns of every row of the block, so
-        // its A rows load as whole wavefronts and its X vector as a
-        // broadcast, and a warp past the chunk's last right-hand side skips
-        // its products (the columns of X there stay zero)
-        const int r = (tid % C::ROWG) * RR, cq = (tid / C::ROWG) * PER;
-        const bool live = cq < cw;
-        T acc[RR][PER];
+        const double inv = (!unitd && lane < nv) ? 1.0 / A[int64_t(r0 + lane) * (sr + sc)] : 1.0;
+        for (int kb = 0; kb < b; kb++) {
+            if (tm.nwu > 1) await_block(tm.solved, kb, known, gave_up);
+            const double *x0 = tm.Xs + size_t(kb) * NBB * CW + col;
+            const double *ac = Ar + int64_t(kb) * NBB * sc;
+            if (nv == NBB) {
+#pragma unroll 2
+                for (int kk = 0; kk < NBB; kk++) {
+                    const double x = x0[kk * CW];
+                    double a[NQ];
 #pragma unroll
-        for (int a = 0; a < RR; a++)
+                    for (int q = 0; q < NQ; q++) a[q] = ac[int64_t(2 * q) * sr + kk * sc];
 #pragma unroll
-            for (int e = 0; e < PER; e++) acc[a][e] = T(0);
-        TilePos cur;  // tile tt
-        for (int tt = 0; tt < ntile; tt++, cur.next()) {
-            // wait until tile tt (and the B chunk) has landed; the barrier
-            // also means every thread is done with tile tt - 1, whose buffer
-            // then takes tile tt + NBUF - 1 (NBUF - 1 tiles stay in flight)
-            cp_async_wait<NBUF - 2>();
-            __syncthreads();
-            if (tt + NBUF - 1 < ntile) {
-                load_tile(u, pf.jb, pf.ib, Ts + ((tt + NBUF - 1) % NBUF) * TS);
-                pf.next();
-            }
-            cp_async_commit();
-            const T *Tb = Ts + (tt % NBUF) * TS;
-            const int jb = cur.jb, ib = cur.ib;
-            const int j0 = jb * NBB, nr = min(NBB, k - j0);
-            if (ib < jb) {
-                // gemm task: acc += Mv'(j, i) X_i
-                if (live) tile_fma<T, RR, PER, LX>(acc, Tb, Xs + ib * NBB * LX, r, cq);
-            } else if (u.Linv) {
-                // X_j -= sum of the gemm tasks, then the TS task as the
-                // product X_j = L_jj^-1 X_j on the register tiles
-#pragma unroll
-                for (int q = 0; q < RR; q++) {
-                    if (r + q < nr) {
-#pragma unroll
-                        for (int e = 0; e < PER; e++) Xs[(j0 + r + q) * LX + cq + e] -= acc[q][e];
-                    }
-#pragma unroll
-                    for (int e = 0; e < PER; e++) acc[q][e] = T(0);
-                }
-                __syncthreads();
-                if (live) tile_fma<T, RR, PER, LX>(acc, Tb, Xs + j0 * LX, r, cq);
-                __syncthreads();  // every thread has read X_j
-#pragma unroll
-                for (int q = 0; q < RR; q++) {
-                    if (r + q < nr) {
-#pragma unroll
-                        for (int e = 0; e < PER; e++) Xs[(j0 + r + q) * LX + cq + e] = acc[q][e];
-                    }
-#pragma unroll
-                    for (int e = 0; e < PER; e++) acc[q][e] = T(0);
+                    for (int q = 0; q < NQ; q++) acc[q] = fma(a[q], x, acc[q]);
                 }
             } else {
-                // X_j -= sum of the gemm tasks, then the TS task: the nr x nr
-                // triangle by warp-shuffle substitution
+                for (int kk = 0; kk < NBB; kk++) {
+                    const double x = x0[kk * CW];
+                    const double *p = ac + kk * sc;
 #pragma unroll
-                for (int q = 0; q < RR; q++) {
-                    if (r + q < nr) {
+                    for (int g = 0; g < NQ; g += 4) {
+                        if (g >= nq) break;
 #pragma unroll
-                        for (int e = 0; e < PER; e++) Xs[(j0 + r + q) * LX + cq + e] -= acc[q][e];
+                        for (int q = g; q < g + 4; q++)
+                            if (q < nq) acc[q] = fma(row(p, q), x, acc[q]);
                     }
-#pragma unroll
-                    for (int e = 0; e < PER; e++) acc[q][e] = T(0);
-                }
-                if (tid < NBB) inv[tid] = (tid < nr && !unitd) ? T(1) / Tb[tid * LT + tid] : T(1);
-                __syncthreads();
-                // warp w solves columns w, w+8, ... (CPW columns, interleaved for ILP)
-                T tv[CPW];
-#pragma unroll
-                for (int e = 0; e < CPW; e++) tv[e] = (lane < nr) ? Xs[(j0 + lane) * LX + warp + 8 * e] : T(0);
-                // columns past the chunk's last right-hand side stay zero
-                for (int kk = 0; kk < (warp < cw ? nr : 0); kk++) {
-                    const T d = inv[kk];
-                    const T lk = Tb[kk * LT + lane];
-#pragma unroll
-                    for (int e = 0; e < CPW; e++) {
-                        const T x = __shfl_sync(0xffffffffu, tv[e], kk) * d;
-                        if (lane == kk) tv[e] = x;
-                        else if (lane > kk) tv[e] -= lk * x;
-                    }
-                }
-                if (lane < nr) {
-#pragma unroll
-                    for (int e = 0; e < CPW; e++) Xs[(j0 + lane) * LX + warp + 8 * e] = tv[e];
                 }
             }
         }
-        cp_async_wait<0>();
-        __syncthreads();  // the last block's X (written by every thread) is complete
-
-        // ---- write back alpha * X (undo reversal / transposition) -----------
-        if (left) {
-            for (int c = warp; c < cw; c += NT / 32) {
-                T *bc = u.B + int64_t(c) * u.ldb;
-                for (int i = lane; i < k; i += 32) bc[rev ? k - 1 - i : i] = u.alpha * Xs[i * LX + c];
-            }
-        } else {
-            for (int idx = tid; idx < k * CW; idx += NT) {
-                const int c = idx % CW, i = idx / CW;
-                if (c < cw) u.B[c + int64_t(rev ? k - 1 - i : i) * u.ldb] = u.alpha * Xs[i * LX + c];
+#pragma unroll
+        for (int q = 0; q < NQ; q++) t[q] -= acc[q];
+        // the triangle: x_k by the lanes of its row's half, the rows below it by all
+        const double *ad = Ar + int64_t(r0) * sc;
+#pragma unroll
+        for (int kk = 0; kk < NBB; kk++) {
+            if (kk < nv) {
+                const double v = t[kk >> 1] * __shfl_sync(0xffffffffu, inv, kk);
+                const double x = __shfl_sync(0xffffffffu, v, (kk & 1) * 16 + col);
+                if (h == (kk & 1)) t[kk >> 1] = x;
+                const double *p = ad + kk * sc;
+#pragma unroll
+                for (int q = 0; q < NQ; q++) {
+                    if (2 * q + 1 <= kk || q >= nq) continue;
+                    // rows 2q (h = 0) and 2q + 1 (h = 1), below kk
+                    const bool below = 2 * q > kk || h == 1;
+                    const double a = below ? row(p, q) : 0.0;
+                    const double r = fma(-a, x, t[q]);
+                    t[q] = below ? r : t[q];
+                }
             }
         }
-        __syncthreads();
-    }
-}
-
-// Diagonal-block inverses of one instance per CTA (FP32): warp w inverts the
-// forward-view blocks w, w + 8, ...: the lower triangle (unit diagonal when
-// flagged) goes to shared memory, lane c solves L x = e_c by forward
-// substitution in registers (x_r = 0 above the diagonal; rows past the
-// instance's order are the identity) and writes column c of the inverse,
-// k-major (Linv[c * 32 + r] = inverse(r, c)).
-struct InvJob {
-    const float *A;
-    float *Linv;
-    int64_t lda;
-    int k;
-    int flags;  // as Unit::flags (bit0 mt, bit1 rev, bit2 unit diagonal)
-};
-
-__global__ void __launch_bounds__(NT) batched_inv_kernel(const InvJob *__restrict__ jobs, int njobs)
-{
-    __shared__ float Ls[NT / 32][NBB][NBB + 1];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int jj = blockIdx.x; jj < njobs; jj += gridDim.x) {
-        const InvJob J = jobs[jj];
-        Unit<float> u{};
-        u.A = J.A;
-        u.lda = J.lda;
-        u.k = J.k;
-        u.flags = J.flags;
-        const bool unitd = J.flags & 4;
-        const bool mt = J.flags & 1;
-        const int nblk = (J.k + NBB - 1) / NBB;
-        for (int b = warp; b < nblk; b += NT / 32) {
-            const int j0 = b * NBB, nr = min(NBB, J.k - j0);
-            // the block's lower triangle, read along A's contiguous dimension
-            for (int idx = lane; idx < NBB * NBB; idx += 32) {
-                const int fast = idx % NBB, slow = idx / NBB;
-                const int rr = mt ? slow : fast, cc = mt ? fast : slow;
-                float v = 0.f;
-                if (rr < nr && cc < nr && cc <= rr) v = *mv_addr(u, j0 + rr, j0 + cc);
-                if (rr == cc && (unitd || rr >= nr)) v = 1.f;
-                Ls[warp][rr][cc] = v;
-            }
-            __syncwarp();
-            float x[NBB];
+        // a reader that gave up (it cannot unless the device is broken) says
+        // so in every row from there on
+        if (gave_up) {
 #pragma unroll
-            for (int r = 0; r < NBB; r++) {
-                float sum = (r == lane) ? 1.f : 0.f;
+            for (int q = 0; q < NQ; q++) t[q] = NAN;
+        }
+        double *xb = tm.Xs + size_t(b) * NBB * CW + h * CW + col;
 #pragma unroll
-                for (int t = 0; t < r; t++) sum -= Ls[warp][r][t] * x[t];
-                x[r] = (r < lane) ? 0.f : sum / Ls[warp][r][r];
-            }
-            float *dst = J.Linv + size_t(b) * NBB * NBB + size_t(lane) * NBB;
+        for (int q = 0; q < NQ; q++) xb[2 * q * CW] = t[q];
+        publish_block(tm.solved, b);
+        if (incol) {
 #pragma unroll
-            for (int r = 0; r < NBB; r++) dst[r] = x[r];
-            __syncwarp();
+            for (int q = 0; q < NQ; q++)
+                if (2 * q + h < nv) B[int64_t(r0 + 2 * q + h) * br] = u.alpha * t[q];
         }
     }
 }
 
-template <typename T, int RR>
+// Shared memory: the warps' rings and inverse diagonals (FP32), then X: KMAX
+// rows, divided among the CTA's teams.
+template <typename T>
 constexpr size_t batched_smem()
 {
-    return sizeof(T) * (size_t(KMAX) * BCfg<T, RR>::LX + nbuf<T>() * NBB * LT + NBB);
+    return sizeof(T) * ((sizeof(T) == 4 ? size_t(NW) * (2 * wide::TILE + 2 * NBB) : 0) + size_t(KMAX) * kStride<T>);
+}
+
+// The units by the team that solves them: [0, n4) a CTA's four warps, [n4, n2)
+// two warps, [n2, n1) one.
+struct Queues {
+    int n4, n2, n1;
+};
+
+// ticket[0..2]: the queues' counters.
+template <typename T>
+__global__ void __launch_bounds__(NT, sizeof(T) == 8 ? 3 : 2)
+batched_kernel(const Unit<T> *__restrict__ units, Queues qs, unsigned *__restrict__ ticket)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int cur[NW], solved[NW];
+    T *sm = reinterpret_cast<T *>(smem_raw);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    Team<T> tm;
+    tm.ring = tm.inv = nullptr;
+    T *Xs = sm;
+    if (sizeof(T) == 4) {
+        tm.ring = sm + warp * 2 * wide::TILE;
+        tm.inv = sm + NW * 2 * wide::TILE + warp * 2 * NBB;
+        Xs = sm + NW * (2 * wide::TILE + 2 * NBB);
+    }
+#pragma unroll 1
+    for (int c = 0; c < 3; c++) {
+        const int nwu = NW >> c, team = warp / nwu;
+        const int lo = c == 0 ? 0 : (c == 1 ? qs.n4 : qs.n2), hi = c == 0 ? qs.n4 : (c == 1 ? qs.n2 : qs.n1);
+        tm.nwu = nwu;
+        tm.wid = warp % nwu;
+        tm.Xs = Xs + size_t(team) * (KMAX / NW) * nwu * kStride<T>;
+        tm.solved = &solved[team];
+        // a team's own barrier (the team of four: the CTA's)
+        auto team_sync = [&]() {
+            if (nwu == NW) __syncthreads();
+            else if (nwu == 2) asm volatile("bar.sync %0, 64;" ::"r"(1 + team) : "memory");
+            else __syncwarp();
+        };
+        __syncthreads();  // the other teams' X space is free
+        for (;;) {
+            team_sync();  // every warp of the team has left its last unit
+            if (tm.wid == 0 && lane == 0) {
+                cur[team] = lo + int(atomicAdd(&ticket[c], 1u));
+                solved[team] = 0;
+            }
+            team_sync();
+            const int t = cur[team];
+            if (t >= hi) break;
+            const Unit<T> u = units[t];
+            solve_unit(u, tm);
+        }
+    }
 }
 
 }  // namespace
@@ -457,10 +391,11 @@ constexpr size_t batched_smem()
 
 struct BatchedPlan {
     int dtype = 0;                 // 0 FP64, 1 FP32
-    int tile = 1;                  // rows per thread in the gemm tasks (1 or 2)
+    int tile = 1;                  // split of the work over teams (see build_units)
     int64_t nunits = 0;
+    Queues queues = {0, 0, 0};     // the units by team size
     void *units = nullptr;         // device array of Unit<T>
-    unsigned *ticket = nullptr;    // device work-queue counter
+    unsigned *ticket = nullptr;    // the device work queues' counters
     int grid = 0;
     // instances too large for shared memory, solved by the regular driver
     struct Big {
@@ -474,11 +409,6 @@ struct BatchedPlan {
     cudaGraphExec_t exec = nullptr;
     uint64_t graph_kernels = 0;
     double flops = 0, bytes = 0;
-    // FP32: inverses of every instance's diagonal blocks, recomputed each run
-    std::vector<InvJob> jobs_h;
-    InvJob *jobs = nullptr;
-    float *linv = nullptr;
-    size_t linv_elems = 0;
 };
 
 namespace {
@@ -488,7 +418,7 @@ void build_units(BatchedPlan &P, int64_t count, const int8_t *side, const int8_t
                  const int8_t *diag, const int64_t *m, const int64_t *n, const T *alpha, const void *const *A,
                  const int64_t *lda, void *const *B, const int64_t *ldb, std::vector<Unit<T>> &units)
 {
-    const int CW = P.tile == 2 ? BCfg<T, 2>::CW : BCfg<T, 1>::CW;
+    constexpr int CW = kChunk<T>;
     for (int64_t i = 0; i < count; i++) {
         if (m[i] == 0 || n[i] == 0) continue;
         const bool left = side[i] == GB_LEFT;
@@ -504,27 +434,11 @@ void build_units(BatchedPlan &P, int64_t count, const int8_t *side, const int8_t
         const bool mt = left ? (trans[i] == GB_TRANS) : (trans[i] == GB_NOTRANS);
         const bool fwd = (uplo[i] == GB_LOWER) != mt;
         const int flags = (mt ? 1 : 0) | (fwd ? 0 : 2) | (diag[i] == GB_UNIT ? 4 : 0) | (left ? 8 : 0);
-        // FP32: the instance's block inverses at this element offset of the
-        // plan's inverse buffer (kept as offset + 1, 0 meaning none, until
-        // the pointer is filled in on upload)
-        size_t linv_off = 0;
-        if (sizeof(T) == 4) {
-            linv_off = P.linv_elems + 1;
-            P.linv_elems += size_t((k + NBB - 1) / NBB) * NBB * NBB;
-            InvJob j;
-            j.A = reinterpret_cast<const float *>(A[i]);
-            j.Linv = reinterpret_cast<float *>(linv_off);
-            j.lda = lda[i];
-            j.k = int(k);
-            j.flags = flags;
-            P.jobs_h.push_back(j);
-        }
         for (int64_t c0 = 0; c0 < ncols; c0 += CW) {
             Unit<T> u;
             u.A = static_cast<const T *>(A[i]);
             T *b = static_cast<T *>(B[i]);
             u.B = left ? b + c0 * ldb[i] : b + c0;
-            u.Linv = sizeof(T) == 4 ? reinterpret_cast<const T *>(linv_off) : nullptr;
             u.lda = lda[i];
             u.ldb = ldb[i];
             u.k = int(k);
@@ -534,57 +448,52 @@ void build_units(BatchedPlan &P, int64_t count, const int8_t *side, const int8_t
             units.push_back(u);
         }
     }
-    // largest first (longest-processing-time order for the work queue)
-    std::stable_sort(units.begin(), units.end(),
-                     [](const Unit<T> &a, const Unit<T> &b) { return a.k * a.cw > b.k * b.cw; });
+    // by team size (warps per unit: X of a team of w warps is w KMAX / 4 rows),
+    // largest first inside (longest-processing-time order for the queues)
+    const int one = P.tile == 2 ? KMAX / 8 : KMAX / 4, two = 2 * one;
+    auto cls = [one, two](const Unit<T> &a) { return a.k > two ? 0 : (a.k > one ? 1 : 2); };
+    std::stable_sort(units.begin(), units.end(), [&](const Unit<T> &a, const Unit<T> &b) {
+        if (cls(a) != cls(b)) return cls(a) < cls(b);
+        return a.k * a.cw > b.k * b.cw;
+    });
+    P.queues.n4 = int(std::count_if(units.begin(), units.end(), [&](const Unit<T> &a) { return cls(a) == 0; }));
+    P.queues.n2 = P.queues.n4 + int(std::count_if(units.begin(), units.end(), [&](const Unit<T> &a) { return cls(a) == 1; }));
+    P.queues.n1 = int(units.size());
 }
 
-template <typename T, int RR>
+template <typename T>
 int upload_and_capture(BatchedPlan &P, std::vector<Unit<T>> &units, cudaStream_t s)
 {
     P.nunits = int64_t(units.size());
     const size_t ub = units.size() * sizeof(Unit<T>);
     GB_CUDA(cudaMalloc(&P.units, ub > 0 ? ub : sizeof(Unit<T>)));
-    GB_CUDA(cudaMalloc(&P.ticket, sizeof(unsigned)));
-    if (!P.jobs_h.empty()) {
-        GB_CUDA(cudaMalloc(&P.linv, P.linv_elems * sizeof(float)));
-        GB_CUDA(cudaMalloc(&P.jobs, P.jobs_h.size() * sizeof(InvJob)));
-        for (auto &j : P.jobs_h) j.Linv = P.linv + (reinterpret_cast<size_t>(j.Linv) - 1);
-        for (auto &u : units)
-            if (u.Linv) u.Linv = reinterpret_cast<const T *>(P.linv) + (reinterpret_cast<size_t>(u.Linv) - 1);
-        GB_CUDA(cudaMemcpyAsync(P.jobs, P.jobs_h.data(), P.jobs_h.size() * sizeof(InvJob), cudaMemcpyHostToDevice,
-                                s));
-    }
+    GB_CUDA(cudaMalloc(&P.ticket, 3 * sizeof(unsigned)));
     if (ub) GB_CUDA(cudaMemcpyAsync(P.units, units.data(), ub, cudaMemcpyHostToDevice, s));
     GB_CUDA(cudaStreamSynchronize(s));
     static PerDeviceOnce attr;
-    GB_TRY(smem_attr_once(attr, batched_kernel<T, RR>, batched_smem<T, RR>()));
+    GB_TRY(smem_attr_once(attr, batched_kernel<T>, batched_smem<T>()));
     int dev = 0, sms = 0, per_sm = 0;
     GB_CUDA(cudaGetDevice(&dev));
     GB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_kernel<T, RR>, NT, batched_smem<T, RR>()));
+    GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_kernel<T>, NT, batched_smem<T>()));
     if (per_sm < 1) per_sm = 1;
     int64_t g = int64_t(sms) * per_sm;
-    if (g > P.nunits) g = P.nunits;
+    // (smaller teams share a CTA)
+    const int64_t need = P.queues.n4 + (P.queues.n2 - P.queues.n4 + 1) / 2 + (P.queues.n1 - P.queues.n2 + 3) / 4;
+    if (g > need) g = need;
     P.grid = int(g);
     if (P.nunits == 0) return 0;
-    // CUDA graph: [reset the queue counter, persistent kernel]
+    // CUDA graph: [reset the queue counters, persistent kernel]
     cudaStream_t cs;
     GB_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     const uint64_t before = capture_count();
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaMemsetAsync(P.ticket, 0, sizeof(unsigned), cs);
-        if (!P.jobs_h.empty()) {
-            const int64_t nj = int64_t(P.jobs_h.size());
-            const int64_t gi = nj < int64_t(sms) * 8 ? nj : int64_t(sms) * 8;
-            LaunchScope ls(KK_BATCHED, cs, 0.0, 4.0 * double(P.linv_elems));
-            batched_inv_kernel<<<(unsigned)gi, NT, 0, cs>>>(P.jobs, int(nj));
-        }
+        cudaMemsetAsync(P.ticket, 0, 3 * sizeof(unsigned), cs);
         {
             LaunchScope ls(KK_BATCHED, cs, P.flops, P.bytes);
-            batched_kernel<T, RR><<<P.grid, NT, batched_smem<T, RR>(), cs>>>(
-                static_cast<const Unit<T> *>(P.units), int(P.nunits), P.ticket);
+            batched_kernel<T><<<P.grid, NT, batched_smem<T>(), cs>>>(
+                static_cast<const Unit<T> *>(P.units), P.queues, P.ticket);
         }
         cudaGraph_t graph = nullptr;
         e = cudaStreamEndCapture(cs, &graph);
@@ -625,8 +534,6 @@ void batched_free(BatchedPlan *P)
     if (P->exec) cudaGraphExecDestroy(P->exec);
     if (P->units) cudaFree(P->units);
     if (P->ticket) cudaFree(P->ticket);
-    if (P->jobs) cudaFree(P->jobs);
-    if (P->linv) cudaFree(P->linv);
     delete P;
 }
 
@@ -665,12 +572,12 @@ int batched_create(int dtype, int64_t count, const int8_t *side, const int8_t *u
         std::vector<Unit<double>> units;
         build_units<double>(*P, count, side, uplo, trans, diag, m, n, static_cast<const double *>(alpha), A, lda, B,
                             ldb, units);
-        st = tile == 2 ? upload_and_capture<double, 2>(*P, units, s) : upload_and_capture<double, 1>(*P, units, s);
+        st = upload_and_capture<double>(*P, units, s);
     } else {
         std::vector<Unit<float>> units;
         build_units<float>(*P, count, side, uplo, trans, diag, m, n, static_cast<const float *>(alpha), A, lda, B,
                            ldb, units);
-        st = tile == 2 ? upload_and_capture<float, 2>(*P, units, s) : upload_and_capture<float, 1>(*P, units, s);
+        st = upload_and_capture<float>(*P, units, s);
     }
     if (st) {
         batched_free(P);

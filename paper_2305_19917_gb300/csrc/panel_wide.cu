@@ -4,33 +4,19 @@
 // As there, a CTA walks a block of up to 1024 rows by itself, left-looking in
 // 32-row blocks, each warp owning every fourth block row and streaming its own
 // tiles of Mv.  But a lane holds one right-hand side and the block's 32 rows of
-// it in registers, instead of one row and CW right-hand sides: a substitution
-// step then has no shuffles and 31 independent multiply-adds behind it (a
-// 32 x 32 block takes 528 multiply-adds for 32 right-hand sides, where the
-// other form spends about 100 instructions a step), and an update step loads
-// one X value per lane and its 32 Mv entries as eight broadcast vectors:
-// nine shared-memory wavefronts per 32 multiply-adds, close to the eight
-// clocks that these take.  Bounded by FFMA issue, those wavefronts and, for
-// few CTAs, the chain of blocks.  Two CTAs of 4 warps share an SM.  Measured,
-// 512 rows: 8192 right-hand sides 138 us (the other form 265), 2500 104.
+// it, instead of one row and CW right-hand sides (wide_tile.cuh).  Bounded by
+// the issue of one warp per sub-partition (two CTAs of 4 warps share an SM)
+// and, for few CTAs, the chain of blocks.  Measured, 512 rows: 8192 right-hand sides
+// 138 us (the other form 265), 2500 104.
 #include <cmath>
 #include "panel.cuh"
-#include "tc_common.cuh"
+#include "wide_tile.cuh"
 
 namespace gb {
 namespace {
 
-constexpr int NB = 32, NW = 4, NS = 2, LD = NB + 4, TILE = NB * LD, CW = 32;
-constexpr int kSpins = 1 << 22;  // polls before a reader gives up
-
-__device__ __forceinline__ void cpa16(float *dst, const float *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cpa4(float *dst, const float *src, bool in)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(tc::smem_u32(dst)), "l"(src), "r"(in ? 4 : 0) : "memory");
-}
+using namespace wide;
+constexpr int NW = 4, NS = 2;
 
 constexpr size_t wide_smem(int nblk) { return sizeof(float) * (size_t(NW) * (NS * TILE + NB) + size_t(nblk) * NB * CW); }
 
@@ -39,7 +25,7 @@ constexpr size_t wide_smem(int nblk) { return sizeof(float) * (size_t(NW) * (NS 
 // 16 bytes at a time.  Rows inside a block are numbered in natural order; a
 // backward solve takes the blocks from the bottom and the rows downwards.
 template <bool AM, bool FWD>
-__global__ void __launch_bounds__(32 * NW)
+__global__ void __launch_bounds__(32 * NW, 2)
 panel_wide_kernel(const float *__restrict__ M, int64_t lda, float *__restrict__ B, int64_t si, int64_t sc, int nr,
                   int64_t ncols, float alpha, int unit, int vec, int vecb)
 {
@@ -58,33 +44,11 @@ panel_wide_kernel(const float *__restrict__ M, int64_t lda, float *__restrict__ 
     __syncthreads();
 
     auto nat = [&](int b) { return FWD ? b * NB : nr - (b + 1) * NB; };
-    // Off-diagonal tiles stay in Mv's storage order ([k][row] for AM, [row][k]
-    // else); a block's triangle is stored [k][row], zero outside the strict
-    // triangle.
-    auto load_tile = [&](int b, int kb, float *t) {
-        const int ri = nat(b), ci = nat(kb);
-        const float *src = AM ? M + ri + int64_t(ci) * lda : M + ci + int64_t(ri) * lda;
-        if (vec && kb < b && ri >= 0 && ri + NB <= nr) {
-#pragma unroll
-            for (int q = 0; q < 8; q++) {
-                const int idx = lane + 32 * q, f = (idx % 8) * 4, s = idx / 8;
-                cpa16(t + s * LD + f, src + f + int64_t(s) * lda);
-            }
-            return;
-        }
-#pragma unroll 8
-        for (int s = 0; s < NB; s++) {
-            const int i = AM ? lane : s, k = AM ? s : lane;
-            bool in = ri + i >= 0 && ri + i < nr && ci + k >= 0 && ci + k < nr;
-            if (kb == b) in = in && (FWD ? k < i : k > i);
-            cpa4(t + (kb == b ? k * LD + i : s * LD + lane), in ? src + lane + int64_t(s) * lda : M, in);
-        }
-    };
     // the warp's tiles in order: block rows warp, warp + NW, ...; in each kb = 0 .. b
     int pb = warp, pk = 0, pn = 0;
     auto prefetch = [&]() {
         if (pb < nblk) {
-            load_tile(pb, pk, ring + (pn % NS) * TILE);
+            load_block<AM>(M, lda, nr, nat(pb), nat(pk), pk < pb ? 0 : (FWD ? 1 : 2), vec, ring + (pn % NS) * TILE);
             if (pk == pb) {
                 pb += NW;
                 pk = 0;
@@ -93,7 +57,7 @@ panel_wide_kernel(const float *__restrict__ M, int64_t lda, float *__restrict__ 
             }
         }
         pn++;
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        commit();
     };
     prefetch();
 
@@ -101,9 +65,8 @@ panel_wide_kernel(const float *__restrict__ M, int64_t lda, float *__restrict__ 
     bool gave_up = false;
     for (int b = warp; b < nblk; b += NW) {
         const int r0 = nat(b);
-        float t[NB];  // first the updates' sum, then the rows
-#pragma unroll
-        for (int i = 0; i < NB; i++) t[i] = 0.f;
+        Sum<AM> sum;
+        sum.clear();
         // the rows' right-hand sides into their place in X (read again by the
         // lane that copied them)
         const float *bc = B + col * sc + int64_t(r0) * si;
@@ -111,16 +74,16 @@ panel_wide_kernel(const float *__restrict__ M, int64_t lda, float *__restrict__ 
 #pragma unroll 8
         for (int i = 0; i < NB; i++) {
             const bool in = incol && r0 + i >= 0 && r0 + i < nr;
-            cpa4(xb + i * CW, in ? bc + i * si : M, in);
+            cp4(xb + i * CW, in ? bc + i * si : M, in);
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        commit();
         {
             const int i = r0 + lane;
             inv[lane] = (!unit && i >= 0 && i < nr) ? 1.f / M[i + int64_t(i) * lda] : 1.f;
         }
         for (int kb = 0; kb <= b; kb++, n++) {
             // everything committed (NS = 2: tile n, and the right-hand sides at kb = 0)
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            wait_all();
             __syncwarp();
             prefetch();  // into the buffer of tile n - 1, which every lane has read
             const float *tile = ring + (n % NS) * TILE;
@@ -130,67 +93,21 @@ panel_wide_kernel(const float *__restrict__ M, int64_t lda, float *__restrict__ 
                     if (spin > kSpins) gave_up = true;
                 }
                 __threadfence_block();
-                const float *x0 = Xs + size_t(kb) * NB * CW + lane;
-                if (AM) {
-#pragma unroll 4
-                    for (int k = 0; k < NB; k++) {
-                        const float x = x0[k * CW];
-#pragma unroll
-                        for (int i = 0; i < NB; i += 4) {
-                            const float4 a = *reinterpret_cast<const float4 *>(tile + k * LD + i);
-                            t[i] = fmaf(a.x, x, t[i]);
-                            t[i + 1] = fmaf(a.y, x, t[i + 1]);
-                            t[i + 2] = fmaf(a.z, x, t[i + 2]);
-                            t[i + 3] = fmaf(a.w, x, t[i + 3]);
-                        }
-                    }
-                } else {
-#pragma unroll 2
-                    for (int k = 0; k < NB; k += 4) {
-                        float x[4];
-#pragma unroll
-                        for (int u = 0; u < 4; u++) x[u] = x0[(k + u) * CW];
-#pragma unroll
-                        for (int i = 0; i < NB; i++) {
-                            const float4 a = *reinterpret_cast<const float4 *>(tile + i * LD + k);
-                            t[i] = fmaf(a.x, x[0], t[i]);
-                            t[i] = fmaf(a.y, x[1], t[i]);
-                            t[i] = fmaf(a.z, x[2], t[i]);
-                            t[i] = fmaf(a.w, x[3], t[i]);
-                        }
-                    }
-                }
+                sum.update(tile, Xs + size_t(kb) * NB * CW + lane);
                 continue;
             }
             // t = alpha B - the updates, then the triangle
             const bool whole = vecb && r0 >= 0 && r0 + NB <= nr;
+            float2 t[NB / 2];
 #pragma unroll
-            for (int i = 0; i < NB; i++) t[i] = alpha * xb[i * CW] - t[i];
-#pragma unroll
-            for (int q = 0; q < NB; q++) {
-                const int k = FWD ? q : NB - 1 - q;
-                t[k] *= inv[k];
-                const float *lk = tile + k * LD;
-#pragma unroll
-                for (int i = 0; i < NB; i += 4) {
-                    // vectors with a row of the triangle's column k
-                    if (FWD ? i + 3 > k : i < k) {
-                        const float4 a = *reinterpret_cast<const float4 *>(lk + i);
-                        if (FWD ? i > k : i < k) t[i] = fmaf(-a.x, t[k], t[i]);
-                        if (FWD ? i + 1 > k : i + 1 < k) t[i + 1] = fmaf(-a.y, t[k], t[i + 1]);
-                        if (FWD ? i + 2 > k : i + 2 < k) t[i + 2] = fmaf(-a.z, t[k], t[i + 2]);
-                        if (FWD ? i + 3 > k : i + 3 < k) t[i + 3] = fmaf(-a.w, t[k], t[i + 3]);
-                    }
-                }
-            }
+            for (int i = 0; i < NB; i++) at(t, i) = sum.row(i);
+            substitute<FWD, false, CW>(t, tile, inv, xb, alpha);
             // a reader that gave up (it cannot unless the device is broken)
             // says so in every row from there on
             if (gave_up) {
 #pragma unroll
-                for (int i = 0; i < NB; i++) t[i] = NAN;
+                for (int i = 0; i < NB; i++) xb[i * CW] = at(t, i) = NAN;
             }
-#pragma unroll
-            for (int i = 0; i < NB; i++) xb[i * CW] = t[i];
             __syncwarp();
             if (lane == 0) {
                 __threadfence_block();
@@ -201,15 +118,15 @@ panel_wide_kernel(const float *__restrict__ M, int64_t lda, float *__restrict__ 
             if (whole) {
 #pragma unroll
                 for (int i = 0; i < NB; i += 4)
-                    *reinterpret_cast<float4 *>(bo + i) = make_float4(t[i], t[i + 1], t[i + 2], t[i + 3]);
+                    *reinterpret_cast<float4 *>(bo + i) = make_float4(t[i / 2].x, t[i / 2].y, t[i / 2 + 1].x, t[i / 2 + 1].y);
             } else {
 #pragma unroll
                 for (int i = 0; i < NB; i++)
-                    if (r0 + i >= 0 && r0 + i < nr) bo[i * si] = t[i];
+                    if (r0 + i >= 0 && r0 + i < nr) bo[i * si] = at(t, i);
             }
         }
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    wait_all();
 }
 
 template <bool AM, bool FWD>
