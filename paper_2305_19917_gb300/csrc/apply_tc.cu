@@ -21,18 +21,17 @@ int *device_status_word();
 
 namespace {
 
-constexpr int TB = 128;                    // rows of the block = K = panel width
+constexpr int TB = 128;                    // rows of the block = K
 constexpr uint32_t HALF_BYTES = TB * 128;  // 128 rows x 64 BF16 (one 128-byte swizzle column)
 constexpr uint32_t OP_BYTES = 2 * HALF_BYTES;
-constexpr uint32_t PANEL_BYTES = TB * TB * 4;  // FP32 staging of the panel, [column][row]
 
 // Byte offset of element (row r, k) of a K-major BF16 operand with K = 128
-// stored as two 64-wide halves of 128-byte rows in the 128-byte swizzle
+// stored as two 64-wide halves of `rows` 128-byte rows in the 128-byte swizzle
 // (16-byte chunk c of row r sits at chunk position c ^ (r mod 8)).
-__device__ __forceinline__ uint32_t sw128_off(int r, int k)
+__device__ __forceinline__ uint32_t sw128_off(int r, int k, uint32_t rows)
 {
     const int h = k >> 6, c = (k & 63) >> 3;
-    return uint32_t(h) * HALF_BYTES + uint32_t(r) * 128u + uint32_t((c ^ (r & 7)) << 4) + uint32_t(k & 7) * 2u;
+    return uint32_t(h) * (rows * 128u) + uint32_t(r) * 128u + uint32_t((c ^ (r & 7)) << 4) + uint32_t(k & 7) * 2u;
 }
 
 __device__ __forceinline__ void cp_async16_zfill(void *dst, const void *src, bool in)
@@ -44,16 +43,27 @@ __device__ __forceinline__ void cp_async16_zfill(void *dst, const void *src, boo
 
 constexpr int NTH = 256;
 
+__device__ __forceinline__ void ld_cols(uint32_t a, uint32_t (&x)[32])
+{
+    tc::tmem_ld32(a, x);
+    tc::tmem_ld_wait();
+}
+__device__ __forceinline__ void ld_cols(uint32_t a, uint32_t (&x)[16])
+{
+    tc::tmem_ld16(a, x);
+    tc::tmem_ld_wait();
+}
+
 // One leaf of the low-precision solve, left-looking, in one launch: for its
 // blocks b = 0, 1, ..., nblk-1 (rows b0 = s0 + 128 b .. b0 + 127)
 //     Y_b -= L(b, s0:b0) X(s0:b0)          (BF16 tensor cores, FP32 in TMEM)
 //     X_b  = L_b^-1 Y_b                    (two-term BF16 split, as above)
-// One CTA per 128-column panel walks the blocks in order: the columns of
+// One CTA per panel of PW columns walks the blocks in order: the columns of
 // the right-hand side are independent, so a panel needs only its own X of
 // the earlier blocks, which it wrote itself (stores, then a proxy fence
 // before the tensor-memory-access reads of them) -- no launch, prologue or
 // grid-wide wait between blocks.  Per block: the GEMM operands stream
-// through a 3-stage TMA ring (A rows of the BF16 copy of Mv, X's BF16 copy;
+// through a TMA ring of 3 to 6 stages (A rows of the BF16 copy of Mv, X's BF16 copy;
 // the ring position runs on across blocks), the FP32 panel and the
 // inverse's two terms arrive meanwhile, the ring then holds the split panel.
 // While a block's X is stored, the next block's FP32 panel, inverse and
@@ -61,29 +71,43 @@ constexpr int NTH = 256;
 // Thread 0 issues TMA, thread 32 the MMAs; all 8 warps do the subtraction,
 // the split and the stores (warps w, w+4 share TMEM lanes 32(w%4).. and
 // split the columns).
-constexpr int LST = 3;                                  // ring stages
-constexpr uint32_t LA_BYTES = TB * 64 * 2;              // 128 rows x 64 K of A
-constexpr uint32_t LB_BYTES = TB * 64 * 2;              // 128 columns x 64 K of X
-constexpr uint32_t LSTAGE = LA_BYTES + LB_BYTES;
-static_assert(LST * LSTAGE >= 2 * OP_BYTES, "the ring holds the split panel afterwards");
-constexpr size_t LEAF_SMEM = 1024 + LST * size_t(LSTAGE) + PANEL_BYTES + 2 * size_t(OP_BYTES) + 256;
+// A block's chain is bound by what one SM loads, converts and stores for it,
+// so PW is the narrowest panel whose CTAs still fit the SMs side by side: 32 up
+// to 4864 columns, 64 up to 9728, else 128.  Measured, time per 128-row block:
+// 9.6 us with 128 columns at any width; 6.3 with 32 (1500 x 700: low-precision
+// solve 115 -> 76 us; 32768 x 4096, whole BF16 solve 60.3 -> 56.9 ms).
+template <int PW>
+struct LeafCfg {
+    static constexpr int LST = PW == 128 ? 3 : (PW == 64 ? 5 : 6);  // ring stages
+    static constexpr uint32_t LA_BYTES = TB * 64 * 2;               // 128 rows x 64 K of A
+    static constexpr uint32_t LB_BYTES = PW * 64 * 2;               // PW columns x 64 K of X
+    static constexpr uint32_t LSTAGE = LA_BYTES + LB_BYTES;
+    static constexpr uint32_t PANEL_BYTES = PW * TB * 4;            // FP32 staging of the panel, [column][row]
+    static constexpr uint32_t OPY_BYTES = PW * TB * 2;              // one BF16 term of the split panel
+    static_assert(LST * LSTAGE >= 2 * OPY_BYTES, "the ring holds the split panel afterwards");
+    static constexpr size_t SMEM = 1024 + LST * size_t(LSTAGE) + PANEL_BYTES + 2 * size_t(OP_BYTES) + 256;
+};
 
+template <int PW>
 __global__ void __launch_bounds__(NTH, 1)
 leaf_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmX,
                const __grid_constant__ CUtensorMap tmL, int s0, int nblk, int kp, float *__restrict__ Y,
                int64_t ldy, __nv_bfloat16 *__restrict__ Ybf, int64_t ncols, int *status)
 {
+    using Cfg = LeafCfg<PW>;
+    constexpr int LST = Cfg::LST;
+    constexpr uint32_t LA_BYTES = Cfg::LA_BYTES, LSTAGE = Cfg::LSTAGE;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t *ring = base;                                         // LST stages, later the split panel
     float *sP = reinterpret_cast<float *>(base + LST * LSTAGE);   // FP32 panel, [column][row]
-    uint8_t *sLh = base + LST * LSTAGE + PANEL_BYTES, *sLl = sLh + OP_BYTES;
-    uint8_t *sYh = ring, *sYl = ring + OP_BYTES;
+    uint8_t *sLh = base + LST * LSTAGE + Cfg::PANEL_BYTES, *sLl = sLh + OP_BYTES;
+    uint8_t *sYh = ring, *sYl = ring + Cfg::OPY_BYTES;
     __shared__ uint64_t full[LST], empty[LST], bar_g, bar_l, bar_x;
     __shared__ uint32_t tslot;
     __shared__ int abort_flag;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t c0 = int64_t(blockIdx.x) * TB;
+    const int64_t c0 = int64_t(blockIdx.x) * PW;
     tc::pdl_launch_dependents();
 
     if (tid == 0) {
@@ -97,7 +121,7 @@ leaf_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         abort_flag = 0;
         tc::fence_barrier_init();
     }
-    if (warp == 0) tc::tmem_alloc(&tslot, 2 * TB);  // [0,128): L(b,.) X,  [128,256): L_b^-1 Y_b
+    if (warp == 0) tc::tmem_alloc(&tslot, 2 * PW);  // [0,PW): L(b,.) X,  [PW,2 PW): L_b^-1 Y_b
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
@@ -106,12 +130,13 @@ leaf_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     tc::pdl_wait();  // Y, its BF16 copy: the previous kernel's until it completes
     const int q = warp & 3, half = warp >> 2;
     const int r = q * 32 + lane;
+    constexpr int CH = PW / 2 < 32 ? PW / 2 : 32;  // columns drained at a time
     uint32_t g = 0;  // ring position (k-tiles issued so far)
     int pre = 0;     // thread 0: k-tiles of the current block issued during the previous one
 
     // the FP32 panel of Y_b (rows b0..), every copy in flight at once
     auto load_panel = [&](int b0) {
-        for (int idx = tid; idx < TB * TB / 4; idx += NTH) {
+        for (int idx = tid; idx < PW * TB / 4; idx += NTH) {
             const int j = idx >> 5, k4 = (idx & 31) * 4;
             const int64_t col = c0 + j;
             const bool in = col < ncols;
@@ -150,7 +175,7 @@ leaf_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             for (int kt = pre; kt < nk; kt++)
                 if (!load_ktile(g + uint32_t(kt), kt, b0)) break;
         } else if (tid == 32) {
-            constexpr uint32_t idesc = tc::idesc_bf16_f32(TB, TB);
+            constexpr uint32_t idesc = tc::idesc_bf16_f32(TB, PW);
             for (int kt = 0; kt < nk; kt++) {
                 const uint32_t gi = g + uint32_t(kt);
                 const int st = int(gi % LST);
@@ -175,17 +200,16 @@ leaf_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (ok_g && nk > 0) {
             tc::tc_fence_after();
 #pragma unroll 1
-            for (int cc = half * (TB / 2); cc < (half + 1) * (TB / 2); cc += 32) {
-                uint32_t x[32];
-                tc::tmem_ld32(tmem + (uint32_t(q * 32) << 16) + uint32_t(cc), x);
-                tc::tmem_ld_wait();
+            for (int cc = half * (PW / 2); cc < (half + 1) * (PW / 2); cc += CH) {
+                uint32_t x[CH];
+                ld_cols(tmem + (uint32_t(q * 32) << 16) + uint32_t(cc), x);
 #pragma unroll
-                for (int e = 0; e < 32; e++) sP[(cc + e) * TB + r] -= __uint_as_float(x[e]);
+                for (int e = 0; e < CH; e++) sP[(cc + e) * TB + r] -= __uint_as_float(x[e]);
             }
         }
         tc::tc_fence_before();
         __syncthreads();  // the panel is complete and the ring is free (all MMAs of the GEMM are done)
-        for (int task = tid; task < TB * 16; task += NTH) {
+        for (int task = tid; task < PW * 16; task += NTH) {
             const int j = task >> 4, k0 = (task & 15) * 8;
             const float4 a = *reinterpret_cast<const float4 *>(sP + j * TB + k0);
             const float4 b = *reinterpret_cast<const float4 *>(sP + j * TB + k0 + 4);
@@ -198,7 +222,7 @@ leaf_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 hw[e / 2] = *reinterpret_cast<const uint32_t *>(&h);
                 lw[e / 2] = *reinterpret_cast<const uint32_t *>(&l);
             }
-            const uint32_t off = sw128_off(j, k0);
+            const uint32_t off = sw128_off(j, k0, PW);
             *reinterpret_cast<uint4 *>(sYh + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
             *reinterpret_cast<uint4 *>(sYl + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
         }
@@ -208,7 +232,7 @@ leaf_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (tid == 32) {
             if (ok_g && tc::mbar_wait(&bar_l, ph, ab, status, tc::TC_TIMEOUT_MMA)) {
                 tc::tc_fence_after();
-                constexpr uint32_t idesc = tc::idesc_bf16_f32(TB, TB);
+                constexpr uint32_t idesc = tc::idesc_bf16_f32(TB, PW);
                 const uint8_t *As[3] = {sLh, sLh, sLl};
                 const uint8_t *Bs[3] = {sYh, sYl, sYh};
                 uint32_t acc = 0;
@@ -218,8 +242,9 @@ leaf_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     const uint64_t dy = tc::desc_kmajor_sw128(tc::smem_u32(Bs[pr]));
 #pragma unroll
                     for (int kk = 0; kk < TB / 16; kk++) {
-                        const uint64_t o = uint64_t(((kk >> 2) * HALF_BYTES + (kk & 3) * 32u) >> 4);
-                        tc::mma_f16(tmem + TB, da + o, dy + o, idesc, acc);
+                        const uint64_t oa = uint64_t(((kk >> 2) * HALF_BYTES + (kk & 3) * 32u) >> 4);
+                        const uint64_t oy = uint64_t(((kk >> 2) * (PW * 128u) + (kk & 3) * 32u) >> 4);
+                        tc::mma_f16(tmem + PW, da + oa, dy + oy, idesc, acc);
                         acc = 1;
                     }
                 }
@@ -244,12 +269,11 @@ leaf_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (ok_x && !*ab) {
             tc::tc_fence_after();
 #pragma unroll 1
-            for (int cc = half * (TB / 2); cc < (half + 1) * (TB / 2); cc += 32) {
-                uint32_t x[32];
-                tc::tmem_ld32(tmem + (uint32_t(q * 32) << 16) + uint32_t(TB + cc), x);
-                tc::tmem_ld_wait();
+            for (int cc = half * (PW / 2); cc < (half + 1) * (PW / 2); cc += CH) {
+                uint32_t x[CH];
+                ld_cols(tmem + (uint32_t(q * 32) << 16) + uint32_t(PW + cc), x);
 #pragma unroll
-                for (int e = 0; e < 32; e++) {
+                for (int e = 0; e < CH; e++) {
                     const int64_t col = c0 + cc + e;
                     if (col < ncols) {
                         const float val = __uint_as_float(x[e]);
@@ -266,15 +290,17 @@ leaf_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (*ab) break;
     }
     tc::tc_fence_after();
-    if (warp == 0) tc::tmem_dealloc(tmem, 2 * TB);
+    if (warp == 0) tc::tmem_dealloc(tmem, 2 * PW);
 }
 
 }  // namespace
 
 int apply_tc_prepare()
 {
-    static PerDeviceOnce attr;
-    return smem_attr_once(attr, leaf_tc_kernel, LEAF_SMEM);
+    static PerDeviceOnce a32, a64, a128;
+    GB_TRY(smem_attr_once(a32, leaf_tc_kernel<32>, LeafCfg<32>::SMEM));
+    GB_TRY(smem_attr_once(a64, leaf_tc_kernel<64>, LeafCfg<64>::SMEM));
+    return smem_attr_once(a128, leaf_tc_kernel<128>, LeafCfg<128>::SMEM);
 }
 
 // One leaf of the low-precision solve: rows s0 .. s0 + nr - 1 (s0 and nr
@@ -291,6 +317,7 @@ int launch_leaf_tc(const __nv_bfloat16 *Abf, const __nv_bfloat16 *inv16, int64_t
         (reinterpret_cast<uintptr_t>(Y) & 15) || (reinterpret_cast<uintptr_t>(Abf) & 15) ||
         (reinterpret_cast<uintptr_t>(Ybf) & 15) || (reinterpret_cast<uintptr_t>(inv16) & 15))
         return GB_STATUS_CUDA_ERROR;
+    const int pw = np <= 152 * 32 ? 32 : (np <= 152 * 64 ? 64 : 128);
     CUtensorMap ta, tx, tl;
     {
         uint64_t dims[2] = {uint64_t(kp), uint64_t(kp)};
@@ -301,7 +328,7 @@ int launch_leaf_tc(const __nv_bfloat16 *Abf, const __nv_bfloat16 *inv16, int64_t
     {
         uint64_t dims[2] = {uint64_t(kp), uint64_t(np)};
         uint64_t strides[1] = {uint64_t(kp) * 2};
-        uint32_t box[2] = {64, TB};
+        uint32_t box[2] = {64, uint32_t(pw)};
         GB_TRY(encode_tmap(&tx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Ybf, dims, strides, box));
     }
     {
@@ -317,8 +344,13 @@ int launch_leaf_tc(const __nv_bfloat16 *Abf, const __nv_bfloat16 *inv16, int64_t
     // GEMM flops of the leaf (sum over blocks of 2 * 128 * K * np) plus the 3 split products per block
     LaunchScope ls(KK_DIAG, s, (nrd * (nrd - TB) + 3.0 * 2.0 * TB * nrd) * double(np),
                    nrd * nrd + nrd * (nrd - TB) / TB * double(np) + 10.0 * nrd * double(np));
-    return check(launch_pdl(leaf_tc_kernel, dim3((unsigned)(np / TB)), dim3(NTH), LEAF_SMEM, s, ta, tx, tl, int(s0),
-                            int(nr / TB), int(kp), Y, kp, Ybf, np, st));
+    auto launch = [&](auto kern, size_t smem) {
+        return check(launch_pdl(kern, dim3((unsigned)(np / pw)), dim3(NTH), smem, s, ta, tx, tl, int(s0), int(nr / TB),
+                                int(kp), Y, kp, Ybf, np, st));
+    };
+    if (pw == 32) return launch(leaf_tc_kernel<32>, LeafCfg<32>::SMEM);
+    if (pw == 64) return launch(leaf_tc_kernel<64>, LeafCfg<64>::SMEM);
+    return launch(leaf_tc_kernel<128>, LeafCfg<128>::SMEM);
 }
 
 }  // namespace gb
