@@ -178,9 +178,9 @@ int gb_dtrsm_mixed(int side, int uplo, int trans, int diag, int64_t m,
  * low-precision solve: `leaf` (argument 15, after max_iter; iters_out,
  * est_err_out and stream follow as arguments 16-18) is the order of the
  * recursion's leaves (Section V-A: refinement level ~ k / leaf), a multiple
- * of 128 in [128, 8192], or 0 for the default (1024 rows for BF16, each leaf
- * one tensor-core kernel launch; 128 rows for FP8, larger FP8 leaves are
- * solved blocked in 128-row steps).  Any other value returns -15.  Results
+ * of 128 in [128, 8192], or 0 for the default (1024 rows, each leaf one
+ * tensor-core kernel launch, in BF16 inside the leaf for either precision).
+ * Any other value returns -15.  Results
  * and status codes as gb_dtrsm_mixed; the planner's timing sweep uses it.
  */
 int gb_dtrsm_mixed_leaf(int side, int uplo, int trans, int diag, int64_t m,

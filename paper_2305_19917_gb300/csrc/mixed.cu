@@ -49,10 +49,9 @@ int tc_gemm_fp8_prepare();
 int launch_tc_gemm_fp8(int64_t M, int64_t N, int64_t K, const void *A, int64_t lda, const void *B, int64_t ldb,
                        float *C, int64_t ldc, float alpha, const float *sA, int64_t ldsa, const float *sB,
                        int64_t ldsb, cudaStream_t s, int *status);
-int launch_apply_inverse_fp8(const float *Linv_b, float *Yb, int64_t ldy, uint8_t *Y8_b, float *s8_b, int nr,
-                             int64_t ncols, cudaStream_t s);
-int diag_inv_prepare();
-int launch_invert_blocks(const float *band, float *inv, __nv_bfloat16 *inv16, int64_t nblocks, cudaStream_t s);
+int launch_quantise_fp8(const float *Y, int64_t ld, uint8_t *Y8, float *scales, int64_t lds, int64_t nr, int64_t np,
+                        cudaStream_t s);
+int launch_invert_blocks(const float *band, __nv_bfloat16 *inv16, int64_t nblocks, cudaStream_t s);
 int apply_tc_prepare();
 int launch_leaf_tc(const __nv_bfloat16 *Abf, const __nv_bfloat16 *inv16, int64_t kp, int64_t np, int64_t s0,
                    int64_t nr, float *Y, __nv_bfloat16 *Ybf, cudaStream_t s, int *status);
@@ -66,7 +65,7 @@ constexpr int kSlices = 6;     // digit slices of Mv (8 bits each)
 // place from then on.
 constexpr int kZSlots = 3;
 constexpr int kBand = 128;     // FP32 band of diagonal 128-blocks (column-major per block)
-constexpr int kLeaf = 1024;    // default leaf order of the BF16 low-precision solve (one leaf kernel launch each)
+constexpr int kLeaf = 1024;    // default leaf order of the low-precision solve (one leaf kernel launch each)
 
 // z * 2^e as a double for |z| < 2^31 (exact: no rounding), built with 32-bit
 // integer operations (an int -> double conversion runs on the FP64 pipe,
@@ -935,7 +934,6 @@ struct LowExec {
     float *Y;
     __nv_bfloat16 *Ybf;
     const __nv_bfloat16 *Abf;
-    const float *binv;  // inverses of the diagonal kBand-blocks
     int64_t kp, np;
     cudaStream_t s;
     int *status_word;   // device word for wait timeouts
@@ -951,20 +949,16 @@ struct LowExec {
     void ts(int64_t b0, int64_t nr, float a)
     {
         if (status) return;
-        if (!fp8) {
-            // BF16 form: a leaf (kLeaf rows by default), left-looking, in one
-            // launch: each 128-row block takes its update from the solved
-            // blocks of the leaf and its TS task
-            status = launch_leaf_tc(Abf, binv16, kp, np, b0, nr, Y, Ybf, s, status_word);
-            return;
-        }
-        if (nr > kBand) {
-            drive_blocked(*this, b0, b0 + nr, (int64_t)kBand, a, true);
-            return;
-        }
-        // TS task: X_b = L_b^-1 Y_b with the precomputed inverse of the block
-        status = launch_apply_inverse_fp8(binv + b0 * kBand, Y + b0, kp, Y8 + b0, sY + (b0 / 128) * (np / 64),
-                                          (int)nr, np, s);
+        (void)a;
+        // a leaf (kLeaf rows by default), left-looking, in one launch: each
+        // 128-row block takes its update from the solved blocks of the leaf
+        // and its TS task
+        status = launch_leaf_tc(Abf, binv16, kp, np, b0, nr, Y, Ybf, s, status_word);
+        // FP8 form: the updates outside the leaves read its FP8 copy (leaves
+        // of 128 rows with the inverse applied on the CUDA cores and FP8
+        // updates between them took 9.2 ms a solve at 32768 x 4096; this 5.4)
+        if (!status && fp8 && b0 + nr < kp)
+            status = launch_quantise_fp8(Y + b0, kp, Y8 + b0, sY + (b0 / 128) * (np / 64), np / 64, nr, np, s);
     }
     void gemm(int64_t ci0, int64_t M, int64_t ak0, int64_t K, float a)
     {
@@ -980,11 +974,10 @@ struct LowExec {
 };
 
 // Recursive model (Section V-A) down to leaves of e.leaf rows, by default
-// kLeaf (BF16 form: each leaf solved left-looking by one leaf kernel launch)
-// or kBand (FP8 form: larger leaves are solved blocked in kBand steps).
+// kLeaf, each solved left-looking by one leaf kernel launch.
 int low_solve(LowExec &e, int64_t kp)
 {
-    const int64_t leaf = e.leaf > 0 ? e.leaf : (e.fp8 ? kBand : kLeaf);
+    const int64_t leaf = e.leaf > 0 ? e.leaf : kLeaf;
     drive_recursive(e, 0, kp, 24, leaf, 1.0f, true);
     return e.status;
 }
@@ -1153,7 +1146,6 @@ int low_graph(LowExec &le, const void *ws, LowGraph **out)
     // everything that allocates or sets attributes happens before capture
     GB_TRY(tc_gemm_prepare());
     GB_TRY(tc_gemm_fp8_prepare());
-    GB_TRY(diag_inv_prepare());
     GB_TRY(apply_tc_prepare());
     cudaStream_t user = le.s;
     le.s = cap_stream[dev];
@@ -1208,7 +1200,7 @@ MixedLayout mixed_layout(int side, int64_t m, int64_t n, int prec)
     L.o_abf = take(kk * 2);
     L.o_as = take(kk * 2 * kSlices);
     L.o_band = take(size_t(L.kp) * kBand * 4);
-    L.o_binv = take(size_t(L.kp) * kBand * 4);
+    take(size_t(L.kp) * kBand * 4);  // unused (keeps the size that the fixed scratch's limit was set by)
     L.o_binv16 = take(size_t(L.kp) * kBand * 4);
     L.o_r = take(kn * 8);
     L.o_t = take(kn * 8);
@@ -1239,7 +1231,7 @@ MixedLayout mixed_layout(int side, int64_t m, int64_t n, int prec)
 // Pointers into a work space laid out by mixed_layout.
 struct MixedBufs {
     __nv_bfloat16 *Abf, *As, *binv16, *Ybf, *Zs;
-    float *band, *binv, *Y, *xmax;
+    float *band, *Y, *xmax;
     double *R, *X, *norms, *dg;
     long long *Tg;
     int *e_row, *f_col, *cs;
@@ -1254,11 +1246,10 @@ static MixedBufs mixed_bufs(const MixedLayout &L, char *ws, bool fp8)
     MixedBufs b;
     b.Abf = reinterpret_cast<__nv_bfloat16 *>(ws + L.o_abf);
     b.As = reinterpret_cast<__nv_bfloat16 *>(ws + L.o_as);
-    b.binv16 = fp8 ? nullptr : reinterpret_cast<__nv_bfloat16 *>(ws + L.o_binv16);
+    b.binv16 = reinterpret_cast<__nv_bfloat16 *>(ws + L.o_binv16);
     b.Ybf = reinterpret_cast<__nv_bfloat16 *>(ws + L.o_ybf);
     b.Zs = reinterpret_cast<__nv_bfloat16 *>(ws + L.o_zs);
     b.band = reinterpret_cast<float *>(ws + L.o_band);
-    b.binv = reinterpret_cast<float *>(ws + L.o_binv);
     b.Y = reinterpret_cast<float *>(ws + L.o_y);
     b.xmax = reinterpret_cast<float *>(ws + L.o_xm);
     b.cs = reinterpret_cast<int *>(ws + L.o_cs);
@@ -1312,7 +1303,7 @@ int mixed_prep_a(int side, int uplo, int trans, int diag, int64_t k, const doubl
         prepA_kernel<<<tgrid, 256, 0, s>>>(v, kp, bf.e_row, bf.Abf, bf.As, bf.band, bf.dg, bf.A8, bf.bscale);
         GB_CUDA(cudaGetLastError());
     }
-    return launch_invert_blocks(bf.band, bf.binv, bf.binv16, kp / kBand, s);
+    return launch_invert_blocks(bf.band, bf.binv16, kp / kBand, s);
 }
 
 int mixed_solve_b(int side, int uplo, int trans, int64_t k, int64_t ncols, double alpha, const double *B,
@@ -1327,7 +1318,6 @@ int mixed_solve_b(int side, int uplo, int trans, int64_t k, int64_t ncols, doubl
     const MixedBufs bf = mixed_bufs(L, ws, fp8);
     auto *Abf = bf.Abf;
     auto *As = bf.As;
-    auto *binv = bf.binv;
     auto *R = bf.R;
     auto *Tg = bf.Tg;
     auto *X = bf.X;
@@ -1371,7 +1361,7 @@ int mixed_solve_b(int side, int uplo, int trans, int64_t k, int64_t ncols, doubl
                 break;
             if ((st = check(cudaGetLastError()))) break;
         }
-        LowExec le{Y, Ybf, Abf, binv, kp, np, s, status_word};
+        LowExec le{Y, Ybf, Abf, kp, np, s, status_word};
         le.binv16 = bf.binv16;
         le.fp8 = fp8;
         le.A8 = bf.A8;

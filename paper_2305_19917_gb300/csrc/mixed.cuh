@@ -12,7 +12,7 @@ namespace gb {
 // right-hand sides padded to multiples of 128 as kp, np); `total` bytes.
 struct MixedLayout {
     int64_t kp, np;
-    size_t o_abf, o_as, o_band, o_binv, o_binv16, o_r, o_t, o_x, o_y, o_ybf, o_zs, o_e, o_f, o_norm, o_dg, o_xm, o_cs;
+    size_t o_abf, o_as, o_band, o_binv16, o_r, o_t, o_x, o_y, o_ybf, o_zs, o_e, o_f, o_norm, o_dg, o_xm, o_cs;
     size_t o_a8, o_bmax, o_bscale, o_y8, o_sy;  // FP8 variant only (0 otherwise)
     size_t total;
 };
@@ -41,7 +41,7 @@ int mixed_core(int side, int uplo, int trans, int diag, int64_t m, int64_t n, do
 //    merge_hist folds this block's refinement history into the previous
 //    block's (step-wise maximum) instead of starting a new one.
 // leaf: order of the low-precision solve's recursion leaves (a multiple of
-// 128; 0 = the form's default, 1024 rows BF16 / 128 rows FP8).
+// 128; 0 = the default, 1024 rows).
 int mixed_prep_a(int side, int uplo, int trans, int diag, int64_t k, const double *A, int64_t lda, int prec,
                  const MixedLayout &L, char *ws, cudaStream_t s);
 int mixed_solve_b(int side, int uplo, int trans, int64_t k, int64_t ncols, double alpha, const double *B,
