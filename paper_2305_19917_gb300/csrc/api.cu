@@ -144,8 +144,13 @@ struct LaunchExec {
         if (nr <= ts_rows<T>(c.ncols)) {
             settle(b0, b0 + nr);
             if (status) return;
-            if (sizeof(T) == 8 && c.ncols > 2432) status = launch_diag_solve(c, b0, (int)nr, a);
-            else status = launch_panel_solve(c, b0, (int)nr, a);
+            if constexpr (sizeof(T) == 8) {
+                if (c.ncols > 2432) {
+                    status = launch_diag_solve(c, b0, (int)nr, a);
+                    return;
+                }
+            }
+            status = launch_panel_solve(c, b0, (int)nr, a);
             return;
         }
         expand_ts(*this, b0, nr, nb, a, c.forward);

@@ -17,8 +17,8 @@
 // coalesced whichever way B is laid out, and the diagonal is inverted once
 // per CTA (nr^2/2 multiply-adds per right-hand side).
 #pragma once
-#include <cuda_bf16.h>
 #include "common.cuh"
+#include "tc_common.cuh"
 
 namespace gb {
 namespace {
@@ -92,14 +92,13 @@ __device__ __forceinline__ void diag_rows(const T *L, const T *inv, T *Bs, int n
 
 // FWD: Mv lower (forward substitution); MT: Mv(i,j) = A(j,i); LEFT: Bv
 // column-major.  Msub = &A(r0, r0), Bsub = &Bv(r0, 0).
-// EMIT: also write a BF16 copy of the solved block to Ebf (column-major,
-// ldb), the operand of the tensor-core GEMM updates (LEFT layout only).
-template <typename T, int NB, bool FWD, bool MT, bool LEFT, bool EMIT, int CW>
+template <typename T, int NB, bool FWD, bool MT, bool LEFT, int CW>
 __global__ void __launch_bounds__(kDiagThreads)
 diag_solve_kernel(const T *__restrict__ Msub, int64_t lda, T *__restrict__ Bsub,
-                  int64_t ldb, int nr, int64_t ncols, T alpha, int unit,
-                  __nv_bfloat16 *__restrict__ Ebf)
+                  int64_t ldb, int nr, int64_t ncols, T alpha, int unit)
 {
+    tc::pdl_wait();
+    tc::pdl_launch_dependents();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *L = reinterpret_cast<T *>(smem_raw);
     T *inv = L + NB * NB;
@@ -170,10 +169,7 @@ diag_solve_kernel(const T *__restrict__ Msub, int64_t lda, T *__restrict__ Bsub,
     if (LEFT) {
         for (int idx = tid; idx < NB * CW; idx += kDiagThreads) {
             int i = idx % NB, c = idx / NB;
-            if (i < nr && c < ncb) {
-                Bsub[i + (c0 + c) * ldb] = Bs[i * BS + c];
-                if (EMIT) Ebf[i + (c0 + c) * ldb] = __float2bfloat16_rn(float(Bs[i * BS + c]));
-            }
+            if (i < nr && c < ncb) Bsub[i + (c0 + c) * ldb] = Bs[i * BS + c];
         }
     } else {
         for (int idx = tid; idx < NB * CW; idx += kDiagThreads) {
@@ -184,36 +180,36 @@ diag_solve_kernel(const T *__restrict__ Msub, int64_t lda, T *__restrict__ Bsub,
 }
 
 // One-time kernel attribute (dynamic shared memory above 48 KB).
-template <typename T, int NB, bool FWD, bool MT, bool LEFT, bool EMIT, int CW>
+template <typename T, int NB, bool FWD, bool MT, bool LEFT, int CW>
 int diag_prepare()
 {
     static PerDeviceOnce attr;  // per instantiation and device
-    return smem_attr_once(attr, diag_solve_kernel<T, NB, FWD, MT, LEFT, EMIT, CW>, diag_smem_bytes<T, NB, CW>());
+    return smem_attr_once(attr, diag_solve_kernel<T, NB, FWD, MT, LEFT, CW>, diag_smem_bytes<T, NB, CW>());
 }
 
-template <typename T, int NB, bool FWD, bool MT, bool LEFT, bool EMIT, int CW>
+template <typename T, int NB, bool FWD, bool MT, bool LEFT, int CW>
 int launch_nb_cw(const T *Msub, int64_t lda, T *Bsub, int64_t ldb, int nr, int64_t ncols, T alpha, int unit,
-                 cudaStream_t s, __nv_bfloat16 *Ebf)
+                 cudaStream_t s)
 {
-    auto kern = diag_solve_kernel<T, NB, FWD, MT, LEFT, EMIT, CW>;
+    auto kern = diag_solve_kernel<T, NB, FWD, MT, LEFT, CW>;
     constexpr size_t smem = diag_smem_bytes<T, NB, CW>();
     {
-        const int pst = diag_prepare<T, NB, FWD, MT, LEFT, EMIT, CW>();
+        const int pst = diag_prepare<T, NB, FWD, MT, LEFT, CW>();
         if (pst) return pst;
     }
     int64_t grid = (ncols + CW - 1) / CW;
     if (grid > 0x7fffffff) return GB_STATUS_CUDA_ERROR;
     LaunchScope ls(KK_DIAG, s, double(nr) * nr * ncols,
                    sizeof(T) * (0.5 * nr * nr + 2.0 * nr * ncols));
-    kern<<<(unsigned)grid, kDiagThreads, smem, s>>>(Msub, lda, Bsub, ldb, nr, ncols, alpha, unit, Ebf);
-    return check(cudaGetLastError());
+    return check(launch_pdl(kern, dim3((unsigned)grid), dim3(kDiagThreads), smem, s, Msub, lda, Bsub, ldb, nr, ncols, alpha,
+                            unit));
 }
 
-template <typename T, int NB, bool FWD, bool MT, bool LEFT, bool EMIT = false>
+template <typename T, int NB, bool FWD, bool MT, bool LEFT>
 int launch_nb(const T *Msub, int64_t lda, T *Bsub, int64_t ldb, int nr, int64_t ncols,
-              T alpha, int unit, cudaStream_t s, __nv_bfloat16 *Ebf = nullptr)
+              T alpha, int unit, cudaStream_t s)
 {
-    return launch_nb_cw<T, NB, FWD, MT, LEFT, EMIT, 64>(Msub, lda, Bsub, ldb, nr, ncols, alpha, unit, s, Ebf);
+    return launch_nb_cw<T, NB, FWD, MT, LEFT, 64>(Msub, lda, Bsub, ldb, nr, ncols, alpha, unit, s);
 }
 
 template <typename T, bool FWD, bool MT, bool LEFT>

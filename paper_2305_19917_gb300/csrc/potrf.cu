@@ -14,8 +14,8 @@
 // library's own TRSM, side Right, transposed).  So every column block meets
 // one TS task, on all its rows at once: splitting the matrix in 2 x 2 blocks
 // instead, with a TRSM of every order, ran 448 of them at n = 8192 instead of
-// 127.  n = 8192 FP64: 128 -> 28.5 ms by the panels and the tasks' digit gemms, 23.7
-// with the leaf below; n = 16384 87 ms (1.34 s before the digit gemms).  The upper form (A = U^T U) is the same with everything stored
+// 127.  n = 8192 FP64: 128 -> 28.5 ms by the panels and the tasks' digit gemms, 20.5
+// with the leaf below and overlapped launches; n = 16384 71 ms (1.34 s before the digit gemms).  The upper form (A = U^T U) is the same with everything stored
 // transposed.  Only the named triangle of A is read and written.
 //
 // A non-positive (or NaN) pivot stops the leaf that meets it; the leaf
@@ -28,6 +28,7 @@
 #include "driver.cuh"
 #include "gemm_digits.cuh"
 #include "mixed.cuh"
+#include "tc_common.cuh"
 
 extern "C" int gb_dtrsm(int side, int uplo, int trans, int diag, int64_t m, int64_t n, double alpha,
                         const double *A, int64_t lda, double *B, int64_t ldb, void *stream);
@@ -38,7 +39,7 @@ namespace gb {
 namespace {
 
 constexpr int kLeafNB = 64;
-constexpr int kLeafThreads = 256;
+constexpr int kLeafThreads = 384;
 
 // Exponent field and its largest value (tests on it are integer operations: a
 // comparison of FP64 values takes 66 clocks as any operation of that unit).
@@ -46,36 +47,58 @@ __device__ __forceinline__ int expo(double x) { return (__double2hiint(x) >> 20)
 __device__ __forceinline__ int expo(float x) { return (__float_as_int(x) >> 23) & 0xFF; }
 template <typename T>
 constexpr int kExpoMax = sizeof(T) == 8 ? 0x7FF : 0xFF;
+// where the corrections below could leave the range
+template <typename T>
+__device__ __forceinline__ bool extreme(T d)
+{
+    const int e = expo(d);
+    return e < kExpoMax<T> / 8 || e == kExpoMax<T>;
+}
 
 // The rare cases by definition.  Out of line: inlined, the compiler evaluates
 // a division beside every ordinary case and selects afterwards.
 template <typename T>
-__device__ __noinline__ void pivot_root_slow(T d, T &l, T &y)
+__device__ __noinline__ T root_slow(T d)
 {
-    l = sqrt(d);
-    y = T(1) / l;
+    return sqrt(d);
 }
 template <typename T>
-__device__ __noinline__ T pivot_scale_slow(T v, T l)
+__device__ __noinline__ T ratio_slow(T v, T l)
 {
     return v / l;
 }
 
-// l = sqrt(d) and y = 1 / sqrt(d) of a pivot d > 0, the reciprocal square root
-// corrected once against d.
-template <typename T>
-__device__ __forceinline__ void pivot_root(T d, T &l, T &y)
+// 1 / sqrt(d) to about 22 bits, for d > 0 in the middle of the range: the FP32
+// unit's approximation, FP64 exponents and mantissas moved by integer operations.
+__device__ __forceinline__ float rsqrt_seed(float d)
 {
-    const int e = expo(d);
-    if (e < kExpoMax<T> / 8 || e == kExpoMax<T>) {  // where the corrections could leave the range
-        pivot_root_slow(d, l, y);
-        return;
-    }
-    y = rsqrt(d);
-    const T h = T(0.5) * y;
-    l = d * y;
-    l = fma(fma(-l, l, d), h, l);
-    y = fma(y, fma(-l, y, T(1)), y);
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(d));
+    return y;
+}
+__device__ __forceinline__ double rsqrt_seed(double d)
+{
+    const int hi = __double2hiint(d), k = ((hi >> 20) - 1023) >> 1;  // d = m 4^k, 1 <= m < 4
+    const unsigned m = unsigned(hi - (k << 21) - (896 << 20));
+    const unsigned y = __float_as_uint(rsqrt_seed(__uint_as_float(__funnelshift_l(__double2loint(d), m, 3))));
+    return __hiloint2double(int((y >> 3) + (896 << 20)) - (k << 20), int(y << 29));
+}
+// y = 1 / sqrt(d) of a pivot d > 0: the seed's residual r = 1 - d y^2 through the
+// series y (1 + r / 2 + 3 r^2 / 8), what follows is below 2^-63.
+template <typename T>
+__device__ __forceinline__ T root_rcp(T d)
+{
+    if (extreme(d)) return ratio_slow(T(1), root_slow(d));
+    const T y = rsqrt_seed(d), r = fma(-(d * y), y, T(1));
+    return fma(y * r, fma(r, T(0.375), T(0.5)), y);
+}
+// sqrt(d) by y, corrected once.
+template <typename T>
+__device__ __forceinline__ T root(T d, T y)
+{
+    if (extreme(d)) return root_slow(d);
+    const T l = d * y;
+    return fma(fma(-l, l, d), T(0.5) * y, l);
 }
 // v / l by the reciprocal y, corrected once: as exact as the division.
 template <typename T>
@@ -83,110 +106,154 @@ __device__ __forceinline__ T pivot_scale(T v, T l, T y)
 {
     T q = v * y;
     q = fma(fma(-q, l, v), y, q);
-    if (expo(q) == kExpoMax<T>) q = pivot_scale_slow(v, l);
+    if (expo(q) == kExpoMax<T>) q = ratio_slow(v, l);
     return q;
 }
 
 // One diagonal block of order nr <= 64 at &A(r0, r0) (A0 points there),
-// factorised right-looking in shared memory.  s[c][i] (i >= c) holds the
-// block's lower triangle by columns: A(i, c) for the lower form, A(c, i) for
-// the upper.  What bounds it is the chain of 64 pivots: a reciprocal square
-// root, its corrections and the next pivot's update are about 18 operations
-// of the FP64 unit, 66 clocks each.  Warp 0 does nothing else: while it forms
-// pivot j + 1 from its own copy of that pivot's column entry, warps 1 and 2
-// scale column j and then all but warps 0 and 4 (the one that shares warp 0's
-// sub-partition) update the columns behind it.  One CTA barrier a column; a
-// finished column goes to A at once.
-// Measured (one 64-column block): FP64 70 us, FP32 27 (one thread's square
+// factorised right-looking: A(i, c) is element (i, c) of the lower form,
+// stored (c, i) for the upper.  What bounds it is the FP64 unit, 66 clocks an
+// operation of a warp however many lanes take part: a chain of 64 pivots of 9
+// operations each, and 43.7k multiply-adds behind them.  Roles, by step j (one CTA barrier each):
+//   warp 0        pivot j + 1 and its reciprocal root, from the entries
+//                 (j+1, j), (j+1, j+1) as of column j - 2 and what columns
+//                 j - 1 and j add to them;
+//   warps 1, 2    bring column j (as of column j - 2) up to date and scale it;
+//   update warps  take column j - 1 off everything behind column j, and hand
+//                 out column j + 1 and pivot entry j + 2.
+// So nobody waits within a step.  The update warps hold the triangle in
+// registers, packed by columns, 32 elements a slot: full lanes to the end
+// (2080 / 32 slots at first; the columns one by one take 94), dealt out by what else
+// a warp's sub-partition (warp mod 4) has to do.
+// Measured (one 64-column block): FP64 46 us, FP32 24 (updates column by column
+// in shared memory, CUDA's rsqrt() in the chain: 70 and 27; one thread's square
 // root, a division per entry and three barriers a column: 107 and 48).
+constexpr int kLeafSlots = kLeafNB * (kLeafNB + 1) / 2 / 32;  // 65
+constexpr int kUpdWarps = 8, kUpdGroups = 3, kUpdPer = 3;     // slots: groups of three a warp
+static_assert(kUpdWarps * kUpdGroups * kUpdPer >= kLeafSlots, "slots");
+
 template <typename T>
 __global__ void __launch_bounds__(kLeafThreads)
 potrf_leaf_kernel(T *__restrict__ A0, int64_t lda, int nr, int upper, int64_t r0, int *info)
 {
-    __shared__ T s[kLeafNB][kLeafNB + 1];
-    __shared__ T piv[2][2];           // l and y of the pivots, by parity of the column
-    __shared__ T col[2][kLeafNB];     // scaled columns, likewise
-    __shared__ int fail;
-    if (*static_cast<volatile int *>(info) != 0) return;  // an earlier leaf failed
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // load the named triangle, reading A along its contiguous dimension
-    // (every load before the first store)
-    {
-        constexpr int PER = kLeafNB * kLeafNB / kLeafThreads;
-        T v[PER];
+    __shared__ T cb[2][kLeafNB];  // column j as of column j - 2, by parity
+    __shared__ T dg[2];           // pivot entry j + 1 as of column j - 2
+    __shared__ T qb[2][kLeafNB];  // scaled columns
+    __shared__ T pd[2], py[2];    // pivots and their reciprocal roots
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // update warps 3, 7, 11 | 5, 9 | 6, 10 | 4 (beside the pivots)
+    const int uw = warp == 3 ? 0 : warp >= 4 && warp <= 7 ? warp - 3 : warp >= 9 ? warp - 4 : -1;
+    T v[kUpdGroups][kUpdPer] = {};
+    int col[kUpdGroups][kUpdPer], row[kUpdGroups][kUpdPer], last[kUpdGroups][kUpdPer];  // last: the slot's last column
+    if (uw >= 0) {
 #pragma unroll
-        for (int u = 0; u < PER; u++) {
-            const int fast = tid % kLeafNB, slow = tid / kLeafNB + u * (kLeafThreads / kLeafNB);  // A(fast, slow)
-            const int i = upper ? slow : fast, c = upper ? fast : slow;
-            v[u] = (i < nr && c <= i) ? A0[fast + int64_t(slow) * lda] : T(0);
-        }
+        for (int g = 0; g < kUpdGroups; g++) {
 #pragma unroll
-        for (int u = 0; u < PER; u++) {
-            const int fast = tid % kLeafNB, slow = tid / kLeafNB + u * (kLeafThreads / kLeafNB);
-            s[upper ? fast : slow][upper ? slow : fast] = v[u];
+            for (int u = 0; u < kUpdPer; u++) {
+                const int slot = (g * kUpdPer + u) * kUpdWarps + uw;
+                // element 32 slot + lane of the columns of 64, 63, 62, ... entries;
+                // from the end column 63 - k starts at k (k + 1) / 2
+                const int f = max(kLeafSlots * 32 - 1 - (32 * slot + lane), 0);
+                const int k = int((sqrtf(8.0f * float(f) + 1.0f) - 1.0f) * 0.5f);
+                const bool in = slot < kLeafSlots;
+                const int c = in ? kLeafNB - 1 - k : 0, i = in ? kLeafNB - 1 - (f - k * (k + 1) / 2) : 0;
+                col[g][u] = c;
+                row[g][u] = i;
+                last[g][u] = __shfl_sync(0xffffffffu, in ? c : -1, 31);
+            }
         }
     }
-    if (tid < 2 * kLeafNB) (&col[0][0])[tid] = T(0);
-    if (tid == 0) fail = kLeafNB;
-    __syncthreads();
-    auto pivot = [&](int j, T d) {  // warp 0
-        T l, y;
-        pivot_root(d, l, y);
-        if (lane == 0) {
-            piv[j & 1][0] = l;
-            piv[j & 1][1] = y;
-            if (!(d > T(0))) fail = j;
-            else A0[j + int64_t(j) * lda] = l;
+    tc::pdl_wait();
+    tc::pdl_launch_dependents();
+    const int before = *static_cast<volatile int *>(info);
+    if (uw >= 0) {
+#pragma unroll
+        for (int g = 0; g < kUpdGroups; g++)
+#pragma unroll
+            for (int u = 0; u < kUpdPer; u++) {
+                const int c = col[g][u], i = row[g][u];
+                if (i < nr) v[g][u] = A0[upper ? c + int64_t(i) * lda : i + int64_t(c) * lda];
+            }
+#pragma unroll
+        for (int u = 0; u < kUpdPer; u++) {  // (columns 0 and 1 lie in the first slots)
+            const int c = col[0][u], i = row[0][u];
+            if (c == 0) cb[0][i] = v[0][u];
+            if (c == i && c < 2) dg[c] = v[0][u];
         }
+    }
+    if (before != 0) return;  // an earlier leaf failed
+    __syncthreads();
+    int fail = kLeafNB;  // first pivot that is not positive (warp 0; what follows it is undefined)
+    auto pivot = [&](int j, T d) {
+        const T y = root_rcp(d);
+        if (lane == 0) {
+            pd[j & 1] = d;
+            py[j & 1] = y;
+        }
+        if (!(d > T(0))) fail = min(fail, j);
     };
-    if (warp == 0) pivot(0, s[0][0]);
+    if (warp == 0) pivot(0, dg[0]);
     for (int j = 0; j < nr; j++) {
         __syncthreads();
-        if (fail <= j) break;
-        const T l = piv[j & 1][0], y = piv[j & 1][1];
+        const T *q1 = qb[(j + 1) & 1];  // column j - 1
         if (warp == 0) {
             if (j + 1 < nr) {
-                const T q = pivot_scale(s[j][j + 1], l, y);
-                pivot(j + 1, fma(-q, q, s[j + 1][j + 1]));
-            }
-        } else if (warp != 4) {
-            const int w = warp - 1 - (warp > 4);  // 0 .. 5
-            T *q = col[j & 1];
-            if (w < 2) {
-                const int i = 32 * w + lane;
-                if (i > j && i < nr) {
-                    const T v = pivot_scale(s[j][i], l, y);
-                    q[i] = v;
-                    A0[upper ? j + int64_t(i) * lda : i + int64_t(j) * lda] = v;
+                T x = cb[j & 1][j + 1], d = dg[(j + 1) & 1];
+                if (j > 0) {
+                    const T a = q1[j + 1];
+                    x = fma(-a, q1[j], x);
+                    d = fma(-a, a, d);
                 }
+                const T q = x * py[j & 1];
+                pivot(j + 1, fma(-q, q, d));
             }
-            asm volatile("bar.sync 1, 192;" ::: "memory");
-            // columns c > j, rows i >= c (but for the pivot (j + 1, j + 1): warp 0's)
-            // (rows past nr hold zeros); columns below 32 in two pieces of
-            // rows, two pieces at a time
-            int c = j + 1 + w;
-            for (; c < 32; c += 6) {
-                const T f = q[c];
-                const int i = c + lane, i2 = i + 32;
-                const T a = s[c][i], b = i2 < kLeafNB ? s[c][i2] : T(0);
-                const T qa = q[i], qb = i2 < kLeafNB ? q[i2] : T(0);
-                const T ra = fma(-qa, f, a), rb = fma(-qb, f, b);
-                if (i > j + 1) s[c][i] = ra;
-                if (i2 < kLeafNB) s[c][i2] = rb;
+        } else if (warp < 3) {
+            const int i = 32 * (warp - 1) + lane;
+            if (32 * warp > j) {
+                const T d = pd[j & 1], y = py[j & 1];
+                T x = cb[j & 1][i];
+                if (j > 0) x = fma(-q1[i], q1[j], x);
+                const T l = root(d, y), q = pivot_scale(x, l, y);
+                if (i > j) qb[j & 1][i] = q;
+                if (i >= j && i < nr) A0[upper ? j + int64_t(i) * lda : i + int64_t(j) * lda] = i > j ? q : l;
             }
-            for (; c < nr; c += 12) {
-                const int i = c + lane, c2 = c + 6, i2 = c2 + lane;
-                const bool in = i < kLeafNB, in2 = c2 < nr && i2 < kLeafNB;
-                const T f = q[c], f2 = c2 < nr ? q[c2] : T(0);
-                const T a = in ? s[c][i] : T(0), b = in2 ? s[c2][i2] : T(0);
-                const T qa = in ? q[i] : T(0), qb = in2 ? q[i2] : T(0);
-                const T ra = fma(-qa, f, a), rb = fma(-qb, f2, b);
-                if (in && i > j + 1) s[c][i] = ra;
-                if (in2) s[c2][i2] = rb;
+        } else if (uw >= 0) {
+            T *cn = cb[(j + 1) & 1];
+            auto publish = [&](int g, int u) {
+                const int c = col[g][u], i = row[g][u];
+                if (c == j + 1) cn[i] = v[g][u];
+                if (c == j + 2 && i == c) dg[j & 1] = v[g][u];
+            };
+#pragma unroll
+            for (int g = 0; g < kUpdGroups; g++) {
+                if (sizeof(T) == 8) {
+                    // slot by slot: an operation for a finished one costs as
+                    // much as any, and loads in a batch gain nothing (52 us)
+#pragma unroll
+                    for (int u = 0; u < kUpdPer; u++)
+                        if (last[g][u] > j) {
+                            if (j > 0) v[g][u] = fma(-q1[row[g][u]], q1[col[g][u]], v[g][u]);
+                            publish(g, u);
+                        }
+                } else if (max(last[g][0], max(last[g][1], last[g][2])) > j) {
+                    // loads of a group at once
+                    if (j > 0) {
+                        T qi[kUpdPer], qc[kUpdPer];
+#pragma unroll
+                        for (int u = 0; u < kUpdPer; u++) {
+                            qi[u] = q1[row[g][u]];
+                            qc[u] = q1[col[g][u]];
+                        }
+#pragma unroll
+                        for (int u = 0; u < kUpdPer; u++) v[g][u] = fma(-qi[u], qc[u], v[g][u]);
+                    }
+#pragma unroll
+                    for (int u = 0; u < kUpdPer; u++) publish(g, u);
+                }
             }
         }
     }
-    if (tid == 0 && fail < nr) atomicCAS(info, 0, int(r0 + fail + 1));
+    if (threadIdx.x == 0 && fail < nr) atomicCAS(info, 0, int(r0 + fail + 1));
 }
 
 int trsm_call(int side, int uplo, int trans, int64_t m, int64_t n, const double *A, int64_t lda, double *B,
@@ -241,8 +308,8 @@ struct PotrfExec {
         const int64_t w = c1 - c0;
         {
             LaunchScope ls(KK_DIAG, s, double(w) * w * w / 3.0, sizeof(T) * double(w) * (w + 1));
-            potrf_leaf_kernel<T><<<1, kLeafThreads, 0, s>>>(at(c0, c0), lda, int(w), upper, c0, info);
-            GB_TRY(check(cudaGetLastError()));
+            GB_TRY(check(launch_pdl(potrf_leaf_kernel<T>, dim3(1), dim3(kLeafThreads), 0, s, at(c0, c0), lda, int(w), int(upper),
+                                    c0, info)));
         }
         if (c1 >= n) return 0;
         // L(c1.., c0..) = A(c1.., c0..) L11^-T, or U(c0.., c1..) = U11^-T A(c0.., c1..)
