@@ -407,9 +407,16 @@ __device__ __forceinline__ uint32_t biased_int(float S)
 // Persistent: one CTA per SM walks the items w = blockIdx.x, + gridDim.x, ...
 // Warp 0 issues the TMA loads, warp 1 the MMAs, warps 2-17 drain the
 // accumulators and finish C.  What bounds it: the tensor cores (28 x 2 flop
-// per multiply-add of the product), fed with 48 KB of digits per 512 clocks;
+// per multiply-add of the product; over an 8192 x 8192 solve 1160 TFLOP/s in FP64,
+// 1010 in FP32, 4096^2 x 8192 alone about 1700), fed with 48 KB of digits per 512 clocks;
 // the drains (12 half accumulators per 28.7k clocks of MMAs) go on beside them.
 // Sixteen drain warps hide the latencies of the accumulators' loads.
+// Issuing is close to the bound too: with the loops of warps 0 and 1 in a branch
+// of one lane a stage's four MMAs, wait and commit took that lane about 700
+// clocks, more than their 512 on the tensor cores (4096 x 8192 x 4096: FP64 6.4
+// ms, FP32 1.94, now 4.96 and 1.52).  CTA pairs (256-row MMAs, cta_group::2)
+// halve the X traffic but came out slower, 5.18 and 1.65 ms; loading the next
+// chunk's slices into L2 ahead changed nothing.
 template <typename T>
 __global__ void __launch_bounds__(MMA_THREADS, 1)
 digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmX,
@@ -456,23 +463,26 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             tc::tma_prefetch_desc(&tmA);
             tc::tma_prefetch_desc(&tmX);
         }
+        // (No loop ends on a wait's result: after one that gave up nothing more
+        // is issued, every further wait returns at once, and the tiles are
+        // listed.  So the loops are the same for all lanes as far as the
+        // compiler can tell, and addresses and descriptors stay in uniform
+        // registers.)
         int n = 0;
-        int ok = 1;
-        for (int w = blockIdx.x; w < nitems && ok; w += gridDim.x) {
+        for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
             const Item it = digit_item(a, w, lane);
             if (it.skip) continue;
-            if (lane == 0) {
-                for (int kb = it.k0; kb < it.k1 && ok; kb += KC) {
-                    const int ke = min(kb + KC, it.k1);
-                    for (int o = 0; o < S::NO && ok; o++) {
-                        const int p = S::p(o), q = S::q(o);
-                        const bool two = o < S::TWO;
-                        for (int kk = kb; kk < ke; kk += BK, n++) {
-                            const int s = n % STAGES;
-                            const uint32_t ph = (n / STAGES) & 1;
-                            ok = tc::mbar_wait(&empty[s], ph ^ 1, ab, a.status, tc::TC_TIMEOUT_PRODUCER);
-                            if (!ok) break;
-                            uint8_t *st = base + s * STAGE_BYTES;
+            for (int kb = it.k0; kb < it.k1; kb += KC) {
+                const int ke = min(kb + KC, it.k1);
+#pragma unroll 1
+                for (int o = 0; o < S::NO; o++) {
+                    const int p = S::p(o), q = S::q(o);
+                    const bool two = o < S::TWO;
+                    for (int kk = kb; kk < ke; kk += BK, n++) {
+                        const int s = n % STAGES;
+                        const bool go = tc::mbar_pass(&empty[s], ((n / STAGES) & 1) ^ 1, ab, a.status, tc::TC_TIMEOUT_PRODUCER);
+                        uint8_t *st = base + s * STAGE_BYTES;
+                        if (tc::elect_one() && go) {
                             tc::mbar_arrive_expect_tx(&full[s], (two ? 3u : 2u) * TILE_BYTES);
                             tc::tma_load_3d(&tmA, &full[s], st, kk, it.i0, p);
                             tc::tma_load_3d(&tmX, &full[s], st + TILE_BYTES, kk, it.j0, q);
@@ -481,11 +491,13 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     }
                 }
             }
-            ok = __shfl_sync(0xffffffffu, ok, 0);
         }
+        __syncwarp();
         if (lane == 0) {
             // tail: wait until the MMAs released every stage, so that no
             // commit is still on its way to this CTA's barriers when it exits
+            const int n0 = n;
+            int ok = 1;
             for (int t = 0; t < STAGES && ok; t++, n++) {
                 const int s = n % STAGES;
                 const uint32_t ph = (n / STAGES) & 1;
@@ -493,8 +505,8 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             }
             // after a wait that gave up: the copies still in flight land
             // before this CTA's shared memory is given away (bounded)
-            if (!ok)
-                for (int t = n > STAGES ? n - STAGES : 0; t < n; t++)
+            if (*ab)
+                for (int t = n0 > STAGES ? n0 - STAGES : 0; t < n0; t++)
                     for (int spin = 0; spin < (1 << 16) && !tc::mbar_try_wait(&full[t % STAGES], (t / STAGES) & 1); spin++) {
                     }
         }
@@ -502,34 +514,31 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const uint64_t d0 = tc::desc_kmajor_sw128(tc::smem_u32(base));
         const uint32_t idesc256 = tc::idesc_bf16_f32(BM, 256), idesc128 = tc::idesc_bf16_f32(BM, 128);
         int n = 0, cp = 0;
-        int ok = 1;
-        for (int w = blockIdx.x; w < nitems && ok; w += gridDim.x) {
+        for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
             const Item it = digit_item(a, w, lane);
             if (it.skip) continue;
-            if (lane == 0) {
-                for (int kb = it.k0; kb < it.k1 && ok; kb += KC) {
-                    const int ke = min(kb + KC, it.k1);
-                    const int nk = (ke - kb) / BK;
-                    for (int j = 0; j < S::NP && ok; j++, cp++) {
-                        const int buf = cp & 1;
-                        ok = tc::mbar_wait(&acce[buf], ((cp >> 1) & 1) ^ 1, ab, a.status, tc::TC_TIMEOUT_MMA);
-                        if (!ok) break;
-                        tc::tc_fence_after();
-                        const uint32_t acc = tmem + uint32_t(buf * 256);
-                        const int o0 = S::first(j), o1 = S::first(j + 1);
-                        for (int o = o0; o < o1 && ok; o++) {
-                            const bool two = o < S::TWO;
-                            const uint32_t d = two ? acc : acc + 128u;
-                            const uint32_t idesc = two ? idesc256 : idesc128;
-                            for (int kt = 0; kt < nk; kt++, n++) {
-                                const int s = n % STAGES;
-                                ok = tc::mbar_wait(&full[s], (n / STAGES) & 1, ab, a.status, tc::TC_TIMEOUT_MMA);
-                                if (!ok) break;
-                                tc::tc_fence_after();
-                                // the start address field counts 16-byte units: a
-                                // 32-byte step along K adds 2
-                                const uint64_t da = d0 + uint64_t(uint32_t(s) * (STAGE_BYTES >> 4));
-                                const uint64_t db = da + uint64_t(TILE_BYTES >> 4);
+            for (int kb = it.k0; kb < it.k1; kb += KC) {
+                const int nk = (min(kb + KC, it.k1) - kb) / BK;
+#pragma unroll 1
+                for (int j = 0; j < S::NP; j++, cp++) {
+                    const int buf = cp & 1;
+                    tc::mbar_pass(&acce[buf], ((cp >> 1) & 1) ^ 1, ab, a.status, tc::TC_TIMEOUT_MMA);
+                    tc::tc_fence_after();
+                    const uint32_t acc = tmem + uint32_t(buf * 256);
+                    const int o0 = S::first(j), o1 = S::first(j + 1);
+                    for (int o = o0; o < o1; o++) {
+                        const bool two = o < S::TWO;
+                        const uint32_t d = two ? acc : acc + 128u;
+                        const uint32_t idesc = two ? idesc256 : idesc128;
+                        for (int kt = 0; kt < nk; kt++, n++) {
+                            const int s = n % STAGES;
+                            const bool go = tc::mbar_pass(&full[s], (n / STAGES) & 1, ab, a.status, tc::TC_TIMEOUT_MMA);
+                            tc::tc_fence_after();
+                            // the start address field counts 16-byte units: a
+                            // 32-byte step along K adds 2
+                            const uint64_t da = d0 + uint64_t(uint32_t(s) * (STAGE_BYTES >> 4));
+                            const uint64_t db = da + uint64_t(TILE_BYTES >> 4);
+                            if (tc::elect_one() && go) {
                                 tc::mma_f16(d, da, db, idesc, o != o0 || kt != 0);
 #pragma unroll
                                 for (int kk = 1; kk < BK / 16; kk++)
@@ -537,12 +546,12 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                                 tc::mma_commit(&empty[s]);
                             }
                         }
-                        if (ok) tc::mma_commit(&accf[buf]);
                     }
+                    if (tc::elect_one()) tc::mma_commit(&accf[buf]);
                 }
             }
-            ok = __shfl_sync(0xffffffffu, ok, 0);
         }
+        __syncwarp();
     } else {
         const int q = warp & 3;                 // TMEM lane group this warp may read
         const int cg = (warp - 2) >> 2;         // columns [32 cg, 32 cg + 32) of the tile

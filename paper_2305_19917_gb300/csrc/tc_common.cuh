@@ -98,6 +98,22 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
     }
 }
 
+// As mbar_wait, for a caller that goes on either way: once the CTA's abort flag
+// is set no further wait lasts.
+__device__ __forceinline__ bool mbar_pass(uint64_t *bar, uint32_t parity, volatile int *abort, int *status, int code)
+{
+    if (mbar_try_wait(bar, parity)) return true;
+    if (*abort) return false;
+    return mbar_wait(bar, parity, abort, status, code);
+}
+// True in one lane of a converged warp.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // ---- TMA -------------------------------------------------------------------
 __device__ __forceinline__ void tma_load_2d(const CUtensorMap *map, uint64_t *bar, void *dst, int x, int y)
 {

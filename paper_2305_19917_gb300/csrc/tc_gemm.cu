@@ -135,38 +135,54 @@ tc_gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     volatile int *ab = &abort_flag;
     tc::pdl_wait();  // A, B and C belong to the previous kernel until it completes
 
+    // Warps 0 and 1 run their loops with all lanes, and no loop ends on a
+    // wait's result (after one that gave up nothing more is issued and every
+    // further wait returns at once): so loop variables, addresses and
+    // descriptors stay in uniform registers, and one lane issues.
     if (warp == 0) {
         if (lane == 0) {
             tc::tma_prefetch_desc(&tmA);
             tc::tma_prefetch_desc(&tmB);
-            for (int kt = 0; kt < nk; kt++) {
-                const int s = kt % STAGES;
-                const uint32_t ph = (kt / STAGES) & 1;
-                if (!tc::mbar_wait(&empty[s], ph ^ 1, ab, status, tc::TC_TIMEOUT_PRODUCER)) break;
+        }
+        int s = 0;
+        uint32_t ph = 1;
+        for (int kt = 0; kt < nk; kt++) {
+            const bool go = tc::mbar_pass(&empty[s], ph, ab, status, tc::TC_TIMEOUT_PRODUCER);
+            if (tc::elect_one() && go) {
                 tc::mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
                 tc::tma_load_2d(&tmA, &full[s], sA + s * A_BYTES, kt * BK, m_blk * BM);
                 tc::tma_load_2d(&tmB, &full[s], sB + s * B_BYTES, kt * BK, n_blk * BN);
             }
+            if (++s == STAGES) {
+                s = 0;
+                ph ^= 1u;
+            }
         }
+        __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = tc::idesc_bf16_f32(BM, BN);
-            // descriptors from the ring's base ones (16-byte units: a 32-byte K step adds 2)
-            const uint64_t dA0 = tc::desc_kmajor_sw128(tc::smem_u32(sA)), dB0 = tc::desc_kmajor_sw128(tc::smem_u32(sB));
-            for (int kt = 0; kt < nk; kt++) {
-                const int s = kt % STAGES;
-                const uint32_t ph = (kt / STAGES) & 1;
-                if (!tc::mbar_wait(&full[s], ph, ab, status, tc::TC_TIMEOUT_MMA)) break;
-                tc::tc_fence_after();
-                const uint64_t da = dA0 + uint64_t(uint32_t(s) * (A_BYTES >> 4));
-                const uint64_t db = dB0 + uint64_t(uint32_t(s) * (B_BYTES >> 4));
+        constexpr uint32_t idesc = tc::idesc_bf16_f32(BM, BN);
+        // descriptors from the ring's base ones (16-byte units: a 32-byte K step adds 2)
+        const uint64_t dA0 = tc::desc_kmajor_sw128(tc::smem_u32(sA)), dB0 = tc::desc_kmajor_sw128(tc::smem_u32(sB));
+        int s = 0;
+        uint32_t ph = 0;
+        for (int kt = 0; kt < nk; kt++) {
+            const bool go = tc::mbar_pass(&full[s], ph, ab, status, tc::TC_TIMEOUT_MMA);
+            tc::tc_fence_after();
+            const uint64_t da = dA0 + uint64_t(uint32_t(s) * (A_BYTES >> 4));
+            const uint64_t db = dB0 + uint64_t(uint32_t(s) * (B_BYTES >> 4));
+            if (tc::elect_one() && go) {
                 tc::mma_f16(tmem, da, db, idesc, kt != 0);
 #pragma unroll
                 for (int kk = 1; kk < BK / 16; kk++) tc::mma_f16(tmem, da + uint64_t(2 * kk), db + uint64_t(2 * kk), idesc, 1);
                 tc::mma_commit(&empty[s]);
             }
-            tc::mma_commit(accf);
+            if (++s == STAGES) {
+                s = 0;
+                ph ^= 1u;
+            }
         }
+        if (tc::elect_one()) tc::mma_commit(accf);
+        __syncwarp();
     } else {
         // epilogue: 4 warps, warp w reads TMEM lanes 32*(w%4) .. +31
         const int q = warp & 3;
@@ -283,65 +299,64 @@ tc_gemm_bf16_persistent_kernel(const __grid_constant__ CUtensorMap tmA, const __
     volatile int *ab = &abort_flag;
     tc::pdl_wait();  // A, B and C belong to the previous kernel until it completes
 
+    // (warps 0 and 1: as in tc_gemm_bf16_kernel)
     if (warp == 0) {
         if (lane == 0) {
             tc::tma_prefetch_desc(&tmA);
             tc::tma_prefetch_desc(&tmB);
-            uint32_t kg = 0;
-            for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-                int m_blk, n_blk;
-                tc::raster_grouped(t, nMt, nNt, 8, m_blk, n_blk);
-                bool ok = true;
-                for (int kt = 0; kt < nk; kt++, kg++) {
-                    const int s = kg % PSTAGES;
-                    const uint32_t ph = (kg / PSTAGES) & 1;
-                    if (!tc::mbar_wait(&empty[s], ph ^ 1, ab, status, tc::TC_TIMEOUT_PRODUCER)) {
-                        ok = false;
-                        break;
-                    }
+        }
+        int s = 0;
+        uint32_t ph = 1;
+        for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+            int m_blk, n_blk;
+            tc::raster_grouped(t, nMt, nNt, 8, m_blk, n_blk);
+            for (int kt = 0; kt < nk; kt++) {
+                const bool go = tc::mbar_pass(&empty[s], ph, ab, status, tc::TC_TIMEOUT_PRODUCER);
+                if (tc::elect_one() && go) {
                     tc::mbar_arrive_expect_tx(&full[s], P_STAGE_BYTES);
                     tc::tma_load_2d(&tmA, &full[s], sA + s * A_BYTES, kt * BK, m_blk * BM);
                     tc::tma_load_2d(&tmB, &full[s], sB + s * P_B_BYTES, kt * BK, n_blk * PBN);
                 }
-                if (!ok) break;
+                if (++s == PSTAGES) {
+                    s = 0;
+                    ph ^= 1u;
+                }
             }
         }
+        __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = tc::idesc_bf16_f32(BM, PBN);
-            // descriptors from the ring's base ones (16-byte units: a 32-byte K step adds
-            // 2), and the ring position kept incrementally (no division per K step)
-            const uint64_t dA0 = tc::desc_kmajor_sw128(tc::smem_u32(sA)), dB0 = tc::desc_kmajor_sw128(tc::smem_u32(sB));
-            int s = 0;
-            uint32_t ph = 0;
-            int it = 0;
-            bool ok = true;
-            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, it++) {
-                const int buf = it & 1;
-                const uint32_t use = uint32_t(it >> 1);
-                if (!tc::mbar_wait(&tempty[buf], (use & 1) ^ 1, ab, status, tc::TC_TIMEOUT_MMA)) break;
+        constexpr uint32_t idesc = tc::idesc_bf16_f32(BM, PBN);
+        // descriptors from the ring's base ones (16-byte units: a 32-byte K step adds
+        // 2), and the ring position kept incrementally (no division per K step)
+        const uint64_t dA0 = tc::desc_kmajor_sw128(tc::smem_u32(sA)), dB0 = tc::desc_kmajor_sw128(tc::smem_u32(sB));
+        int s = 0;
+        uint32_t ph = 0;
+        int it = 0;
+        for (int t = blockIdx.x; t < ntiles; t += gridDim.x, it++) {
+            const int buf = it & 1;
+            tc::mbar_pass(&tempty[buf], (uint32_t(it >> 1) & 1) ^ 1, ab, status, tc::TC_TIMEOUT_MMA);
+            tc::tc_fence_after();
+            const uint32_t d = tmem + uint32_t(buf * PBN);
+            for (int kt = 0; kt < nk; kt++) {
+                const bool go = tc::mbar_pass(&full[s], ph, ab, status, tc::TC_TIMEOUT_MMA);
                 tc::tc_fence_after();
-                const uint32_t d = tmem + uint32_t(buf * PBN);
-                for (int kt = 0; kt < nk; kt++) {
-                    if (!tc::mbar_wait(&full[s], ph, ab, status, tc::TC_TIMEOUT_MMA)) {
-                        ok = false;
-                        break;
-                    }
-                    tc::tc_fence_after();
-                    const uint64_t da = dA0 + uint64_t(uint32_t(s) * (A_BYTES >> 4));
-                    const uint64_t db = dB0 + uint64_t(uint32_t(s) * (P_B_BYTES >> 4));
+                const uint64_t da = dA0 + uint64_t(uint32_t(s) * (A_BYTES >> 4));
+                const uint64_t db = dB0 + uint64_t(uint32_t(s) * (P_B_BYTES >> 4));
+                if (tc::elect_one() && go) {
                     tc::mma_f16(d, da, db, idesc, kt != 0);
 #pragma unroll
-                    for (int kk = 1; kk < BK / 16; kk++) tc::mma_f16(d, da + uint64_t(2 * kk), db + uint64_t(2 * kk), idesc, 1);
+                    for (int kk = 1; kk < BK / 16; kk++)
+                        tc::mma_f16(d, da + uint64_t(2 * kk), db + uint64_t(2 * kk), idesc, 1);
                     tc::mma_commit(&empty[s]);
-                    if (++s == PSTAGES) {
-                        s = 0;
-                        ph ^= 1u;
-                    }
                 }
-                if (ok) tc::mma_commit(&tfull[buf]);
+                if (++s == PSTAGES) {
+                    s = 0;
+                    ph ^= 1u;
+                }
             }
+            if (tc::elect_one()) tc::mma_commit(&tfull[buf]);
         }
+        __syncwarp();
     } else {
         const int q = warp & 3;                 // TMEM lane quadrant of this warp
         const int half = (warp - 2) >> 2;       // which 128 columns of the tile

@@ -137,105 +137,90 @@ tc_residual_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     const uint32_t tmem = *tslot;
     volatile int *ab = &abort_flag;
 
+    // Warps 0 and 1 run their loops with all lanes, and no loop ends on a
+    // wait's result (after one that gave up nothing more is issued and every
+    // further wait returns at once): so loop variables, addresses and
+    // descriptors stay in uniform registers, and one lane issues (a branch on
+    // one lane around the loops: 35.2 ms for the two residuals of 16384^2, 33.3 so).
     if (warp == 0) {
         if (lane == 0) {
             tc::tma_prefetch_desc(&tmA);
             tc::tma_prefetch_desc(&tmZ);
-            int g = 0;
-            bool ok = true;
-            // one ring entry: slice p's A tile and the first nsl z tiles
-            auto load = [&](int kk, int p, int nsl) {
-                const int s = g % STAGES;
-                const uint32_t ph = (g / STAGES) & 1;
-                if (!tc::mbar_wait(&empty[s], ph ^ 1, ab, status, tc::TC_TIMEOUT_PRODUCER)) return false;
+        }
+        int g = 0;
+        // one ring entry: slice p's A tile and the first nsl z tiles
+        auto load = [&](int kk, int p, int nsl) {
+            const int s = g % STAGES;
+            const bool go = tc::mbar_pass(&empty[s], ((g / STAGES) & 1) ^ 1, ab, status, tc::TC_TIMEOUT_PRODUCER);
+            if (tc::elect_one() && go) {
                 tc::mbar_arrive_expect_tx(&full[s], A_BYTES + uint32_t(nsl) * ZS_BYTES);
                 tc::tma_load_3d(&tmA, &full[s], sA + s * A_BYTES, kk, i0, p);
-                for (int q = 0; q < nsl; q++)
-                    tc::tma_load_3d(&tmZ, &full[s], sB + s * B_BYTES + q * ZS_BYTES, kk, j0, q);
-                g++;
-                return true;
-            };
-            for (int c = 0; c < nchunks && ok; c++) {
-                const int kc0 = k_lo + c * KC, kc1 = min(kc0 + KC, k_end);
-                const int nj = chunk_passes(kc0, kc1, P, merge);
-                for (int j = 0; j < nj && ok; j++) {
-                    const Pass ps = chunk_pass(j, kc0, kc1, P, P2, merge);
-                    for (int kk = ps.kb; kk < ps.ke && ok; kk += BK) {
-                        ok = load(kk, ps.p, ps.nsl);
-                        if (ok && ps.merged) ok = load(kk, ps.p + 1, 1);
-                    }
+                tc::tma_load_3d(&tmZ, &full[s], sB + s * B_BYTES, kk, j0, 0);
+                if (nsl == 2) tc::tma_load_3d(&tmZ, &full[s], sB + s * B_BYTES + ZS_BYTES, kk, j0, 1);
+            }
+            g++;
+        };
+        for (int c = 0; c < nchunks; c++) {
+            const int kc0 = k_lo + c * KC, kc1 = min(kc0 + KC, k_end);
+            const int nj = chunk_passes(kc0, kc1, P, merge);
+            for (int j = 0; j < nj; j++) {
+                const Pass ps = chunk_pass(j, kc0, kc1, P, P2, merge);
+                for (int kk = ps.kb; kk < ps.ke; kk += BK) {
+                    load(kk, ps.p, ps.nsl);
+                    if (ps.merged) load(kk, ps.p + 1, 1);
                 }
             }
-            // tail: wait until the MMAs released every stage, so that no
-            // commit is still on its way to this CTA's barriers when it exits
-            for (int t = 0; t < STAGES && ok; t++, g++) {
-                const int s = g % STAGES;
-                const uint32_t ph = (g / STAGES) & 1;
-                if (!tc::mbar_wait(&empty[s], ph ^ 1, ab, status, tc::TC_TIMEOUT_PRODUCER)) break;
-            }
         }
+        __syncwarp();
+        // tail: wait until the MMAs released every stage, so that no
+        // commit is still on its way to this CTA's barriers when it exits
+        if (lane == 0)
+            for (int t = 0; t < STAGES; t++, g++)
+                if (!tc::mbar_pass(&empty[g % STAGES], ((g / STAGES) & 1) ^ 1, ab, status, tc::TC_TIMEOUT_PRODUCER)) break;
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint64_t dA0 = tc::desc_kmajor_sw128(tc::smem_u32(sA)), dB0 = tc::desc_kmajor_sw128(tc::smem_u32(sB));
-            const uint32_t idesc256 = tc::idesc_bf16_f32(BM, 256), idesc128 = tc::idesc_bf16_f32(BM, 128);
-            int g = 0, cp = 0;
-            bool ok = true;
-            // ring entry g: wait until its copies landed, return its stage
-            auto take = [&](int &s) {
-                s = g % STAGES;
-                const uint32_t ph = (g / STAGES) & 1;
-                g++;
-                if (!tc::mbar_wait(&full[s], ph, ab, status, tc::TC_TIMEOUT_MMA)) return false;
+        const uint64_t dA0 = tc::desc_kmajor_sw128(tc::smem_u32(sA)), dB0 = tc::desc_kmajor_sw128(tc::smem_u32(sB));
+        const uint32_t idesc256 = tc::idesc_bf16_f32(BM, 256), idesc128 = tc::idesc_bf16_f32(BM, 128);
+        int g = 0, cp = 0;
+        // ring entry g, once its copies have landed, into the accumulator d:
+        // the stage's descriptors from the ring's base ones (the start address
+        // field counts 16-byte units, so a 32-byte step along K adds 2)
+        auto mma = [&](uint32_t d, uint32_t idesc, uint32_t acc) {
+            const int s = g % STAGES;
+            const bool go = tc::mbar_pass(&full[s], (g / STAGES) & 1, ab, status, tc::TC_TIMEOUT_MMA);
+            tc::tc_fence_after();
+            const uint64_t da = dA0 + uint64_t(uint32_t(s) * (A_BYTES >> 4));
+            const uint64_t db = dB0 + uint64_t(uint32_t(s) * (B_BYTES >> 4));
+            if (tc::elect_one() && go) {
+                tc::mma_f16(d, da, db, idesc, acc);
+#pragma unroll
+                for (int kk = 1; kk < BK / 16; kk++)
+                    tc::mma_f16(d, da + uint64_t(2 * kk), db + uint64_t(2 * kk), idesc, 1);
+                tc::mma_commit(&empty[s]);
+            }
+            g++;
+        };
+        for (int c = 0; c < nchunks; c++) {
+            const int kc0 = k_lo + c * KC, kc1 = min(kc0 + KC, k_end);
+            const int nj = chunk_passes(kc0, kc1, P, merge);
+            for (int j = 0; j < nj; j++, cp++) {
+                const Pass ps = chunk_pass(j, kc0, kc1, P, P2, merge);
+                const int nk = (ps.ke - ps.kb) / BK;
+                const int buf = cp & 1;
+                tc::mbar_pass(&acce[buf], ((cp >> 1) & 1) ^ 1, ab, status, tc::TC_TIMEOUT_MMA);
                 tc::tc_fence_after();
-                return true;
-            };
-            for (int c = 0; c < nchunks && ok; c++) {
-                const int kc0 = k_lo + c * KC, kc1 = min(kc0 + KC, k_end);
-                const int nj = chunk_passes(kc0, kc1, P, merge);
-                for (int j = 0; j < nj && ok; j++, cp++) {
-                    const Pass ps = chunk_pass(j, kc0, kc1, P, P2, merge);
-                    const int nk = (ps.ke - ps.kb) / BK;
-                    const int buf = cp & 1;
-                    const uint32_t use = cp >> 1;
-                    if (!tc::mbar_wait(&acce[buf], (use & 1) ^ 1, ab, status, tc::TC_TIMEOUT_MMA)) {
-                        ok = false;
-                        break;
-                    }
-                    tc::tc_fence_after();
-                    // pair (p+1, 2) formed: one N = 256 MMA over [z_1; z_2]
-                    const uint32_t idesc = ps.nsl == 2 ? idesc256 : idesc128;
-                    const uint32_t d = tmem + uint32_t(buf * 256);
-                    for (int kt = 0; kt < nk; kt++) {
-                        int s;
-                        if (!(ok = take(s))) break;
-                        // the stage's descriptors from the ring's base ones: the start
-                        // address field counts 16-byte units, so a 32-byte step along
-                        // K adds 2 (few instructions per MMA: an N = 128 MMA takes
-                        // 64 tensor-core clocks)
-                        const uint64_t da = dA0 + uint64_t(uint32_t(s) * (A_BYTES >> 4));
-                        const uint64_t db = dB0 + uint64_t(uint32_t(s) * (B_BYTES >> 4));
-                        tc::mma_f16(d, da, db, idesc, kt != 0);
-#pragma unroll
-                        for (int kk = 1; kk < BK / 16; kk++)
-                            tc::mma_f16(d, da + uint64_t(2 * kk), db + uint64_t(2 * kk), idesc, 1);
-                        tc::mma_commit(&empty[s]);
-                        if (ps.merged) {
-                            // slice p+2 (1-based) times its own copy of z_1, added
-                            // into the z_2 half (the same pair weight)
-                            int s2;
-                            if (!(ok = take(s2))) break;
-                            const uint64_t da2 = dA0 + uint64_t(uint32_t(s2) * (A_BYTES >> 4));
-                            const uint64_t db2 = dB0 + uint64_t(uint32_t(s2) * (B_BYTES >> 4));
-#pragma unroll
-                            for (int kk = 0; kk < BK / 16; kk++)
-                                tc::mma_f16(d + 128u, da2 + uint64_t(2 * kk), db2 + uint64_t(2 * kk), idesc128, 1);
-                            tc::mma_commit(&empty[s2]);
-                        }
-                    }
-                    tc::mma_commit(&accf[buf]);
+                // pair (p+1, 2) formed: one N = 256 MMA over [z_1; z_2]
+                const uint32_t idesc = ps.nsl == 2 ? idesc256 : idesc128;
+                const uint32_t d = tmem + uint32_t(buf * 256);
+                for (int kt = 0; kt < nk; kt++) {
+                    mma(d, idesc, kt != 0);
+                    // merged: slice p+2 (1-based) times its own copy of z_1, added
+                    // into the z_2 half (the same pair weight)
+                    if (ps.merged) mma(d + 128u, idesc128, 1);
                 }
+                if (tc::elect_one()) tc::mma_commit(&accf[buf]);
             }
         }
+        __syncwarp();
     } else {
         const int q = warp & 3;                 // TMEM lane group this warp may read
         const int half = (warp - 2) >> 2;       // output columns [half*64, half*64+64)
