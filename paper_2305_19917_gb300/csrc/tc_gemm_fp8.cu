@@ -21,17 +21,24 @@ int *device_status_word();
 
 namespace {
 
-constexpr int BM = 128, BN = 128, BK = 128, STAGES = 6;
-constexpr uint32_t A_BYTES = BM * BK, B_BYTES = BN * BK;
-constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
-constexpr size_t SMEM_BYTES = 1024 + STAGES * size_t(STAGE_BYTES) + 256;
+constexpr int BM = 128, BK = 128, NTHR = 320;
+constexpr uint32_t A_BYTES = BM * BK;
+template <int BN>
+struct Cfg8 {
+    static constexpr uint32_t B_BYTES = BN * BK, STAGE_BYTES = A_BYTES + B_BYTES;
+    static constexpr int STAGES = int(192 * 1024 / STAGE_BYTES);
+    static constexpr size_t SMEM = 1024 + STAGES * size_t(STAGE_BYTES) + 256;
+};
 
-__global__ void __launch_bounds__(192, 1)
+template <int BN>
+__global__ void __launch_bounds__(NTHR, 1)
 tc_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    float *__restrict__ C, int64_t ldc, int M, int N, int K, float alpha,
                    const float *__restrict__ sA, int64_t ldsa, const float *__restrict__ sB, int64_t ldsb,
                    int nMt, int nNt, int *status)
 {
+    constexpr int STAGES = Cfg8<BN>::STAGES;
+    constexpr uint32_t B_BYTES = Cfg8<BN>::B_BYTES, STAGE_BYTES = Cfg8<BN>::STAGE_BYTES;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t *sAm = base;
@@ -47,6 +54,7 @@ tc_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     int m_blk, n_blk;
     tc::raster_grouped(int(blockIdx.x), nMt, nNt, 8, m_blk, n_blk);
     const int nk = K / BK;
+    tc::pdl_launch_dependents();
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; s++) {
@@ -55,7 +63,7 @@ tc_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         }
         for (int b = 0; b < 2; b++) {
             tc::mbar_init(&accf[b], 1);
-            tc::mbar_init(&acce[b], 4);  // one arrival per epilogue warp
+            tc::mbar_init(&acce[b], 8);  // one arrival per epilogue warp
         }
         abort_flag = 0;
         tc::fence_barrier_init();
@@ -66,34 +74,40 @@ tc_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     tc::tc_fence_after();
     const uint32_t tmem = *tslot;
     volatile int *ab = &abort_flag;
+    tc::pdl_wait();  // the operands and C belong to the previous kernel until it completes
 
+    // Warps 0 and 1 run their loops with all lanes, and no loop ends on a
+    // wait's result (after one that gave up nothing more is issued and every
+    // further wait returns at once): so loop variables, addresses and
+    // descriptors stay in uniform registers, and one lane issues.
     if (warp == 0) {
         if (lane == 0) {
             tc::tma_prefetch_desc(&tmA);
             tc::tma_prefetch_desc(&tmB);
-            for (int kt = 0; kt < nk; kt++) {
-                const int s = kt % STAGES;
-                const uint32_t ph = (kt / STAGES) & 1;
-                if (!tc::mbar_wait(&empty[s], ph ^ 1, ab, status, tc::TC_TIMEOUT_PRODUCER)) break;
+        }
+        for (int kt = 0; kt < nk; kt++) {
+            const int s = kt % STAGES;
+            const bool go = tc::mbar_pass(&empty[s], ((kt / STAGES) & 1) ^ 1, ab, status, tc::TC_TIMEOUT_PRODUCER);
+            if (tc::elect_one() && go) {
                 tc::mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
                 tc::tma_load_2d(&tmA, &full[s], sAm + s * A_BYTES, kt * BK, m_blk * BM);
                 tc::tma_load_2d(&tmB, &full[s], sBm + s * B_BYTES, kt * BK, n_blk * BN);
             }
         }
+        __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = tc::idesc_e4m3_f32(BM, BN);
-            // descriptors from the ring's base ones (16-byte units: a 32-byte K step adds 2)
-            const uint64_t dA0 = tc::desc_kmajor_sw128(tc::smem_u32(sAm)), dB0 = tc::desc_kmajor_sw128(tc::smem_u32(sBm));
-            for (int kt = 0; kt < nk; kt++) {
-                const int s = kt % STAGES;
-                const uint32_t ph = (kt / STAGES) & 1;
-                const int buf = kt & 1;
-                if (!tc::mbar_wait(&acce[buf], ((kt >> 1) & 1) ^ 1, ab, status, tc::TC_TIMEOUT_MMA)) break;
-                if (!tc::mbar_wait(&full[s], ph, ab, status, tc::TC_TIMEOUT_MMA)) break;
-                tc::tc_fence_after();
-                const uint64_t da = dA0 + uint64_t(uint32_t(s) * (A_BYTES >> 4));
-                const uint64_t db = dB0 + uint64_t(uint32_t(s) * (B_BYTES >> 4));
+        constexpr uint32_t idesc = tc::idesc_e4m3_f32(BM, BN);
+        // descriptors from the ring's base ones (16-byte units: a 32-byte K step adds 2)
+        const uint64_t dA0 = tc::desc_kmajor_sw128(tc::smem_u32(sAm)), dB0 = tc::desc_kmajor_sw128(tc::smem_u32(sBm));
+        for (int kt = 0; kt < nk; kt++) {
+            const int s = kt % STAGES;
+            const int buf = kt & 1;
+            tc::mbar_pass(&acce[buf], ((kt >> 1) & 1) ^ 1, ab, status, tc::TC_TIMEOUT_MMA);
+            const bool go = tc::mbar_pass(&full[s], (kt / STAGES) & 1, ab, status, tc::TC_TIMEOUT_MMA);
+            tc::tc_fence_after();
+            const uint64_t da = dA0 + uint64_t(uint32_t(s) * (A_BYTES >> 4));
+            const uint64_t db = dB0 + uint64_t(uint32_t(s) * (B_BYTES >> 4));
+            if (tc::elect_one() && go) {
 #pragma unroll
                 for (int kk = 0; kk < BK / 32; kk++)
                     tc::mma_f8(tmem + uint32_t(buf * BN), da + uint64_t(2 * kk), db + uint64_t(2 * kk), idesc, kk != 0);
@@ -101,33 +115,50 @@ tc_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                 tc::mma_commit(&accf[buf]);
             }
         }
+        __syncwarp();
     } else {
-        const int q = warp & 3;
+        constexpr int HN = BN / 2, NS = HN / 64;  // columns and scale blocks of this warp
+        const int q = warp & 3, half = (warp - 2) >> 2;
         const int row = q * 32 + lane;
         const int64_t gi = int64_t(m_blk) * BM + row;
-        float acc[BN];
+        const int64_t gh = int64_t(n_blk) * BN + half * HN;
+        float acc[HN];
 #pragma unroll
-        for (int c = 0; c < BN; c++) acc[c] = 0.f;
+        for (int c = 0; c < HN; c++) acc[c] = 0.f;
+        const float *pa = sA + int64_t(m_blk) * ldsa, *pb[NS];
+#pragma unroll
+        for (int u = 0; u < NS; u++) {
+            const int64_t last = N / 64 - 1, c = gh / 64 + u;
+            pb[u] = sB + (c < last ? c : last);
+        }
+        float sa = pa[0], sb[NS];
+#pragma unroll
+        for (int u = 0; u < NS; u++) sb[u] = pb[u][0];
         bool ok = true;
         for (int kt = 0; kt < nk; kt++) {
+            float sc[NS];
+#pragma unroll
+            for (int u = 0; u < NS; u++) sc[u] = sa * sb[u];
+            if (kt + 1 < nk) {
+                sa = pa[kt + 1];
+#pragma unroll
+                for (int u = 0; u < NS; u++) sb[u] = pb[u][int64_t(kt + 1) * ldsb];
+            }
             const int buf = kt & 1;
             if (!tc::mbar_wait(&accf[buf], (kt >> 1) & 1, ab, status, tc::TC_TIMEOUT_EPILOGUE)) {
                 ok = false;
                 break;
             }
             tc::tc_fence_after();
-            const float sa = sA[int64_t(m_blk) * ldsa + kt];
-            const float sb0 = sB[int64_t(kt) * ldsb + 2 * n_blk], sb1 = sB[int64_t(kt) * ldsb + 2 * n_blk + 1];
-            const float s0 = sa * sb0, s1 = sa * sb1;
-            const uint32_t tb = tmem + (uint32_t(q * 32) << 16) + uint32_t(buf * BN);
+            const uint32_t tb = tmem + (uint32_t(q * 32) << 16) + uint32_t(buf * BN + half * HN);
 #pragma unroll
-            for (int c0 = 0; c0 < BN; c0 += 32) {
-                uint32_t r[32];
-                tc::tmem_ld32(tb + c0, r);
+            for (int c0 = 0; c0 < HN; c0 += 16) {
+                uint32_t r[2][8];
+                tc::tmem_ld8(tb + c0, r[0]);
+                tc::tmem_ld8(tb + c0 + 8, r[1]);
                 tc::tmem_ld_wait();
-                const float sc = c0 < 64 ? s0 : s1;
 #pragma unroll
-                for (int j = 0; j < 32; j++) acc[c0 + j] = fmaf(sc, __uint_as_float(r[j]), acc[c0 + j]);
+                for (int j = 0; j < 16; j++) acc[c0 + j] = fmaf(sc[c0 / 64], __uint_as_float(r[j / 8][j % 8]), acc[c0 + j]);
             }
             tc::tc_fence_before();
             __syncwarp();
@@ -135,9 +166,9 @@ tc_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         }
         if (ok && gi < M) {
 #pragma unroll
-            for (int c0 = 0; c0 < BN; c0 += 16) {
+            for (int c0 = 0; c0 < HN; c0 += 16) {
                 float cv[16];
-                const int64_t gj0 = int64_t(n_blk) * BN + c0;
+                const int64_t gj0 = gh + c0;
 #pragma unroll
                 for (int j = 0; j < 16; j++) cv[j] = (gj0 + j < N) ? C[gi + (gj0 + j) * ldc] : 0.f;
 #pragma unroll
@@ -158,8 +189,9 @@ tc_gemm_fp8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
 
 int tc_gemm_fp8_prepare()
 {
-    static PerDeviceOnce attr;
-    return smem_attr_once(attr, tc_gemm_fp8_kernel, SMEM_BYTES);
+    static PerDeviceOnce a128, a256;
+    GB_TRY(smem_attr_once(a128, tc_gemm_fp8_kernel<128>, Cfg8<128>::SMEM));
+    return smem_attr_once(a256, tc_gemm_fp8_kernel<256>, Cfg8<256>::SMEM);
 }
 
 // C (M x N FP32 column-major) = alpha*C - A8*B8 with the block scales above;
@@ -173,9 +205,12 @@ int launch_tc_gemm_fp8(int64_t M, int64_t N, int64_t K, const void *A, int64_t l
                        int64_t ldsb, cudaStream_t s, int *status)
 {
     if (M <= 0 || N <= 0) return 0;
-    if (K <= 0 || K % BK || N % BN || lda % 16 || ldb % 16 || (reinterpret_cast<uintptr_t>(A) & 15) ||
+    if (K <= 0 || K % BK || N % 128 || lda % 16 || ldb % 16 || (reinterpret_cast<uintptr_t>(A) & 15) ||
         (reinterpret_cast<uintptr_t>(B) & 15))
         return GB_STATUS_CUDA_ERROR;
+    const int64_t nM = (M + BM - 1) / BM;
+    const bool wide = nM * ((N + 255) / 256) >= 152;
+    const int bn = wide ? 256 : 128;
     CUtensorMap ta, tb;
     {
         uint64_t dims[2] = {uint64_t(K), uint64_t(M)};
@@ -186,18 +221,21 @@ int launch_tc_gemm_fp8(int64_t M, int64_t N, int64_t K, const void *A, int64_t l
     {
         uint64_t dims[2] = {uint64_t(K), uint64_t(N)};
         uint64_t strides[1] = {uint64_t(ldb)};
-        uint32_t box[2] = {BK, BN};
+        uint32_t box[2] = {BK, uint32_t(bn)};
         GB_TRY(encode_tmap(&tb, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, B, dims, strides, box));
     }
     GB_TRY(tc_gemm_fp8_prepare());
     int *st = status ? status : device_status_word();
     if (!st) return GB_STATUS_CUDA_ERROR;
-    const int64_t nM = (M + BM - 1) / BM, nN = (N + BN - 1) / BN;
+    const int64_t nN = (N + bn - 1) / bn;
     if (nM * nN > 0x7fffffffLL) return GB_STATUS_CUDA_ERROR;
     LaunchScope ls(KK_GEMM_TC, s, 2.0 * M * N * K, double(M) * K + double(K) * N + 8.0 * M * N);
-    tc_gemm_fp8_kernel<<<(unsigned)(nM * nN), 192, SMEM_BYTES, s>>>(ta, tb, C, ldc, (int)M, (int)N, (int)K, alpha,
-                                                                     sA, ldsa, sB, ldsb, (int)nM, (int)nN, st);
-    return check(cudaGetLastError());
+    const dim3 grid((unsigned)(nM * nN));
+    if (wide)
+        return check(launch_pdl(tc_gemm_fp8_kernel<256>, grid, dim3(NTHR), Cfg8<256>::SMEM, s, ta, tb, C, ldc, int(M), int(N),
+                                int(K), alpha, sA, ldsa, sB, ldsb, int(nM), int(nN), st));
+    return check(launch_pdl(tc_gemm_fp8_kernel<128>, grid, dim3(NTHR), Cfg8<128>::SMEM, s, ta, tb, C, ldc, int(M), int(N),
+                            int(K), alpha, sA, ldsa, sB, ldsb, int(nM), int(nN), st));
 }
 
 }  // namespace gb
