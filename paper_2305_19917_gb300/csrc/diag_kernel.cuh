@@ -2,12 +2,12 @@
 // and 3; the white triangles of Figs. 2-4), for one nr x nr block with
 // nr <= 64 and all right-hand sides of the canonical view.
 //
-// Design (GB300): a CTA solves 64 right-hand sides with 8 warps; warp w
+// Design (GB300): a CTA solves 64 (or 32) right-hand sides with 8 (4) warps; warp w
 // handles 32 of them (column group w / 4) and the rows i = w % 4 (mod 4) of
-// the block, in registers, by column-oriented substitution: at step k the
-// warp owning row k forms x_k = t_k / a_kk, publishes it in shared memory
-// (a named barrier per column group), and the four warps update their own
-// rows.  Splitting each right-hand side's rows over four warps matters on
+// the block, in registers, by column-oriented substitution: the warp owning
+// row k forms x_k = t_k / a_kk and publishes it in shared memory, and the four
+// warps update their own rows.  What bounds it is the FP64 unit (64 x 8192: 33
+// of 43 us; 46 when every step waited for its x_k).  Splitting each right-hand side's rows over four warps matters on
 // this GPU: a warp runs on one SM sub-partition, whose FP64 unit takes about
 // 64 clocks per warp instruction (a quarter of the SM's 1.9 DFMA per clock),
 // so one warp per column would leave three quarters of the FP64 throughput
@@ -23,9 +23,11 @@
 namespace gb {
 namespace {
 
-// Threads per CTA (8 warps: 2 column groups x 4 row groups); a CTA solves
-// CW = 64 right-hand sides.
-constexpr int kDiagThreads = 256;
+// Threads per CTA: column groups of 32 x 4 row groups.  A CTA solves CW = 64
+// right-hand sides, or 32 where such CTAs still fit the SMs side by side (up to
+// 4864): FP64 64 x 4096 33 us instead of 43.
+template <int CW>
+constexpr int kDiagThreads = 4 * CW;
 
 // Asynchronous copy of one 4- or 8-byte element into shared memory; `in`
 // false writes zero (the source is not read).
@@ -52,13 +54,17 @@ constexpr size_t diag_smem_bytes()
 }
 
 // The substitution of one warp: rows i = 4 m + RG of right-hand side `col`
-// (column group cg).  At step k the warp owning row k forms x_k = t_k / a_kk
-// and publishes it in Bs (row k); after the column group's named barrier the
-// four warps subtract a_ik x_k from their rows below (forward) or above
-// (backward) k.  Fully unrolled with RG fixed, so t stays in registers and
-// every row test is a compile-time constant.  The four warps of a column
-// group run different instantiations and meet at the same named barrier
-// (a counting barrier of 128 threads) from their own code.
+// (column group cg).  At step k the four warps subtract a_ik x_k from their rows
+// below (forward) or above (backward) k; the warp of the next row does that row
+// first, forms x_next = t / a, publishes it in Bs (row next) and signals it
+// before its other rows, so that a step costs its multiply-adds and no
+// latency of the chain.  A signal is an arrival of the owner on a named barrier
+// of the column group (128 threads) that the other three warps wait on; it
+// alternates between two, since the owner may be a step ahead.  Fully unrolled
+// with RG fixed, so t stays in registers and every row test is a compile-time
+// constant (the four warps run different instantiations); rows from nr on are
+// solved too, to zero: a test of nr at every step kept the compiler from moving
+// anything across it.
 template <typename T, int NB, bool FWD, bool MT, int CW, int RG>
 __device__ __forceinline__ void diag_rows(const T *L, const T *inv, T *Bs, int nr, int col, int cg, T alpha)
 {
@@ -68,24 +74,35 @@ __device__ __forceinline__ void diag_rows(const T *L, const T *inv, T *Bs, int n
     // a warp reads only its own rows of B, and x_k overwrites row k, owned by
     // the warp that writes it: no barrier needed before the steps
 #pragma unroll
-    for (int m = 0; m < NM; m++) t[m] = alpha * Bs[(4 * m + RG) * BS + col];
-    const uint32_t bar_id = 1u + uint32_t(cg);
+    for (int m = 0; m < NM; m++) t[m] = 4 * m + RG < nr ? alpha * Bs[(4 * m + RG) * BS + col] : T(0);
+    const uint32_t bar = 1u + 2u * uint32_t(cg);
 #pragma unroll
     for (int s = 0; s < NB; s++) {
-        const int k = FWD ? s : NB - 1 - s;
-        if (k < nr) {
-            if ((k & 3) == RG) {
-                const T x = t[k >> 2] * inv[k];
-                t[k >> 2] = x;
-                Bs[k * BS + col] = x;
+        const int k = FWD ? s : NB - 1 - s, kn = FWD ? k + 1 : k - 1;
+        T x;
+        if ((k & 3) == RG) {
+            if (s == 0) {
+                t[k >> 2] *= inv[k];
+                Bs[k * BS + col] = t[k >> 2];
+                asm volatile("bar.arrive %0, 128;" ::"r"(bar + uint32_t(k & 1)) : "memory");
             }
-            asm volatile("bar.sync %0, 128;" ::"r"(bar_id) : "memory");
-            const T x = Bs[k * BS + col];
+            x = t[k >> 2];
+        } else {
+            asm volatile("bar.sync %0, 128;" ::"r"(bar + uint32_t(k & 1)) : "memory");
+            x = Bs[k * BS + col];
+        }
 #pragma unroll
-            for (int m = 0; m < NM; m++) {
-                const int i = 4 * m + RG;
-                if (FWD ? (i > k) : (i < k)) t[m] -= (MT ? L[i * NB + k] : L[k * NB + i]) * x;
+        for (int m = 0; m < NM; m++)
+            if (4 * m + RG == kn) {
+                t[m] -= (MT ? L[kn * NB + k] : L[k * NB + kn]) * x;
+                t[m] *= inv[kn];
+                Bs[kn * BS + col] = t[m];
+                asm volatile("bar.arrive %0, 128;" ::"r"(bar + uint32_t(kn & 1)) : "memory");
             }
+#pragma unroll
+        for (int m = 0; m < NM; m++) {
+            const int i = 4 * m + RG;
+            if ((FWD ? (i > k) : (i < k)) && i != kn) t[m] -= (MT ? L[i * NB + k] : L[k * NB + i]) * x;
         }
     }
 }
@@ -93,7 +110,7 @@ __device__ __forceinline__ void diag_rows(const T *L, const T *inv, T *Bs, int n
 // FWD: Mv lower (forward substitution); MT: Mv(i,j) = A(j,i); LEFT: Bv
 // column-major.  Msub = &A(r0, r0), Bsub = &Bv(r0, 0).
 template <typename T, int NB, bool FWD, bool MT, bool LEFT, int CW>
-__global__ void __launch_bounds__(kDiagThreads)
+__global__ void __launch_bounds__(kDiagThreads<CW>)
 diag_solve_kernel(const T *__restrict__ Msub, int64_t lda, T *__restrict__ Bsub,
                   int64_t ldb, int nr, int64_t ncols, T alpha, int unit)
 {
@@ -115,7 +132,7 @@ diag_solve_kernel(const T *__restrict__ Msub, int64_t lda, T *__restrict__ Bsub,
     // column-major; Mv(i,k) = MT ? A(k,i) : A(i,k).  The loop index runs
     // fastest over A's contiguous dimension; entries outside the referenced
     // strict triangle are zero-filled.
-    for (int idx = tid; idx < NB * NB; idx += kDiagThreads) {
+    for (int idx = tid; idx < NB * NB; idx += kDiagThreads<CW>) {
         int fast = idx % NB, slow = idx / NB;  // fast = row of A, slow = col of A
         int i = MT ? slow : fast;              // row of Mv
         int k = MT ? fast : slow;              // col of Mv
@@ -125,20 +142,20 @@ diag_solve_kernel(const T *__restrict__ Msub, int64_t lda, T *__restrict__ Bsub,
     }
     // B panel, coalesced
     if (LEFT) {  // Bv(i,c) = Bsub[i + c*ldb]: contiguous in i
-        for (int idx = tid; idx < NB * CW; idx += kDiagThreads) {
+        for (int idx = tid; idx < NB * CW; idx += kDiagThreads<CW>) {
             int i = idx % NB, c = idx / NB;
             const bool in = i < nr && c < ncb;
             diag_cp_async(&Bs[i * BS + c], in ? Bsub + i + (c0 + c) * ldb : Bsub, in);
         }
     } else {     // Bv(i,c) = Bsub[c + i*ldb]: contiguous in c
-        for (int idx = tid; idx < NB * CW; idx += kDiagThreads) {
+        for (int idx = tid; idx < NB * CW; idx += kDiagThreads<CW>) {
             int c = idx % CW, i = idx / CW;
             const bool in = i < nr && c < ncb;
             diag_cp_async(&Bs[i * BS + c], in ? Bsub + (c0 + c) + int64_t(i) * ldb : Bsub, in);
         }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
-    for (int i = tid; i < NB; i += kDiagThreads) {
+    for (int i = tid; i < NB; i += kDiagThreads<CW>) {
         T d = T(1);
         if (i < nr && !unit) d = T(1) / Msub[i + int64_t(i) * lda];
         inv[i] = d;
@@ -167,12 +184,12 @@ diag_solve_kernel(const T *__restrict__ Msub, int64_t lda, T *__restrict__ Bsub,
 
     // ---- write back, coalesced --------------------------------------------
     if (LEFT) {
-        for (int idx = tid; idx < NB * CW; idx += kDiagThreads) {
+        for (int idx = tid; idx < NB * CW; idx += kDiagThreads<CW>) {
             int i = idx % NB, c = idx / NB;
             if (i < nr && c < ncb) Bsub[i + (c0 + c) * ldb] = Bs[i * BS + c];
         }
     } else {
-        for (int idx = tid; idx < NB * CW; idx += kDiagThreads) {
+        for (int idx = tid; idx < NB * CW; idx += kDiagThreads<CW>) {
             int c = idx % CW, i = idx / CW;
             if (i < nr && c < ncb) Bsub[(c0 + c) + int64_t(i) * ldb] = Bs[i * BS + c];
         }
@@ -201,7 +218,7 @@ int launch_nb_cw(const T *Msub, int64_t lda, T *Bsub, int64_t ldb, int nr, int64
     if (grid > 0x7fffffff) return GB_STATUS_CUDA_ERROR;
     LaunchScope ls(KK_DIAG, s, double(nr) * nr * ncols,
                    sizeof(T) * (0.5 * nr * nr + 2.0 * nr * ncols));
-    return check(launch_pdl(kern, dim3((unsigned)grid), dim3(kDiagThreads), smem, s, Msub, lda, Bsub, ldb, nr, ncols, alpha,
+    return check(launch_pdl(kern, dim3((unsigned)grid), dim3(kDiagThreads<CW>), smem, s, Msub, lda, Bsub, ldb, nr, ncols, alpha,
                             unit));
 }
 
@@ -209,6 +226,7 @@ template <typename T, int NB, bool FWD, bool MT, bool LEFT>
 int launch_nb(const T *Msub, int64_t lda, T *Bsub, int64_t ldb, int nr, int64_t ncols,
               T alpha, int unit, cudaStream_t s)
 {
+    if (ncols <= 152 * 32) return launch_nb_cw<T, NB, FWD, MT, LEFT, 32>(Msub, lda, Bsub, ldb, nr, ncols, alpha, unit, s);
     return launch_nb_cw<T, NB, FWD, MT, LEFT, 64>(Msub, lda, Bsub, ldb, nr, ncols, alpha, unit, s);
 }
 
