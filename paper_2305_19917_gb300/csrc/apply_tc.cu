@@ -68,14 +68,18 @@ __device__ __forceinline__ void ld_cols(uint32_t a, uint32_t (&x)[16])
 // inverse's two terms arrive meanwhile, the ring then holds the split panel.
 // While a block's X is stored, the next block's FP32 panel, inverse and
 // first k-tiles (those not needing that X) are already on their way.
-// Thread 0 issues TMA, thread 32 the MMAs; all 8 warps do the subtraction,
+// Warp 0 issues TMA, warp 1 the MMAs; all 8 warps do the subtraction,
 // the split and the stores (warps w, w+4 share TMEM lanes 32(w%4).. and
 // split the columns).
 // A block's chain is bound by what one SM loads, converts and stores for it,
 // so PW is the narrowest panel whose CTAs still fit the SMs side by side: 32 up
 // to 4864 columns, 64 up to 9728, else 128.  Measured, time per 128-row block:
 // 9.6 us with 128 columns at any width; 6.3 with 32 (1500 x 700: low-precision
-// solve 115 -> 76 us; 32768 x 4096, whole BF16 solve 60.3 -> 56.9 ms).
+// solve 115 -> 76 us; 32768 x 4096, whole BF16 solve 60.3 -> 56.9 ms).  About half
+// of the chain is issuing MMAs (some 70 clocks each with 32 columns, 24 with the
+// inverse and four a k-tile): the issue loops in uniform registers took the
+// 1500 x 700 solve from 74 to 66 us.  X kept in shared memory as well, so that
+// it need not come back through the ring, gained 1 % on top.
 template <int PW>
 struct LeafCfg {
     static constexpr int LST = PW == 128 ? 3 : (PW == 64 ? 5 : 6);  // ring stages
@@ -132,7 +136,6 @@ leaf_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int r = q * 32 + lane;
     constexpr int CH = PW / 2 < 32 ? PW / 2 : 32;  // columns drained at a time
     uint32_t g = 0;  // ring position (k-tiles issued so far)
-    int pre = 0;     // thread 0: k-tiles of the current block issued during the previous one
 
     // the FP32 panel of Y_b (rows b0..), every copy in flight at once
     auto load_panel = [&](int b0) {
@@ -144,59 +147,73 @@ leaf_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    // thread 0: the inverse's two terms for block b0
+    // Warps 0 and 1 issue the loads and the MMAs with all lanes in the loops
+    // and no branch on a wait's result (after one that gave up nothing more is
+    // issued and every further wait returns at once), so that loop variables and
+    // descriptors stay in uniform registers; one lane issues.
+    // warp 0: the inverse's two terms for block b0
     auto load_inverse = [&](int b0) {
-        tc::mbar_arrive_expect_tx(&bar_l, 2 * OP_BYTES);
-        tc::tma_load_2d(&tmL, &bar_l, sLh, 0, b0);
-        tc::tma_load_2d(&tmL, &bar_l, sLh + HALF_BYTES, 64, b0);
-        tc::tma_load_2d(&tmL, &bar_l, sLl, 0, kp + b0);
-        tc::tma_load_2d(&tmL, &bar_l, sLl + HALF_BYTES, 64, kp + b0);
+        if (tc::elect_one()) {
+            tc::mbar_arrive_expect_tx(&bar_l, 2 * OP_BYTES);
+            tc::tma_load_2d(&tmL, &bar_l, sLh, 0, b0);
+            tc::tma_load_2d(&tmL, &bar_l, sLh + HALF_BYTES, 64, b0);
+            tc::tma_load_2d(&tmL, &bar_l, sLl, 0, kp + b0);
+            tc::tma_load_2d(&tmL, &bar_l, sLl + HALF_BYTES, 64, kp + b0);
+        }
     };
-    // thread 0: k-tile kt of the GEMM of block b0 into ring position gi
-    auto load_ktile = [&](uint32_t gi, int kt, int b0) -> bool {
+    // warp 0: k-tile kt of the GEMM of block b0 into ring position gi
+    auto load_ktile = [&](uint32_t gi, int kt, int b0) {
         const int st = int(gi % LST);
-        const uint32_t phs = (gi / LST) & 1u;
-        if (!tc::mbar_wait(&empty[st], phs ^ 1, ab, status, tc::TC_TIMEOUT_PRODUCER)) return false;
-        tc::mbar_arrive_expect_tx(&full[st], LSTAGE);
-        tc::tma_load_2d(&tmA, &full[st], ring + st * LSTAGE, s0 + kt * 64, b0);
-        tc::tma_load_2d(&tmX, &full[st], ring + st * LSTAGE + LA_BYTES, s0 + kt * 64, int(c0));
-        return true;
+        const bool go = tc::mbar_pass(&empty[st], ((gi / LST) & 1u) ^ 1, ab, status, tc::TC_TIMEOUT_PRODUCER);
+        if (tc::elect_one() && go) {
+            tc::mbar_arrive_expect_tx(&full[st], LSTAGE);
+            tc::tma_load_2d(&tmA, &full[st], ring + st * LSTAGE, s0 + kt * 64, b0);
+            tc::tma_load_2d(&tmX, &full[st], ring + st * LSTAGE + LA_BYTES, s0 + kt * 64, int(c0));
+        }
     };
+    const uint64_t dring = tc::desc_kmajor_sw128(tc::smem_u32(ring));
+    // warp 1: the products with k-tile kt, from ring position gi
+    auto mma_ktile = [&](uint32_t gi, int kt) {
+        constexpr uint32_t idesc = tc::idesc_bf16_f32(TB, PW);
+        const int st = int(gi % LST);
+        const bool go = tc::mbar_pass(&full[st], (gi / LST) & 1u, ab, status, tc::TC_TIMEOUT_MMA);
+        tc::tc_fence_after();
+        // descriptors in 16-byte units: a 32-byte K step adds 2
+        const uint64_t da = dring + uint64_t(uint32_t(st) * (LSTAGE >> 4));
+        const uint64_t dx = da + uint64_t(LA_BYTES >> 4);
+        if (tc::elect_one() && go) {
+            tc::mma_f16(tmem, da, dx, idesc, kt != 0);
+#pragma unroll
+            for (int kk = 1; kk < 4; kk++) tc::mma_f16(tmem, da + uint64_t(2 * kk), dx + uint64_t(2 * kk), idesc, 1);
+            tc::mma_commit(&empty[st]);
+        }
+    };
+    // k-tiles of a block (nk of them) loaded during the previous one: those that
+    // need no X of it
+    auto loaded_ahead = [&](int nk) { return min(LST, max(nk - TB / 64, 0)); };
     load_panel(s0);
-    if (tid == 0) {
-        tc::tma_prefetch_desc(&tmL);
+    if (warp == 0) {
+        if (lane == 0) tc::tma_prefetch_desc(&tmL);
         load_inverse(s0);
     }
 
     for (int blk = 0; blk < nblk; blk++) {
         const int b0 = s0 + blk * TB, nk = blk * (TB / 64);
         const uint32_t ph = uint32_t(blk) & 1u;
-        if (tid == 0) {
-            for (int kt = pre; kt < nk; kt++)
-                if (!load_ktile(g + uint32_t(kt), kt, b0)) break;
-        } else if (tid == 32) {
-            constexpr uint32_t idesc = tc::idesc_bf16_f32(TB, PW);
-            for (int kt = 0; kt < nk; kt++) {
-                const uint32_t gi = g + uint32_t(kt);
-                const int st = int(gi % LST);
-                const uint32_t phs = (gi / LST) & 1u;
-                if (!tc::mbar_wait(&full[st], phs, ab, status, tc::TC_TIMEOUT_MMA)) break;
-                tc::tc_fence_after();
-                // descriptors in 16-byte units: a 32-byte K step adds 2
-                const uint32_t a0 = tc::smem_u32(ring + st * LSTAGE);
-                const uint64_t da = tc::desc_kmajor_sw128(a0), dx = tc::desc_kmajor_sw128(a0 + LA_BYTES);
-                tc::mma_f16(tmem, da, dx, idesc, kt != 0);
-#pragma unroll
-                for (int kk = 1; kk < 4; kk++) tc::mma_f16(tmem, da + uint64_t(2 * kk), dx + uint64_t(2 * kk), idesc, 1);
-                tc::mma_commit(&empty[st]);
-            }
-            tc::mma_commit(&bar_g);  // also when nk == 0: arrives once the earlier MMAs are done
+        if (warp == 0) {
+            for (int kt = loaded_ahead(nk); kt < nk; kt++) load_ktile(g + uint32_t(kt), kt, b0);
+            __syncwarp();
+        } else if (warp == 1) {
+            for (int kt = 0; kt < nk; kt++) mma_ktile(g + uint32_t(kt), kt);
+            if (tc::elect_one()) tc::mma_commit(&bar_g);  // also when nk == 0: arrives once the earlier MMAs are done
+            __syncwarp();
         }
         g += uint32_t(nk);
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();
         // Y_b - L(b, s0:b0) X(s0:b0), in place in the panel
-        const bool ok_g = tc::mbar_wait(&bar_g, ph, ab, status, tc::TC_TIMEOUT_EPILOGUE);
+        // (one answer per warp: its lanes go on together)
+        const bool ok_g = __all_sync(0xffffffffu, tc::mbar_wait(&bar_g, ph, ab, status, tc::TC_TIMEOUT_EPILOGUE));
         if (ok_g && nk > 0) {
             tc::tc_fence_after();
 #pragma unroll 1
@@ -229,44 +246,40 @@ leaf_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
         if (blk + 1 < nblk) load_panel(b0 + TB);  // the panel is free again: the next block's
-        if (tid == 32) {
-            if (ok_g && tc::mbar_wait(&bar_l, ph, ab, status, tc::TC_TIMEOUT_MMA)) {
-                tc::tc_fence_after();
-                constexpr uint32_t idesc = tc::idesc_bf16_f32(TB, PW);
-                const uint8_t *As[3] = {sLh, sLh, sLl};
-                const uint8_t *Bs[3] = {sYh, sYl, sYh};
-                uint32_t acc = 0;
+        if (warp == 1) {
+            const bool go = ok_g && tc::mbar_pass(&bar_l, ph, ab, status, tc::TC_TIMEOUT_MMA);
+            tc::tc_fence_after();
+            constexpr uint32_t idesc = tc::idesc_bf16_f32(TB, PW);
+            const uint64_t dLh = tc::desc_kmajor_sw128(tc::smem_u32(sLh)), dYh = tc::desc_kmajor_sw128(tc::smem_u32(sYh));
+            if (tc::elect_one()) {
+                if (go) {
 #pragma unroll
-                for (int pr = 0; pr < 3; pr++) {
-                    const uint64_t da = tc::desc_kmajor_sw128(tc::smem_u32(As[pr]));
-                    const uint64_t dy = tc::desc_kmajor_sw128(tc::smem_u32(Bs[pr]));
+                    for (int pr = 0; pr < 3; pr++) {  // Lh Yh, Lh Yl, Ll Yh
+                        const uint64_t da = dLh + uint64_t(pr == 2 ? OP_BYTES >> 4 : 0u);
+                        const uint64_t dy = dYh + uint64_t(pr == 1 ? Cfg::OPY_BYTES >> 4 : 0u);
 #pragma unroll
-                    for (int kk = 0; kk < TB / 16; kk++) {
-                        const uint64_t oa = uint64_t(((kk >> 2) * HALF_BYTES + (kk & 3) * 32u) >> 4);
-                        const uint64_t oy = uint64_t(((kk >> 2) * (PW * 128u) + (kk & 3) * 32u) >> 4);
-                        tc::mma_f16(tmem + PW, da + oa, dy + oy, idesc, acc);
-                        acc = 1;
+                        for (int kk = 0; kk < TB / 16; kk++) {
+                            const uint64_t oa = uint64_t(((kk >> 2) * HALF_BYTES + (kk & 3) * 32u) >> 4);
+                            const uint64_t oy = uint64_t(((kk >> 2) * (PW * 128u) + (kk & 3) * 32u) >> 4);
+                            tc::mma_f16(tmem + PW, da + oa, dy + oy, idesc, pr + kk > 0);
+                        }
                     }
                 }
+                tc::mma_commit(&bar_x);
             }
-            tc::mma_commit(&bar_x);
+            __syncwarp();
         }
-        const bool ok_x = tc::mbar_wait(&bar_x, ph, ab, status, tc::TC_TIMEOUT_EPILOGUE);
-        pre = 0;
-        if (ok_x && tid == 0 && blk + 1 < nblk) {
+        const bool ok_x = __all_sync(0xffffffffu, tc::mbar_wait(&bar_x, ph, ab, status, tc::TC_TIMEOUT_EPILOGUE));
+        if (warp == 0 && ok_x && blk + 1 < nblk) {
             // the split panel and the inverse are consumed: the next block's
             // inverse, and its first k-tiles that do not need this block's X
             // (rows below b0), go out while this block's X is stored
             load_inverse(b0 + TB);
-            const int nkn = (blk + 1) * (TB / 64);
-            pre = min(LST, nkn - TB / 64);
-            for (int kt = 0; kt < pre; kt++)
-                if (!load_ktile(g + uint32_t(kt), kt, b0 + TB)) {
-                    pre = nkn;  // stop issuing: the wait has timed out and set the abort flag
-                    break;
-                }
+            const int nkn = nk + TB / 64;
+            for (int kt = 0; kt < loaded_ahead(nkn); kt++) load_ktile(g + uint32_t(kt), kt, b0 + TB);
+            __syncwarp();
         }
-        if (ok_x && !*ab) {
+        if (__all_sync(0xffffffffu, ok_x && !*ab)) {
             tc::tc_fence_after();
 #pragma unroll 1
             for (int cc = half * (PW / 2); cc < (half + 1) * (PW / 2); cc += CH) {
