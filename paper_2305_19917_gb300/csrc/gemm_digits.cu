@@ -87,6 +87,10 @@ struct Fmt<float> {
     __device__ static int field(float a) { return int((__float_as_uint(a) >> 23) & 0xFF); }
 };
 
+// a != 0 by its bits (a comparison of FP64 values takes 66 clocks of that unit).
+__device__ __forceinline__ bool nonzero(double a) { return ((__double2hiint(a) << 1) | __double2loint(a)) != 0; }
+__device__ __forceinline__ bool nonzero(float a) { return (__float_as_uint(a) << 1) != 0u; }
+
 // Digits of a (exponent field of the row's largest entry: emax), most
 // significant first, as the bit patterns of exact FP32 integers.
 // e' = emax - BIAS + 1: |a| < 2^e', N = round(a 2^(8P - e')).
@@ -155,8 +159,11 @@ struct DigitSrc {
     int *cnt;             // entries within 2^-kNear of the largest; kCntBad; >= 2K for a zero or padding row
 };
 
-// cp.async-free: what bounds this kernel is the latency of its loads (8 per
-// thread in flight) and the integer work of the digits.  A CTA takes 32 rows
+// What bounds this kernel is the integer work of the digits (about half the
+// issue slots) and the latency of its loads.  The next tile's loads go out before
+// this one's digits are formed, and zeros are told by integer operations: the
+// factors of 4096 x 8192 x 4096 take 362 us in FP64 (411 before; 165 at the HBM
+// rate), 181 in FP32 (206).  A CTA takes 32 rows
 // and a share of K; the CTAs of one row block form a cluster along K (so that
 // a few rows of a long K still fill the chip) and exchange the rows' largest
 // exponents and counts through distributed shared memory.  The second read of
@@ -166,7 +173,7 @@ __global__ void __launch_bounds__(DTHREADS, sizeof(T) == 8 ? 3 : 4)
 digits_kernel(DigitSrc<T> a, DigitSrc<T> x, int ablocks, int K, int kp, int *zero, int nzero, ulonglong2 *sums, int64_t nsums)
 {
     constexpr int P = Fmt<T>::P;
-    __shared__ T t[DROWS][65];
+    __shared__ T t[2][DROWS][65];
     __shared__ int key[DROWS];   // 2 * largest exponent field + (any nonzero entry)
     __shared__ int num[DROWS];
     __shared__ int emx[DROWS];
@@ -207,10 +214,11 @@ digits_kernel(DigitSrc<T> a, DigitSrc<T> x, int ablocks, int K, int kp, int *zer
 #pragma unroll
     for (int u = 0; u < 8; u++) mx[u] = 0;
     T v[8];
+#pragma unroll 2
     for (int tile = t0; tile < t1; tile++) {
         load(tile, v);
 #pragma unroll
-        for (int u = 0; u < 8; u++) mx[u] = max(mx[u], 2 * Fmt<T>::field(v[u]) + (v[u] != T(0) ? 1 : 0));
+        for (int u = 0; u < 8; u++) mx[u] = max(mx[u], 2 * Fmt<T>::field(v[u]) + (nonzero(v[u]) ? 1 : 0));
     }
     if (s.kc) {  // a warp's lanes share the rows (tid >> 6) + 4u
 #pragma unroll
@@ -246,24 +254,26 @@ digits_kernel(DigitSrc<T> a, DigitSrc<T> x, int ablocks, int K, int kp, int *zer
     const int em = emx[row] >> 1;
     int near = 0;
     const size_t plane = size_t(s.rp) * size_t(kp);
-    for (int tile = t0; tile < t1; tile++) {
-        if (t1 - t0 > 1) load(tile, v);  // (a single tile is still in registers)
-        __syncthreads();  // the previous tile has been read
+    // (backwards: the last tile is still in registers; the next one's loads go
+    // out before the digits of this one are formed)
+    for (int tile = t1 - 1; tile >= t0; tile--) {
+        T(*tb)[65] = t[tile & 1];
 #pragma unroll
         for (int u = 0; u < 8; u++) {
             const int r = s.kc ? (tid >> 6) + 4 * u : (tid & 31);
             const int k = s.kc ? (tid & 63) : (tid >> 5) + 8 * u;
-            t[r][k] = v[u];
+            tb[r][k] = v[u];
         }
+        if (tile > t0) load(tile - 1, v);
         __syncthreads();
         uint32_t w[P][4];
 #pragma unroll
         for (int u = 0; u < 8; u += 2) {
             uint32_t d0[P], d1[P];
-            const T a0 = t[row][lk + u], a1 = t[row][lk + u + 1];
+            const T a0 = tb[row][lk + u], a1 = tb[row][lk + u + 1];
             digits_of(a0, em, d0);
             digits_of(a1, em, d1);
-            near += (Fmt<T>::field(a0) + kNear >= em && a0 != T(0)) + (Fmt<T>::field(a1) + kNear >= em && a1 != T(0));
+            near += (Fmt<T>::field(a0) + kNear >= em && nonzero(a0)) + (Fmt<T>::field(a1) + kNear >= em && nonzero(a1));
 #pragma unroll
             for (int p = 0; p < P; p++) w[p][u >> 1] = pack_hi16(d0[p], d1[p]);
         }
@@ -408,7 +418,7 @@ __device__ __forceinline__ uint32_t biased_int(float S)
 // Warp 0 issues the TMA loads, warp 1 the MMAs, warps 2-17 drain the
 // accumulators and finish C.  What bounds it: the tensor cores (28 x 2 flop
 // per multiply-add of the product; over an 8192 x 8192 solve 1160 TFLOP/s in FP64,
-// 1010 in FP32, 4096^2 x 8192 alone about 1700), fed with 48 KB of digits per 512 clocks;
+// 1010 in FP32, 4096 x 8192 x 4096 alone 1650 and 1260), fed with 48 KB of digits per 512 clocks;
 // the drains (12 half accumulators per 28.7k clocks of MMAs) go on beside them.
 // Sixteen drain warps hide the latencies of the accumulators' loads.
 // Issuing is close to the bound too: with the loops of warps 0 and 1 in a branch
@@ -975,13 +985,13 @@ void digit_pool_trim()
     if (pool) cudaMemPoolTrimTo(pool, 0);
 }
 
-// FP64: from K = 64 on at every M and N: measured, 64 x 32 x 64 takes 40 us
-// (CUDA cores 74), 64 x 256 x 512 82 (531), 2048 x 8192 x 64 0.22 ms (1.79),
-// 2048 x 8192 x 2048 1.7 ms (55).  FP32: from K = 128, where the digits'
+// FP64: from K = 64 on at every M and N: measured, 64 x 32 x 64 takes 37 us
+// (CUDA cores 74), 64 x 256 x 512 42 (531), 2048 x 8192 x 64 0.20 ms (1.79),
+// 2048 x 8192 x 2048 1.36 ms (55).  FP32: from K = 128, where the digits'
 // rounding (1.7e-7 of a normally distributed sum) falls below that of the
 // CUDA-core sum (2.1e-7; at K = 64 it would be above), and from 64 x 256
 // outputs, where they are the faster ones: 64 x 256 x 128 30 us (36), 512 x
-// 8192 x 128 44 (94), 2048 x 8192 x 2048 0.56 ms (2.6).
+// 8192 x 128 42 (94), 2048 x 8192 x 2048 0.45 ms (2.6).
 template <typename T>
 bool digit_gemm_wanted(int64_t M, int64_t N, int64_t K, int)
 {
