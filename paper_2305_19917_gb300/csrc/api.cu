@@ -40,8 +40,8 @@ int side_stream(cudaStream_t *out)
 // per right-hand side, FP64 252 per clock on the whole chip, FP32 about 10000)
 // take longer than the digit gemm that would replace them (50 and 30 us at
 // these sizes).  FP64 beyond 2432 right-hand sides: the 64-row diagonal kernel
-// (512 rows: 2400 right-hand sides 504 us with panels, 607 with it; 4096 962
-// with panels of 16, 646 with it).
+// (4096 rows: 1300 right-hand sides 4.5 ms with panels, 4.7 with it, 2400 4.84 and
+// 4.90; beyond, panels of eight columns need a third round of CTAs).
 template <typename T>
 int64_t ts_rows(int64_t ncols)
 {

@@ -27,8 +27,8 @@
 // Mv through a ring of asynchronous copies, packed multiply-adds
 // (wide_tile.cuh); two CTAs of four warps fill an SM's shared memory, and the
 // latencies that eight warps leave open are the time.  Measured, 4096 uneven
-// instances (m log-uniform in [16, 512], n in [1, 256]): FP64 22.2 -> 16.4 ms
-// (the FP64 unit 89 % busy; 12.9 ms at its peak), FP32 1.79 -> 1.19 ms.
+// instances (m log-uniform in [16, 512], n in [1, 256]): FP64 22.2 -> 16.6 ms
+// (the FP64 unit 89 % busy; 12.9 ms at its peak), FP32 1.80 -> 1.2-1.3 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
