@@ -19,7 +19,8 @@
 //     the largest product).  K advances in chunks of 256, over which every
 //     sum of one weight p + q stays an exact integer of at most 2^24 in the
 //     FP32 accumulators; so all pairs of one weight share an accumulator
-//     (FP64: 28 pairs in 12 accumulators, six passes over the chunk), and
+//     (FP64: 28 pairs in 12 accumulators, six passes over the chunk; in seven,
+//     four passes, where a CTA's share of K is at most 128), and
 //     the chunk's sums are added into int64 sums T = sum 2^(W-8(p+q)) S_pq.
 //     The two lowest weights of FP64 (2^-56, 2^-64 of the product) are scaled
 //     and rounded before they are added; W is the largest weight for which T
@@ -45,6 +46,7 @@
 // CUDA-core tile of gemm_tile.cuh: the operations of gemm_simt.cu.  So is a
 // tile whose bounded waits gave up.
 #include <mutex>
+#include <type_traits>
 #include <cuda_bf16.h>
 #include "common.cuh"
 #include "fixed.cuh"
@@ -301,25 +303,44 @@ digits_kernel(DigitSrc<T> a, DigitSrc<T> x, int ablocks, int K, int kp, int *zer
 // ---- pass 2: digit products ----------------------------------------------------
 
 // The schedule of a chunk: products in order, grouped into passes (pass j:
-// weight j + 2 in the low half of the accumulator, j + 3 in the high half).
-// Product o takes A slice p(o) (0-based) with X slices q(o) and q(o) + 1 into
-// both halves (o < TWO), or with X slice q(o) alone into the high half.
+// weight base(j) in the low half of the accumulator, base(j) + 1 in the high
+// half).  Product o takes A slice p(o) (0-based) with X slices q(o) and q(o) + 1
+// into both halves (two(o)), or with X slice q(o) alone into the high half.
+//
+// Full: every sum of a half stays within 2^24 over K = 256 (the last weight's
+// within 2^25.2).  Thin, for shares of at most 128 of K: there all pairs of a
+// weight fit one half, so that four passes are drained instead of six.  It
+// matters where the drains are the chain: 64 x 8192 x 64 24.5 us instead of 28.5,
+// 128 x 8192 x 128 31 instead of 35.
 template <typename T>
 struct Sched;
 template <>
-struct Sched<double> {  // (p, q): (0,0) | (1,0) | (0,2) (2,0) | (1,2) (3,0) | (0,4) (2,2) (4,0) |
-                        // (1,4) (3,2) (5,0) and alone (0,6) (2,4) (4,2) (6,0)
-    static constexpr int NP = 6, NO = 16, TWO = 12;
-    __device__ static int p(int o) { return int(0x6420531420312010ull >> (4 * o)) & 15; }
-    __device__ static int q(int o) { return int(0x0246024024020200ull >> (4 * o)) & 15; }
-    __device__ static int first(int j) { return int(0x10090604020100ull >> (8 * j)) & 255; }
+struct Sched<double> {
+    static constexpr int THIN_K = 128;
+    // full, (p, q): (0,0) | (1,0) | (0,2) (2,0) | (1,2) (3,0) | (0,4) (2,2) (4,0) |
+    //               (1,4) (3,2) (5,0) and alone (0,6) (2,4) (4,2) (6,0)
+    // thin: (0,0) alone (1,0) | (0,2) (1,1) (2,0) alone (3,0) | (0,4) .. (4,0) alone (5,0) | alone (0,6) .. (6,0)
+    __device__ static int passes(bool thin) { return thin ? 4 : 6; }
+    __device__ static int first(int j, bool thin) { return int((thin ? 0x130c060200ull : 0x10090604020100ull) >> (8 * j)) & 255; }
+    __device__ static int base(int j, bool thin) { return thin ? min(2 + 2 * j, 7) : j + 2; }
+    __device__ static bool low(int j, bool thin) { return !thin || j < 3; }  // the low half is used
+    __device__ static bool two(int o, bool thin) { return thin ? (0x7DD >> o) & 1 : o < 12; }
+    __device__ static int p(int o, int j, bool thin) { return thin ? o - first(j, true) : int(0x6420531420312010ull >> (4 * o)) & 15; }
+    __device__ static int q(int o, int j, bool thin)
+    {
+        return thin ? base(j, true) - (two(o, true) ? 2 : 1) - p(o, j, true) : int(0x0246024024020200ull >> (4 * o)) & 15;
+    }
 };
 template <>
 struct Sched<float> {  // (0,0) | (1,0) and alone (0,2) (2,0)
-    static constexpr int NP = 2, NO = 4, TWO = 2;
-    __device__ static int p(int o) { return (0x2010 >> (4 * o)) & 15; }
-    __device__ static int q(int o) { return (0x0200 >> (4 * o)) & 15; }
-    __device__ static int first(int j) { return (0x040100 >> (8 * j)) & 255; }
+    static constexpr int THIN_K = 0;
+    __device__ static int passes(bool) { return 2; }
+    __device__ static int first(int j, bool) { return (0x040100 >> (8 * j)) & 255; }
+    __device__ static int base(int j, bool) { return j + 2; }
+    __device__ static bool low(int, bool) { return true; }
+    __device__ static bool two(int o, bool) { return o < 2; }
+    __device__ static int p(int o, int, bool) { return (0x2010 >> (4 * o)) & 15; }
+    __device__ static int q(int o, int, bool) { return (0x0200 >> (4 * o)) & 15; }
 };
 
 // The tiles' words, cleared by pass 1: [0] number of listed tiles, then per
@@ -374,6 +395,7 @@ __device__ __forceinline__ float scale_sum(float, long long t, int e)
 struct Item {
     int tile, i0, j0, sp, k0, k1;
     bool skip;  // the digits may not represent this tile
+    bool thin;  // schedule
 };
 // Evaluated by every warp for itself (all lanes).
 template <typename T>
@@ -389,6 +411,7 @@ __device__ __forceinline__ Item digit_item(const MmaArgs<T> &a, int w, int lane)
     const int kt = a.kp / BK, per = (kt + a.split - 1) / a.split;
     it.k0 = min(it.sp * per, kt) * BK;
     it.k1 = min(it.k0 + per * BK, a.kp);
+    it.thin = it.k1 - it.k0 <= Sched<T>::THIN_K;
     const int4 ca = reinterpret_cast<const int4 *>(a.cnt_a + it.i0)[lane];
     const int4 cx = reinterpret_cast<const int4 *>(a.cnt_x + it.j0)[lane];
     const int ma = __reduce_min_sync(0xffffffffu, min(min(ca.x, ca.y), min(ca.z, ca.w)));
@@ -479,15 +502,14 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         // compiler can tell, and addresses and descriptors stay in uniform
         // registers.)
         int n = 0;
-        for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
-            const Item it = digit_item(a, w, lane);
-            if (it.skip) continue;
-            for (int kb = it.k0; kb < it.k1; kb += KC) {
-                const int ke = min(kb + KC, it.k1);
+        auto chunk = [&](auto thin, const Item &it, int kb, int ke) {
+            constexpr bool TH = decltype(thin)::value;
 #pragma unroll 1
-                for (int o = 0; o < S::NO; o++) {
-                    const int p = S::p(o), q = S::q(o);
-                    const bool two = o < S::TWO;
+            for (int j = 0; j < S::passes(TH); j++) {
+                const int o1 = S::first(j + 1, TH);
+                for (int o = S::first(j, TH); o < o1; o++) {
+                    const int p = S::p(o, j, TH), q = S::q(o, j, TH);
+                    const bool two = S::two(o, TH);
                     for (int kk = kb; kk < ke; kk += BK, n++) {
                         const int s = n % STAGES;
                         const bool go = tc::mbar_pass(&empty[s], ((n / STAGES) & 1) ^ 1, ab, a.status, tc::TC_TIMEOUT_PRODUCER);
@@ -501,6 +523,13 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     }
                 }
             }
+        };
+        for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
+            const Item it = digit_item(a, w, lane);
+            if (it.skip) continue;
+            if (S::THIN_K && it.thin) chunk(std::true_type(), it, it.k0, it.k1);
+            else
+                for (int kb = it.k0; kb < it.k1; kb += KC) chunk(std::false_type(), it, kb, min(kb + KC, it.k1));
         }
         __syncwarp();
         if (lane == 0) {
@@ -524,42 +553,45 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const uint64_t d0 = tc::desc_kmajor_sw128(tc::smem_u32(base));
         const uint32_t idesc256 = tc::idesc_bf16_f32(BM, 256), idesc128 = tc::idesc_bf16_f32(BM, 128);
         int n = 0, cp = 0;
+        auto chunk = [&](auto thin, int nk) {
+            constexpr bool TH = decltype(thin)::value;
+#pragma unroll 1
+            for (int j = 0; j < S::passes(TH); j++, cp++) {
+                const int buf = cp & 1;
+                tc::mbar_pass(&acce[buf], ((cp >> 1) & 1) ^ 1, ab, a.status, tc::TC_TIMEOUT_MMA);
+                tc::tc_fence_after();
+                const uint32_t acc = tmem + uint32_t(buf * 256);
+                const int o0 = S::first(j, TH), o1 = S::first(j + 1, TH);
+                for (int o = o0; o < o1; o++) {
+                    const bool two = S::two(o, TH);
+                    const uint32_t d = two ? acc : acc + 128u;
+                    const uint32_t idesc = two ? idesc256 : idesc128;
+                    for (int kt = 0; kt < nk; kt++, n++) {
+                        const int s = n % STAGES;
+                        const bool go = tc::mbar_pass(&full[s], (n / STAGES) & 1, ab, a.status, tc::TC_TIMEOUT_MMA);
+                        tc::tc_fence_after();
+                        // the start address field counts 16-byte units: a
+                        // 32-byte step along K adds 2
+                        const uint64_t da = d0 + uint64_t(uint32_t(s) * (STAGE_BYTES >> 4));
+                        const uint64_t db = da + uint64_t(TILE_BYTES >> 4);
+                        if (tc::elect_one() && go) {
+                            tc::mma_f16(d, da, db, idesc, o != o0 || kt != 0);
+#pragma unroll
+                            for (int kk = 1; kk < BK / 16; kk++)
+                                tc::mma_f16(d, da + uint64_t(2 * kk), db + uint64_t(2 * kk), idesc, 1);
+                            tc::mma_commit(&empty[s]);
+                        }
+                    }
+                }
+                if (tc::elect_one()) tc::mma_commit(&accf[buf]);
+            }
+        };
         for (int w = blockIdx.x; w < nitems; w += gridDim.x) {
             const Item it = digit_item(a, w, lane);
             if (it.skip) continue;
-            for (int kb = it.k0; kb < it.k1; kb += KC) {
-                const int nk = (min(kb + KC, it.k1) - kb) / BK;
-#pragma unroll 1
-                for (int j = 0; j < S::NP; j++, cp++) {
-                    const int buf = cp & 1;
-                    tc::mbar_pass(&acce[buf], ((cp >> 1) & 1) ^ 1, ab, a.status, tc::TC_TIMEOUT_MMA);
-                    tc::tc_fence_after();
-                    const uint32_t acc = tmem + uint32_t(buf * 256);
-                    const int o0 = S::first(j), o1 = S::first(j + 1);
-                    for (int o = o0; o < o1; o++) {
-                        const bool two = o < S::TWO;
-                        const uint32_t d = two ? acc : acc + 128u;
-                        const uint32_t idesc = two ? idesc256 : idesc128;
-                        for (int kt = 0; kt < nk; kt++, n++) {
-                            const int s = n % STAGES;
-                            const bool go = tc::mbar_pass(&full[s], (n / STAGES) & 1, ab, a.status, tc::TC_TIMEOUT_MMA);
-                            tc::tc_fence_after();
-                            // the start address field counts 16-byte units: a
-                            // 32-byte step along K adds 2
-                            const uint64_t da = d0 + uint64_t(uint32_t(s) * (STAGE_BYTES >> 4));
-                            const uint64_t db = da + uint64_t(TILE_BYTES >> 4);
-                            if (tc::elect_one() && go) {
-                                tc::mma_f16(d, da, db, idesc, o != o0 || kt != 0);
-#pragma unroll
-                                for (int kk = 1; kk < BK / 16; kk++)
-                                    tc::mma_f16(d, da + uint64_t(2 * kk), db + uint64_t(2 * kk), idesc, 1);
-                                tc::mma_commit(&empty[s]);
-                            }
-                        }
-                    }
-                    if (tc::elect_one()) tc::mma_commit(&accf[buf]);
-                }
-            }
+            if (S::THIN_K && it.thin) chunk(std::true_type(), (it.k1 - it.k0) / BK);
+            else
+                for (int kb = it.k0; kb < it.k1; kb += KC) chunk(std::false_type(), (min(kb + KC, it.k1) - kb) / BK);
         }
         __syncwarp();
     } else {
@@ -580,13 +612,12 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             long long T64[32];
             {
                 unsigned long long bias = 0;
-#pragma unroll
-                for (int j = 0; j < S::NP; j++)
+                for (int j = 0; j < S::passes(it.thin); j++)
 #pragma unroll
                     for (int h = 0; h < 2; h++) {
-                        const int s = a.W - 8 * (j + 2 + h);
-                        if (s >= 0) bias += kIntBias << s;
-                        else if (h == 1) bias += kIntBias;
+                        const int s = a.W - 8 * (S::base(j, it.thin) + h);
+                        if (s < 0) bias += h ? kIntBias : 0;
+                        else if (h || S::low(j, it.thin)) bias += kIntBias << s;
                     }
                 bias *= (unsigned long long)((it.k1 - it.k0 + KC - 1) / KC);
 #pragma unroll
@@ -614,27 +645,29 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             };
             for (int kb = it.k0; kb < it.k1 && ok; kb += KC) {
 #pragma unroll 1
-                for (int j = 0; j < S::NP; j++, cp++) {
+                for (int j = 0; j < S::passes(it.thin); j++, cp++) {
                     const int buf = cp & 1;
                     ok = tc::mbar_wait(&accf[buf], (cp >> 1) & 1, ab, a.status, tc::TC_TIMEOUT_EPILOGUE);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     tc::tc_fence_after();
                     const uint32_t tb = lbase + uint32_t(buf * 256);
-                    const int s1 = a.W - 8 * (j + 2), s2 = s1 - 8;
-                    if (s1 >= 0) add_half(tb, s1);
+                    const int s1 = a.W - 8 * S::base(j, it.thin), s2 = s1 - 8;
+                    const bool low = S::low(j, it.thin);
+                    if (s1 >= 0 && low) add_half(tb, s1);
                     if (sizeof(T) == 4 || s2 >= 0) {
                         add_half(tb + 128, s2);
                     } else {
                         // a weight below the sums' last bit: scaled, and both
                         // halves rounded as one number when neither is above it
                         // (|S| 2^s2 <= 2^25-4: the sum stays within 2^22)
-                        const float m1 = s1 < 0 ? __int_as_float((127 + s1) << 23) : 0.f;
+                        const float m1 = s1 < 0 && low ? __int_as_float((127 + s1) << 23) : 0.f;
                         const float m2 = __int_as_float((127 + s2) << 23);
 #pragma unroll
                         for (int c0 = 0; c0 < 32; c0 += 8) {
                             uint32_t r1[8], r2[8];
-                            tc::tmem_ld8(tb + c0, r1);
+                            // (an unused low half may hold anything: the high one in its place, times 0)
+                            tc::tmem_ld8(low ? tb + c0 : tb + 128 + c0, r1);
                             tc::tmem_ld8(tb + 128 + c0, r2);
                             tc::tmem_ld_wait();
 #pragma unroll

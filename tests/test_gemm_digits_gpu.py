@@ -111,3 +111,19 @@ def test_what_digits_cannot_hold(dtype, change):
     u = 2.0 ** (-53 if dtype == 0 else -24)
     tiny = np.finfo(A.dtype).smallest_subnormal
     assert np.all(np.abs(got - want)[ok] <= K * (u * bound[ok] + tiny))
+
+
+@pytest.mark.parametrize("M,N,K", [(1700, 1500, 64), (1700, 1500, 128), (1700, 1500, 129), (1700, 1500, 300)])
+def test_schedules_by_share_of_k(M, N, K):
+    """Enough tiles that K is not split: up to 128 of it the schedule with one
+    accumulator per weight, from 129 the one for 256, with a last chunk of 44;
+    entries of one sign, so that the sums come near their bounds."""
+    A, B, C = _factors(0, M, N, K, seed=K)
+    A, B = 1 - np.abs(A) / 64, 1 - np.abs(B) / 64
+    got = _update(0, A, B, C, 1.0)
+    L = np.longdouble
+    rows, cols = np.r_[0:3, 126:131, M - 2:M], np.r_[0:2, 127:129, N - 2:N]
+    want = C[np.ix_(rows, cols)].astype(L) - A[rows].astype(L) @ B[:, cols].astype(L)
+    norms = np.linalg.norm(A[rows], axis=1)[:, None] * np.linalg.norm(B[:, cols], axis=0)[None, :]
+    u = 2.0 ** -53
+    assert np.all(np.abs(got[np.ix_(rows, cols)] - want) <= NORM[0] * norms + 2 * u * np.abs(want))
