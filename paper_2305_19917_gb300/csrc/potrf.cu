@@ -14,7 +14,7 @@
 // library's own TRSM, side Right, transposed).  So every column block meets
 // one TS task, on all its rows at once: splitting the matrix in 2 x 2 blocks
 // instead, with a TRSM of every order, ran 448 of them at n = 8192 instead of
-// 127.  n = 8192 FP64: 128 -> 28.5 ms by the panels and the tasks' digit gemms, 18.4
+// 127.  n = 8192 FP64: 128 -> 28.5 ms by the panels and the tasks' digit gemms, 18.0
 // with the leaf below and overlapped launches; n = 16384 62 ms (1.34 s before the digit gemms).  The upper form (A = U^T U) is the same with everything stored
 // transposed.  Only the named triangle of A is read and written.
 //
