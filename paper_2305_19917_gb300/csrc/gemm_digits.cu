@@ -49,6 +49,7 @@
 #include <type_traits>
 #include <cuda_bf16.h>
 #include "common.cuh"
+#include "digit_plan.cuh"
 #include "fixed.cuh"
 #include "gemm_digits.cuh"
 #include "gemm_tile.cuh"
@@ -56,9 +57,11 @@
 
 namespace gb {
 
+using namespace digits;
+
 namespace {
 
-constexpr int BM = 128, BK = 64, STAGES = 4;
+constexpr int STAGES = 4;
 constexpr int KC = 256;                        // K of one exact accumulation
 constexpr uint32_t TILE_BYTES = BM * BK * 2;   // one digit tile of 128 rows
 constexpr uint32_t STAGE_BYTES = 3 * TILE_BYTES;
@@ -379,10 +382,6 @@ __device__ __forceinline__ void digit_tile(int t, int nMt, int nNt, int tri, int
     }
     tc::raster_grouped(t, nMt, nNt, 8, m, n);
 }
-inline int64_t digit_tiles(int64_t nMt, int64_t nNt, int tri)
-{
-    return tri ? nNt * (nNt + 1) / 2 + (nMt - nNt) * nNt : nMt * nNt;
-}
 
 __device__ __forceinline__ double scale_sum(double, long long t, int e) { return scaled_i64_to_f64(t, e); }
 // |T| 2^e with a normal scale factor (EMAX bounds e): one rounding, of T
@@ -408,10 +407,12 @@ __device__ __forceinline__ Item digit_item(const MmaArgs<T> &a, int w, int lane)
     digit_tile(it.tile, a.nMt, a.nNt, a.g.tri, m, n);
     it.i0 = m * BM;
     it.j0 = n * BM;
-    const int kt = a.kp / BK, per = (kt + a.split - 1) / a.split;
-    it.k0 = min(it.sp * per, kt) * BK;
-    it.k1 = min(it.k0 + per * BK, a.kp);
-    it.thin = it.k1 - it.k0 <= Sched<T>::THIN_K;
+    share_range(a.kp / BK, a.split, it.sp, it.k0, it.k1);
+    it.k0 *= BK;
+    it.k1 *= BK;
+    // (an empty share, of which the host makes none, runs no pass in any warp:
+    // the other schedule's loops go over its chunks)
+    it.thin = it.k0 < it.k1 && it.k1 - it.k0 <= Sched<T>::THIN_K;
     const int4 ca = reinterpret_cast<const int4 *>(a.cnt_a + it.i0)[lane];
     const int4 cx = reinterpret_cast<const int4 *>(a.cnt_x + it.j0)[lane];
     const int ma = __reduce_min_sync(0xffffffffu, min(min(ca.x, ca.y), min(ca.z, ca.w)));
@@ -793,8 +794,6 @@ digit_fallback_kernel(DigitGemm<T> g, TileWords w, int nMt, int nNt)
 
 // ---- host ------------------------------------------------------------------------
 
-inline int64_t up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
-
 // SMs of the current device.
 inline int sm_count()
 {
@@ -804,58 +803,6 @@ inline int sm_count()
     int v = n.done[dev].load(std::memory_order_relaxed);
     if (!v && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) n.done[dev].store(v);
     return v > 0 ? v : 152;
-}
-
-// Largest piece of one launch sequence: the digits of both factors and the
-// sums stay within the work space's cap, K within 16384 (the sums' weight W).
-constexpr size_t kWsCap = size_t(2) << 30;
-constexpr int64_t kMaxK = 16384;
-
-struct Piece {
-    int64_t mc, nc, kc;  // extents of one piece (mc, nc multiples of 128 unless whole)
-    int split;
-    size_t bytes;
-};
-
-template <typename T>
-size_t piece_bytes(int64_t M, int64_t N, int64_t K, int tri, int split)
-{
-    constexpr int P = Fmt<T>::P;
-    const size_t mp = size_t(up(M, BM)), np = size_t(up(N, BM)), kp = size_t(up(K, BK));
-    const size_t nt = size_t(digit_tiles(int64_t(mp / BM), int64_t(np / BM), tri));
-    size_t b = 256 + 2 * P * mp * kp + (tri ? 0 : 2 * P * np * kp) + (split > 1 ? nt * BM * BM * 8 : 0);
-    b += 4 * (2 * mp + 2 * np) + 4 * (3 * nt + 2) + 8 * 256;
-    return b;
-}
-
-// K is split over CTAs, down to 64 of it each, while the tiles alone leave SMs
-// idle: 9 tiles of K = 512 on 72 CTAs instead of 9.
-inline int pick_split(int64_t ntiles, int64_t K)
-{
-    const int64_t kt = (K + BK - 1) / BK;
-    int64_t s = 152 / ntiles;
-    if (s > kt) s = kt;
-    if (s < 2) return 1;
-    const int64_t per = (kt + s - 1) / s;
-    return int((kt + per - 1) / per);
-}
-
-template <typename T>
-Piece plan_piece(int64_t M, int64_t N, int64_t K, int tri)
-{
-    Piece p;
-    p.kc = K < kMaxK ? K : kMaxK;
-    p.mc = M;
-    p.nc = N;
-    // halve the longer of the two extents until the piece fits (of a triangle, K)
-    while (!tri && piece_bytes<T>(p.mc, p.nc, p.kc, 0, 1) > kWsCap && (p.mc > 1024 || p.nc > 1024)) {
-        if (p.nc >= p.mc) p.nc = up((p.nc + 1) / 2, BM);
-        else p.mc = up((p.mc + 1) / 2, BM);
-    }
-    while (tri && piece_bytes<T>(M, N, p.kc, 1, 1) > kWsCap && p.kc > 1024) p.kc = up((p.kc + 1) / 2, BK);
-    p.split = pick_split(digit_tiles(up(p.mc, BM) / BM, up(p.nc, BM) / BM, tri), p.kc);
-    p.bytes = piece_bytes<T>(p.mc, p.nc, p.kc, tri, p.split);
-    return p;
 }
 
 template <typename T>
@@ -1035,28 +982,24 @@ bool digit_gemm_wanted(int64_t M, int64_t N, int64_t K, int)
 template <typename T>
 size_t digit_gemm_bytes(int64_t M, int64_t N, int64_t K, int tri)
 {
-    return plan_piece<T>(M, N, K, tri).bytes;
+    return plan_piece<Fmt<T>::P>(M, N, K, tri).bytes;
 }
 
 template <typename T>
 int launch_digit_gemm(const DigitGemm<T> &g, char *ws, size_t ws_bytes, cudaStream_t s)
 {
-    const Piece pc = plan_piece<T>(g.M, g.N, g.K, g.tri);
-    for (int64_t i = 0; i < g.M; i += pc.mc)
-        for (int64_t j = 0; j < g.N; j += pc.nc)
-            for (int64_t k = 0; k < g.K; k += pc.kc) {
-                DigitGemm<T> d = g;
-                d.M = g.M - i < pc.mc ? g.M - i : pc.mc;
-                d.N = g.N - j < pc.nc ? g.N - j : pc.nc;
-                d.K = g.K - k < pc.kc ? g.K - k : pc.kc;
-                d.A = g.am ? g.A + i + k * g.lda : g.A + k + i * g.lda;
-                d.B = g.bc ? g.B + k + j * g.ldb : g.B + j + k * g.ldb;
-                d.C = g.cl ? g.C + i + j * g.ldc : g.C + j + i * g.ldc;
-                if (k > 0) d.alpha = T(1);
-                // a ragged last piece needs no more than the full one
-                GB_TRY(digit_piece<T>(d, ws, ws_bytes, pc.split, s));
-            }
-    return 0;
+    const Piece pc = plan_piece<Fmt<T>::P>(g.M, g.N, g.K, g.tri);
+    return for_pieces(pc, g.M, g.N, g.K, g.tri, [&](int64_t i, int64_t j, int64_t k, int64_t m, int64_t n, int64_t kk, int split) {
+        DigitGemm<T> d = g;
+        d.M = m;
+        d.N = n;
+        d.K = kk;
+        d.A = g.am ? g.A + i + k * g.lda : g.A + k + i * g.lda;
+        d.B = g.bc ? g.B + k + j * g.ldb : g.B + j + k * g.ldb;
+        d.C = g.cl ? g.C + i + j * g.ldc : g.C + j + i * g.ldc;
+        if (k > 0) d.alpha = T(1);
+        return digit_piece<T>(d, ws, ws_bytes, split, s);
+    });
 }
 
 template bool digit_gemm_wanted<double>(int64_t, int64_t, int64_t, int);

@@ -127,3 +127,31 @@ def test_schedules_by_share_of_k(M, N, K):
     norms = np.linalg.norm(A[rows], axis=1)[:, None] * np.linalg.norm(B[:, cols], axis=0)[None, :]
     u = 2.0 ** -53
     assert np.all(np.abs(got[np.ix_(rows, cols)] - want) <= NORM[0] * norms + 2 * u * np.abs(want))
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+@pytest.mark.parametrize("M,N,K", [(70, 50, 17000), (512, 64, 17000), (40, 40, 16385)])
+def test_ragged_last_piece_of_k(M, N, K, dtype):
+    """K beyond one piece on few tiles: the last piece is split by its own K.
+    No wait runs out: those last two seconds, these updates a few hundred
+    microseconds."""
+    import torch
+    from paper_2305_19917_gb300 import api
+    A, B, C = _factors(dtype, M, N, K, seed=K)
+    dev = [api.to_device_colmajor(x, torch.float64 if dtype == 0 else torch.float32) for x in (A, B, C)]
+    t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    torch.cuda.synchronize()
+    for _ in range(2):  # the first call may load the kernels
+        t0.record()
+        st = api.gb_gemm_update(dtype, M, N, K, dev[0].data_ptr(), M, dev[1].data_ptr(), K, dev[2].data_ptr(), M, 1.0,
+                                torch.cuda.current_stream().cuda_stream)
+        t1.record()
+        torch.cuda.synchronize()
+        assert st == 0
+    assert t0.elapsed_time(t1) < 200.0
+    L = np.longdouble
+    want = C[:16].astype(L) - 2 * (A[:16].astype(L) @ B.astype(L))
+    norms = np.linalg.norm(A[:16].astype(L), axis=1)[:, None] * np.linalg.norm(B.astype(L), axis=0)[None, :]
+    u = 2.0 ** (-53 if dtype == 0 else -24)
+    err = np.abs(dev[2].cpu().numpy()[:16] - want)
+    assert np.all(err <= 2 * NORM[dtype] * norms * K / 4096 + 4 * u * (np.abs(want) + np.abs(C[:16])))
