@@ -682,11 +682,11 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     if (lane == 0) tc::mbar_arrive(&acce[buf]);
                 }
             }
-            // one answer for all sixteen warps (a bounded wait that gave up
-            // in one of them leaves the tile to the last pass)
-            asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS) : "memory");
-            ok = ok && *ab == 0;
-            asm volatile("bar.sync 1, %0;" ::"n"(32 * EPI_WARPS) : "memory");
+            // one answer for all sixteen warps (a bounded wait that gave up in
+            // any of them leaves the tile to the last pass): the barrier's own
+            // AND, since warps 0 and 1, which take no part in it, may set the
+            // flag while these read it
+            ok = tc::bar_and(1, 32 * EPI_WARPS, ok && *ab == 0);
             if (!ok) {
                 if (first && atomicExch(&a.w.listed[it.tile], 1) == 0) a.w.list[atomicAdd(a.w.count, 1)] = it.tile;
                 continue;
