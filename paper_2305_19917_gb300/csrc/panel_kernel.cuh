@@ -15,8 +15,11 @@
 // through a ring of asynchronous copies of its own), then solves its triangle
 // by substitution, one step per row, x broadcast from its lane.  Each x goes
 // to shared memory as soon as it is known and the next block row's warp takes
-// it from there at once: X starts out as a pattern that no computation
-// produces, and a reader polls the value itself.  So the critical chain is
+// it from there at once: X starts out as a pattern that stands for "not
+// known yet", and a reader polls the value itself.  The pattern is a NaN, and
+// FP64 arithmetic hands on the payload of a NaN in B or Mv: so one with this
+// payload is replaced by another before it can get into X (once per block row
+// where the triangle's entries are finite, else at every step).  So the critical chain is
 // the substitution alone, the updates go on beside it, and the warps never
 // meet at a barrier.
 //
@@ -42,19 +45,24 @@ struct PanelCfg;
 template <>
 struct PanelCfg<double> {
     static constexpr int NW = 4, LD = NB + 2;  // warps, row stride of a tile
-    static constexpr unsigned long long EMPTY = 0xFFF8DEADBEEF5A5Aull;  // X not known yet
+    static constexpr unsigned long long EMPTY = 0xFFF8DEADBEEF5A5Aull;  // X not known yet (a NaN)
     using Bits = unsigned long long;
     __device__ static Bits bits(double x) { return static_cast<Bits>(__double_as_longlong(x)); }
     __device__ static double from(Bits b) { return __longlong_as_double(static_cast<long long>(b)); }
+    // x, or another NaN where its payload is EMPTY's (of either sign: arithmetic
+    // may hand it on with the other one)
+    __device__ static double other(double x)
+    {
+        const int lo = __double2loint(x), hi = __double2hiint(x);
+        const bool is = lo == int(EMPTY & 0xFFFFFFFFu) && (hi & 0x7FFFFFFF) == int((EMPTY >> 32) & 0x7FFFFFFFu);
+        return __hiloint2double(hi, is ? lo ^ 1 : lo);
+    }
     __device__ static int field(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
 };
 template <>
 struct PanelCfg<float> {
     static constexpr int NW = 8, LD = NB + 4;
-    static constexpr unsigned EMPTY = 0xFFC5AD5Au;
-    using Bits = unsigned;
-    __device__ static Bits bits(float x) { return __float_as_uint(x); }
-    __device__ static float from(Bits b) { return __uint_as_float(b); }
+    __device__ static float other(float x) { return x; }
 };
 
 // Tiles in a warp's ring: two CTAs with their X share an SM.
@@ -204,7 +212,7 @@ panel_kernel(const T *__restrict__ M, int64_t lda, T *__restrict__ B, int64_t si
         bool scaled = false;
         if constexpr (sizeof(T) == 8) {
             // scaled rows: exponents within 2^+-400 of the diagonal's, the
-            // diagonal's within 2^+-400
+            // diagonal's within 2^+-400 (so no infinity or NaN)
             const int fd = C::field(diag);
             bool ok = fd > 623 && fd < 1423;
 #pragma unroll
@@ -263,7 +271,7 @@ panel_kernel(const T *__restrict__ M, int64_t lda, T *__restrict__ B, int64_t si
             }
         }
 #pragma unroll
-        for (int c = 0; c < CW; c++) t[c] = alpha * t[c] - acc[c];
+        for (int c = 0; c < CW; c++) t[c] = C::other(alpha * t[c] - acc[c]);
         // a reader that gave up (it cannot unless the device is broken) says
         // so in every row from there on
         if (gave_up) {
@@ -299,7 +307,7 @@ panel_kernel(const T *__restrict__ M, int64_t lda, T *__restrict__ B, int64_t si
                 const T d = __shfl_sync(0xffffffffu, inv, k);
                 T x[CW];
 #pragma unroll
-                for (int c = 0; c < CW; c++) x[c] = __shfl_sync(0xffffffffu, t[c], k) * d;
+                for (int c = 0; c < CW; c++) x[c] = C::other(__shfl_sync(0xffffffffu, t[c], k) * d);
                 if (lane == k) {
 #pragma unroll
                     for (int c = 0; c < CW; c++) *const_cast<volatile T *>(xb + k * CW + c) = x[c];

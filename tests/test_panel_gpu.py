@@ -66,3 +66,24 @@ def test_extreme_rows(form):
     if side == 1:
         A, B = np.asfortranarray(A.T), np.asfortranarray(B.T)
     _check(form, *B.shape, "f64", A, B)
+
+
+@pytest.mark.parametrize("cols", [3, 310, 610, 1220])
+@pytest.mark.parametrize("where", ["B", "diagonal", "triangle", "below"])
+def test_nan_of_any_payload(where, cols):
+    """FP64: a NaN in B reaches its own column from its row on, one in A every
+    column from its row on, and nothing else, whatever its payload; the word
+    that stands for an X not yet known is one of them."""
+    k = 100
+    A, B = inputs.make_problem(0, 0, 0, 0, k, cols, seed=7)
+    want, _ = gpu_solve(0, 0, 0, 0, 1.5, A, B)
+    at = {"B": (37, 1), "diagonal": (37, 37), "triangle": (37, 33), "below": (37, 3)}[where]
+    for word in (0xFFF8DEADBEEF5A5A, 0x7FF8DEADBEEF5A5A, 0xFFF0DEADBEEF5A5A, 0x7FF8000000000000):
+        An, Bn = A.copy(), B.copy()
+        (Bn if where == "B" else An)[at] = np.array([word], dtype=np.uint64).view(np.float64)[0]
+        X, _ = gpu_solve(0, 0, 0, 0, 1.5, An, Bn)
+        hit = (slice(37, None), slice(1, 2) if where == "B" else slice(None))
+        assert np.all(np.isnan(X[hit]))
+        X[hit] = want[hit]
+        # (a row with a NaN keeps its block from being scaled: rounding only)
+        assert np.all(np.isfinite(X)) and np.all(np.abs(X - want) <= 1e-13 * np.abs(want).max())
