@@ -98,9 +98,13 @@ typedef struct gb_plan {
  * The plan is picked by the planner (cost model if loaded, else the
  * built-in default).  Asynchronous.  Off-diagonal updates of 64 (FP64) / 128
  * (FP32) products per entry or more run on the tensor cores, by exact
- * products of 8-bit digits whose error is below that of the CUDA-core sum
- * (input for which it would not be is found on the device and taken by the
- * CUDA cores).  Their work space (14 (M + N) K bytes FP64, 6 (M + N) K FP32
+ * products of 8-bit digits of fixed-point factors (63 bits and a sign FP64,
+ * 31 FP32, each row and column to the scale of its largest entry).  Rows and
+ * columns of which too few entries are near their largest one, or whose
+ * exponents lie near the ends of the range, are found on the device and taken
+ * by the CUDA cores; on the others the update's root mean square error was
+ * measured at 0.02 to 0.8 of that of the CUDA-core sum, which rounds every
+ * step.  Their work space (16 (M + N) K bytes FP64, 8 (M + N) K FP32
  * for the largest update, at most about 2 GiB) is taken from and given back
  * to a stream-ordered pool of the library, which keeps up to 2.5 GiB
  * (gb_mixed_workspace_release returns it); while `stream` is being captured,

@@ -155,3 +155,97 @@ def test_ragged_last_piece_of_k(M, N, K, dtype):
     u = 2.0 ** (-53 if dtype == 0 else -24)
     err = np.abs(dev[2].cpu().numpy()[:16] - want)
     assert np.all(err <= 2 * NORM[dtype] * norms * K / 4096 + 4 * u * (np.abs(want) + np.abs(C[:16])))
+
+
+def _edge(kind, dtype, M, N, K, r):
+    """Factors that the digits take, near the edge of the rule for it: entries of
+    2^-5 to 2^-4 of the scales, and one entry near the scale per row ("spike"); all
+    but the least number of them 2^-12 smaller, at opposite places ("count"); as
+    large as the scale, against ones of 2^-30 ("big")."""
+    def small(*n):
+        return r.choice([-1.0, 1.0], n) * r.uniform(1 / 16, 1 / 8, n)
+
+    def large(*n):
+        return r.choice([-1.0, 1.0], n) * r.uniform(1, 2, n)
+    A, B = small(M, K), small(K, N)
+    rest = K - (K * (6 if dtype == 0 and K > 1024 else 5) // 8 + 2)
+    if kind == "spike":
+        A[:, 3] = B[7, :] = 1.9
+    elif kind == "count":
+        A[:, :rest] *= 2.0 ** -12
+        B[-rest:] *= 2.0 ** -12
+        A[:, 0] = B[-1, :] = 1.9
+    else:
+        A[:, :rest], A[:, -rest:] = large(M, rest), A[:, -rest:] * 2.0 ** -30
+        B[-rest:], B[:rest] = large(rest, N), B[:rest] * 2.0 ** -30
+    nt = np.float64 if dtype == 0 else np.float32
+    return A.astype(nt), B.astype(nt)
+
+
+@pytest.mark.parametrize("dtype,K", [(0, 64), (0, 200), (0, 1000), (0, 2500), (1, 128), (1, 500), (1, 2500)])
+@pytest.mark.parametrize("kind", ["spike", "count", "big"])
+def test_error_below_the_cuda_core_sum(kind, dtype, K):
+    """The claim itself, on what the rule lets pass: the root mean square error
+    over a tile's entries is at most that of the CUDA-core sum of the same
+    factors (the path taken while a stream is being captured)."""
+    import torch
+    from paper_2305_19917_gb300 import api
+    M = N = 130  # (FP32 takes digits from 16384 entries on)
+    A, B = _edge(kind, dtype, M, N, K, np.random.default_rng(K))
+    td = torch.float64 if dtype == 0 else torch.float32
+    a, b = api.to_device_colmajor(A, td), api.to_device_colmajor(B, td)
+    got = _update(dtype, A, B, np.zeros((M, N), A.dtype), 1.0)
+    c = torch.zeros(N, M, dtype=td, device="cuda").t()
+    s, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        st = api.gb_gemm_update(dtype, M, N, K, a.data_ptr(), M, b.data_ptr(), K, c.data_ptr(), M, 1.0, s.cuda_stream)
+    assert st == 0
+    graph.replay()
+    torch.cuda.synchronize()
+    L = np.longdouble
+    i, j = np.r_[0:20, 120:130], np.r_[0:10, 110:130]
+    want = -(A[i].astype(L) @ B[:, j].astype(L))
+    scale = np.abs(A[i]).astype(L) @ np.abs(B[:, j]).astype(L)
+    rms = [float(np.sqrt(np.mean(((x[np.ix_(i, j)] - want) / scale) ** 2))) for x in (got, c.cpu().numpy())]
+    assert not np.array_equal(got, c.cpu().numpy())  # the digits did take it
+    assert rms[0] <= rms[1], rms
+
+
+def test_weights_of_the_int64_sums():
+    """FP64: the sums' weight W follows the factors' 2-norms, from 50 for the
+    longest rows of large entries up to 62; one value too high would overflow.
+    Tolerance as for dense factors."""
+    seen = set()
+    for K in (64, 129, 300, 1000, 4000, 9000, 16384):
+        for f in (1.0, 0.5, 0.25, 0.125, 0.0625):
+            r = np.random.default_rng(int(K / f))
+            A, B = r.choice([-1.0, 1.0], (9, K)), r.choice([-1.0, 1.0], (K, 7))
+            A, B = A * r.uniform(1.9, 1.999, A.shape), B * r.uniform(1.9, 1.999, B.shape)
+            A[:, 1:] *= f
+            B[1:] *= f
+            n2 = [int(np.max(np.sum((np.round(np.abs(X) * 64) + 1) ** 2, axis=ax))) for X, ax in ((A, 1), (B, 0))]
+            seen.add(min(62, int(78.95 - 0.5 * np.log2(float(n2[0]) * n2[1]))))
+            got = _update(0, A, B, np.zeros((9, 7)), 1.0)
+            L = np.longdouble
+            want = -(A.astype(L) @ B.astype(L))
+            norms = np.linalg.norm(A, axis=1)[:, None] * np.linalg.norm(B, axis=0)[None, :]
+            assert np.all(np.abs(got - want) <= NORM[0] * norms + 2.0 ** -52 * np.abs(want)), (K, f)
+    assert seen == set(range(50, 63)), seen
+
+
+@pytest.mark.parametrize("dtype,K", [(0, 64), (0, 128), (0, 256), (0, 700), (1, 128), (1, 256), (1, 700)])
+def test_digits_at_their_bounds(dtype, K):
+    """All digits of all entries 127 (as far as the type's bits go) or all -128
+    but the first, every product of one sign: the accumulators reach their
+    bounds.  Tolerance: the last bits of T and the result's rounding."""
+    n = 6 if dtype == 0 else 3
+    up = sum(127 * 256.0 ** -(p + 1) for p in range(n))
+    dn = 127 * 256.0 ** -1 - sum(128 * 256.0 ** -(p + 1) for p in range(1, n))
+    nt = np.float64 if dtype == 0 else np.float32
+    for a, x in ((up, up), (up, dn), (dn, dn)):
+        A, B = np.full((130, K), 2 * a, nt), np.full((K, 130), 2 * x, nt)
+        assert A[0, 0] == 2 * a and B[0, 0] == 2 * x
+        got = _update(dtype, A, B, np.zeros((130, 130), nt), 1.0)
+        want = -np.longdouble(2 * a) * np.longdouble(2 * x) * K
+        u = 2.0 ** (-53 if dtype == 0 else -24)
+        assert np.all(np.abs(got - want) <= 1.01 * u * abs(want))
