@@ -64,7 +64,7 @@ size_t piece_bytes(int64_t M, int64_t N, int64_t K, int tri, int split)
     const size_t mp = size_t(up(M, BM)), np = size_t(up(N, BM)), kp = size_t(up(K, BK));
     const size_t nt = size_t(digit_tiles(int64_t(mp / BM), int64_t(np / BM), tri));
     size_t b = 256 + 2 * P * mp * kp + (tri ? 0 : 2 * P * np * kp) + (split > 1 ? nt * BM * BM * 8 : 0);
-    b += 4 * 3 * (mp + np) + 4 * (3 * nt + 2) + 10 * 256;
+    b += 4 * 3 * (mp + np) + 4 * (3 * nt + 3) + 10 * 256;
     return b;
 }
 

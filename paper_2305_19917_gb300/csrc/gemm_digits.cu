@@ -369,11 +369,12 @@ struct Sched<float> {
     __device__ static int p(int o, int j, bool) { return o - first(j, false); }
 };
 
-// The tiles' words, cleared by pass 1: [0] number of listed tiles, then per
+// The tiles' words, cleared by pass 1: number of listed tiles, how many parts of
+// them the last pass has handed out, then per
 // tile: partial sums stored (split > 1), listed or not, and the list; last the
 // bounded waits' status (nobody reads it: a tile whose wait gave up is listed).
 struct TileWords {
-    int *count, *done, *listed, *list;
+    int *count, *next, *done, *listed, *list;
 };
 
 template <typename T>
@@ -803,22 +804,30 @@ digit_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
 // ---- pass 3: the listed tiles on the CUDA cores ------------------------------------
 
-template <typename T, bool AM, bool BC, bool CL>
-__global__ void __launch_bounds__(256)
-digit_fallback_kernel(DigitGemm<T> g, TileWords w, int nMt, int nNt)
+// A listed tile is cut into parts of G::BM x G::BN, handed out one by one: with a
+// fixed share per CTA the last round left half the SMs idle while others took two
+// parts (512 x 8192 x 512 FP64, all tiles listed, 1024 parts: 4.22 ms instead of
+// 3.66).
+template <typename T, bool AM, bool BC, bool CL, class G>
+__global__ void __launch_bounds__(G::NT)
+digit_fallback_kernel(const T *__restrict__ A, const T *__restrict__ B, T *__restrict__ C, DigitGemm<T> g, TileWords w, int nMt, int nNt)
 {
-    constexpr int FB = GemmTile<T>::BM, PER = BM / FB;
-    __shared__ __align__(16) T smem[gemm_tile_smem<T>()];
+    constexpr int FB = G::BM, PER = BM / FB;
+    __shared__ __align__(16) T smem[gemm_tile_smem<T, G>()];
+    __shared__ int part;
     tc::pdl_wait();
     tc::pdl_launch_dependents();
     const int n = *w.count * PER * PER;
-    for (int t = blockIdx.x; t < n; t += gridDim.x) {
+    for (int t = blockIdx.x; t < n;) {
         const int tile = w.list[t / (PER * PER)], sub = t % (PER * PER);
+        if (threadIdx.x == 0) part = int(gridDim.x) + atomicAdd(w.next, 1);
         int m_blk, n_blk;
         digit_tile(tile, nMt, nNt, g.tri, m_blk, n_blk);
         const int64_t i0 = int64_t(m_blk) * BM + (sub % PER) * FB, j0 = int64_t(n_blk) * BM + (sub / PER) * FB;
-        if (i0 >= g.M || j0 >= g.N || (g.tri && j0 > i0 + FB - 1)) continue;
-        gemm_tile<T, AM, BC, CL>(smem, i0, j0, g.M, g.N, g.K, g.A, g.lda, g.B, g.ldb, g.C, g.ldc, g.alpha, g.tri);
+        if (i0 < g.M && j0 < g.N && !(g.tri && j0 > i0 + FB - 1))
+            gemm_tile<T, AM, BC, CL, G>(smem, i0, j0, g.M, g.N, g.K, A, g.lda, B, g.ldb, C, g.ldc, g.alpha, g.tri);
+        __syncthreads();
+        t = part;
         __syncthreads();
     }
 }
@@ -836,20 +845,23 @@ inline int sm_count()
     return v > 0 ? v : 152;
 }
 
-template <typename T>
-int launch_fallback(const DigitGemm<T> &g, const TileWords &w, int nMt, int nNt, int ntiles, cudaStream_t s)
+// G: parts of the CUDA-core update's own tiles, or of a quarter of them where
+// those would not fill the SMs (a part of 64 x 64 x 64 FP64 takes its SM 69 us
+// whatever the others do).
+template <typename T, class G>
+int launch_fallback(const DigitGemm<T> &g, const TileWords &w, int nMt, int nNt, int64_t ntiles, cudaStream_t s)
 {
-    void (*k)(DigitGemm<T>, TileWords, int, int) = nullptr;
-    if (g.am && g.bc && g.cl) k = digit_fallback_kernel<T, true, true, true>;
-    else if (g.am && !g.bc && !g.cl) k = digit_fallback_kernel<T, true, false, false>;
-    else if (!g.am && g.bc && g.cl) k = digit_fallback_kernel<T, false, true, true>;
-    else if (!g.am && !g.bc && !g.cl) k = digit_fallback_kernel<T, false, false, false>;
-    else if (g.am && !g.bc && g.cl) k = digit_fallback_kernel<T, true, false, true>;    // P P^T
-    else if (!g.am && g.bc && !g.cl) k = digit_fallback_kernel<T, false, true, false>;  // the same, stored transposed
+    void (*k)(const T *, const T *, T *, DigitGemm<T>, TileWords, int, int) = nullptr;
+    if (g.am && g.bc && g.cl) k = digit_fallback_kernel<T, true, true, true, G>;
+    else if (g.am && !g.bc && !g.cl) k = digit_fallback_kernel<T, true, false, false, G>;
+    else if (!g.am && g.bc && g.cl) k = digit_fallback_kernel<T, false, true, true, G>;
+    else if (!g.am && !g.bc && !g.cl) k = digit_fallback_kernel<T, false, false, false, G>;
+    else if (g.am && !g.bc && g.cl) k = digit_fallback_kernel<T, true, false, true, G>;    // P P^T
+    else if (!g.am && g.bc && !g.cl) k = digit_fallback_kernel<T, false, true, false, G>;  // the same, stored transposed
     if (!k) return GB_STATUS_CUDA_ERROR;
-    constexpr int PER = BM / GemmTile<T>::BM;
-    const int grid = ntiles * PER * PER < 304 ? ntiles * PER * PER : 304;
-    return check(launch_pdl(k, dim3((unsigned)grid), dim3(256), 0, s, g, w, nMt, nNt));
+    constexpr int PER = BM / G::BM;
+    const int64_t parts = ntiles * PER * PER, most = int64_t(2) * sm_count() * (GemmTile<T>::NT / G::NT);
+    return check(launch_pdl(k, dim3((unsigned)(parts < most ? parts : most)), dim3(G::NT), 0, s, g.A, g.B, g.C, g, w, nMt, nNt));
 }
 
 template <typename T>
@@ -874,8 +886,8 @@ int digit_piece(const DigitGemm<T> &g, char *ws, size_t ws_bytes, int split, cud
     int *ex = g.tri ? ea : reinterpret_cast<int *>(take(4 * size_t(np)));
     int *cx = g.tri ? ca : reinterpret_cast<int *>(take(4 * size_t(np)));
     int *nx = g.tri ? na : reinterpret_cast<int *>(take(4 * size_t(np)));
-    int *words = reinterpret_cast<int *>(take(4 * (3 * size_t(nt) + 2)));
-    const TileWords w{words, words + 1, words + 1 + nt, words + 1 + 2 * nt};
+    int *words = reinterpret_cast<int *>(take(4 * (3 * size_t(nt) + 3)));
+    const TileWords w{words, words + 1, words + 2, words + 2 + nt, words + 2 + 2 * nt};
     if (off > ws_bytes || nt * split > 0x3fffffff) return GB_STATUS_CUDA_ERROR;
 
     CUtensorMap ta, tx;
@@ -912,7 +924,7 @@ int digit_piece(const DigitGemm<T> &g, char *ws, size_t ws_bytes, int split, cud
         attr[1].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 2;
-        GB_CUDA(cudaLaunchKernelEx(&cfg, digits_kernel<T>, sa, sx, ab, int(g.K), int(kp), words, int(2 * nt + 1),
+        GB_CUDA(cudaLaunchKernelEx(&cfg, digits_kernel<T>, sa, sx, ab, int(g.K), int(kp), words, int(2 * nt + 2),
                                    reinterpret_cast<ulonglong2 *>(Tg), split > 1 ? nt * (BM * BM / 2) : int64_t(0)));
     }
     {
@@ -920,13 +932,15 @@ int digit_piece(const DigitGemm<T> &g, char *ws, size_t ws_bytes, int split, cud
         GB_TRY(smem_attr_once(attr, digit_mma_kernel<T>, MMA_SMEM));
         constexpr double pairs = P * (P + 1) / 2;
         LaunchScope ls(KK_GEMM_TC, s, 2.0 * pairs * double(nt) * BM * BM * double(kp), 8.0 * double(nt) * BM * BM);
-        MmaArgs<T> a{g, Tg, ca, cx, na, nx, ea, ex, w, int(kp), nMt, nNt, int(nt), split, words + 3 * nt + 1};
+        MmaArgs<T> a{g, Tg, ca, cx, na, nx, ea, ex, w, int(kp), nMt, nNt, int(nt), split, words + 3 * nt + 2};
         const int64_t items = nt * split;
         GB_CUDA(launch_pdl(digit_mma_kernel<T>, dim3((unsigned)(items < sm_count() ? items : sm_count())), dim3(MMA_THREADS),
                            MMA_SMEM, s, ta, tx, a));
     }
     LaunchScope ls(KK_GEMM_SIMT, s, 0, 0);
-    return launch_fallback<T>(g, w, nMt, nNt, int(nt), s);
+    constexpr int PER = BM / GemmTile<T>::BM;
+    if (nt * PER * PER < 2 * sm_count()) return launch_fallback<T, GemmTileSmall<T>>(g, w, nMt, nNt, nt, s);
+    return launch_fallback<T, GemmTile<T>>(g, w, nMt, nNt, nt, s);
 }
 
 cudaMemPool_t digit_pool()

@@ -27,6 +27,14 @@ struct GemmTile<double> {  // DFMA: 64x64 tile, 4x4 per thread, 256 threads
     static constexpr int BM = 64, BN = 64, BK = 16, TM = 4, TN = 4, NT = 256;
 };
 
+// A quarter of that by a quarter of the threads, the same micro-tiles: for
+// updates of which the large tiles leave SMs idle.
+template <typename T>
+struct GemmTileSmall {
+    static constexpr int BM = GemmTile<T>::BM / 2, BN = GemmTile<T>::BN / 2, BK = GemmTile<T>::BK;
+    static constexpr int TM = GemmTile<T>::TM, TN = GemmTile<T>::TN, NT = GemmTile<T>::NT / 4;
+};
+
 template <typename T, int W>
 struct VecT;
 template <>
@@ -40,22 +48,22 @@ struct VecT<double, 2> {
 
 // AM: A-operand contiguous along M (Mv(i,k) = A(i,k), i.e. !mt).
 // BC: Bop contiguous along K, else along N.  CL: C contiguous along M, else
-// along N.  tri: only the entries on and below the diagonal of C.  smem: gemm_tile_smem<T>() elements, 16-byte aligned.
+// along N.  tri: only the entries on and below the diagonal of C.  smem: gemm_tile_smem<T, G>() elements, 16-byte aligned.
 // Every thread of the CTA takes part; shared memory is free on return only
 // after a barrier.
-template <typename T>
+template <typename T, class G = GemmTile<T>>
 constexpr int gemm_tile_smem()
 {
-    return 2 * GemmTile<T>::BK * (GemmTile<T>::BM + GemmTile<T>::BN + GemmTile<T>::TM);
+    return 2 * G::BK * (G::BM + G::BN + G::TM);
 }
 
-template <typename T, bool AM, bool BC, bool CL>
+template <typename T, bool AM, bool BC, bool CL, class G = GemmTile<T>>
 __device__ __forceinline__ void gemm_tile(T *smem, int64_t m0, int64_t n0, int64_t M, int64_t N, int64_t K,
                                           const T *__restrict__ A, int64_t lda, const T *__restrict__ B, int64_t ldb,
                                           T *__restrict__ C, int64_t ldc, T alpha, int tri)
 {
-    constexpr int BM = GemmTile<T>::BM, BN = GemmTile<T>::BN, BK = GemmTile<T>::BK;
-    constexpr int TM = GemmTile<T>::TM, TN = GemmTile<T>::TN;
+    constexpr int BM = G::BM, BN = G::BN, BK = G::BK;
+    constexpr int TM = G::TM, TN = G::TN;
     constexpr int NTX = BN / TN, NTY = BM / TM;
     constexpr int NT = NTX * NTY;
     constexpr int VW = TM / 2;  // vector width of one half micro-tile

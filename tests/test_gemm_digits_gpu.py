@@ -249,3 +249,27 @@ def test_digits_at_their_bounds(dtype, K):
         want = -np.longdouble(2 * a) * np.longdouble(2 * x) * K
         u = 2.0 ** (-53 if dtype == 0 else -24)
         assert np.all(np.abs(got - want) <= 1.01 * u * abs(want))
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+@pytest.mark.parametrize("M,N,K", [(1, 1, 512), (70, 300, 128), (130, 260, 512), (1000, 1100, 128), (1300, 2200, 130)])
+def test_all_tiles_listed(M, N, K, dtype):
+    """Half of A's columns zero, the other half meeting zeros of B: every tile is
+    left to the CUDA cores, in parts of a quarter of their tiles where there are
+    few and in whole ones, more parts than CTAs among them.  Componentwise K u,
+    as for the CUDA-core sum."""
+    A, B, C = _factors(dtype, M, N, K, seed=M + K)
+    A[:, ::2] = 0
+    B[1::4] = 0
+    got = _update(dtype, A, B, C, 0.5)
+    rows, cols = (np.unique(np.minimum(np.r_[0:5, n // 2, max(n - 70, 0):n], n - 1)) for n in (M, N))
+    i = np.ix_(rows, cols)
+    L = np.longdouble
+    want = L(0.5) * C[i] - A[rows].astype(L) @ B[:, cols].astype(L)
+    bound = np.abs(A[rows]).astype(L) @ np.abs(B[:, cols]).astype(L) + np.abs(C[i])
+    u = 2.0 ** (-53 if dtype == 0 else -24)
+    assert np.all(np.abs(got[i] - want) <= K * u * bound)
+    assert np.all(np.isfinite(got))
+    # and all of C: a probe against a product by another path
+    full = 0.5 * C.astype(np.float64) - A.astype(np.float64) @ B.astype(np.float64)
+    assert np.allclose(got, full, rtol=0, atol=(1e-11 if dtype == 0 else 1e-3))
