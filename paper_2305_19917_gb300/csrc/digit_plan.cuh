@@ -17,9 +17,12 @@ namespace digits {
 constexpr int BM = 128, BK = 64;  // tile of C, K of one load
 
 // Largest piece of one launch sequence: the digits of both factors and the
-// sums stay within the work space's cap, K within 16384 (the sums' weight W).
+// sums stay within the work space's cap, K within 16384, with eight digits (FP64)
+// 8192, where the rounding of the sums' last bits still leaves room for normally
+// distributed factors (gemm_digits.cu, "Accuracy").
 constexpr size_t kWsCap = size_t(2) << 30;
-constexpr int64_t kMaxK = 16384;
+template <int P>
+constexpr int64_t kMaxK = P == 8 ? 8192 : 16384;
 
 inline int64_t up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
@@ -38,13 +41,15 @@ GB_HD void share_range(int kt, int split, int sp, int &k0, int &k1)
 }
 
 // K is split over CTAs, down to 64 of it each, while the tiles alone leave SMs
-// idle: 9 tiles of K = 512 on 72 CTAs instead of 9.  At most `most` shares, and
-// none of them empty.
+// idle: 9 tiles of K = 512 on 72 CTAs instead of 9.  Beyond K = 2048 a share is at
+// least a whole chunk of 256: every share rounds the sums' last bits once.  At most
+// `most` shares, and none of them empty.
 inline int pick_split(int64_t ntiles, int64_t K, int64_t most = 152)
 {
     const int64_t kt = (K + BK - 1) / BK;
     int64_t s = 152 / ntiles;
-    if (s > kt) s = kt;
+    const int64_t least = K > 2048 ? 4 : 1;
+    if (s > kt / least) s = kt / least;
     if (s > most) s = most;
     if (s < 2) return 1;
     const int64_t per = (kt + s - 1) / s;
@@ -64,7 +69,7 @@ size_t piece_bytes(int64_t M, int64_t N, int64_t K, int tri, int split)
     const size_t mp = size_t(up(M, BM)), np = size_t(up(N, BM)), kp = size_t(up(K, BK));
     const size_t nt = size_t(digit_tiles(int64_t(mp / BM), int64_t(np / BM), tri));
     size_t b = 256 + 2 * P * mp * kp + (tri ? 0 : 2 * P * np * kp) + (split > 1 ? nt * BM * BM * 8 : 0);
-    b += 4 * 3 * (mp + np) + 4 * (3 * nt + 3) + 10 * 256;
+    b += 4 * 4 * (mp + np) + 4 * (3 * nt + 3) + 12 * 256;
     return b;
 }
 
@@ -72,7 +77,7 @@ template <int P>
 Piece plan_piece(int64_t M, int64_t N, int64_t K, int tri)
 {
     Piece p;
-    p.kc = K < kMaxK ? K : kMaxK;
+    p.kc = K < kMaxK<P> ? K : kMaxK<P>;
     p.mc = M;
     p.nc = N;
     // halve the longer of the two extents until the piece fits (of a triangle, K)

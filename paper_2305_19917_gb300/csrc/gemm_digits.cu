@@ -39,22 +39,24 @@
 // at 2^-54 (2^-25) of the partial sum.  That is relative to the largest entries,
 // not to each product: for a sum in which large entries of Aop meet only small
 // ones of Bop it would be worse.  Pass 1 therefore counts the entries of every
-// row and column within 2^-4 of its largest; where the counts of a row and a
-// column add up to more than 5/4 K (FP64 beyond K = 1024, where T's last bit
-// weighs more: 3/2 K), at least K/4 (K/2) products of the sum have both factors
-// within 2^-4 of their largest ones.  A tile with a row and a column for which
-// that cannot be said, with an infinity or a NaN, or with exponents near the ends
-// of the range, is listed for the last pass, which computes it with the
-// CUDA-core tile of gemm_tile.cuh: the operations of gemm_simt.cu.  So is a
-// tile whose bounded waits gave up.
+// row and column within 2^-4 (and 2^-2) of its largest; where the counts of a row
+// and a column add up to K + n, at least n products of the sum have both factors
+// so near their scales, and n has to outweigh what is left out (kLeftOut,
+// kLastBit).  A tile with a row and a column for which it does not, with an
+// infinity or a NaN, or with exponents near the ends of the range, is listed for
+// the last pass, which computes it with the CUDA-core tile of gemm_tile.cuh: the
+// operations of gemm_simt.cu.  So is a tile whose bounded waits gave up.
 //
 // Measured, rms error over u sum |a||x|, digits / CUDA-core sum: uniform times
 // normal entries 0.08 / 0.39 (FP64, K = 64), 0.016 / 0.38 (4096), 0.05 / 0.49 (FP32,
-// K = 128); at the edge of what the rule lets pass (a quarter of the products at
-// 2^-4 of the scales each, the other large entries against ones of 2^-30) 0.22 /
-// 0.61 (FP64, K = 64), 0.50 / 0.64 (1024), 0.20 / 0.31 (FP32, 128).  With a digit
-// less (seven and three: 28 and 6 pairs, 4.95 instead of 5.9 ms for 4096 x 8192 x
-// 4096 FP64, 1.49 instead of 2.14 FP32) and W at most 52 those were 17, 6.0 and 8.9.
+// K = 128).  At the edge of what the rule lets pass (n products at 2^-4 of the
+// scales each, the other large entries against ones of 2^-30) 0.10 / 0.40 (FP64, K =
+// 64, n = 32), 0.24 / 0.34 (1024, n = 512), 0.15 / 0.30 (FP32, 128, n = 64).  A rule of
+// 5/4 K counted entries let pass, with a digit less (28 and 6 pairs: 4.95 instead of
+// 5.9 ms for 4096 x 8192 x 4096 FP64, 1.49 instead of 2.14 FP32) and W at most 52,
+// factors with 17 / 0.6 and 8.9 / 0.3; one of 3/2 K beyond K = 1024 listed tiles of
+// exponential-kernel factors that the digits hold well (4096 x 4096 solve 33.8 ms,
+// now 6.6).
 #include <mutex>
 #include <type_traits>
 #include <cuda_bf16.h>
@@ -83,7 +85,19 @@ constexpr int DROWS = 32;                      // rows of one digits_kernel CTA
 constexpr int DTHREADS = 256;
 constexpr int kMaxCluster = 8;
 constexpr int kCntBad = -(1 << 28);            // a row the digits must not represent
-constexpr int kNear = 4;                       // "within 2^-4 of the largest"
+// The rule for what the digits may take ("Accuracy" above; digit_item): entries
+// within 2^-kNear (FP64 also: 2^-kNear2) of their row's largest are counted, and
+// the products of two such must number kLeftOut sqrt(K) + kLastBit times T's last
+// bit, in units of 2^-53 of the scales' product, times the root of how often it
+// is rounded.  By rms: what the digits leave out is 0.0005 sqrt(K) (FP32 0.0022) of
+// that unit, T's rounding 0.3 to 0.45 of its last bit; the CUDA-core sum's error 0.35
+// to 0.6 of sum |a||x|, of which a product of two counted entries has 2^-8.8 of the
+// scales' product (both within 2^-kNear2: 2^-4.8, one of them: 2^-6.8) if they are
+// spread over their binades.
+constexpr int kNear = 4, kNear2 = 2;
+template <typename T>
+constexpr float kLeftOut = sizeof(T) == 8 ? 0.8f : 3.0f;
+constexpr float kLastBit = 640.f;
 
 template <typename T>
 struct Fmt;
@@ -181,6 +195,7 @@ struct DigitSrc {
     __nv_bfloat16 *out;   // P planes of rp x kp, row-major
     int *e;               // exponent e' + 1 per row
     int *cnt;             // entries within 2^-kNear of the largest; kCntBad; >= 2K for a zero or padding row
+    int *cnt2;            // FP64: those within 2^-kNear2
     int *nrm;             // FP64: sum of (|d[0]| + 1)^2, above 2^16 times that of the squared entries over 2^(e' + 1)
 };
 
@@ -213,8 +228,6 @@ digits_kernel(DigitSrc<T> a, DigitSrc<T> x, int ablocks, int K, int kp, int *zer
 
     if (tid < DROWS) {
         key[tid] = 0;
-        num[tid] = 0;
-        sqs[tid] = 0;
     }
     tc::pdl_wait();
     tc::pdl_launch_dependents();
@@ -279,7 +292,7 @@ digits_kernel(DigitSrc<T> a, DigitSrc<T> x, int ablocks, int K, int kp, int *zer
     // digits, 8 consecutive k of one row per thread and tile
     const int row = tid >> 3, lk = (tid & 7) * 8;
     const int em = emx[row] >> 1;
-    int near = 0, sq = 0;
+    int near = 0, sq = 0;  // FP64: within 2^-kNear2 counted in the upper half of near
     const size_t plane = size_t(s.rp) * size_t(kp);
     // (backwards: the last tile is still in registers; the next one's loads go
     // out before the digits of this one are formed)
@@ -299,8 +312,12 @@ digits_kernel(DigitSrc<T> a, DigitSrc<T> x, int ablocks, int K, int kp, int *zer
             uint32_t d0[P], d1[P];
             const T a0 = tb[row][lk + u], a1 = tb[row][lk + u + 1];
             const int g0 = digits_of(a0, em, d0) + 1, g1 = digits_of(a1, em, d1) + 1;
-            if (sizeof(T) == 8) sq += g0 * g0 + g1 * g1;
-            near += (Fmt<T>::field(a0) + kNear >= em && nonzero(a0)) + (Fmt<T>::field(a1) + kNear >= em && nonzero(a1));
+            const int f0 = nonzero(a0) ? Fmt<T>::field(a0) - em : -kNear - 1, f1 = nonzero(a1) ? Fmt<T>::field(a1) - em : -kNear - 1;
+            near += (f0 >= -kNear) + (f1 >= -kNear);
+            if (sizeof(T) == 8) {
+                near += ((f0 >= -kNear2) + (f1 >= -kNear2)) << 16;
+                sq += g0 * g0 + g1 * g1;
+            }
 #pragma unroll
             for (int p = 0; p < P; p++) w[p][u >> 1] = pack_hi16(d0[p], d1[p]);
         }
@@ -326,11 +343,16 @@ digits_kernel(DigitSrc<T> a, DigitSrc<T> x, int ablocks, int K, int kp, int *zer
             if (sizeof(T) == 8) n2 += peer(&sqs[tid], q);
         }
         const int k2 = emx[tid], f = k2 >> 1, e = f - Fmt<T>::BIAS;
-        if (k2 == 0) c = 2 * K;                                         // a zero row: exact
+        int c2 = c >> 16;
+        c &= 0xFFFF;
+        if (k2 == 0) c = c2 = 2 * K;                                    // a zero row: exact
         else if (f == 0 || e > Fmt<T>::EMAX || e < -Fmt<T>::EMAX) c = kCntBad;  // infinities and NaN too
         s.cnt[r0 + tid] = c;
         s.e[r0 + tid] = k2 == 0 ? 0 : e + 2;
-        if (sizeof(T) == 8) s.nrm[r0 + tid] = n2;
+        if (sizeof(T) == 8) {
+            s.cnt2[r0 + tid] = c2;
+            s.nrm[r0 + tid] = n2;
+        }
     }
     cluster_sync();  // no CTA leaves while its shared memory may be read
 }
@@ -381,7 +403,7 @@ template <typename T>
 struct MmaArgs {
     DigitGemm<T> g;
     long long *Tg;      // split > 1: the tiles' sums (128 x 128, column-major), cleared by pass 1
-    const int *cnt_a, *cnt_x, *nrm_a, *nrm_x, *e_a, *e_x;
+    const int *cnt_a, *cnt_x, *cnt2_a, *cnt2_x, *nrm_a, *nrm_x, *e_a, *e_x;
     TileWords w;
     int kp, nMt, nNt, ntiles, split;
     int *status;
@@ -438,21 +460,33 @@ __device__ __forceinline__ Item digit_item(const MmaArgs<T> &a, int w, int lane)
     // (an empty share, of which the host makes none, runs no pass in any warp:
     // the other schedule's loops go over its chunks)
     it.thin = it.k0 < it.k1 && it.k1 - it.k0 <= Sched<T>::THIN_K;
-    const int4 ca = reinterpret_cast<const int4 *>(a.cnt_a + it.i0)[lane];
-    const int4 cx = reinterpret_cast<const int4 *>(a.cnt_x + it.j0)[lane];
-    const int ma = __reduce_min_sync(0xffffffffu, min(min(ca.x, ca.y), min(ca.z, ca.w)));
-    const int mx = __reduce_min_sync(0xffffffffu, min(min(cx.x, cx.y), min(cx.z, cx.w)));
+    // four rows (columns) a lane, everything loaded before anything is reduced
+    auto four = [&](const int *p, int at) { return reinterpret_cast<const int4 *>(p + at)[lane]; };
+    auto least = [](int4 x) { return __reduce_min_sync(0xffffffffu, min(min(x.x, x.y), min(x.z, x.w))); };
+    auto most = [](int4 x) { return __reduce_max_sync(0xffffffffu, max(max(x.x, x.y), max(x.z, x.w))); };
     const int K = int(a.g.K);
-    it.skip = ma < 0 || mx < 0 || ma + mx < K + (sizeof(T) == 8 && K > 1024 ? K / 2 : K / 4);
+    const float need = kLeftOut<T> * sqrtf(float(K));
+    const int4 va = four(a.cnt_a, it.i0), vx = four(a.cnt_x, it.j0);
     it.W = 40;  // FP32: every weight is an integer, |T| <= K 2^38
-    if (sizeof(T) == 8) {
+    bool skip;
+    if constexpr (sizeof(T) == 8) {
+        const int4 va2 = four(a.cnt2_a, it.i0), vx2 = four(a.cnt2_x, it.j0), wa = four(a.nrm_a, it.i0), wx = four(a.nrm_x, it.j0);
         // by the rows' and columns' 2-norms: |T| <= 2^(W - 16) sqrt(na nx) <= 2^62.95
-        const int4 va = reinterpret_cast<const int4 *>(a.nrm_a + it.i0)[lane];
-        const int4 vx = reinterpret_cast<const int4 *>(a.nrm_x + it.j0)[lane];
-        const int na = __reduce_max_sync(0xffffffffu, max(max(va.x, va.y), max(va.z, va.w)));
-        const int nx = __reduce_max_sync(0xffffffffu, max(max(vx.x, vx.y), max(vx.z, vx.w)));
-        it.W = min(62, int(78.95f - 0.5f * log2f(float(na) * float(nx))));
+        const float n2 = float(most(wa)) * float(most(wx));
+        it.W = __reduce_max_sync(0xffffffffu, min(62, int(78.95f - 0.5f * log2f(n2))));
+        // T's last bit: rounded once per chunk of every share
+        const int per = (a.kp / BK + a.split - 1) / a.split, rounds = a.split * ((per * BK + KC - 1) / KC);
+        const float last = kLastBit * __int_as_float((127 + 55 - it.W) << 23) * sqrtf(float(rounds));
+        const int ca = least(va), cx = least(vx), ca2 = least(va2), cx2 = least(vx2);
+        const float both = fmaxf(fmaxf(float(ca + cx - K), 4.f * float(max(ca2 + cx, ca + cx2) - K)), 16.f * float(ca2 + cx2 - K));
+        skip = ca < 0 || cx < 0 || float(ca + cx - K) < need || both < need + last;
+    } else {
+        const int ca = least(va), cx = least(vx);
+        skip = ca < 0 || cx < 0 || float(ca + cx - K) < need;
     }
+    // (the reductions say to the compiler that all lanes agree: the loops over an
+    // item keep their uniform registers, 1 % of the tensor time)
+    it.skip = __reduce_max_sync(0xffffffffu, int(skip)) != 0;
     return it;
 }
 
@@ -882,9 +916,10 @@ int digit_piece(const DigitGemm<T> &g, char *ws, size_t ws_bytes, int split, cud
     long long *Tg = reinterpret_cast<long long *>(take(split > 1 ? size_t(nt) * BM * BM * 8 : 0));
     // (128-row arrays of int4 reads: each starts on a 256-byte boundary)
     int *ea = reinterpret_cast<int *>(take(4 * size_t(mp))), *ca = reinterpret_cast<int *>(take(4 * size_t(mp)));
-    int *na = reinterpret_cast<int *>(take(4 * size_t(mp)));
+    int *ca2 = reinterpret_cast<int *>(take(4 * size_t(mp))), *na = reinterpret_cast<int *>(take(4 * size_t(mp)));
     int *ex = g.tri ? ea : reinterpret_cast<int *>(take(4 * size_t(np)));
     int *cx = g.tri ? ca : reinterpret_cast<int *>(take(4 * size_t(np)));
+    int *cx2 = g.tri ? ca2 : reinterpret_cast<int *>(take(4 * size_t(np)));
     int *nx = g.tri ? na : reinterpret_cast<int *>(take(4 * size_t(np)));
     int *words = reinterpret_cast<int *>(take(4 * (3 * size_t(nt) + 3)));
     const TileWords w{words, words + 1, words + 2, words + 2 + nt, words + 2 + 2 * nt};
@@ -905,8 +940,8 @@ int digit_piece(const DigitGemm<T> &g, char *ws, size_t ws_bytes, int split, cud
     {
         LaunchScope ls(KK_CONVERT, s, 0,
                        (sizeof(T) + 2.0 * P) * (double(g.M) + (g.tri ? 0.0 : double(g.N))) * double(g.K));
-        DigitSrc<T> sa{g.A, g.lda, g.am ? 0 : 1, int(g.M), int(mp), da, ea, ca, na};
-        DigitSrc<T> sx{g.B, g.ldb, g.bc ? 1 : 0, int(g.N), int(np), dx, ex, cx, nx};
+        DigitSrc<T> sa{g.A, g.lda, g.am ? 0 : 1, int(g.M), int(mp), da, ea, ca, ca2, na};
+        DigitSrc<T> sx{g.B, g.ldb, g.bc ? 1 : 0, int(g.N), int(np), dx, ex, cx, cx2, nx};
         const int ab = int(mp / DROWS), xb = g.tri ? 0 : int(np / DROWS);
         const int64_t ktiles = kp / BK;
         int cl = 1;
@@ -932,7 +967,7 @@ int digit_piece(const DigitGemm<T> &g, char *ws, size_t ws_bytes, int split, cud
         GB_TRY(smem_attr_once(attr, digit_mma_kernel<T>, MMA_SMEM));
         constexpr double pairs = P * (P + 1) / 2;
         LaunchScope ls(KK_GEMM_TC, s, 2.0 * pairs * double(nt) * BM * BM * double(kp), 8.0 * double(nt) * BM * BM);
-        MmaArgs<T> a{g, Tg, ca, cx, na, nx, ea, ex, w, int(kp), nMt, nNt, int(nt), split, words + 3 * nt + 2};
+        MmaArgs<T> a{g, Tg, ca, cx, ca2, cx2, na, nx, ea, ex, w, int(kp), nMt, nNt, int(nt), split, words + 3 * nt + 2};
         const int64_t items = nt * split;
         GB_CUDA(launch_pdl(digit_mma_kernel<T>, dim3((unsigned)(items < sm_count() ? items : sm_count())), dim3(MMA_THREADS),
                            MMA_SMEM, s, ta, tx, a));

@@ -157,58 +157,69 @@ def test_ragged_last_piece_of_k(M, N, K, dtype):
     assert np.all(err <= 2 * NORM[dtype] * norms * K / 4096 + 4 * u * (np.abs(want) + np.abs(C[:16])))
 
 
-def _edge(kind, dtype, M, N, K, r):
-    """Factors that the digits take, near the edge of the rule for it: entries of
-    2^-5 to 2^-4 of the scales, and one entry near the scale per row ("spike"); all
-    but the least number of them 2^-12 smaller, at opposite places ("count"); as
-    large as the scale, against ones of 2^-30 ("big")."""
-    def small(*n):
-        return r.choice([-1.0, 1.0], n) * r.uniform(1 / 16, 1 / 8, n)
+def _edge(kind, n, M, N, K, r):
+    """Factors of which n products have both entries 2^-5 to 2^-4 of the scales;
+    the other entries there meet ones 2^-12 smaller ("count": one entry per row is
+    near the scale), or they are as large as the scale and meet ones of 2^-30
+    ("big")."""
+    def small(*size):
+        return r.choice([-1.0, 1.0], size) * r.uniform(1 / 16, 1 / 8, size)
 
-    def large(*n):
-        return r.choice([-1.0, 1.0], n) * r.uniform(1, 2, n)
+    def large(*size):
+        return r.choice([-1.0, 1.0], size) * r.uniform(1, 1.99, size)
     A, B = small(M, K), small(K, N)
-    rest = K - (K * (6 if dtype == 0 and K > 1024 else 5) // 8 + 2)
-    if kind == "spike":
-        A[:, 3] = B[7, :] = 1.9
-    elif kind == "count":
+    rest = (K - n) // 2
+    if kind == "count":
         A[:, :rest] *= 2.0 ** -12
-        B[-rest:] *= 2.0 ** -12
+        B[K - rest:] *= 2.0 ** -12
         A[:, 0] = B[-1, :] = 1.9
     else:
-        A[:, :rest], A[:, -rest:] = large(M, rest), A[:, -rest:] * 2.0 ** -30
-        B[-rest:], B[:rest] = large(rest, N), B[:rest] * 2.0 ** -30
-    nt = np.float64 if dtype == 0 else np.float32
-    return A.astype(nt), B.astype(nt)
+        A[:, :rest], A[:, K - rest:] = large(M, rest), A[:, K - rest:] * 2.0 ** -30
+        B[K - rest:], B[:rest] = large(rest, N), B[:rest] * 2.0 ** -30
+    return A, B
 
 
-@pytest.mark.parametrize("dtype,K", [(0, 64), (0, 200), (0, 1000), (0, 2500), (1, 128), (1, 500), (1, 2500)])
-@pytest.mark.parametrize("kind", ["spike", "count", "big"])
+@pytest.mark.parametrize("dtype,K", [(0, 64), (0, 200), (0, 1000), (0, 2500), (0, 9000), (1, 128), (1, 500), (1, 2500)])
+@pytest.mark.parametrize("kind", ["count", "big", "normal", "uniform"])
 def test_error_below_the_cuda_core_sum(kind, dtype, K):
-    """The claim itself, on what the rule lets pass: the root mean square error
-    over a tile's entries is at most that of the CUDA-core sum of the same
-    factors (the path taken while a stream is being captured)."""
+    """The claim itself, on both sides of the rule's edge: the root mean square
+    error over a tile's entries is at most that of the CUDA-core sum of the same
+    factors (the path taken while a stream is being captured; the same bits where
+    the rule lists the tile).  Normal and uniform entries are the digits', and so
+    are factors of which half of the products have a counted pair and no other
+    entry is large."""
     import torch
     from paper_2305_19917_gb300 import api
     M = N = 130  # (FP32 takes digits from 16384 entries on)
-    A, B = _edge(kind, dtype, M, N, K, np.random.default_rng(K))
+    r = np.random.default_rng(K)
+    nt = np.float64 if dtype == 0 else np.float32
     td = torch.float64 if dtype == 0 else torch.float32
-    a, b = api.to_device_colmajor(A, td), api.to_device_colmajor(B, td)
-    got = _update(dtype, A, B, np.zeros((M, N), A.dtype), 1.0)
-    c = torch.zeros(N, M, dtype=td, device="cuda").t()
-    s, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
-    with torch.cuda.graph(graph, stream=s):
-        st = api.gb_gemm_update(dtype, M, N, K, a.data_ptr(), M, b.data_ptr(), K, c.data_ptr(), M, 1.0, s.cuda_stream)
-    assert st == 0
-    graph.replay()
-    torch.cuda.synchronize()
     L = np.longdouble
-    i, j = np.r_[0:20, 120:130], np.r_[0:10, 110:130]
-    want = -(A[i].astype(L) @ B[:, j].astype(L))
-    scale = np.abs(A[i]).astype(L) @ np.abs(B[:, j]).astype(L)
-    rms = [float(np.sqrt(np.mean(((x[np.ix_(i, j)] - want) / scale) ** 2))) for x in (got, c.cpu().numpy())]
-    assert not np.array_equal(got, c.cpu().numpy())  # the digits did take it
-    assert rms[0] <= rms[1], rms
+    i, j = np.r_[0:15, 120:130], np.r_[0:10, 115:130]
+    taken = []
+    for part in ((64, 16, 8, 4, 2) if kind in ("count", "big") else (1,)):
+        if kind in ("count", "big"):
+            A, B = _edge(kind, max(K // part, 2), M, N, K, r)
+        else:
+            A = r.standard_normal((M, K)) if kind == "normal" else r.uniform(-1, 1, (M, K))
+            B = r.standard_normal((K, N))
+        A, B = A.astype(nt), B.astype(nt)
+        a, b = api.to_device_colmajor(A, td), api.to_device_colmajor(B, td)
+        got = _update(dtype, A, B, np.zeros((M, N), nt), 1.0)
+        c = torch.zeros(N, M, dtype=td, device="cuda").t()
+        s, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            st = api.gb_gemm_update(dtype, M, N, K, a.data_ptr(), M, b.data_ptr(), K, c.data_ptr(), M, 1.0, s.cuda_stream)
+        assert st == 0
+        graph.replay()
+        torch.cuda.synchronize()
+        cuda = c.cpu().numpy()
+        want = -(A[i].astype(L) @ B[:, j].astype(L))
+        scale = np.abs(A[i]).astype(L) @ np.abs(B[:, j]).astype(L)
+        rms = [float(np.sqrt(np.mean(((x[np.ix_(i, j)] - want) / scale) ** 2))) for x in (got, cuda)]
+        assert rms[0] <= rms[1], (part, rms)
+        taken.append(not np.array_equal(got, cuda))
+    assert taken[-1] or kind == "big", taken
 
 
 def test_weights_of_the_int64_sums():
