@@ -52,6 +52,18 @@ int64_t ts_rows(int64_t ncols)
     return r;
 }
 
+// Whether a TS task of at most 64 rows goes to the diagonal kernel instead of the
+// panel kernel, whose blocks are 32 rows whatever the task's: FP64 16 rows 4.3 us
+// with any number of right-hand sides (panels 6.7 with 300, 12.8 with 1200, 21 with
+// 2400); 32 rows 9.3 (6.8, 8.7 with 600, 12.8, 21); 64 rows 27.5 (11, 25 with 1200, 42).
+// FP32 16 rows 2.5 us (2.9, 5.0 with 1200), 32 rows 5 (2.9, 4.9).
+template <typename T>
+bool diag_wanted(int64_t nr, int64_t ncols)
+{
+    if (sizeof(T) == 4) return nr <= 16;
+    return nr <= 16 || ncols > (nr <= 32 ? 608 : 1216);
+}
+
 // A larger TS task is itself solved: by the recursive model down to such
 // tasks, whose updates are wide enough for the digit gemm, or, for a plan
 // that asks for smaller blocks, blocked by them.
@@ -144,13 +156,8 @@ struct LaunchExec {
         if (nr <= ts_rows<T>(c.ncols)) {
             settle(b0, b0 + nr);
             if (status) return;
-            if constexpr (sizeof(T) == 8) {
-                if (c.ncols > 2432) {
-                    status = launch_diag_solve(c, b0, (int)nr, a);
-                    return;
-                }
-            }
-            status = launch_panel_solve(c, b0, (int)nr, a);
+            status = nr <= 64 && diag_wanted<T>(nr, c.ncols) ? launch_diag_solve(c, b0, (int)nr, a)
+                                                             : launch_panel_solve(c, b0, (int)nr, a);
             return;
         }
         expand_ts(*this, b0, nr, nb, a, c.forward);

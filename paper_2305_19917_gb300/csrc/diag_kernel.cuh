@@ -235,8 +235,11 @@ int launch_dir(const T *Msub, int64_t lda, T *Bsub, int64_t ldb, int nr, int64_t
                T alpha, int unit, cudaStream_t s)
 {
     if (nr <= 16) return launch_nb<T, 16, FWD, MT, LEFT>(Msub, lda, Bsub, ldb, nr, ncols, alpha, unit, s);
-    if (nr <= 32) return launch_nb<T, 32, FWD, MT, LEFT>(Msub, lda, Bsub, ldb, nr, ncols, alpha, unit, s);
-    return launch_nb<T, 64, FWD, MT, LEFT>(Msub, lda, Bsub, ldb, nr, ncols, alpha, unit, s);
+    if constexpr (sizeof(T) == 8) {
+        if (nr <= 32) return launch_nb<T, 32, FWD, MT, LEFT>(Msub, lda, Bsub, ldb, nr, ncols, alpha, unit, s);
+        return launch_nb<T, 64, FWD, MT, LEFT>(Msub, lda, Bsub, ldb, nr, ncols, alpha, unit, s);
+    }
+    return GB_STATUS_CUDA_ERROR;  // FP32: the driver asks for at most 16 rows
 }
 
 }  // namespace

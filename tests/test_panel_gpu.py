@@ -87,3 +87,15 @@ def test_nan_of_any_payload(where, cols):
         X[hit] = want[hit]
         # (a row with a NaN keeps its block from being scaled: rounding only)
         assert np.all(np.isfinite(X)) and np.all(np.abs(X - want) <= 1e-13 * np.abs(want).max())
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("k,cols", [(1, 700), (8, 1), (15, 2500), (16, 33), (17, 608), (17, 609), (32, 609), (32, 65), (33, 1216),
+                                    (33, 1217), (48, 2000), (64, 1300), (64, 5000)])
+def test_small_orders(k, cols, dtype):
+    """Orders of at most 64: the diagonal kernel and the panel kernel on both
+    sides of the lines between them."""
+    for i, form in enumerate(FORMS):
+        m, n = (k, cols) if form[0] == 0 else (cols, k)
+        A, B = inputs.make_problem(*form, m, n, seed=k + cols + i)
+        _check(form, m, n, dtype, A, B, ldpad=i % 2)
