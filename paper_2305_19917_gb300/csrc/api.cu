@@ -64,14 +64,21 @@ bool diag_wanted(int64_t nr, int64_t ncols)
     return nr <= 16 || ncols > (nr <= 32 ? 608 : 1216);
 }
 
-// A larger TS task is itself solved: by the recursive model down to such
-// tasks, whose updates are wide enough for the digit gemm, or, for a plan
-// that asks for smaller blocks, blocked by them.
+// FP64 right-hand sides from which updates on the CUDA cores (a stream that is
+// being captured: no work space for digits) go with 64-row blocks, one update
+// behind each, rather than with panels and the recursive model's small updates,
+// whose few tiles leave SMs idle: captured, 1500 x 1500 4.47 ms (5.11 with panels),
+// 700 x 2400 1.57 (2.09), 1024 x 3000 3.68 (4.18); 2048 x 1000 panels 5.08, blocks 6.5.
+constexpr int64_t kBlockedColumns = 1216;
+
+// A TS task larger than e.rows() is itself solved: by the recursive model down to
+// such tasks, whose updates are wide enough for the digit gemm, or, for a plan
+// that asks for smaller blocks or without digits, blocked.
 template <class E, typename T>
 void expand_ts(E &e, int64_t b0, int64_t nr, int64_t nb, T a, bool fwd)
 {
-    if (nb < 64) drive_blocked(e, b0, b0 + nr, nb, a, fwd);
-    else drive_recursive(e, b0, b0 + nr, 24, ts_rows<T>(e.columns()), a, fwd);
+    if (nb < 64 || e.blocked) drive_blocked(e, b0, b0 + nr, nb < nr ? nb : 64, a, fwd);
+    else drive_recursive(e, b0, b0 + nr, 24, e.rows(), a, fwd);
 }
 
 // Executor that finds the work space of a schedule's largest digit gemm.
@@ -79,12 +86,13 @@ template <typename T>
 struct DigitBytesExec {
     int64_t nb, ncols;
     bool forward;
+    bool blocked;
     size_t bytes = 0;
     bool ok() const { return true; }
-    int64_t columns() const { return ncols; }
+    int64_t rows() const { return ts_rows<T>(ncols); }
     void ts(int64_t b0, int64_t nr, T a)
     {
-        if (nr > ts_rows<T>(ncols)) expand_ts(*this, b0, nr, nb, a, forward);
+        if (nr > rows()) expand_ts(*this, b0, nr, nb, a, forward);
     }
     void gemm(int64_t, int64_t M, int64_t, int64_t K, T)
     {
@@ -118,16 +126,17 @@ struct LaunchExec {
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_tail = nullptr;
     int64_t pend_lo = 0, pend_hi = 0;  // rows written by tails not yet waited for
+    bool blocked = false;              // no digits, and wide (kBlockedColumns)
     size_t digit_bytes = 0;            // work space of the schedule's largest digit gemm (0: none)
-    DigitWorkspace dws;
-    LaunchExec(const Canon<T> &c_, int64_t nb_) : c(c_), nb(nb_), dws(c_.stream) {}
+    DigitWorkspace &dws;
+    LaunchExec(const Canon<T> &c_, int64_t nb_, DigitWorkspace &dws_) : c(c_), nb(nb_), dws(dws_) {}
     ~LaunchExec()
     {
         if (ev_fork) cudaEventDestroy(ev_fork);
         if (ev_tail) cudaEventDestroy(ev_tail);
     }
     bool ok() const { return status == 0; }
-    int64_t columns() const { return c.ncols; }
+    int64_t rows() const { return blocked ? 64 : ts_rows<T>(c.ncols); }
     int enable_lookahead()
     {
         GB_TRY(side_stream(&side));
@@ -153,7 +162,7 @@ struct LaunchExec {
     void ts(int64_t b0, int64_t nr, T a)
     {
         if (status) return;
-        if (nr <= ts_rows<T>(c.ncols)) {
+        if (nr <= rows()) {
             settle(b0, b0 + nr);
             if (status) return;
             status = nr <= 64 && diag_wanted<T>(nr, c.ncols) ? launch_diag_solve(c, b0, (int)nr, a)
@@ -245,15 +254,18 @@ int trsm_impl(int side, int uplo, int trans, int diag, int64_t m, int64_t n, T a
     c.stream = static_cast<cudaStream_t>(stream);
 
     if (alpha == T(0)) return launch_zero(c);
+    DigitWorkspace dws(c.stream);
+    const bool blocked = sizeof(T) == 8 && k > 64 && c.ncols > kBlockedColumns && !dws.usable();
     if (plan == nullptr || plan->driver == GB_DRIVER_AUTO)
-        p = choose_plan(sizeof(T) == 8 ? GB_DTYPE_F64 : GB_DTYPE_F32, side, uplo, trans, m, n);
-    LaunchExec<T> e(c, p.nb);
+        p = choose_plan(sizeof(T) == 8 ? GB_DTYPE_F64 : GB_DTYPE_F32, side, uplo, trans, m, n, blocked);
+    LaunchExec<T> e(c, p.nb, dws);
+    e.blocked = blocked;
     // lookahead where a split update can overlap the next diagonal block:
     // the blocked and recursive models on more than four blocks of rows
     if (g_lookahead.load() && p.driver != GB_DRIVER_ITERATIVE && k > 4 * p.nb)
         GB_TRY(e.enable_lookahead());
-    DigitBytesExec<T> db{p.nb, c.ncols, c.forward};
-    drive_plan(db, p.driver, k, p.nb, p.depth, alpha, c.forward);
+    DigitBytesExec<T> db{p.nb, c.ncols, c.forward, blocked};
+    if (!blocked) drive_plan(db, p.driver, k, p.nb, p.depth, alpha, c.forward);
     e.digit_bytes = db.bytes;
     drive_plan(e, p.driver, k, p.nb, p.depth, alpha, c.forward);
     if (e.status) {

@@ -1004,17 +1004,18 @@ cudaMemPool_t digit_pool()
 
 }  // namespace
 
-char *DigitWorkspace::get(size_t bytes)
+bool DigitWorkspace::usable()
 {
-    if (state_ < 0) return nullptr;
     if (state_ == 0) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(s_, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-            state_ = -1;
-            return nullptr;
-        }
-        state_ = 1;
+        state_ = cudaStreamIsCapturing(s_, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ? -1 : 1;
     }
+    return state_ > 0;
+}
+
+char *DigitWorkspace::get(size_t bytes)
+{
+    if (!usable()) return nullptr;
     if (size_ >= bytes) return p_;
     release();
     cudaMemPool_t pool = digit_pool();

@@ -50,6 +50,8 @@ class DigitWorkspace {
 public:
     explicit DigitWorkspace(cudaStream_t s) : s_(s) {}
     ~DigitWorkspace() { release(); }
+    // The stream is not being captured.
+    bool usable();
     char *get(size_t bytes);
     size_t size() const { return size_; }
     void release();

@@ -28,13 +28,14 @@ const int kNbs[6] = {16, 32, 64, 128, 256, 512};
 
 // One TS task up to the panel kernel's order (512 rows, FP32 1024), else
 // recursive halving to tasks of at least 512 rows, which are solved down to
-// the panel or diagonal kernel's rows inside (api.cu).
-gb_plan default_plan(int dtype, int64_t k)
+// the panel or diagonal kernel's rows inside (api.cu).  `blocked` (wide FP64
+// solves without digits): those tasks in blocks of 64 rows.
+gb_plan default_plan(int dtype, int64_t k, bool blocked = false)
 {
     gb_plan p;
     p.reserved = 0;
-    p.nb = 512;
-    p.driver = GB_DRIVER_RECURSIVE;
+    p.nb = blocked ? 64 : 512;
+    p.driver = blocked && k <= 512 ? GB_DRIVER_BLOCKED : GB_DRIVER_RECURSIVE;
     int d = 0;
     if (k > (dtype == GB_DTYPE_F32 ? 1024 : 512))
         while ((k >> (d + 1)) >= 512 && d < 8) d++;
@@ -111,7 +112,7 @@ static int model_choose(int dtype, int side, int uplo, int trans, int64_t m, int
     return 0;
 }
 
-gb_plan choose_plan(int dtype, int side, int uplo, int trans, int64_t m, int64_t n)
+gb_plan choose_plan(int dtype, int side, int uplo, int trans, int64_t m, int64_t n, bool blocked)
 {
     const int64_t k = side == GB_LEFT ? m : n;
     {
@@ -123,7 +124,7 @@ gb_plan choose_plan(int dtype, int side, int uplo, int trans, int64_t m, int64_t
             if (model_choose(dtype, side, uplo, trans, m, n, &p, nullptr) == 0) return p;
         }
     }
-    return default_plan(dtype, k);
+    return default_plan(dtype, k, blocked);
 }
 
 }  // namespace gb
