@@ -81,13 +81,16 @@ void expand_ts(E &e, int64_t b0, int64_t nr, int64_t nb, T a, bool fwd)
     else drive_recursive(e, b0, b0 + nr, 24, e.rows(), a, fwd);
 }
 
-// Executor that finds the work space of a schedule's largest digit gemm.
+// Executor that finds the work space of a schedule's largest digit gemm, and
+// whether an update is tall enough that lookahead would split it: any, or one
+// that goes to the CUDA cores although digits can be had.
 template <typename T>
 struct DigitBytesExec {
     int64_t nb, ncols;
     bool forward;
     bool blocked;
     size_t bytes = 0;
+    bool tall = false, tall_cuda = false;
     bool ok() const { return true; }
     int64_t rows() const { return ts_rows<T>(ncols); }
     void ts(int64_t b0, int64_t nr, T a)
@@ -96,7 +99,10 @@ struct DigitBytesExec {
     }
     void gemm(int64_t, int64_t M, int64_t, int64_t K, T)
     {
-        if (digit_gemm_wanted<T>(M, ncols, K, 0)) bytes = std::max(bytes, digit_gemm_bytes<T>(M, ncols, K, 0));
+        const bool digits = !blocked && digit_gemm_wanted<T>(M, ncols, K, 0);
+        if (digits) bytes = std::max(bytes, digit_gemm_bytes<T>(M, ncols, K, 0));
+        tall = tall || M > 2 * nb;
+        tall_cuda = tall_cuda || (!digits && M > 2 * nb);
     }
 };
 
@@ -260,13 +266,15 @@ int trsm_impl(int side, int uplo, int trans, int diag, int64_t m, int64_t n, T a
         p = choose_plan(sizeof(T) == 8 ? GB_DTYPE_F64 : GB_DTYPE_F32, side, uplo, trans, m, n, blocked);
     LaunchExec<T> e(c, p.nb, dws);
     e.blocked = blocked;
-    // lookahead where a split update can overlap the next diagonal block:
-    // the blocked and recursive models on more than four blocks of rows
-    if (g_lookahead.load() && p.driver != GB_DRIVER_ITERATIVE && k > 4 * p.nb)
-        GB_TRY(e.enable_lookahead());
     DigitBytesExec<T> db{p.nb, c.ncols, c.forward, blocked};
-    if (!blocked) drive_plan(db, p.driver, k, p.nb, p.depth, alpha, c.forward);
+    drive_plan(db, p.driver, k, p.nb, p.depth, alpha, c.forward);
     e.digit_bytes = db.bytes;
+    // lookahead where a split update can overlap the next diagonal block: the
+    // blocked and recursive models on more than four blocks of rows, with
+    // updates on the CUDA cores (digit gemms are not split)
+    if (g_lookahead.load() && p.driver != GB_DRIVER_ITERATIVE && k > 4 * p.nb &&
+        (db.tall_cuda || (db.tall && db.bytes && !dws.usable())))
+        GB_TRY(e.enable_lookahead());
     drive_plan(e, p.driver, k, p.nb, p.depth, alpha, c.forward);
     if (e.status) {
         e.join();  // leave no work of this call on the second stream unordered
