@@ -348,8 +348,9 @@ int gb_mixed_history(double *rho, int *levels, int cap);
  *  14 stream
  * A negative status -a names the argument a whose entry is invalid (or
  * whose array is NULL).  Problems of order (m for Left, n for Right) up to
- * 512 are solved in shared memory by the persistent kernel, in chunks of 16
- * (FP64) or 32 (FP32) right-hand sides, largest first; larger problems are
+ * 512 are solved in shared memory by the persistent kernel, in chunks of up
+ * to 16 (FP64: narrower in small batches) or 32 (FP32) right-hand sides,
+ * largest first; larger problems are
  * solved one after the other by the regular driver on the same stream.
  * Synchronous (returns after the solves completed).
  *
@@ -378,8 +379,10 @@ int gb_batched_plan_create(int dtype, int64_t count, const int8_t *side,
  * gb_batched_plan_create_tiled: as gb_batched_plan_create with the split of
  * the work as argument 14 (stream 15, plan_out 16): tile = 1 (chunks of
  * problems of order up to 128 are solved by a warp each, up to 256 by two, the
- * others by the four warps of a CTA) or 2 (up to 64, up to 128); 0 = 1.  Any other value returns -15; a NULL plan_out
- * -17.
+ * others by the four warps of a CTA; FP32: up to 64 and 128, or all by four,
+ * in batches that would leave SMs idle) or 2 (up to 64, up to 128); 0 = 1.
+ * Any other value returns -15; a NULL plan_out -17.  Results do not depend on
+ * the split.
  * gb_batched_plan_create is this with tile 1.
  * gb_batched_plan_tile(plan): the plan's tile (or -1 for NULL).
  *

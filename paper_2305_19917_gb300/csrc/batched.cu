@@ -2,18 +2,19 @@
 // TS" (Section IV, many right-hand sides) generalised to many independent
 // problems of different order and width.
 //
-// Work units are (instance, chunk of CW right-hand sides, 16 FP64 / 32 FP32); a
-// chunk of an order-k instance costs ~k^2 CW / 2 multiply-adds, so units are
-// sorted by cost (largest first) and handed out through a device-side work
-// queue (atomic tickets; no CTA waits on another).  A unit is solved by the
-// blocked model of Section V-C in left-looking order on 32-row blocks, X in
-// shared memory, by a team of warps: warp w of n owns the block rows w, w + n,
-// ..., each taking its updates from the solved blocks as these are published
-// (no barrier inside a unit).  The more warps share a unit, the more of their
-// time goes into waiting for its chain of blocks; but X has to stay in shared
-// memory.  So teams are as small as that allows: the four warps of a CTA for
-// orders above 256, two above 128, one below (tile 1; half these orders with
-// tile 2), the CTA's X space divided among its teams.  Instances of order above KMAX are solved by the regular driver.
+// Work units are (instance, chunk of right-hand sides), 32 wide in FP32, 16, 8, 4, 2
+// or 1 in FP64 (width_of); sorted by cost (largest first), the first ones go to
+// the teams by number, the others through a device-side work queue (atomic
+// tickets; no CTA waits on another).  A unit is solved by the blocked model of
+// Section V-C in left-looking order on 32-row blocks, X in shared memory, by a
+// team of warps: warp w of n owns the block rows w, w + n, ..., each taking its
+// updates from the solved blocks as these are published (no barrier inside a
+// unit).  The more warps share a unit, the more of their time goes into waiting
+// for its chain of blocks; but X has to stay in shared memory.  So teams are as
+// small as that allows: the four warps of a CTA for orders above 256, two above
+// 128, one below (half these orders with tile 2; FP32 batches that would leave SMs
+// idle take larger teams, team_order), the CTA's X space divided among its teams.  Instances of order above KMAX are solved by the
+// regular driver.
 //
 // A lane holds one right-hand side and its rows of the block in registers, so
 // that the 32 x 32 triangle is solved by multiply-adds on independent rows,
@@ -22,13 +23,16 @@
 // and the multiply-adds are the time, a block's triangle takes 18 instructions
 // per right-hand side instead of the 64 of a substitution with one row per
 // lane.  FP64: 16 right-hand sides times the two halves of the rows (odd and
-// even), Mv read from L1 / L2 as it is needed (two addresses per warp and load;
-// the loads hide behind the arithmetic).  FP32: 32 right-hand sides, tiles of
-// Mv through a ring of asynchronous copies, packed multiply-adds
-// (wide_tile.cuh); two CTAs of four warps fill an SM's shared memory, and the
-// latencies that eight warps leave open are the time.  Measured, 4096 uneven
-// instances (m log-uniform in [16, 512], n in [1, 256]): FP64 22.2 -> 16.6 ms
-// (the FP64 unit 89 % busy; 12.9 ms at its peak), FP32 1.80 -> 1.2-1.3 ms.
+// even), or fewer times more parts, Mv read from L1 / L2 as it is needed (the
+// loads hide behind the arithmetic, of narrow units behind each other).  FP32:
+// 32 right-hand sides, tiles of Mv through a ring of asynchronous copies, packed
+// multiply-adds (wide_tile.cuh); two CTAs of four warps fill an SM's shared
+// memory, and the latencies that eight warps leave open are the time.  Measured,
+// 4096 uneven instances (m log-uniform in [16, 512], n in [1, 256]): FP64 22.2 ->
+// 16.0 ms (12.9 at the unit's peak), FP32 1.80 -> 1.29 ms.  With units always 16 wide
+// small or narrow FP64 batches were up to 4.5 times slower than with one row per
+// lane, 8 warps a unit (644 instances of order <= 128 and <= 5 right-hand sides 363 us
+// against 81).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -221,12 +225,15 @@ __device__ __forceinline__ void solve_unit(const Unit<float> &u, const Team<floa
     __syncwarp();  // X, the ring and the inverses are free for the next unit
 }
 
-// FP64, in solution order (a backward problem by negative strides): lane l
-// holds rows 2q + h (h = l / 16) of the block for right-hand side l % 16.
+// FP64, in solution order (a backward problem by negative strides): G lanes share
+// a right-hand side, lane l holding rows G q + l / (32 / G) of the block for right-
+// hand side l % (32 / G).  So a unit's instructions are as many as its right-hand
+// sides are wide, 16, 8, 4 or 1 of them: G = 2, 4, 8, 32.
+template <int G>
 __device__ __forceinline__ void solve_unit(const Unit<double> &u, const Team<double> &tm)
 {
-    constexpr int CW = kChunk<double>, NQ = NBB / 2;
-    const int lane = threadIdx.x & 31, h = lane >> 4, col = lane & 15;
+    constexpr int CW = kChunk<double>, W = 32 / G, NQ = NBB / G;
+    const int lane = threadIdx.x & 31, h = lane / W, col = lane % W;
     const int k = u.k, nblk = (k + NBB - 1) / NBB;
     const bool mt = u.flags & 1, rev = u.flags & 2, unitd = u.flags & 4, left = u.flags & 8;
     int64_t sr = mt ? u.lda : 1, sc = mt ? 1 : u.lda, br = left ? 1 : u.ldb;
@@ -243,16 +250,21 @@ __device__ __forceinline__ void solve_unit(const Unit<double> &u, const Team<dou
     int known = 0;
     bool gave_up = false;
     for (int b = tm.wid; b < nblk; b += tm.nwu) {
-        const int r0 = b * NBB, nv = min(NBB, k - r0), nq = (nv + 1) / 2;
-        // entry (row 2q + h, column) of the block row; a row past the last one
-        // reads the row before it (its results are not used)
+        const int r0 = b * NBB, nv = min(NBB, k - r0), nq = (nv + G - 1) / G;
+        // entry (row G q + h, column) of the block row; a row past the last one
+        // reads the last one (its results are not used)
         const double *Ar = A + int64_t(r0 + h) * sr;
-        const int64_t last = (nv & 1) && h ? (nv - 1) : -1;  // 2q of the lane's row past the end
-        auto row = [&](const double *p, int q) { return p[(2 * q == last ? int64_t(2 * q - 1) : int64_t(2 * q)) * sr]; };
+        auto row = [&](const double *p, int q) { return p[int64_t(min(G * q, nv - 1 - h)) * sr]; };
+        if (G >= 8 && lane < nv) {
+            // a narrow unit is a chain of latencies: the triangle's lines on their way
+            const double *d = A + int64_t(r0) * (sr + sc) + lane * (mt ? sr : sc);
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(d));
+            if (nv > 16) asm volatile("prefetch.global.L1 [%0];" ::"l"(d + 16 * (mt ? sc : sr)));
+        }
         double t[NQ], acc[NQ];
 #pragma unroll
         for (int q = 0; q < NQ; q++) {
-            t[q] = (incol && 2 * q + h < nv) ? B[int64_t(r0 + 2 * q + h) * br] : 0.0;
+            t[q] = (incol && G * q + h < nv) ? B[int64_t(r0 + G * q + h) * br] : 0.0;
             acc[q] = 0.0;
         }
         const double inv = (!unitd && lane < nv) ? 1.0 / A[int64_t(r0 + lane) * (sr + sc)] : 1.0;
@@ -260,17 +272,37 @@ __device__ __forceinline__ void solve_unit(const Unit<double> &u, const Team<dou
             if (tm.nwu > 1) await_block(tm.solved, kb, known, gave_up);
             const double *x0 = tm.Xs + size_t(kb) * NBB * CW + col;
             const double *ac = Ar + int64_t(kb) * NBB * sc;
+            constexpr int U = G <= 4 ? 2 : 8;  // steps whose entries are loaded at once
             if (nv == NBB) {
-#pragma unroll 2
+#pragma unroll U
                 for (int kk = 0; kk < NBB; kk++) {
                     const double x = x0[kk * CW];
                     double a[NQ];
 #pragma unroll
-                    for (int q = 0; q < NQ; q++) a[q] = ac[int64_t(2 * q) * sr + kk * sc];
+                    for (int q = 0; q < NQ; q++) a[q] = ac[int64_t(G * q) * sr + kk * sc];
 #pragma unroll
                     for (int q = 0; q < NQ; q++) acc[q] = fma(a[q], x, acc[q]);
                 }
+            } else if (G >= 8 || nv > 24) {
+#pragma unroll 1
+                for (int k0 = 0; k0 < NBB; k0 += U) {
+                    double x[U], a[U][NQ];
+#pragma unroll
+                    for (int i = 0; i < U; i++) {
+                        x[i] = x0[(k0 + i) * CW];
+#pragma unroll
+                        for (int q = 0; q < NQ; q++) a[i][q] = row(ac + (k0 + i) * sc, q);
+                    }
+#pragma unroll
+                    for (int q = 0; q < NQ; q++)
+                        if (q < nq) {
+#pragma unroll
+                            for (int i = 0; i < U; i++) acc[q] = fma(a[i][q], x[i], acc[q]);
+                        }
+                }
             } else {
+                // few rows: their entries only
+#pragma unroll 1
                 for (int kk = 0; kk < NBB; kk++) {
                     const double x = x0[kk * CW];
                     const double *p = ac + kk * sc;
@@ -278,7 +310,7 @@ __device__ __forceinline__ void solve_unit(const Unit<double> &u, const Team<dou
                     for (int g = 0; g < NQ; g += 4) {
                         if (g >= nq) break;
 #pragma unroll
-                        for (int q = g; q < g + 4; q++)
+                        for (int q = g; q < (g + 4 < NQ ? g + 4 : NQ); q++)
                             if (q < nq) acc[q] = fma(row(p, q), x, acc[q]);
                     }
                 }
@@ -286,23 +318,39 @@ __device__ __forceinline__ void solve_unit(const Unit<double> &u, const Team<dou
         }
 #pragma unroll
         for (int q = 0; q < NQ; q++) t[q] -= acc[q];
-        // the triangle: x_k by the lanes of its row's half, the rows below it by all
+        // the triangle: x_k by the lanes of its row's group, the rows below it by all
         const double *ad = Ar + int64_t(r0) * sc;
+        auto step = [&](int kk, auto entry) {
+            const double v = t[kk / G] * __shfl_sync(0xffffffffu, inv, kk);
+            const double x = __shfl_sync(0xffffffffu, v, (kk % G) * W + col);
+            if (h == kk % G) t[kk / G] = x;
 #pragma unroll
-        for (int kk = 0; kk < NBB; kk++) {
-            if (kk < nv) {
-                const double v = t[kk >> 1] * __shfl_sync(0xffffffffu, inv, kk);
-                const double x = __shfl_sync(0xffffffffu, v, (kk & 1) * 16 + col);
-                if (h == (kk & 1)) t[kk >> 1] = x;
-                const double *p = ad + kk * sc;
+            for (int q = 0; q < NQ; q++) {
+                if (G * q + G - 1 <= kk || q >= nq) continue;
+                // this lane's row G q + h below kk
+                const bool below = G * q > kk || G * q + h > kk;
+                const double r = fma(-entry(kk, q, below), x, t[q]);
+                t[q] = below ? r : t[q];
+            }
+        };
+        if constexpr (G <= 4) {
 #pragma unroll
-                for (int q = 0; q < NQ; q++) {
-                    if (2 * q + 1 <= kk || q >= nq) continue;
-                    // rows 2q (h = 0) and 2q + 1 (h = 1), below kk
-                    const bool below = 2 * q > kk || h == 1;
-                    const double a = below ? row(p, q) : 0.0;
-                    const double r = fma(-a, x, t[q]);
-                    t[q] = below ? r : t[q];
+            for (int kk = 0; kk < NBB; kk++)
+                if (kk < nv) step(kk, [&](int kk, int q, bool below) { return below ? row(ad + kk * sc, q) : 0.0; });
+        } else {
+            // a step is short here: eight steps' entries are fetched at once
+            constexpr int KS = 8;
+#pragma unroll
+            for (int k0 = 0; k0 < NBB; k0 += KS) {
+                if (k0 < nv) {
+                    double a[KS][NQ];
+#pragma unroll
+                    for (int i = 0; i < KS; i++)
+#pragma unroll
+                        for (int q = 0; q < NQ; q++)
+                            a[i][q] = G * q + h > k0 + i && k0 + i < nv ? row(ad + (k0 + i) * sc, q) : 0.0;
+#pragma unroll
+                    for (int i = 0; i < KS; i++) step(k0 + i, [&](int kk, int q, bool) { return a[kk % KS][q]; });
                 }
             }
         }
@@ -314,13 +362,23 @@ __device__ __forceinline__ void solve_unit(const Unit<double> &u, const Team<dou
         }
         double *xb = tm.Xs + size_t(b) * NBB * CW + h * CW + col;
 #pragma unroll
-        for (int q = 0; q < NQ; q++) xb[2 * q * CW] = t[q];
+        for (int q = 0; q < NQ; q++) xb[G * q * CW] = t[q];
         publish_block(tm.solved, b);
         if (incol) {
 #pragma unroll
             for (int q = 0; q < NQ; q++)
-                if (2 * q + h < nv) B[int64_t(r0 + 2 * q + h) * br] = u.alpha * t[q];
+                if (G * q + h < nv) B[int64_t(r0 + G * q + h) * br] = u.alpha * t[q];
         }
+    }
+}
+__device__ __forceinline__ void solve_unit(const Unit<double> &u, const Team<double> &tm)
+{
+    switch (u.flags >> 4) {
+    case 0: solve_unit<2>(u, tm); break;
+    case 1: solve_unit<4>(u, tm); break;
+    case 2: solve_unit<8>(u, tm); break;
+    case 3: solve_unit<16>(u, tm); break;
+    default: solve_unit<32>(u, tm);
     }
 }
 
@@ -359,8 +417,8 @@ batched_kernel(const Unit<T> *__restrict__ units, Queues qs, unsigned *__restric
     for (int c = 0; c < 3; c++) {
         const int nwu = NW >> c, team = warp / nwu;
         const int lo = c == 0 ? 0 : (c == 1 ? qs.n4 : qs.n2), hi = c == 0 ? qs.n4 : (c == 1 ? qs.n2 : qs.n1);
+        if (lo == hi) continue;
         tm.nwu = nwu;
-        tm.wid = warp % nwu;
         tm.Xs = Xs + size_t(team) * (KMAX / NW) * nwu * kStride<T>;
         tm.solved = &solved[team];
         // a team's own barrier (the team of four: the CTA's)
@@ -370,17 +428,20 @@ batched_kernel(const Unit<T> *__restrict__ units, Queues qs, unsigned *__restric
             else __syncwarp();
         };
         __syncthreads();  // the other teams' X space is free
-        for (;;) {
-            team_sync();  // every warp of the team has left its last unit
-            if (tm.wid == 0 && lane == 0) {
-                cur[team] = lo + int(atomicAdd(&ticket[c], 1u));
-                solved[team] = 0;
-            }
+        // The first unit of every team by its number, the others by ticket; the
+        // CTAs in turn from class to class, so that few units meet no busy one.
+        const int grid = gridDim.x, nteams = grid << c;
+        for (int t = lo + team * grid + (int(blockIdx.x) + grid - lo % grid) % grid; t < hi; t = cur[team]) {
+            if (warp % nwu == 0 && lane == 0) solved[team] = 0;
             team_sync();
-            const int t = cur[team];
-            if (t >= hi) break;
             const Unit<T> u = units[t];
+            // (a warp is a sub-partition with its own FP64 unit, and the team's last
+            // warps own the longest rows: they take turns)
+            tm.wid = (warp + t + t / 152) % nwu;
             solve_unit(u, tm);
+            team_sync();  // every warp of the team has left the unit
+            if (warp % nwu == 0 && lane == 0) cur[team] = lo + nteams + int(atomicAdd(&ticket[c], 1u));
+            team_sync();
         }
     }
 }
@@ -413,12 +474,130 @@ struct BatchedPlan {
 
 namespace {
 
+// FP64 unit of order k, w right-hand sides wide: FP64 warp instructions, those of
+// its longest chain on a team of nt warps.
+double unit_slots(int64_t k, int64_t w)
+{
+    const double nb = double((k + NBB - 1) / NBB);
+    return nb * (nb - 1) / 2 * double(32 * w) + nb * double(48 + 15 * w);
+}
+double unit_chain(int64_t k, int64_t w, int nt)
+{
+    if (nt == 1) return unit_slots(k, w);
+    const int nb = int((k + NBB - 1) / NBB);
+    double load = 0;
+    for (int i = 0; i < nt; i++) {
+        double row = 0;
+        for (int b = i; b < nb; b += nt) row += double(b * 32 * w + 48 + 15 * w);
+        load = std::max(load, row);
+    }
+    return std::max(load, double(nb) * double(48 + 15 * w + (nb > 1 ? 32 * w : 0)));
+}
+// Width of the next unit of `rest` right-hand sides: the narrowest that holds
+// them, at most cap.
+int64_t width_of(int64_t rest, int64_t cap)
+{
+    int64_t w = 1;
+    while (w < rest && w < cap) w *= 2;
+    return w;
+}
+int sm_count()
+{
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+// FP64: the largest width of the batch's units.  Sixteen right-hand sides make
+// the fewest instructions per right-hand side, narrower units a shorter chain and
+// more of them: the width with the least of all instructions, spread over the
+// sub-partitions, and the longest unit's chain (as a 1.5-norm: most of either
+// hides behind the other; on 30 batches the widths so chosen were 1.6 % slower
+// than the best ones on average).  Measured (orders x right-hand sides): 1125 of
+// 169 x 200 6.5 ms (16 wide; 8.4 with four), 20 of 86 x 8 30 us (one wide; 92 with
+// 16), 595 of up to 312 x 174 1.12 ms (8; 1.39 with 16).
+int64_t unit_width(int64_t count, const int8_t *side, const int64_t *m, const int64_t *n, int one)
+{
+    const double parts = 4.0 * sm_count();
+    int64_t best = 16;
+    double least = 0;
+    double chains[KMAX / NBB + 1][17] = {};  // by blocks and width (a block's orders share a team size)
+    for (int64_t cap = 16; cap >= 1; cap /= 2) {
+        double all = 0, chain = 0;
+        for (int64_t i = 0; i < count; i++) {
+            const int64_t k = side[i] == GB_LEFT ? m[i] : n[i], ncols = side[i] == GB_LEFT ? n[i] : m[i];
+            if (k == 0 || ncols == 0 || k > KMAX) continue;
+            const int nt = k > 2 * one ? 4 : (k > one ? 2 : 1);
+            auto add = [&](int64_t w, double units) {
+                all += units * unit_slots(k, w);
+                double &c = chains[(k + NBB - 1) / NBB][w];
+                if (c == 0) c = unit_chain(k, w, nt);
+                chain = std::max(chain, c);
+            };
+            if (ncols / cap) add(cap, double(ncols / cap));
+            for (int64_t rest = ncols % cap; rest > 0;) {
+                const int64_t w = width_of(rest, cap);
+                add(w, 1);
+                rest -= std::min(rest, w);
+            }
+        }
+        const double t = std::pow(all / parts, 1.5) + std::pow(chain, 1.5);
+        if (cap == 16 || t < least) {
+            least = t;
+            best = cap;
+        }
+    }
+    return best;
+}
+// FP32: the order up to which a unit is one warp's, 128, 64 or none.  Larger
+// teams have shorter chains and idle warps (a unit of one warp: its tiles one after
+// the other; of a team: 0.8 of a tile's time per block, or its busiest warp's
+// tiles; two warps cost 1.3, four 1.7 times the work, eight warps of an SM take
+// 1.5 times as long each as one alone): the order with the least of both (2-norm).
+// 104 of up to 87 x 5 19.5 us (teams of four; 28.6 of one), 563 of up to 255 x 183
+// 408 us (one; 509).
+int team_order(int64_t count, const int8_t *side, const int64_t *m, const int64_t *n)
+{
+    const double warps = 8.0 * sm_count();
+    int best = KMAX / 4;
+    double least = 0;
+    for (int one : {KMAX / 4, KMAX / 8, 0}) {
+        double all = 0, chain = 0, chains[KMAX / NBB + 1] = {};
+        for (int64_t i = 0; i < count; i++) {
+            const int64_t k = side[i] == GB_LEFT ? m[i] : n[i], ncols = side[i] == GB_LEFT ? n[i] : m[i];
+            if (k == 0 || ncols == 0 || k > KMAX) continue;
+            const int nt = k > 2 * one ? 4 : (k > one ? 2 : 1), nb = int((k + NBB - 1) / NBB);
+            const double tiles = nb * (nb + 1) / 2;
+            double &c = chains[nb];
+            if (c == 0) {
+                double busiest = 0;
+                for (int w = 0; w < nt; w++) {
+                    double row = 0;
+                    for (int b = w; b < nb; b += nt) row += b + 1;
+                    busiest = std::max(busiest, row);
+                }
+                c = nt == 1 ? tiles : std::max(busiest, 0.8 * nb);
+            }
+            all += double((ncols + kChunk<float> - 1) / kChunk<float>) * tiles * (nt == 1 ? 1.0 : (nt == 2 ? 1.3 : 1.7));
+            chain = std::max(chain, c);
+        }
+        const double t = std::hypot(1.5 * all / warps, chain);
+        if (one == KMAX / 4 || t < least) {
+            least = t;
+            best = one;
+        }
+    }
+    return best;
+}
+
 template <typename T>
 void build_units(BatchedPlan &P, int64_t count, const int8_t *side, const int8_t *uplo, const int8_t *trans,
                  const int8_t *diag, const int64_t *m, const int64_t *n, const T *alpha, const void *const *A,
                  const int64_t *lda, void *const *B, const int64_t *ldb, std::vector<Unit<T>> &units)
 {
     constexpr int CW = kChunk<T>;
+    // orders up to which a unit is one warp's, two warps'
+    const int one = P.tile == 2 ? KMAX / 8 : (sizeof(T) == 8 ? KMAX / 4 : team_order(count, side, m, n)), two = 2 * one;
+    const int64_t cap = sizeof(T) == 8 ? unit_width(count, side, m, n, one) : CW;
     for (int64_t i = 0; i < count; i++) {
         if (m[i] == 0 || n[i] == 0) continue;
         const bool left = side[i] == GB_LEFT;
@@ -434,7 +613,13 @@ void build_units(BatchedPlan &P, int64_t count, const int8_t *side, const int8_t
         const bool mt = left ? (trans[i] == GB_TRANS) : (trans[i] == GB_NOTRANS);
         const bool fwd = (uplo[i] == GB_LOWER) != mt;
         const int flags = (mt ? 1 : 0) | (fwd ? 0 : 2) | (diag[i] == GB_UNIT ? 4 : 0) | (left ? 8 : 0);
-        for (int64_t c0 = 0; c0 < ncols; c0 += CW) {
+        int64_t w = CW;
+        for (int64_t c0 = 0; c0 < ncols; c0 += w) {
+            int g = 0;  // FP64: the unit is 16 / 2^g wide
+            if (sizeof(T) == 8) {
+                w = width_of(ncols - c0, cap);
+                while (16 >> g > w) g++;
+            }
             Unit<T> u;
             u.A = static_cast<const T *>(A[i]);
             T *b = static_cast<T *>(B[i]);
@@ -442,15 +627,14 @@ void build_units(BatchedPlan &P, int64_t count, const int8_t *side, const int8_t
             u.lda = lda[i];
             u.ldb = ldb[i];
             u.k = int(k);
-            u.cw = int(std::min<int64_t>(CW, ncols - c0));
-            u.flags = flags;
+            u.cw = int(std::min<int64_t>(w, ncols - c0));
+            u.flags = flags | g << 4;
             u.alpha = alpha[i];
             units.push_back(u);
         }
     }
     // by team size (warps per unit: X of a team of w warps is w KMAX / 4 rows),
     // largest first inside (longest-processing-time order for the queues)
-    const int one = P.tile == 2 ? KMAX / 8 : KMAX / 4, two = 2 * one;
     auto cls = [one, two](const Unit<T> &a) { return a.k > two ? 0 : (a.k > one ? 1 : 2); };
     std::stable_sort(units.begin(), units.end(), [&](const Unit<T> &a, const Unit<T> &b) {
         if (cls(a) != cls(b)) return cls(a) < cls(b);
@@ -478,9 +662,7 @@ int upload_and_capture(BatchedPlan &P, std::vector<Unit<T>> &units, cudaStream_t
     GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_kernel<T>, NT, batched_smem<T>()));
     if (per_sm < 1) per_sm = 1;
     int64_t g = int64_t(sms) * per_sm;
-    // (smaller teams share a CTA)
-    const int64_t need = P.queues.n4 + (P.queues.n2 - P.queues.n4 + 1) / 2 + (P.queues.n1 - P.queues.n2 + 3) / 4;
-    if (g > need) g = need;
+    if (g > P.nunits) g = P.nunits;
     P.grid = int(g);
     if (P.nunits == 0) return 0;
     // CUDA graph: [reset the queue counters, persistent kernel]
