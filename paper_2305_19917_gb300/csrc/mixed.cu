@@ -946,10 +946,9 @@ struct LowExec {
     int64_t leaf = 0;   // leaf order of the recursion (0 = the form's default)
     int status = 0;
     bool ok() const { return status == 0; }
-    void ts(int64_t b0, int64_t nr, float a)
+    void ts(int64_t b0, int64_t nr, float)
     {
         if (status) return;
-        (void)a;
         // a leaf (kLeaf rows by default), left-looking, in one launch: each
         // 128-row block takes its update from the solved blocks of the leaf
         // and its TS task
@@ -1107,6 +1106,12 @@ extern "C" int gb_mixed_workspace_release(void *stream)
     if (dev < 0 || dev >= 64) return GB_STATUS_CUDA_ERROR;
     gb::DeviceWorkspace &w = gb::g_ws[dev];
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (!w.base) {
+        // nothing of the mixed path to free: no error while `stream` is being
+        // captured, when the pool cannot be waited for
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone) return 0;
+    }
     GB_CUDA(cudaStreamSynchronize(s));
     gb::digit_pool_trim();
     if (!w.base) return 0;

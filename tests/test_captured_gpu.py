@@ -70,3 +70,22 @@ def test_captured_plan_and_lookahead(plan):
         api.gb_set_lookahead(old)
     assert np.array_equal(on, off)
     assert bwd_err(*form, 1.5, A, B, on) <= 10 * k * U64
+
+
+def test_release_while_capturing():
+    """With no work space of the mixed path kept there is nothing to free:
+    the call returns 0 and leaves the capture as it is."""
+    import torch
+    from paper_2305_19917_gb300 import api
+    A, B = inputs.make_problem(0, 0, 0, 0, 600, 100, seed=2)
+    a, b = api.to_device_colmajor(A, torch.float64), api.to_device_colmajor(B, torch.float64)
+    api.trsm(0, 0, 0, 0, 1.0, a, b)  # the digits' pool exists
+    assert api.gb_mixed_workspace_release(torch.cuda.current_stream().cuda_stream) == 0
+    x = torch.zeros(8, device="cuda")
+    s, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        x.add_(1.0)
+        assert api.gb_mixed_workspace_release(s.cuda_stream) == 0
+    graph.replay()
+    torch.cuda.synchronize()
+    assert bool(torch.all(x == 1.0))
