@@ -33,8 +33,8 @@ struct DigitGemm {
 // measurements stand at the definition).
 template <typename T>
 bool digit_gemm_wanted(int64_t M, int64_t N, int64_t K, int tri);
-// Work space of one update, at most kDigitWsCap + what a minimal pass needs
-// (larger updates are done in pieces).
+// Work space of one update, at most about kWsCap (digit_plan.cuh; larger updates
+// are done in pieces).
 template <typename T>
 size_t digit_gemm_bytes(int64_t M, int64_t N, int64_t K, int tri);
 // The update on stream s, with `ws` at least digit_gemm_bytes<T> long and

@@ -9,8 +9,8 @@ template <typename T>
 constexpr int kPanelRows = sizeof(T) == 8 ? 512 : 1024;
 
 // FP32: the right-hand sides from which a lane holds one of them (512 rows:
-// 2048 right-hand sides 93 us with eight per CTA, 115 with one per lane; 8192
-// 265 with sixteen per CTA, 138).
+// 2048 right-hand sides 93 us with eight per CTA, 115 with one per lane; 8192 265
+// with sixteen per CTA and 138, now 104).
 constexpr int64_t kWideColumns = 2432;
 
 // Solve Mv[r0:r0+nr, r0:r0+nr] X = alpha Bv[r0:r0+nr, :] in place, nr <=

@@ -4,7 +4,7 @@
 //
 // Used where the right-hand sides are few enough that the chain of 64-row
 // blocks (a diagonal kernel and an update launch each, on a handful of SMs)
-// is the time: a CTA takes only CW = 1..16 right-hand sides, so that 64 of
+// is the time: a CTA takes only CW = 1..8 right-hand sides, so that 64 of
 // them already occupy 64 SMs, and walks the whole block by itself, without a
 // launch or a grid-wide wait in between.
 //
