@@ -8,9 +8,12 @@
 // A block scale changes at every 128-wide K block, so partial products cannot
 // simply accumulate in tensor memory: each K block (one 128-byte swizzle row
 // of FP8, 4 MMAs of K = 32) goes to one of two TMEM accumulators, and the
-// four epilogue warps read it back, multiply by the block's two scales
+// eight epilogue warps read it back, multiply by the block's two scales
 // (exact) and add it to FP32 registers while the MMAs of the next block run
-// into the other accumulator.  Tile 128 x 128, 6-stage TMA ring.
+// into the other accumulator.  Tile 128 x 256 with a TMA ring of four stages, or
+// 128 x 128 with six (the rule stands at the launch).  That turn of MMAs and
+// drain is the limit, not a unit: 4096 x 4096 x 4096 109 us (1257 TFLOP/s), tensor
+// pipe 31 % active, L1 34 %, issue slots 31 %, L2 24 %.
 #include <cuda_fp8.h>
 #include "common.cuh"
 #include "tc_common.cuh"
@@ -209,6 +212,10 @@ int launch_tc_gemm_fp8(int64_t M, int64_t N, int64_t K, const void *A, int64_t l
         (reinterpret_cast<uintptr_t>(B) & 15))
         return GB_STATUS_CUDA_ERROR;
     const int64_t nM = (M + BM - 1) / BM;
+    // 256 columns read A half as often: the operands of 128 x 128 outputs take three
+    // quarters of the bytes.  Where such tiles are fewer than the SMs, 128.  With eight
+    // epilogue warps and the scales loaded ahead: the low-precision solves of a 16384 x
+    // 16384 solve 20.2 -> 13.7 ms.
     const bool wide = nM * ((N + 255) / 256) >= 152;
     const int bn = wide ? 256 : 128;
     CUtensorMap ta, tb;
